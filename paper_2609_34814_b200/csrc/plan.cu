@@ -317,51 +317,220 @@ __device__ __forceinline__ void gather_rows(const u64* __restrict__ bits, int n_
 }
 
 // Q factor of the thin QR of an m x 2 block: Gram-Schmidt with one re-orthogonalisation
-// pass; numerically dependent columns become zero.  Returns the column sums of Q.
-__device__ __forceinline__ double2 thin_qr2(const double2* zin, double2* xout, int m, double* scratch) {
+// pass; numerically dependent columns become zero.  Only the coefficients are computed here, in
+// two reductions (the kernel's serial part: one pass and one reduction per coefficient, five in
+// all, cost more than the products on short sequences); the entries follow from them one by one:
+//   q1 = z1 / n1,  x2 = ((z2 - d q1) - e q1) / n2   with  d = q1.z2,  e = q1.(z2 - d q1),
+//   n2^2 = |z2 - d q1|^2 - e^2   (e is a rounding error of the first projection, so nothing cancels)
+struct Qr2 {
+  double inv1, inv2, d, e;      // inv1 / inv2 = 0: that column is dropped
+  double2 colsum;
+  __device__ __forceinline__ double2 entry(double2 z) const {
+    const double q1 = z.x * inv1;
+    return make_double2(q1, ((z.y - d * q1) - e * q1) * inv2);
+  }
+};
+__device__ __forceinline__ Qr2 thin_qr2(const double2* z_in, int m, double* scratch) {
   const double tiny = 1e-30 * sqrt((double)m);
-  int tid = threadIdx.x;
-  double a[2] = {0, 0};
-  for (int i = tid; i < m; i += kPlanThreads) { double2 z = zin[i]; a[0] += z.x * z.x; a[1] += z.y * z.y; }
-  block_sum<2>(a, scratch);
-  double n1 = sqrt(a[0]), n2_before = sqrt(a[1]);
-  bool ok1 = n1 > tiny;
-  double d[1] = {0};
+  const int tid = threadIdx.x;
+  double a[3] = {0, 0, 0};
+  for (int i = tid; i < m; i += kPlanThreads) { const double2 z = z_in[i]; a[0] += z.x * z.x; a[1] += z.x * z.y; a[2] += z.y * z.y; }
+  block_sum<3>(a, scratch);
+  Qr2 r;
+  const double n1 = sqrt(a[0]), n2_before = sqrt(a[2]);
+  r.inv1 = n1 > tiny ? 1.0 / n1 : 0.0;
+  r.d = a[1] * r.inv1;
+  double s[4] = {0, 0, 0, 0};
   for (int i = tid; i < m; i += kPlanThreads) {
-    double2 z = zin[i];
-    double q1 = ok1 ? z.x / n1 : 0.0;
-    xout[i] = make_double2(q1, z.y);
-    d[0] += q1 * z.y;
+    const double2 z = z_in[i];
+    const double q1 = z.x * r.inv1, y = z.y - r.d * q1;
+    s[0] += q1 * y; s[1] += y * y; s[2] += q1; s[3] += y;
   }
-  block_sum<1>(d, scratch);
-  double e[1] = {0};
-  for (int i = tid; i < m; i += kPlanThreads) {
-    double2 x = xout[i];
-    x.y = x.y - d[0] * x.x;
-    xout[i] = x;
-    e[0] += x.x * x.y;
+  block_sum<4>(s, scratch);
+  r.e = s[0];
+  const double n2 = sqrt(fmax(s[1] - r.e * r.e, 0.0));
+  const bool ok2 = n2 > tiny && n2 > 1e-9 * n2_before;
+  r.inv2 = ok2 ? 1.0 / n2 : 0.0;
+  r.colsum = make_double2(s[2], (s[3] - r.e * s[2]) * r.inv2);
+  return r;
+}
+
+// ---- mask products on the integer matrix units
+// A product of a 0/1 mask with two columns of fp64 numbers is a contraction, and an exact one once
+// the numbers are fixed point: every entry becomes a 64-bit integer q = round(v * 2^e), q is cut
+// into eight signed 8-bit digits, and mask x digits accumulates in int32 without rounding, in any
+// order and with any split of the columns.  The digits of both columns are the 16 columns of the
+// B operand (two n8 tiles), 32 mask bits are the k of one mma.m16n8k32.  e is chosen from a bound on the entries, not from their maximum (which
+// would take one more exchange between the CTAs): the quantisation error is 2^-63 of that bound,
+// less than the rounding of the fp64 sums it replaces.
+// Set bits cost nothing here, a row costs the same at any density: the bit walk (gather_rows) takes
+// ~10 instructions per set bit with three quarters of the lanes idle.
+//
+// Operand layout (256 columns = four 64-bit words of a row per chunk): lane (g, t) = (lane / 4,
+// lane % 4) of a warp loads word 4*chunk + t of rows g and g + 8.  Step s of a chunk takes the bits
+// with index s modulo 8 of every 32-bit half: (half << (7 - s)) & 0x80808080 is four bytes, so the
+// k slots of that step are the columns 256*chunk + 64*t + 32*(low/high half) + s + 8*j, j = 0..3,
+// and one mask and one multiply expand four bits.  A set bit counts 128; the sums are divided at the
+// end.  The digits lie in shared memory in the order the fragments need, one 16-byte item per lane
+// and step: {column 0 low half, high half, column 1 low half, high half}; items are XORed with s so that
+// the stores of pack_digits meet no bank conflict.
+constexpr int kChunkCols = 256;
+constexpr int kUnitRows = 32;            // rows one warp multiplies at a time (two m16 tiles)
+
+__device__ __forceinline__ unsigned prmt(unsigned a, unsigned b, unsigned sel) { return __byte_perm(a, b, sel); }
+
+// bytes of four words transposed: out[i] = byte i of w0..w3
+__device__ __forceinline__ void transpose4(unsigned w0, unsigned w1, unsigned w2, unsigned w3, unsigned (&o)[4]) {
+  const unsigned a = prmt(w0, w1, 0x5140), b = prmt(w2, w3, 0x5140);   // {w0.0 w1.0 w0.1 w1.1}
+  const unsigned c = prmt(w0, w1, 0x7362), d = prmt(w2, w3, 0x7362);   // {w0.2 w1.2 w0.3 w1.3}
+  o[0] = prmt(a, b, 0x5410); o[1] = prmt(a, b, 0x7632);
+  o[2] = prmt(c, d, 0x5410); o[3] = prmt(c, d, 0x7632);
+}
+
+// digits of entry(k), k < n, into `items`; entry returns the two columns' values, `scale` = 2^e.
+// One thread packs eight entries of one column.
+template <class Entry>
+__device__ __forceinline__ void pack_digits(uint4* items, int n, double scale, Entry entry) {
+  const int total = (n + kChunkCols - 1) / kChunkCols * 64;            // (chunk, t, s, column)
+  for (int w = threadIdx.x; w < total; w += kPlanThreads) {
+    const int col = w & 1, s = (w >> 1) & 7, t = (w >> 4) & 3, chunk = w >> 6;
+    unsigned lo[8], hi[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int k = chunk * kChunkCols + t * 64 + s + 8 * j;           // j >= 4: the high half of the word
+      const double v = k < n ? entry(k, col) : 0.0;
+      // balanced digits: add 128 to each of the lower seven bytes, then take it off byte by byte
+      const u64 q = ((u64)__double2ll_rn(v * scale) + 0x0080808080808080ull) ^ 0x0080808080808080ull;
+      lo[j] = (unsigned)q; hi[j] = (unsigned)(q >> 32);
+    }
+    unsigned d0[4], d1[4];
+    uint2* base = reinterpret_cast<uint2*>(items + (size_t)(chunk * 8 + s) * 32);
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {                             // digits 0..3, 4..7
+      const unsigned* q = half ? hi : lo;
+      transpose4(q[0], q[1], q[2], q[3], d0);
+      transpose4(q[4], q[5], q[6], q[7], d1);
+#pragma unroll
+      for (int g = 0; g < 4; ++g) base[((((half * 4 + g) * 4 + t) ^ s) << 1) + col] = make_uint2(d0[g], d1[g]);
+    }
   }
-  block_sum<1>(e, scratch);
-  double f[1] = {0};
-  for (int i = tid; i < m; i += kPlanThreads) {
-    double2 x = xout[i];
-    x.y = x.y - e[0] * x.x;
-    xout[i] = x;
-    f[0] += x.y * x.y;
+}
+
+__device__ __forceinline__ void imma(int (&c)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3, unsigned b0, unsigned b1) {
+  asm volatile("mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+r"(c[0]), "+r"(c[1]), "+r"(c[2]), "+r"(c[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+// value of sum_k digit_sum[k] 256^k from two integers of four digits each (both below 2^53)
+__device__ __forceinline__ double join_digits(long long lo, long long hi) { return (double)hi * 4294967296.0 + (double)lo; }
+
+// dst[r] = (sum_{c : bit (r, c) set} q[c]) / scale - rowscale(r) * corr, the q from `items`.
+// A warp takes 32 rows and a share of the chunks; the CTAs of a cluster take the groups of 32 rows in
+// turn.  ksplit > 1: that many warps share the rows of a group (by columns) and meet in `part`
+// ([32 / ksplit groups][32 rows][16 digits] int32, zero on entry and on exit): integer sums,
+// so neither the split nor the cluster size shows in the result.
+__device__ __forceinline__ void multiply_rows(const u64* __restrict__ bits, int n_rows, int wpr, const uint4* items,
+                                              int* part, int ksplit, double inv_scale, double2* dst,
+                                              const int* __restrict__ cnt, double2 corr, int crank, int csize, bool peers) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
+  const int units = (n_rows + kUnitRows - 1) / kUnitRows, chunks = (wpr + 3) >> 2;
+  const int slots = kPlanWarps / ksplit, slot = warp / ksplit, kp = warp - slot * ksplit;
+  auto put = [&](int r, double x, double y) {
+    const double sc = cnt ? (double)cnt[r] : 1.0;
+    const double2 v = make_double2(x * inv_scale - sc * corr.x, y * inv_scale - sc * corr.y);
+    dst[r] = v;
+    if (peers)
+      for (int c = 0; c < csize; ++c)
+        if (c != crank) store_peer(dst + r, (unsigned)c, v);
+  };
+  for (int u0 = crank; u0 < units; u0 += csize * slots) {              // (the same trips for every warp)
+    const int u = u0 + slot * csize;
+    if (slot < slots && u < units) {
+      int acc[2][2][4];                                                // [m16 tile][column][fragment]
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+          for (int e = 0; e < 4; ++e) acc[i][c][e] = 0;
+      const int r0 = u * kUnitRows + g;
+      for (int ch = kp * chunks / ksplit; ch < (kp + 1) * chunks / ksplit; ++ch) {
+        u64 w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = r0 + i * 8, wi = ch * 4 + t;
+          w[i] = (r < n_rows && wi < wpr) ? bits[(size_t)r * wpr + wi] : 0ull;
+        }
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+          const uint4 b = items[(size_t)(ch * 8 + s) * 32 + (lane ^ s)];
+          unsigned a[4][2];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            a[i][0] = ((unsigned)w[i] * (128u >> s)) & 0x80808080u;
+            a[i][1] = ((unsigned)(w[i] >> 32) * (128u >> s)) & 0x80808080u;
+          }
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            imma(acc[i][0], a[2 * i][0], a[2 * i + 1][0], a[2 * i][1], a[2 * i + 1][1], b.x, b.y);
+            imma(acc[i][1], a[2 * i][0], a[2 * i + 1][0], a[2 * i][1], a[2 * i + 1][1], b.z, b.w);
+          }
+        }
+      }
+      // fragment: element 2*half + e of lane (g, t) is row g + 8*half, digit 2*t + e
+      if (ksplit == 1) {
+        double val[2][2][2];                                           // [tile][row half][column]
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int half = 0; half < 2; ++half)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+              long long v = (long long)(acc[i][c][2 * half] >> 7) + ((long long)(acc[i][c][2 * half + 1] >> 7) << 8);
+              v <<= (t & 1) * 16;
+              v += __shfl_xor_sync(0xffffffffu, v, 1);                 // lanes t = 0, 1: digits 0..3; t = 2, 3: digits 4..7
+              const long long o = __shfl_xor_sync(0xffffffffu, v, 2);
+              val[i][half][c] = t < 2 ? join_digits(v, o) : join_digits(o, v);
+            }
+        // lane t of a quad stores row g + 8t of the group
+        const double x = t == 0 ? val[0][0][0] : t == 1 ? val[0][1][0] : t == 2 ? val[1][0][0] : val[1][1][0];
+        const double y = t == 0 ? val[0][0][1] : t == 1 ? val[0][1][1] : t == 2 ? val[1][0][1] : val[1][1][1];
+        const int r = r0 + t * 8;
+        if (r < n_rows) put(r, x, y);
+      } else {
+        int* pp = part + slot * (kUnitRows * 16);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              atomicAdd(&pp[(i * 16 + g + 8 * (e >> 1)) * 16 + c * 8 + 2 * t + (e & 1)], acc[i][c][e] >> 7);
+      }
+    }
+    if (ksplit > 1) {
+      __syncthreads();
+      for (int i = threadIdx.x; i < slots * kUnitRows; i += kPlanThreads) {
+        const int uu = u0 + (i / kUnitRows) * csize, r = uu * kUnitRows + i % kUnitRows;
+        if (uu < units && r < n_rows) {
+          int4* pr = reinterpret_cast<int4*>(part + i * 16);
+          double v[2];
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            const int4 l = pr[2 * c], h = pr[2 * c + 1];
+            v[c] = join_digits((long long)l.x + ((long long)l.y << 8) + ((long long)l.z << 16) + ((long long)l.w << 24),
+                               (long long)h.x + ((long long)h.y << 8) + ((long long)h.z << 16) + ((long long)h.w << 24));
+          }
+          put(r, v[0], v[1]);
+        }
+        int4* pz = reinterpret_cast<int4*>(part + i * 16);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) pz[c] = make_int4(0, 0, 0, 0);
+      }
+      __syncthreads();
+    }
   }
-  block_sum<1>(f, scratch);
-  double n2 = sqrt(f[0]);
-  bool ok2 = n2 > tiny && n2 > 1e-9 * n2_before;
-  double s[2] = {0, 0};
-  for (int i = tid; i < m; i += kPlanThreads) {
-    double2 x = xout[i];
-    x.y = ok2 ? x.y / n2 : 0.0;
-    xout[i] = x;
-    s[0] += x.x;
-    s[1] += x.y;
-  }
-  block_sum<2>(s, scratch);
-  return make_double2(s[0], s[1]);
 }
 
 __device__ __forceinline__ u64 splitmix64(u64 x) {
@@ -402,6 +571,11 @@ struct PlanParams {
   int m_b, n_b, wq, wk, wave, iters, mode, n_pow2, state_in_smem;
   int ring_cut;         // open the angular ring at its largest gap instead of at -pi
   int csize;            // CTAs per head (thread-block cluster size)
+  int mma;              // mask products on the integer matrix units (else: walk over the set bits)
+  int alias_yz;         // Y and Z share one buffer (two barriers more per iteration)
+  int ksplit_y, ksplit_z, part_ints;
+  unsigned off_items, off_part;     // bytes from the start of shared memory
+  double y_scale;       // power of two: |y| y_scale < 2^62
   u64 seed;
   long long kv_bytes, l2_bytes, min_nnz;
   int fit_num, fit_den, min_ppm, loc_num, loc_den;
@@ -493,7 +667,14 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
     double2* X = p.state_in_smem ? reinterpret_cast<double2*>(region)
                                  : p.ws_state + (size_t)h * (2 * (size_t)m_b + n_b);
     double2* Z = X + m_b;
-    double2* Y = Z + m_b;
+    double2* Y = p.alias_yz ? Z : Z + m_b;
+    uint4* items = reinterpret_cast<uint4*>(smem + p.off_items);
+    int* part = reinterpret_cast<int*>(smem + p.off_part);
+    const double y_scale = p.y_scale, x_scale = 4611686018427387904.0;     // 2^62: |x| <= 1
+    const bool peers = csize > 1 && p.state_in_smem;
+    auto sync_head = [&]() { if (csize > 1) cluster_sync_all(); else __syncthreads(); };
+    if (p.mma)
+      for (int i = tid; i < p.part_ints; i += kPlanThreads) part[i] = 0;
     const double inv_m = 1.0 / (double)m_b;
     // ---- start block (counter-based) and its orthonormalisation (Algorithm 1, step 3)
     const u64 hk = (u64)h * 0x9E3779B97F4A7C15ull;
@@ -503,19 +684,35 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
       Z[i] = make_double2(2.0 * u0 - 1.0, 2.0 * u1 - 1.0);
     }
     __syncthreads();
-    double2 colsum = thin_qr2(Z, X, m_b, scratch);
     // ---- T sweeps + one more for the Rayleigh-Ritz step
     for (int it = 0; it <= p.iters; ++it) {
+      const Qr2 qr = thin_qr2(Z, m_b, scratch);
       // Y = M^T X - c (1^T X)/m
-      gather_rows(Mt, n_b, p.wk, X, Y, cnt, make_double2(colsum.x * inv_m, colsum.y * inv_m), crank, csize, csize > 1);
-      if (csize > 1) cluster_sync_all(); else __syncthreads();
+      const double2 corr_y = make_double2(qr.colsum.x * inv_m, qr.colsum.y * inv_m);
+      if (!p.mma || (it == p.iters && lead))                     // (the digits are taken from Z directly)
+        for (int i = tid; i < m_b; i += kPlanThreads) X[i] = qr.entry(Z[i]);
+      if (p.mma) {
+        pack_digits(items, m_b, x_scale, [&](int k, int col) { const double2 x = qr.entry(Z[k]); return col ? x.y : x.x; });
+        if (p.alias_yz) sync_head(); else __syncthreads();
+        multiply_rows(Mt, n_b, p.wk, items, part, p.ksplit_y, 1.0 / x_scale, Y, cnt, corr_y, crank, csize, peers);
+      } else {
+        __syncthreads();
+        gather_rows(Mt, n_b, p.wk, X, Y, cnt, corr_y, crank, csize, peers);
+      }
+      sync_head();
       double cy[2] = {0, 0};
       for (int j = tid; j < n_b; j += kPlanThreads) { double2 y = Y[j]; double c = (double)cnt[j]; cy[0] += c * y.x; cy[1] += c * y.y; }
+      if (p.mma) pack_digits(items, n_b, y_scale, [&](int k, int col) { return col ? Y[k].y : Y[k].x; });
       block_sum<2>(cy, scratch);
       // Z = M Y - 1 (c^T Y)/m
-      gather_rows(M, m_b, p.wq, Y, Z, nullptr, make_double2(cy[0] * inv_m, cy[1] * inv_m), crank, csize, csize > 1);
-      if (csize > 1) cluster_sync_all(); else __syncthreads();
-      if (it < p.iters) colsum = thin_qr2(Z, X, m_b, scratch);
+      const double2 corr_z = make_double2(cy[0] * inv_m, cy[1] * inv_m);
+      if (p.mma) {
+        if (p.alias_yz) sync_head();                             // (else: the barriers of the sum above)
+        multiply_rows(M, m_b, p.wq, items, part, p.ksplit_z, 1.0 / y_scale, Z, nullptr, corr_z, crank, csize, peers);
+      } else {
+        gather_rows(M, m_b, p.wq, Y, Z, nullptr, corr_z, crank, csize, peers);
+      }
+      sync_head();
     }
     // the rest (ordering, angles, sorts, outputs) is cheap: the lead CTA finishes alone.  No CTA
     // touches another's shared memory after the last exchange above.
@@ -647,6 +844,10 @@ struct PlanLayout {
   size_t off_bitmap, off_mt, off_nnz, off_cnt, off_state, total;
   int wq, wk, n_pow2, state_in_smem;
   size_t smem;
+  // shared memory of the matrix-unit form: does it fit, the iteration blocks behind `region`, the
+  // digits behind them (the partial sums of the column split come last, launch_shape() adds them)
+  int mma, alias_yz;
+  size_t off_items, items_end;
 };
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -675,6 +876,17 @@ waveal_status plan_layout(const waveal_plan_desc* d, PlanLayout* L) {
   size_t sort_bytes = (size_t)p2 * 12, state_bytes = (2 * m + n) * 16;
   L->state_in_smem = 2048 + (state_bytes > sort_bytes ? state_bytes : sort_bytes) <= kSmemMax;
   L->smem = 2048 + (L->state_in_smem ? (state_bytes > sort_bytes ? state_bytes : sort_bytes) : sort_bytes);
+  // The matrix-unit form also keeps the digits of one block, 16 bytes an entry.  On square masks it
+  // fits up to ~3,580 blocks as it is, up to ~4,730 with Y and Z in one buffer and up to 14,336
+  // with the blocks in the workspace; between and beyond (the state fits shared memory, the digits
+  // do not) the set bits are walked.
+  const size_t big = m > n ? m : n, items = (big + kChunkCols - 1) / kChunkCols * kChunkCols * 16;
+  L->mma = 1; L->alias_yz = 0;
+  size_t before = L->state_in_smem ? state_bytes : 0;
+  if (2048 + before + items > kSmemMax && L->state_in_smem) { L->alias_yz = 1; before = (m + big) * 16; }
+  if (2048 + before + items > kSmemMax) { L->mma = 0; L->alias_yz = 0; }
+  L->off_items = 2048 + before;
+  L->items_end = L->off_items + items;
   size_t o = 0;
   L->off_bitmap = o; o = align_up(o + H * m * L->wq * 8, 256);
   L->off_mt = o;     o = align_up(o + H * n * L->wk * 8, 256);
@@ -682,6 +894,37 @@ waveal_status plan_layout(const waveal_plan_desc* d, PlanLayout* L) {
   L->off_cnt = o;    o = align_up(o + H * n * 4, 256);
   L->off_state = o;  o = align_up(o + (L->state_in_smem ? 0 : H * (2 * m + n) * 16), 256);
   L->total = o;
+  return WAVEAL_OK;
+}
+
+// Largest cluster (up to 16 CTAs, at most `limit`) of which the device holds `heads` at once; one
+// CTA per SM is assumed (the shared memory of the larger shapes).  How many clusters of a size fit
+// depends on the device alone (its SMs come in groups of unequal size), so it is asked once.
+waveal_status cluster_size(int dev, int heads, int limit, int* out) {
+  constexpr int kMaxCluster = 16, kMaxDev = 64;
+  static std::mutex mu;
+  static int fit[kMaxDev][kMaxCluster + 1] = {};      // clusters of a size the device holds, + 1; 0: not asked
+  if (dev < 0 || dev >= kMaxDev) { *out = 1; return WAVEAL_OK; }
+  std::lock_guard<std::mutex> lock(mu);
+  for (int c = limit < kMaxCluster ? limit : kMaxCluster; c > 1; --c) {
+    if (!fit[dev][c]) {
+      WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_plan_head, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+      WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_plan_head, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3((unsigned)c);
+      cfg.blockDim = dim3(kPlanThreads);
+      cfg.dynamicSmemBytes = kSmemMax;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = (unsigned)c; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+      cfg.attrs = attr; cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, k_plan_head, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+      fit[dev][c] = n + 1;
+    }
+    if (fit[dev][c] - 1 >= heads) { *out = c; return WAVEAL_OK; }
+  }
+  *out = 1;
   return WAVEAL_OK;
 }
 
@@ -699,7 +942,6 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
   WAVEAL_CUDA_OK(cudaGetDevice(&dev));
   WAVEAL_CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   WAVEAL_CUDA_OK(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev));
-  WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_plan_head, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem));
   unsigned char* w = static_cast<unsigned char*>(ws);
   int launches = 0;
   const size_t H = d->heads, m = d->n_q_blocks, n = d->n_kv_blocks;
@@ -729,21 +971,45 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
   p.ws_state = reinterpret_cast<double2*>(w + L.off_state);
   p.row_order = out->row_order; p.row_nnz = out->row_nnz; p.flags = out->skip_flags; p.col_count = out->col_count;
   p.order1 = out->order1; p.embedding = out->embedding; p.stats = reinterpret_cast<long long*>(out->stats);
-  // CTAs per head: as many as fit the device at once (clusters of 1 to 4 CTAs on neighbouring
-  // SMs), when the iteration blocks live in shared memory and some head may be planned at all
+  // CTAs per head: the largest cluster of which the device holds one per head at once, when some
+  // head may be planned at all, and no more than there are groups of 32 rows
   int csize = 1;
-  if (L.state_in_smem && p.mode != WAVEAL_FORCE_NATURAL && p.mode != WAVEAL_STAGE2_ONLY) {
-    csize = (int)(sms / (long long)H);
-    csize = csize < 1 ? 1 : csize > 4 ? 4 : csize;
+  if ((L.mma || L.state_in_smem) && p.mode != WAVEAL_FORCE_NATURAL && p.mode != WAVEAL_STAGE2_ONLY) {
+    const int groups = (int)(((m > n ? m : n) + kUnitRows - 1) / kUnitRows);
+    s = cluster_size(dev, (int)H, L.mma ? groups : (groups < 4 ? groups : 4), &csize);
+    if (s != WAVEAL_OK) return s;
   }
+  p.mma = L.mma; p.alias_yz = L.alias_yz; p.off_items = (unsigned)L.off_items;
+  p.ksplit_y = p.ksplit_z = 1;
+  int y_exp = 0;
+  while ((1ll << (2 * y_exp)) < (long long)m) ++y_exp;       // 2^y_exp >= sqrt(m) >= 2 |y| (rows of X have norm 1 by column)
+  p.y_scale = ldexp(1.0, 63 - y_exp);
+  size_t smem = L.smem;
+  if (L.mma) {
+    // fewer groups of rows than warps: the warps of a CTA share the columns of a group
+    auto split = [&](size_t rows, int words) {
+      const int groups = (int)((rows + kUnitRows - 1) / kUnitRows), per_cta = (groups + csize - 1) / csize;
+      const int chunks = (words + 3) / 4, ks = per_cta >= kPlanWarps ? 1 : kPlanWarps / per_cta;
+      return ks < chunks ? ks : chunks;
+    };
+    p.ksplit_y = split(n, L.wk); p.ksplit_z = split(m, L.wq);
+    int ints = 0;
+    for (int ks : {p.ksplit_y, p.ksplit_z})
+      if (ks > 1) ints = ints > kPlanWarps / ks * kUnitRows * 16 ? ints : kPlanWarps / ks * kUnitRows * 16;
+    if (L.items_end + (size_t)ints * 4 > kSmemMax) { p.ksplit_y = p.ksplit_z = 1; ints = 0; }
+    p.off_part = (unsigned)L.items_end; p.part_ints = ints;
+    const size_t need = L.items_end + (size_t)ints * 4;
+    smem = smem > need ? smem : need;
+  }
+  WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_plan_head, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   p.csize = csize;
   if (csize == 1) {
-    k_plan_head<<<(unsigned)H, kPlanThreads, L.smem, st>>>(p);
+    k_plan_head<<<(unsigned)H, kPlanThreads, smem, st>>>(p);
   } else {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(H * csize));
     cfg.blockDim = dim3(kPlanThreads);
-    cfg.dynamicSmemBytes = L.smem;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
