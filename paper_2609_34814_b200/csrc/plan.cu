@@ -55,20 +55,71 @@ __global__ void k_csr_to_bitmap(const int* __restrict__ row_ptr, const int* __re
   }
 }
 
-// Mt[h][j][i>>6] bit (i&63) = M[h][i][j>>6] bit (j&63); one 64x64-bit tile per CTA of 64 threads
-__global__ void k_transpose_bits(const u64* __restrict__ M, u64* __restrict__ Mt, int m_b, int n_b,
-                                 int wq, int wk) {
-  __shared__ u64 tile[64];
-  int h = blockIdx.z, jw = blockIdx.x, iw = blockIdx.y, t = threadIdx.x;
-  int i = iw * 64 + t;
-  tile[t] = i < m_b ? M[((size_t)h * m_b + i) * wq + jw] : 0ull;
+// 32 x 32 bits transposed inside a warp (lane = row on entry, column on exit): five exchanges
+__device__ __forceinline__ unsigned transpose_bits32(unsigned x, int lane) {
+#pragma unroll
+  for (int j = 16; j; j >>= 1) {
+    const unsigned m = j == 16 ? 0x0000FFFFu : j == 8 ? 0x00FF00FFu : j == 4 ? 0x0F0F0F0Fu : j == 2 ? 0x33333333u : 0x55555555u;
+    const unsigned y = __shfl_xor_sync(0xffffffffu, x, j);
+    x = (lane & j) ? ((x & ~m) | ((y & ~m) >> j)) : ((x & m) | ((y & m) << j));
+  }
+  return x;
+}
+
+// One pass over the mask: its bit transpose Mt[h][j][i>>6] bit (i&63) = M[h][i][j>>6] bit (j&63), the
+// column counts c = M^T 1 and the row counts n_i = M 1.
+// blockIdx.x < wq: a strip of 64 columns and all rows; a warp transposes 32 rows at a time by
+// shuffles, the strip is collected in shared memory ([64 columns][stride] words of 32 rows) so that
+// the columns leave in whole lines and are counted on the way.  The other blocks count 32 rows each.
+// Counting here spreads what every CTA of a head's cluster used to do for itself over the whole chip.
+constexpr int kStatThreads = 256, kStatRows = 32;
+__global__ void __launch_bounds__(kStatThreads) k_mask_stats(const u64* __restrict__ M, u64* __restrict__ Mt, int m_b, int n_b,
+                                                             int wq, int wk, int* __restrict__ nnz, int* __restrict__ cnt,
+                                                             int* __restrict__ nnz_out, int* __restrict__ cnt_out) {
+  extern __shared__ unsigned strip[];
+  const int h = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const u64* Mh = M + (size_t)h * m_b * wq;
+  if ((int)blockIdx.x >= wq) {
+    constexpr int kPer = kStatRows * 32 / kStatThreads;             // rows of a warp, loads of all in flight
+    const int r0 = ((int)blockIdx.x - wq) * kStatRows + warp * kPer;
+    int c[kPer] = {};
+    for (int w = lane; w < wq; w += 32)
+#pragma unroll
+      for (int k = 0; k < kPer; ++k)
+        if (r0 + k < m_b) c[k] += __popcll(Mh[(size_t)(r0 + k) * wq + w]);
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      c[k] = __reduce_add_sync(0xffffffffu, c[k]);
+      if (lane == 0 && r0 + k < m_b) {
+        nnz[(size_t)h * m_b + r0 + k] = c[k];
+        if (nnz_out) nnz_out[(size_t)h * m_b + r0 + k] = c[k];
+      }
+    }
+    return;
+  }
+  const int jw = blockIdx.x, stride = 2 * wk + 1;                   // odd: the columns of a warp hit all banks
+  for (int i0 = warp * 32; i0 < wk * 64; i0 += kStatThreads) {
+    const int i = i0 + lane;
+    const u64 w = i < m_b ? Mh[(size_t)i * wq + jw] : 0ull;
+    strip[lane * stride + (i0 >> 5)] = transpose_bits32((unsigned)w, lane);
+    strip[(lane + 32) * stride + (i0 >> 5)] = transpose_bits32((unsigned)(w >> 32), lane);
+  }
   __syncthreads();
-  int j = jw * 64 + t;
-  if (j < n_b) {
-    u64 o = 0;
-#pragma unroll 8
-    for (int r = 0; r < 64; ++r) o |= ((tile[r] >> t) & 1ull) << r;
-    Mt[((size_t)h * n_b + j) * wk + iw] = o;
+  for (int c0 = warp; c0 < 64; c0 += kStatThreads / 32) {
+    const int j = jw * 64 + c0;
+    if (j >= n_b) break;
+    const unsigned* col = strip + c0 * stride;
+    int c = 0;
+    for (int w = lane; w < wk; w += 32) {
+      const u64 v = (u64)col[2 * w] | (u64)col[2 * w + 1] << 32;
+      Mt[((size_t)h * n_b + j) * wk + w] = v;
+      c += __popcll(v);
+    }
+    c = __reduce_add_sync(0xffffffffu, c);
+    if (lane == 0) {
+      cnt[(size_t)h * n_b + j] = c;
+      if (cnt_out) cnt_out[(size_t)h * n_b + j] = c;
+    }
   }
 }
 
@@ -176,16 +227,24 @@ __device__ __forceinline__ void block_sum(double (&v)[N], double* scratch) {
   __syncthreads();
 }
 
-__device__ __forceinline__ long long block_sum_i64(long long v, long long* scratch) {
-  int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// the same for whole numbers
+template <int N>
+__device__ __forceinline__ void block_sum_i64(long long (&v)[N], long long* scratch) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if (lane == 0) scratch[warp] = v;
+  for (int k = 0; k < N; ++k) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    if (lane == 0) scratch[warp * N + k] = v[k];
+  }
   __syncthreads();
-  long long s = 0;
-  for (int w = 0; w < kPlanWarps; ++w) s += scratch[w];
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    v[k] = scratch[lane * N + k];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+  }
   __syncthreads();
-  return s;
 }
 
 __device__ __forceinline__ double block_max(double v, double* scratch) {
@@ -219,14 +278,20 @@ __device__ __forceinline__ unsigned cluster_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync_all() { cluster_arrive(); cluster_wait(); }
 // store a double2 at the same shared-memory offset of CTA `rank` of this cluster
 __device__ __forceinline__ void store_peer(const double2* local_ptr, unsigned rank, double2 v) {
   unsigned laddr = (unsigned)__cvta_generic_to_shared(local_ptr), raddr;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(raddr) : "r"(laddr), "r"(rank));
   asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(raddr), "d"(v.x), "d"(v.y) : "memory");
+}
+
+__device__ __forceinline__ void store_peer(const long long* local_ptr, unsigned rank, long long v) {
+  unsigned laddr = (unsigned)__cvta_generic_to_shared(local_ptr), raddr;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(raddr) : "r"(laddr), "r"(rank));
+  asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(raddr), "l"(v) : "memory");
 }
 
 // number of set bits with index in [lo, hi) of a bit row
@@ -579,10 +644,10 @@ struct PlanParams {
   u64 seed;
   long long kv_bytes, l2_bytes, min_nnz;
   int fit_num, fit_den, min_ppm, loc_num, loc_den;
-  int* ws_nnz;          // [heads][m_b]
-  int* ws_cnt;          // [heads][n_b]
+  const int* ws_nnz;    // [heads][m_b], k_mask_stats
+  const int* ws_cnt;    // [heads][n_b], k_mask_stats
   double2* ws_state;    // [heads][2*m_b + n_b] when the blocks do not fit shared memory
-  int* row_order; int* row_nnz; unsigned char* flags; int* col_count; int* order1;
+  int* row_order; unsigned char* flags; int* order1;
   double* embedding; long long* stats;
 };
 
@@ -595,48 +660,51 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
   // same order, so the copies stay identical bit for bit; only the two mask sweeps of an
   // iteration, where the time goes, are split, and their results exchanged.
   const int csize = p.csize, crank = csize > 1 ? (int)cluster_rank() : 0;
-  const int h = blockIdx.x / csize, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int h = blockIdx.x / csize, tid = threadIdx.x;
   const bool lead = crank == 0;         // writes the outputs
   const int m_b = p.m_b, n_b = p.n_b;
   const u64* M = p.M + (size_t)h * m_b * p.wq;
   const u64* Mt = p.Mt + (size_t)h * n_b * p.wk;
-  int* nnz = p.ws_nnz + (size_t)h * m_b;
-  int* cnt = p.ws_cnt + (size_t)h * n_b;
+  const int* nnz = p.ws_nnz + (size_t)h * m_b;
+  const int* cnt = p.ws_cnt + (size_t)h * n_b;
   int* order_out = p.row_order + (size_t)h * m_b;
   int* order1_out = p.order1 ? p.order1 + (size_t)h * m_b : nullptr;
 
-  // ---- n_i = sum_j M_ij and c = M^T 1 (Section 2.2; Algorithm 1 step 1)
-  long long my_nnz = 0;
-  for (int r = warp; r < m_b; r += kPlanWarps) {
-    int c = 0;
-    for (int w = lane; w < p.wq; w += 32) c += __popcll(M[(size_t)r * p.wq + w]);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if (lane == 0) { nnz[r] = c; if (p.row_nnz && lead) p.row_nnz[(size_t)h * m_b + r] = c; my_nnz += c; }
-  }
-  for (int j = warp; j < n_b; j += kPlanWarps) {
-    int c = 0;
-    for (int w = lane; w < p.wk; w += 32) c += __popcll(Mt[(size_t)j * p.wk + w]);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if (lane == 0) { cnt[j] = c; if (p.col_count && lead) p.col_count[(size_t)h * n_b + j] = c; }
-  }
-  // ---- guard statistics over natural-order waves (Section 4.5)
+  // (a CTA writes into another's shared memory only once that one runs: waited for below)
+  if (csize > 1) cluster_arrive();
+  // ---- guard statistics over natural-order waves (Section 4.5): selected pairs, and for the overlap
+  // sum_l (w_l - 1) t_l from the row counts, sum_l,j c_lj (c_lj - 1) / 2 from the columns (split
+  // over the CTAs of the cluster; whole numbers, so the split does not show)
   const int n_waves = (m_b + p.wave - 1) / p.wave;
-  long long ov = 0, pair2 = 0;
-  for (int j = warp; j < n_b; j += kPlanWarps) {
-    const u64* col = Mt + (size_t)j * p.wk;
-    for (int l = lane; l < n_waves; l += 32) {
-      int lo = l * p.wave, hi = min(lo + p.wave, m_b);
-      long long c = popcount_range(col, lo, hi);
-      ov += c * (c - 1) / 2;
-      pair2 += (long long)(hi - lo - 1) * c;
+  long long sums[3] = {0, 0, 0};
+  for (int i = tid; i < m_b; i += kPlanThreads) {
+    const int lo = i / p.wave * p.wave;
+    const long long c = nnz[i];
+    sums[0] += c;
+    sums[1] += (long long)(min(p.wave, m_b - lo) - 1) * c;
+  }
+  {
+    const int dj = kPlanThreads / n_waves, dl = kPlanThreads % n_waves;
+    int col = tid / n_waves, l = tid % n_waves;           // (column of this CTA's share, wave), 1024 such pairs a step
+    for (long long j = (long long)col * csize + crank; j < n_b; j = (long long)col * csize + crank) {
+      const int lo = l * p.wave;
+      const long long c = popcount_range(Mt + (size_t)j * p.wk, lo, min(lo + p.wave, m_b));
+      sums[2] += c * (c - 1) / 2;
+      col += dj; l += dl;
+      if (l >= n_waves) { l -= n_waves; ++col; }
     }
   }
-  long long* iscratch = reinterpret_cast<long long*>(scratch);
-  long long nnz_total = block_sum_i64(my_nnz, iscratch);
-  ov = block_sum_i64(ov, iscratch);
-  pair2 = block_sum_i64(pair2, iscratch);
+  block_sum_i64<3>(sums, reinterpret_cast<long long*>(scratch));
+  const long long nnz_total = sums[0], pair2 = sums[1];
+  long long ov = sums[2];
+  if (csize > 1) {
+    cluster_wait();
+    long long* slots = reinterpret_cast<long long*>(smem + 1280);      // one per CTA of the cluster
+    if (tid < csize) store_peer(slots + crank, (unsigned)tid, ov);
+    cluster_sync_all();
+    ov = 0;
+    for (int c = 0; c < csize; ++c) ov += slots[c];
+  }
   unsigned flags = 0;
   if (p.kv_bytes > 0 && p.l2_bytes > 0 && p.kv_bytes * p.fit_den <= p.l2_bytes * p.fit_num)
     flags |= WAVEAL_FLAG_SHORT_SEQ;
@@ -658,7 +726,6 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
     }
     return;
   }
-  __syncthreads();   // nnz[] / cnt[] (global) written by this CTA are visible to all its threads
 
   u64* keys = reinterpret_cast<u64*>(region);
   int* vals = reinterpret_cast<int*>(region + (size_t)p.n_pow2 * 8);
@@ -955,7 +1022,12 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
     M = bm;
   }
   u64* Mt = reinterpret_cast<u64*>(w + L.off_mt);
-  k_transpose_bits<<<dim3(L.wq, L.wk, (unsigned)H), 64, 0, st>>>(M, Mt, (int)m, (int)n, L.wq, L.wk);
+  int* nnz = reinterpret_cast<int*>(w + L.off_nnz);
+  int* cnt = reinterpret_cast<int*>(w + L.off_cnt);
+  const size_t strip_bytes = (size_t)64 * (2 * L.wk + 1) * 4;       // at most 131,328: wk <= kMaxSort / 64
+  WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_mask_stats, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)strip_bytes));
+  k_mask_stats<<<dim3(L.wq + (unsigned)((m + kStatRows - 1) / kStatRows), (unsigned)H), kStatThreads, strip_bytes, st>>>(
+      M, Mt, (int)m, (int)n, L.wq, L.wk, nnz, cnt, out->row_nnz, out->col_count);
   ++launches;
   PlanParams p{};
   p.M = M; p.Mt = Mt; p.m_b = (int)m; p.n_b = (int)n; p.wq = L.wq; p.wk = L.wk;
@@ -966,15 +1038,15 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
   p.kv_bytes = d->kv_bytes_per_head; p.l2_bytes = d->l2_bytes > 0 ? d->l2_bytes : (long long)l2;
   p.min_nnz = d->min_nnz; p.fit_num = d->l2_fit_num; p.fit_den = d->l2_fit_den; p.min_ppm = d->min_density_ppm;
   p.loc_num = d->local_num; p.loc_den = d->local_den;
-  p.ws_nnz = reinterpret_cast<int*>(w + L.off_nnz);
-  p.ws_cnt = reinterpret_cast<int*>(w + L.off_cnt);
+  p.ws_nnz = nnz;
+  p.ws_cnt = cnt;
   p.ws_state = reinterpret_cast<double2*>(w + L.off_state);
-  p.row_order = out->row_order; p.row_nnz = out->row_nnz; p.flags = out->skip_flags; p.col_count = out->col_count;
+  p.row_order = out->row_order; p.flags = out->skip_flags;
   p.order1 = out->order1; p.embedding = out->embedding; p.stats = reinterpret_cast<long long*>(out->stats);
-  // CTAs per head: the largest cluster of which the device holds one per head at once, when some
-  // head may be planned at all, and no more than there are groups of 32 rows
+  // CTAs per head: the largest cluster of which the device holds one per head at once, and no more than
+  // there are groups of 32 rows
   int csize = 1;
-  if ((L.mma || L.state_in_smem) && p.mode != WAVEAL_FORCE_NATURAL && p.mode != WAVEAL_STAGE2_ONLY) {
+  {
     const int groups = (int)(((m > n ? m : n) + kUnitRows - 1) / kUnitRows);
     s = cluster_size(dev, (int)H, L.mma ? groups : (groups < 4 ? groups : 4), &csize);
     if (s != WAVEAL_OK) return s;
