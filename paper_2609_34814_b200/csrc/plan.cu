@@ -32,6 +32,7 @@ constexpr int kPlanThreads = 1024;
 constexpr int kPlanWarps = kPlanThreads / 32;
 constexpr int kMaxSort = 16384;          // largest padded row count the in-smem sort takes
 constexpr size_t kSmemMax = 232448;      // 227 KB opt-in limit per CTA on sm_100
+constexpr int kMaxMerge = (kSmemMax - 2048) / 24;     // rows whose two sort buffers fit: 9,600
 
 // ------------------------------------------------------------------ format conversion
 
@@ -611,7 +612,54 @@ __device__ __forceinline__ u64 sortable(double v) {
   return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
 }
 
-// ascending bitonic sort of (key, val) pairs, ties by val; n is a power of two
+// Ascending merge sort of n (key, val) pairs, stable, between two buffers; the result is in the buffer
+// returned (0 or 1).  Runs of 32 by counting (a warp's own elements, read as broadcasts), then
+// every element finds its place in the neighbouring run by a binary search.  Against the bitonic
+// network below: 8 barriers instead of 78 at 4096 elements, no padding to a power of two, and an
+// element is moved 8 times.
+__device__ __forceinline__ int merge_sort(u64* k0, int* v0, u64* k1, int* v1, int n) {
+  for (int i = threadIdx.x; i < n; i += kPlanThreads) {
+    const int g0 = i & ~31, g1 = min(g0 + 32, n);
+    const u64 key = k0[i];
+    int pos = g0;
+    for (int j = g0; j < g1; ++j) {
+      const u64 kj = k0[j];
+      pos += (kj < key || (kj == key && j < i)) ? 1 : 0;
+    }
+    k1[pos] = key;
+    v1[pos] = v0[i];
+  }
+  int at = 1;
+  for (int len = 32; len < n; len <<= 1, at ^= 1) {
+    __syncthreads();
+    const u64* ks = at ? k1 : k0;
+    const int* vs = at ? v1 : v0;
+    u64* kd = at ? k0 : k1;
+    int* vd = at ? v0 : v1;
+    for (int i = threadIdx.x; i < n; i += kPlanThreads) {
+      const u64 key = ks[i];
+      const bool right = (i & len) != 0;               // of the two runs: equal keys of the left one come first
+      const int sib = right ? (i & ~(len - 1)) - len : (i & ~(len - 1)) + len;
+      int lo = min(sib, n), hi = min(sib + len, n);
+      const int s0 = lo;
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        const u64 km = ks[mid];
+        const bool before = km < key || (right && km == key);
+        lo = before ? mid + 1 : lo;
+        hi = before ? hi : mid;
+      }
+      const int pos = (right ? i - len : i) + (lo - s0);
+      kd[pos] = key;
+      vd[pos] = vs[i];
+    }
+  }
+  __syncthreads();
+  return at;
+}
+
+// ascending bitonic sort of (key, val) pairs, ties by val; n is a power of two (row counts whose
+// second buffer does not fit shared memory)
 __device__ __forceinline__ void bitonic_sort(u64* keys, int* vals, int n) {
   for (int k = 2; k <= n; k <<= 1) {
     for (int j = k >> 1; j > 0; j >>= 1) {
@@ -727,8 +775,20 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
     return;
   }
 
+  // pairs to sort: two buffers of m_b (merge sort), or one of n_pow2 (bitonic)
   u64* keys = reinterpret_cast<u64*>(region);
-  int* vals = reinterpret_cast<int*>(region + (size_t)p.n_pow2 * 8);
+  const bool merging = m_b <= kMaxMerge;
+  const int n_sort = merging ? m_b : p.n_pow2;
+  u64* keys2 = keys + (merging ? m_b : 0);
+  int* vals = reinterpret_cast<int*>(keys + (merging ? 2 * m_b : p.n_pow2));
+  int* vals2 = vals + m_b;
+  auto sort_pairs = [&]() {
+    if (!merging) { bitonic_sort(keys, vals, p.n_pow2); return; }
+    if (merge_sort(keys, vals, keys2, vals2, m_b)) {
+      u64* k = keys; keys = keys2; keys2 = k;
+      int* v = vals; vals = vals2; vals2 = v;
+    }
+  };
 
   if (p.mode != WAVEAL_STAGE2_ONLY) {
     double2* X = p.state_in_smem ? reinterpret_cast<double2*>(region)
@@ -835,13 +895,13 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
       int i = tid + k * kPlanThreads;
-      if (i < p.n_pow2) {
+      if (i < n_sort) {
         keys[i] = i < m_b ? sortable(ang[k]) : ~0ull;
         vals[i] = i < m_b ? i : INT_MAX;
       }
     }
     __syncthreads();
-    bitonic_sort(keys, vals, p.n_pow2);     // Stage 1: rows by ascending angle, ties by row index
+    sort_pairs();                           // Stage 1: rows by ascending angle, ties by row index
     if (p.ring_cut && m_b >= 2) {
       // Variant: the sorted rows form a ring (Section 4.3.1); open it at the largest gap between
       // neighbouring angles (the gap around the back, first + 2 pi - last, included; the first
@@ -880,7 +940,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
     if (!lead) return;
     if (p.embedding)
       for (int i = tid; i < m_b; i += kPlanThreads) { p.embedding[((size_t)h * m_b + i) * 2] = 0.0; p.embedding[((size_t)h * m_b + i) * 2 + 1] = 0.0; }
-    for (int i = tid; i < p.n_pow2; i += kPlanThreads) vals[i] = i < m_b ? i : INT_MAX;
+    for (int i = tid; i < n_sort; i += kPlanThreads) vals[i] = i < m_b ? i : INT_MAX;
     __syncthreads();
   }
   if (order1_out)
@@ -891,7 +951,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
   }
   // ---- Stage 2: inside each bucket of `wave` consecutive positions, descending n_i, ties by
   //      Stage-1 position: one sort on the key (bucket, max_count - n_i, position)
-  for (int i = tid; i < p.n_pow2; i += kPlanThreads) {
+  for (int i = tid; i < n_sort; i += kPlanThreads) {
     if (i < m_b) {
       u64 bucket = (u64)(i / p.wave);
       u64 inv = (u64)(0x3FFFFF - min(nnz[vals[i]], 0x3FFFFF));
@@ -901,7 +961,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
     }
   }
   __syncthreads();
-  bitonic_sort(keys, vals, p.n_pow2);
+  sort_pairs();
   for (int i = tid; i < m_b; i += kPlanThreads) order_out[i] = vals[i];
 }
 
@@ -942,6 +1002,7 @@ waveal_status plan_layout(const waveal_plan_desc* d, PlanLayout* L) {
   L->n_pow2 = p2;
   size_t sort_bytes = (size_t)p2 * 12, state_bytes = (2 * m + n) * 16;
   L->state_in_smem = 2048 + (state_bytes > sort_bytes ? state_bytes : sort_bytes) <= kSmemMax;
+  if (m <= (size_t)kMaxMerge) sort_bytes = m * 24;
   L->smem = 2048 + (L->state_in_smem ? (state_bytes > sort_bytes ? state_bytes : sort_bytes) : sort_bytes);
   // The matrix-unit form also keeps the digits of one block, 16 bytes an entry.  On square masks it
   // fits up to ~3,580 blocks as it is, up to ~4,730 with Y and Z in one buffer and up to 14,336
