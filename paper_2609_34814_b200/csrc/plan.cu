@@ -248,28 +248,38 @@ __device__ __forceinline__ void block_sum_i64(long long (&v)[N], long long* scra
   __syncthreads();
 }
 
-__device__ __forceinline__ double block_max(double v, double* scratch) {
-  int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// maxima of N non-negative doubles / minima of N ints over the CTA, same result in every thread
+template <int N>
+__device__ __forceinline__ void block_max(double (&v)[N], double* scratch) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int o = 16; o; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if (lane == 0) scratch[warp] = v;
+  for (int k = 0; k < N; ++k) {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v[k] = fmax(v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
+    if (lane == 0) scratch[warp * N + k] = v[k];
+  }
   __syncthreads();
-  double s = scratch[0];
-  for (int w = 1; w < kPlanWarps; ++w) s = fmax(s, scratch[w]);
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    v[k] = scratch[lane * N + k];
+#pragma unroll
+    for (int o = 16; o; o >>= 1) v[k] = fmax(v[k], __shfl_xor_sync(0xffffffffu, v[k], o));
+  }
   __syncthreads();
-  return s;
 }
 
-__device__ __forceinline__ int block_min_int(int v, int* scratch) {
-  int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+template <int N>
+__device__ __forceinline__ void block_min(int (&v)[N], int* scratch) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int o = 16; o; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
-  if (lane == 0) scratch[warp] = v;
+  for (int k = 0; k < N; ++k) {
+    v[k] = __reduce_min_sync(0xffffffffu, v[k]);
+    if (lane == 0) scratch[warp * N + k] = v[k];
+  }
   __syncthreads();
-  int s = scratch[0];
-  for (int w = 1; w < kPlanWarps; ++w) s = min(s, scratch[w]);
+#pragma unroll
+  for (int k = 0; k < N; ++k) v[k] = __reduce_min_sync(0xffffffffu, scratch[lane * N + k]);
   __syncthreads();
-  return s;
 }
 
 // ---- thread-block cluster helpers: the CTAs of a cluster split the rows of the two mask sweeps
@@ -397,14 +407,13 @@ struct Qr2 {
   }
 };
 __device__ __forceinline__ Qr2 thin_qr2(const double2* z_in, int m, double* scratch) {
-  const double tiny = 1e-30 * sqrt((double)m);
+  const double tiny_sq = 1e-60 * (double)m;      // a column of norm 1e-30 sqrt(m) or less is dropped
   const int tid = threadIdx.x;
   double a[3] = {0, 0, 0};
   for (int i = tid; i < m; i += kPlanThreads) { const double2 z = z_in[i]; a[0] += z.x * z.x; a[1] += z.x * z.y; a[2] += z.y * z.y; }
   block_sum<3>(a, scratch);
   Qr2 r;
-  const double n1 = sqrt(a[0]), n2_before = sqrt(a[2]);
-  r.inv1 = n1 > tiny ? 1.0 / n1 : 0.0;
+  r.inv1 = a[0] > tiny_sq ? rsqrt(a[0]) : 0.0;
   r.d = a[1] * r.inv1;
   double s[4] = {0, 0, 0, 0};
   for (int i = tid; i < m; i += kPlanThreads) {
@@ -414,9 +423,8 @@ __device__ __forceinline__ Qr2 thin_qr2(const double2* z_in, int m, double* scra
   }
   block_sum<4>(s, scratch);
   r.e = s[0];
-  const double n2 = sqrt(fmax(s[1] - r.e * r.e, 0.0));
-  const bool ok2 = n2 > tiny && n2 > 1e-9 * n2_before;
-  r.inv2 = ok2 ? 1.0 / n2 : 0.0;
+  const double n2_sq = s[1] - r.e * r.e;         // dropped too: 1e-9 or less of the norm before the projection
+  r.inv2 = n2_sq > tiny_sq && n2_sq > 1e-18 * a[2] ? rsqrt(n2_sq) : 0.0;
   r.colsum = make_double2(s[2], (s[3] - r.e * s[2]) * r.inv2);
   return r;
 }
@@ -853,28 +861,25 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
     block_sum<4>(b, scratch);
     double th = 0.5 * atan2(2.0 * (0.5 * (b[1] + b[2])), b[0] - b[3]);
     double cs = cos(th), sn = sin(th);
-    double mx1 = 0, mx2 = 0;
+    double mx[2] = {0, 0};
     for (int i = tid; i < m_b; i += kPlanThreads) {
       double2 x = X[i];
       double2 u = make_double2(x.x * cs + x.y * sn, x.y * cs - x.x * sn);
       X[i] = u;
-      mx1 = fmax(mx1, fabs(u.x));
-      mx2 = fmax(mx2, fabs(u.y));
+      mx[0] = fmax(mx[0], fabs(u.x));
+      mx[1] = fmax(mx[1], fabs(u.y));
     }
-    mx1 = block_max(mx1, scratch);
-    mx2 = block_max(mx2, scratch);
+    block_max<2>(mx, scratch);
     // ---- sign: the first entry reaching half of the largest magnitude is made positive
-    int f1 = INT_MAX, f2 = INT_MAX;
+    int f[2] = {INT_MAX, INT_MAX};
     for (int i = tid; i < m_b; i += kPlanThreads) {
       double2 u = X[i];
-      if (mx1 > 0.0 && fabs(u.x) >= 0.5 * mx1) f1 = min(f1, i);
-      if (mx2 > 0.0 && fabs(u.y) >= 0.5 * mx2) f2 = min(f2, i);
+      if (mx[0] > 0.0 && fabs(u.x) >= 0.5 * mx[0]) f[0] = min(f[0], i);
+      if (mx[1] > 0.0 && fabs(u.y) >= 0.5 * mx[1]) f[1] = min(f[1], i);
     }
-    int* mscratch = reinterpret_cast<int*>(scratch);
-    f1 = block_min_int(f1, mscratch);
-    f2 = block_min_int(f2, mscratch);
-    double s1 = (f1 != INT_MAX && X[f1].x < 0.0) ? -1.0 : 1.0;
-    double s2 = (f2 != INT_MAX && X[f2].y < 0.0) ? -1.0 : 1.0;
+    block_min<2>(f, reinterpret_cast<int*>(scratch));
+    double s1 = (f[0] != INT_MAX && X[f[0]].x < 0.0) ? -1.0 : 1.0;
+    double s2 = (f[1] != INT_MAX && X[f[1]].y < 0.0) ? -1.0 : 1.0;
     __syncthreads();
     // ---- polar angle a_i = atan2(u_2[i], u_1[i]) (Eq. 4); kept in registers across the
     //      re-use of the shared region by the sort
@@ -910,20 +915,21 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
         const u64 k = keys[i];
         return __longlong_as_double((long long)((k >> 63) ? (k & 0x7FFFFFFFFFFFFFFFull) : ~k));
       };
-      double best = -1.0;
+      double best[1] = {0.0};
       for (int i = tid; i < m_b; i += kPlanThreads) {
         const double g = i + 1 < m_b ? angle_at(i + 1) - angle_at(i)
                                      : (angle_at(0) + 2.0 * 3.14159265358979323846) - angle_at(m_b - 1);
-        best = fmax(best, g);
+        best[0] = fmax(best[0], g);
       }
-      best = block_max(best, scratch);
-      int at = INT_MAX;
+      block_max<1>(best, scratch);
+      int first[1] = {INT_MAX};
       for (int i = tid; i < m_b; i += kPlanThreads) {
         const double g = i + 1 < m_b ? angle_at(i + 1) - angle_at(i)
                                      : (angle_at(0) + 2.0 * 3.14159265358979323846) - angle_at(m_b - 1);
-        if (g == best) at = min(at, i);
+        if (g == best[0]) first[0] = min(first[0], i);
       }
-      at = block_min_int(at, reinterpret_cast<int*>(scratch));
+      block_min<1>(first, reinterpret_cast<int*>(scratch));
+      const int at = first[0];
       // rotate: the row behind the gap comes first (the key array is free until Stage 2 refills it)
       int* tmp = reinterpret_cast<int*>(keys);
       __syncthreads();
