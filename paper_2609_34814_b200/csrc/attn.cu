@@ -528,6 +528,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     // ============================================================== producer
     if (lane == 0) { prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmV); prefetch_tmap(&tmK2); prefetch_tmap(&tmV2); }
     uint32_t task_it = 0, q_it = 0, k_it = 0, v_it = 0;
+    int n_tiles = 0, n_pairs = 0;        // words 7 and 6 of the workspace: KV tiles (128 rows x 128 keys) and shared tiles this call ran
     bool ok = true;
     uint32_t k_armed = 0, k_parity = 0, v_armed = 0, v_parity = 0;   // per stage: parity of the last load armed on it
     bool q_armed = false; uint32_t q_armed_parity = 0;
@@ -587,6 +588,8 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       if (tk.n < 0) break;
       if (tk.n <= kDrawAhead) { tk_next = draw(t_next); drawn = true; }
       if (tk.n == 0) continue;
+      n_tiles += tk.n;
+      n_pairs += G::KB == 2 && tk.row2 >= 0;
       // Q tile
       ok = warp_wait(ctx, BAR(B_Q_EMPTY), (q_it & 1) ^ 1, 2);
       if (!ok) break;
@@ -632,6 +635,10 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                                               &tmK, &tmK2, k_it, k_armed, k_parity, chunk_base, my_idx);
         }
       }
+    }
+    if (lane == 0 && !p.redo_pass) {
+      if (n_tiles) atomicAdd(&p.ws[7], n_tiles);
+      if (n_pairs) atomicAdd(&p.ws[6], n_pairs);
     }
     if (*abort_smem) {
       // leave no bulk copy in flight into this CTA's shared memory (bounded)
@@ -1099,17 +1106,13 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 // Task of every ticket (head-major or position-major over the planned order), so that the
 // persistent CTAs need one load behind a ticket instead of a chain through row_order, the row
 // pointers and the index list.
-// The inputs are checked on the way (one thread per task, so it costs nothing): an entry of
+// The inputs are checked on the way (a thread per task, so it costs nothing): an entry of
 // row_order outside [0, M_B), a row-pointer pair that is negative, decreasing or beyond the end
 // of the index list, or a last index outside [0, N_B) is reported as
 // {WAVEAL_ERR_BAD_MASK, site, head, offending value} and the task is given an empty list
 // (its output rows become 0) instead of reading out of range.
-__global__ void k_task_table(AttnParams p, int block_k, Task* table) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= p.total_tasks) return;
-  int h, pos;
-  if (p.interleaved) { pos = (int)(t / p.heads); h = (int)(t % p.heads); }
-  else { h = (int)(t / p.m_b); pos = (int)(t % p.m_b); }
+// It also clears the call's counters (the launch before it on the stream has ended).
+__device__ __forceinline__ Task make_task(const AttnParams& p, int block_k, int h, int pos) {
   auto report = [&](int site, int value) {
     if (p.dev_status && atomicCAS(p.dev_status, 0, WAVEAL_ERR_BAD_MASK) == 0) {
       p.dev_status[1] = site; p.dev_status[2] = h; p.dev_status[3] = value;
@@ -1129,48 +1132,140 @@ __global__ void k_task_table(AttnParams p, int block_k, Task* table) {
     if (last < 0 || last >= p.n_b) { report(33, last); len = 0; }
   }
   fill_tiles(tk, len, block_k, last, p.n_b, p.seq_kv);
-  // 64-row query blocks: two blocks with the very same list share one 128-row tile.  Candidates:
-  //  - rows that select every KV block (list length = N_B: rows that attend to everything), wherever
-  //    they stand: the 1st and 2nd, the 3rd and 4th, ... such row of the head's order form pairs,
-  //    run at the position of the first of the two;
-  //  - any other two rows at positions 2i and 2i+1 of the order (Stage 2 of the plan puts rows of
-  //    equal count side by side).
-  // A pair is formed only if the two lists are equal entry by entry; both threads of a pair run
-  // the same comparison, the first keeps the task, the second one's ticket is absorbed.
-  if (block_k == 64 && len > 0 && !bad && !p.no_pairing) {
-    const size_t hb = (size_t)h * p.m_b;
-    auto row_at = [&](int ps) {
-      const int r = p.row_order ? p.row_order[hb + ps] : ps;
-      return (r < 0 || r >= p.m_b) ? -1 : r;
-    };
-    auto len_of = [&](int r) { return p.row_ptr[hb + r + 1] - p.row_ptr[hb + r]; };
-    int mate = -1;            // the other row of the candidate pair
-    bool first = true;        // this thread's row is the first of the two
-    if (len == p.n_b) {
-      int before = 0;
-      for (int ps = 0; ps < pos; ++ps) { const int r = row_at(ps); if (r >= 0 && len_of(r) == p.n_b) ++before; }
-      first = (before & 1) == 0;
-      if (first) {
-        for (int ps = pos + 1; ps < p.m_b && mate < 0; ++ps) { const int r = row_at(ps); if (r >= 0 && len_of(r) == p.n_b) mate = r; }
-      } else {
-        for (int ps = pos - 1; ps >= 0 && mate < 0; --ps) { const int r = row_at(ps); if (r >= 0 && len_of(r) == p.n_b) mate = r; }
-      }
-    } else if ((pos ^ 1) < p.m_b) {
-      const int r = row_at(pos ^ 1);
-      if (r >= 0 && len_of(r) == len) { mate = r; first = (pos & 1) == 0; }
+  if (bad) tk.pad2 = 1;                             // takes no part in pairing
+  return tk;
+}
+
+__device__ __forceinline__ void clear_counters(const AttnParams& p) {
+  if (blockIdx.x == 0 && threadIdx.x < 8) p.ws[threadIdx.x] = 0;
+}
+
+__global__ void k_task_table(AttnParams p, int block_k, Task* table) {
+  clear_counters(p);
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= p.total_tasks) return;
+  int h, pos;
+  if (p.interleaved) { pos = (int)(t / p.heads); h = (int)(t % p.heads); }
+  else { h = (int)(t / p.m_b); pos = (int)(t % p.m_b); }
+  Task tk = make_task(p, block_k, h, pos);
+  tk.pad2 = 0;
+  table[t] = tk;
+}
+
+// The same for 64-row query blocks, where two blocks with the very same list share one 128-row tile.
+// Candidates:
+//  - rows that select every KV block (list length = N_B: rows that attend to everything), wherever
+//    they stand: the 1st and 2nd, the 3rd and 4th, ... such row of the head's order form pairs,
+//    run at the position of the first of the two;
+//  - any other two rows at positions 2i and 2i+1 of the order (Stage 2 of the plan puts rows of
+//    equal count side by side).
+// A pair is formed only if the two lists are equal entry by entry; the first row keeps the task, the
+// second one's ticket is absorbed.
+// A block takes 64 consecutive positions of a head.  Its warps compare the lists 32 entries at a time;
+// rows that select everything know their number in the head's order from a count over the positions
+// before the block's own (a thread each, so the block reads the row lengths of its head once).  One thread
+// per row that counted and compared alone took 488 us on 32 heads of 1536 rows, a tenth of them full.
+constexpr int kPairRows = 64, kPairThreads = 256;
+__global__ void __launch_bounds__(kPairThreads) k_task_table_pairs(AttnParams p, Task* table, int chunks) {
+  __shared__ int s_row[kPairRows], s_lo[kPairRows], s_len[kPairRows];      // (len -1: takes no part)
+  __shared__ int s_mate[kPairRows];                 // list start of the candidate partner, -1: none
+  __shared__ int s_mate_row[kPairRows], s_mate_pos[kPairRows], s_same[kPairRows];   // its row; its position here, -1: elsewhere
+  __shared__ int s_full[kPairRows];                 // positions of the full rows of this block, in order
+  __shared__ int s_before, s_prev, s_next, s_n_full;
+  clear_counters(p);
+  const int h = blockIdx.x / chunks, c0 = (blockIdx.x - h * chunks) * kPairRows, tid = threadIdx.x;
+  const int lane = tid & 31, warp = tid >> 5;
+  const size_t hb = (size_t)h * p.m_b;
+  const long long nnz = p.row_ptr[p.total_tasks];
+  Task tk{};
+  const int pos = c0 + tid;
+  const bool live = tid < kPairRows && pos < p.m_b;
+  if (tid == 0) { s_before = 0; s_prev = -1; s_next = p.m_b; s_n_full = 0; }
+  if (live) tk = make_task(p, 64, h, pos);
+  const bool open = live && !tk.pad2 && tk.len > 0 && !p.no_pairing;
+  auto full_at = [&](int ps) {                      // the row at position ps if it selects everything by its length, else -1
+    const int r = p.row_order ? p.row_order[hb + ps] : ps;
+    return (r < 0 || r >= p.m_b || p.row_ptr[hb + r + 1] - p.row_ptr[hb + r] != p.n_b) ? -1 : r;
+  };
+  __syncthreads();
+  if (tid < kPairRows) {
+    s_row[tid] = tk.row; s_lo[tid] = tk.lo; s_len[tid] = open ? tk.len : -1;
+    s_mate[tid] = -1; s_mate_pos[tid] = -1; s_same[tid] = 0;
+  }
+  __syncthreads();
+  // ---- full rows of this block in order, and those of the head around it.  All of them count, also
+  // malformed ones (every block must number them alike); those form no pair.
+  const bool full = open && tk.len == p.n_b;
+  if (warp == 0) {
+    const bool any = !p.no_pairing;
+    const unsigned a = __ballot_sync(0xffffffffu, any && c0 + lane < p.m_b && full_at(c0 + lane) >= 0);
+    const unsigned b = __ballot_sync(0xffffffffu, any && c0 + lane + 32 < p.m_b && full_at(c0 + lane + 32) >= 0);
+    const unsigned below = (1u << lane) - 1u;
+    if (a >> lane & 1u) s_full[__popc(a & below)] = lane;
+    if (b >> lane & 1u) s_full[__popc(a) + __popc(b & below)] = lane + 32;
+    if (lane == 0) s_n_full = __popc(a) + __popc(b);
+  }
+  __syncthreads();
+  const int n_full = s_n_full;
+  if (n_full > 0) {
+    int before = 0, prev = -1, next = p.m_b;
+#pragma unroll 4
+    for (int ps = tid; ps < p.m_b; ps += kPairThreads) {
+      if (ps >= c0 && ps < c0 + kPairRows) continue;
+      if (full_at(ps) < 0) continue;
+      if (ps < c0) { ++before; prev = max(prev, ps); } else { next = min(next, ps); }
     }
-    if (mate >= 0 && mate != row) {
-      const int lo2 = p.row_ptr[hb + mate], hi2 = p.row_ptr[hb + mate + 1];
-      bool same = lo2 >= 0 && hi2 - lo2 == len && (long long)hi2 <= nnz;
-      for (int e = 0; same && e < len; ++e) same = p.kv_idx[lo + e] == p.kv_idx[lo2 + e];
-      if (same) {
-        if (first) { tk.row2 = mate; atomicAdd(&p.ws[6], 1); }     // word 6: pairs formed by this call
-        else tk.n = kAbsorbed;
-      }
+    before = __reduce_add_sync(0xffffffffu, before);
+    prev = __reduce_max_sync(0xffffffffu, prev);
+    next = __reduce_min_sync(0xffffffffu, next);
+    if (lane == 0) { atomicAdd(&s_before, before); atomicMax(&s_prev, prev); atomicMin(&s_next, next); }
+    __syncthreads();
+    if (tid < n_full) {
+      const int e = s_full[tid], k = ((s_before + tid) ^ 1) - s_before;      // the partner's number here
+      int mrow = -1, mpos = -1;
+      if (k >= 0 && k < n_full) { mpos = s_full[k]; mrow = s_len[mpos] == p.n_b ? s_row[mpos] : -1; }
+      else if (k < 0 && s_prev >= 0) mrow = full_at(s_prev);
+      else if (k >= n_full && s_next < p.m_b) mrow = full_at(s_next);
+      if (mrow >= 0 && s_len[e] == p.n_b) { s_mate[e] = p.row_ptr[hb + mrow]; s_mate_row[e] = mrow; s_mate_pos[e] = mpos; }
     }
   }
-  if (tk.n > 0) atomicAdd(&p.ws[7], tk.n);    // word 7: KV tiles (128 rows x 128 keys) this call runs
-  table[t] = tk;
+  if (open && !full && pos + 1 - 2 * (pos & 1) < p.m_b && s_len[tid ^ 1] == tk.len) {
+    s_mate[tid] = s_lo[tid ^ 1]; s_mate_row[tid] = s_row[tid ^ 1]; s_mate_pos[tid] = tid ^ 1;
+  }
+  __syncthreads();
+  // ---- comparisons: a warp per pair, by the first of the two where both are here
+  for (int e = warp; e < kPairRows; e += kPairThreads / 32) {
+    const int lo2 = s_mate[e], mpos = s_mate_pos[e], len = s_len[e], lo = s_lo[e];
+    if (lo2 < 0 || mpos >= 0 && mpos < e || s_mate_row[e] == s_row[e] || (long long)lo2 + len > nnz) continue;
+    // the first 32 entries tell most pairs apart; behind them 256 at a time
+    bool same = __all_sync(0xffffffffu, lane >= len || p.kv_idx[lo + lane] == p.kv_idx[lo2 + lane]);
+    for (int i0 = 32; i0 < len && same; i0 += 256) {
+      bool eq = true;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int i = i0 + k * 32 + lane;
+        eq &= i >= len || p.kv_idx[lo + i] == p.kv_idx[lo2 + i];
+      }
+      same = __all_sync(0xffffffffu, eq);
+    }
+    if (lane == 0) { s_same[e] = same; if (mpos >= 0) s_same[mpos] = same; }
+  }
+  __syncthreads();
+  if (!live) return;
+  if (s_same[tid]) {
+    const int mpos = s_mate_pos[tid];
+    // the first of the two in the order: partners elsewhere stand before (odd number) or behind (even)
+    bool first = mpos > tid;
+    if (mpos < 0) {
+      int k = 0;
+      while (s_full[k] != tid) ++k;
+      first = ((s_before + k) & 1) == 0;
+    }
+    if (first) tk.row2 = s_mate_row[tid];
+    else tk.n = kAbsorbed;
+  }
+  tk.pad2 = 0;
+  table[p.interleaved ? (long long)pos * p.heads + h : (long long)hb + pos] = tk;
 }
 
 // ------------------------------------------------------------------ host side
@@ -1241,7 +1336,6 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   if ((s = make_map(&tv2, V, D, d->seq_kv, d->heads, d->v_stride[0], d->v_stride[1], 128, "V (128-row boxes)")) != WAVEAL_OK) return s;
   WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd<BLOCK, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES));
   WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd<BLOCK, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES));
-  WAVEAL_CUDA_OK(cudaMemsetAsync(p.ws, 0, 32, st));  // ticket counters, abort flag, redo count
   long long grid = p.total_tasks < sms ? p.total_tasks : sms;
   Task* table = reinterpret_cast<Task*>(reinterpret_cast<char*>(p.ws) + table_offset(p.total_tasks));
   p.table = table;
@@ -1250,7 +1344,12 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   p.drop_tile = 0;
   if (d->flags & WAVEAL_ATTN_SELFTEST_LOST_TILE) { p.wait_limit = kSelfTestCycles; p.drop_tile = 1; }
   p.no_pairing = (d->flags & WAVEAL_ATTN_NO_ROW_PAIRING) ? 1 : 0;
-  k_task_table<<<(unsigned)((p.total_tasks + 255) / 256), 256, 0, st>>>(p, BLOCK, table);
+  if (BLOCK == 64) {
+    const int chunks = (p.m_b + kPairRows - 1) / kPairRows;
+    k_task_table_pairs<<<(unsigned)((long long)p.heads * chunks), kPairThreads, 0, st>>>(p, table, chunks);
+  } else {
+    k_task_table<<<(unsigned)((p.total_tasks + 255) / 256), 256, 0, st>>>(p, BLOCK, table);
+  }
   WAVEAL_CUDA_OK(cudaGetLastError());
   if (d->flags & WAVEAL_ATTN_ONLINE_MAX_ONLY) {
     p.redo_pass = 0;

@@ -36,23 +36,38 @@ constexpr int kMaxMerge = (kSmemMax - 2048) / 24;     // rows whose two sort buf
 
 // ------------------------------------------------------------------ format conversion
 
-// index lists -> bitmap (bitmap zeroed beforehand); one warp per (head, row)
-__global__ void k_csr_to_bitmap(const int* __restrict__ row_ptr, const int* __restrict__ idx,
-                                u64* __restrict__ bits, long long n_rows, int wq, int n_kv,
-                                int m_b, int* dev_status) {
-  long long row = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  int lane = threadIdx.x & 31;
+// index lists -> bitmap; one warp per (head, row), which collects the row in shared memory, kCsrCols
+// columns at a time, and writes whole words: no zeroing pass and no atomics on global memory (109 us
+// for 79 M indices that way)
+constexpr int kCsrCols = 8192, kCsrWarps = 8;
+__global__ void __launch_bounds__(kCsrWarps * 32) k_csr_to_bitmap(const int* __restrict__ row_ptr, const int* __restrict__ idx,
+                                                                  u64* __restrict__ bits, long long n_rows, int wq, int n_kv,
+                                                                  int m_b, int* dev_status) {
+  __shared__ __align__(8) unsigned words[kCsrWarps][kCsrCols / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long row = (long long)blockIdx.x * kCsrWarps + warp;
   if (row >= n_rows) return;
-  int lo = row_ptr[row], hi = row_ptr[row + 1];
-  for (int e = lo + lane; e < hi; e += 32) {
-    int j = idx[e];
-    if (j < 0 || j >= n_kv) {
-      if (dev_status && atomicCAS(dev_status, 0, WAVEAL_ERR_BAD_MASK) == 0) {
-        dev_status[1] = 1; dev_status[2] = (int)(row / m_b); dev_status[3] = j;
+  unsigned* my = words[warp];
+  const int lo = row_ptr[row], hi = row_ptr[row + 1];
+  for (int c0 = 0; c0 < n_kv; c0 += kCsrCols) {
+    const int cols = min(kCsrCols, n_kv - c0), n = (cols + 63) / 64;
+    for (int w = lane; w < 2 * n; w += 32) my[w] = 0u;
+    __syncwarp();
+#pragma unroll 4
+    for (int e = lo + lane; e < hi; e += 32) {
+      const int j = idx[e];
+      if (j < 0 || j >= n_kv) {
+        if (c0 == 0 && dev_status && atomicCAS(dev_status, 0, WAVEAL_ERR_BAD_MASK) == 0) {
+          dev_status[1] = 1; dev_status[2] = (int)(row / m_b); dev_status[3] = j;
+        }
+        continue;
       }
-      continue;
+      const unsigned k = (unsigned)(j - c0);
+      if (k < (unsigned)cols) atomicOr(&my[k >> 5], 1u << (k & 31));
     }
-    atomicOr(&bits[row * wq + (j >> 6)], 1ull << (j & 63));
+    __syncwarp();
+    for (int w = lane; w < n; w += 32) bits[row * wq + (c0 >> 6) + w] = reinterpret_cast<const u64*>(my)[w];
+    __syncwarp();
   }
 }
 
@@ -99,11 +114,21 @@ __global__ void __launch_bounds__(kStatThreads) k_mask_stats(const u64* __restri
     return;
   }
   const int jw = blockIdx.x, stride = 2 * wk + 1;                   // odd: the columns of a warp hit all banks
-  for (int i0 = warp * 32; i0 < wk * 64; i0 += kStatThreads) {
-    const int i = i0 + lane;
-    const u64 w = i < m_b ? Mh[(size_t)i * wq + jw] : 0ull;
-    strip[lane * stride + (i0 >> 5)] = transpose_bits32((unsigned)w, lane);
-    strip[(lane + 32) * stride + (i0 >> 5)] = transpose_bits32((unsigned)(w >> 32), lane);
+  constexpr int kFly = 4;                                           // loads in flight
+  for (int i0 = warp * 32; i0 < wk * 64; i0 += kFly * kStatThreads) {
+    u64 w[kFly];
+#pragma unroll
+    for (int k = 0; k < kFly; ++k) {
+      const int i = i0 + k * kStatThreads + lane;
+      w[k] = i < m_b ? Mh[(size_t)i * wq + jw] : 0ull;
+    }
+#pragma unroll
+    for (int k = 0; k < kFly; ++k) {
+      const int i = i0 + k * kStatThreads;
+      if (i >= wk * 64) break;
+      strip[lane * stride + (i >> 5)] = transpose_bits32((unsigned)w[k], lane);
+      strip[(lane + 32) * stride + (i >> 5)] = transpose_bits32((unsigned)(w[k] >> 32), lane);
+    }
   }
   __syncthreads();
   for (int c0 = warp; c0 < 64; c0 += kStatThreads / 32) {
@@ -124,70 +149,103 @@ __global__ void __launch_bounds__(kStatThreads) k_mask_stats(const u64* __restri
   }
 }
 
-// per-row popcount over all heads (used by bitmap -> index lists)
-__global__ void k_row_popcount(const u64* __restrict__ bits, long long n_rows, int wq, int* __restrict__ cnt) {
-  long long row = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  int lane = threadIdx.x & 31;
-  if (row >= n_rows) return;
-  int c = 0;
-  for (int w = lane; w < wq; w += 32) c += __popcll(bits[row * wq + w]);
-#pragma unroll
-  for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if (lane == 0) cnt[row] = c;
-}
+// bitmap -> ascending index lists.  The lists of all rows lie one behind the other, so the conversion
+// is one compaction of the flat word array: the place of a word's first index is the number of bits
+// set before it, and the row pointer is that place at the first word of a row.  Rows shorter than a
+// warp leave no lane idle.  k_count_words adds up the share of every block, k_fill_lists starts from
+// the sum of the shares before its own; up to kListDirect words (128 KB) a block counts the words before its own
+// itself, which is quicker than a second launch.  A serial scan over the rows in one CTA, as before, took longer
+// than both passes over the data.
+constexpr int kListThreads = 256;             // threads of a block = words of one of its steps
+constexpr int kListBlocks = 2048;             // most blocks (every one reads the shares before its own)
+constexpr int kListDirect = 16384;
 
-// exclusive scan of cnt[0..n) into ptr[0..n]; single CTA
-__global__ void k_exclusive_scan(const int* __restrict__ cnt, long long n, int* __restrict__ ptr) {
-  __shared__ int warp_tot[32];
-  __shared__ int carry_s;
-  int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) carry_s = 0;
+// total over the block of a value per thread; before: the sum over the warps before this one
+__device__ __forceinline__ int list_sum(int v, int* part, int& before) {
+  const int warp = threadIdx.x >> 5;
+  v = __reduce_add_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) part[warp] = v;
   __syncthreads();
-  for (long long base = 0; base < n; base += blockDim.x) {
-    long long i = base + tid;
-    int v = i < n ? cnt[i] : 0;
-    int incl = v;
+  int t = 0;
+  before = 0;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
-    }
-    if (lane == 31) warp_tot[warp] = incl;
-    __syncthreads();
-    int carry = carry_s, pre = 0;
-    for (int w = 0; w < warp; ++w) pre += warp_tot[w];
-    if (i < n) ptr[i] = carry + pre + incl - v;
-    __syncthreads();
-    if (tid == blockDim.x - 1) carry_s = carry + pre + incl;
-    __syncthreads();
-  }
-  if (tid == 0) ptr[n] = carry_s;
+  for (int i = 0; i < kListThreads / 32; ++i) { before += i < warp ? part[i] : 0; t += part[i]; }
+  __syncthreads();
+  return t;
 }
 
-// bitmap -> ascending index lists; one warp per (head, row)
-__global__ void k_fill_indices(const u64* __restrict__ bits, long long n_rows, int wq,
-                               const int* __restrict__ ptr, int* __restrict__ idx, long long capacity) {
-  long long row = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  int lane = threadIdx.x & 31;
-  if (row >= n_rows) return;
-  long long out = ptr[row];
-  for (int w0 = 0; w0 < wq; w0 += 32) {
-    int w = w0 + lane;
-    u64 word = w < wq ? bits[row * wq + w] : 0ull;
-    int c = __popcll(word), incl = c;
+__global__ void __launch_bounds__(kListThreads) k_count_words(const u64* __restrict__ bits, long long n_words, int steps,
+                                                              int* __restrict__ share) {
+  __shared__ int part[kListThreads / 32];
+  const long long w0 = (long long)blockIdx.x * steps * kListThreads;
+  int c = 0, ignored;
+#pragma unroll 4
+  for (int s = 0; s < steps; ++s) {
+    const long long w = w0 + s * kListThreads + threadIdx.x;
+    if (w < n_words) c += __popcll(bits[w]);
+  }
+  c = list_sum(c, part, ignored);
+  if (threadIdx.x == 0) share[blockIdx.x] = c;
+}
+
+// a warp takes 32 words at a time: every lane writes the bit positions of its word into the warp's
+// staging area ((lane, bit) in 16 bits), which then leaves in whole lines
+__global__ void __launch_bounds__(kListThreads) k_fill_lists(const u64* __restrict__ bits, long long n_words, int wq,
+                                                             int steps, const int* __restrict__ share,
+                                                             int* __restrict__ ptr, long long n_rows,
+                                                             int* __restrict__ idx, long long capacity) {
+  __shared__ unsigned short stage[kListThreads / 32][32 * 64];
+  __shared__ int part[kListThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long w0 = (long long)blockIdx.x * steps * kListThreads;
+  int base = 0, pos;
+  if (share) {
+    for (int i = threadIdx.x; i < (int)blockIdx.x; i += kListThreads) base += share[i];
+  } else {
+#pragma unroll 4
+    for (int w = threadIdx.x; w < (int)w0; w += kListThreads) base += __popcll(bits[w]);
+  }
+  base = list_sum(base, part, pos);
+  const long long row0 = w0 / wq;
+  const unsigned rem0 = (unsigned)(w0 - row0 * wq);
+  u64 next = w0 + threadIdx.x < n_words ? bits[w0 + threadIdx.x] : 0ull;
+  for (int s = 0; s < steps && w0 + s * kListThreads < n_words; ++s) {
+    const unsigned off = (unsigned)(s * kListThreads) + threadIdx.x;
+    const long long w = w0 + off;
+    const u64 x = next;
+    next = s + 1 < steps && w + kListThreads < n_words ? bits[w + kListThreads] : 0ull;
+    const int n = __popcll(x);
+    const int total = list_sum(n, part, pos);
+    pos += base;
+    base += total;
+    int incl = n;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      int t = __shfl_up_sync(0xffffffffu, incl, o);
+      const int t = __shfl_up_sync(0xffffffffu, incl, o);
       if (lane >= o) incl += t;
     }
-    long long pos = out + incl - c;
-    while (word) {
-      int b = __ffsll((long long)word) - 1;
-      word &= word - 1;
-      if (pos < capacity) idx[pos] = w * 64 + b;
-      ++pos;
+    const unsigned flat = rem0 + off, row = flat / (unsigned)wq, col = flat - row * (unsigned)wq;
+    if (w < n_words && col == 0) ptr[row0 + row] = pos + incl - n;
+    if (w == n_words - 1) ptr[n_rows] = pos + incl;
+    if (idx) {
+      unsigned short* st = stage[warp] + (incl - n);
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        unsigned y = half ? (unsigned)(x >> 32) : (unsigned)x;
+        while (y) {
+          *st++ = (unsigned short)(lane * 64 + half * 32 + __ffs((int)y) - 1);
+          y &= y - 1;
+        }
+      }
+      __syncwarp();
+      const int here = __shfl_sync(0xffffffffu, incl, 31);
+      for (int i0 = 0; i0 < here; i0 += 32) {
+        const int i = i0 + lane, e = i < here ? stage[warp][i] : 0;
+        const int v = (int)__shfl_sync(0xffffffffu, col, e >> 6) * 64 + (e & 63);
+        if (i < here && pos + i < capacity) idx[pos + i] = v;
+      }
+      __syncwarp();
     }
-    out += __shfl_sync(0xffffffffu, incl, 31);
   }
 }
 
@@ -1082,9 +1140,8 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
   const u64* M = mask_bits;
   if (!M) {
     u64* bm = reinterpret_cast<u64*>(w + L.off_bitmap);
-    WAVEAL_CUDA_OK(cudaMemsetAsync(bm, 0, H * m * L.wq * 8, st));
     long long rows = (long long)(H * m);
-    k_csr_to_bitmap<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(row_ptr, idx, bm, rows, L.wq, (int)n, (int)m, out->dev_status);
+    k_csr_to_bitmap<<<(unsigned)((rows + kCsrWarps - 1) / kCsrWarps), kCsrWarps * 32, 0, st>>>(row_ptr, idx, bm, rows, L.wq, (int)n, (int)m, out->dev_status);
     ++launches;
     M = bm;
   }
@@ -1214,14 +1271,21 @@ extern "C" waveal_status waveal_bitmap_to_csr(int32_t heads, int32_t n_q_blocks,
   int wq = (n_kv_blocks + 63) / 64;
   int* cnt = static_cast<int*>(ws);
   int launches = 0;
-  k_row_popcount<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(reinterpret_cast<const u64*>(mask_bits), rows, wq, cnt);
-  k_exclusive_scan<<<1, 1024, 0, st>>>(cnt, rows, kv_row_ptr_out);
-  launches += 2;
-  if (kv_block_indices_out) {
-    k_fill_indices<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(reinterpret_cast<const u64*>(mask_bits), rows, wq,
-                                                              kv_row_ptr_out, kv_block_indices_out, capacity);
+  // steps of a block: as few as keep the number of blocks (and of their shares) below kListBlocks and
+  // within the workspace of one int per row
+  const u64* bits = reinterpret_cast<const u64*>(mask_bits);
+  const long long words = rows * wq, steps_all = (words + kListThreads - 1) / kListThreads;
+  const bool direct = words <= kListDirect;
+  const long long most = direct ? steps_all : rows < kListBlocks ? rows : kListBlocks;
+  const long long steps = (steps_all + most - 1) / most;
+  const unsigned blocks = (unsigned)((steps_all + steps - 1) / steps);
+  if (!direct) {
+    k_count_words<<<blocks, kListThreads, 0, st>>>(bits, words, (int)steps, cnt);
     ++launches;
   }
+  k_fill_lists<<<blocks, kListThreads, 0, st>>>(bits, words, wq, (int)steps, direct ? nullptr : cnt, kv_row_ptr_out, rows,
+                                                kv_block_indices_out, capacity);
+  ++launches;
   WAVEAL_CUDA_OK(cudaGetLastError());
   waveal::launch_counter() = launches;
   return WAVEAL_OK;
