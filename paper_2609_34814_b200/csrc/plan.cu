@@ -53,17 +53,33 @@ __global__ void __launch_bounds__(kCsrWarps * 32) k_csr_to_bitmap(const int* __r
     const int cols = min(kCsrCols, n_kv - c0), n = (cols + 63) / 64;
     for (int w = lane; w < 2 * n; w += 32) my[w] = 0u;
     __syncwarp();
-#pragma unroll 4
-    for (int e = lo + lane; e < hi; e += 32) {
-      const int j = idx[e];
-      if (j < 0 || j >= n_kv) {
-        if (c0 == 0 && dev_status && atomicCAS(dev_status, 0, WAVEAL_ERR_BAD_MASK) == 0) {
-          dev_status[1] = 1; dev_status[2] = (int)(row / m_b); dev_status[3] = j;
+    // a lane takes kRun consecutive entries and hands a word over once for all of them that fall into it
+    // (ascending lists: one entry per lane would send a whole warp to the same word in dense rows)
+    constexpr int kRun = 8;
+    for (int e0 = lo + lane * kRun; e0 < hi; e0 += 32 * kRun) {
+      int j[kRun];
+#pragma unroll
+      for (int i = 0; i < kRun; ++i) j[i] = e0 + i < hi ? idx[e0 + i] : INT_MAX;
+      unsigned at = 0, acc = 0;
+#pragma unroll
+      for (int i = 0; i < kRun; ++i) {
+        if (e0 + i >= hi) break;
+        if (j[i] < 0 || j[i] >= n_kv) {
+          if (c0 == 0 && dev_status && atomicCAS(dev_status, 0, WAVEAL_ERR_BAD_MASK) == 0) {
+            dev_status[1] = 1; dev_status[2] = (int)(row / m_b); dev_status[3] = j[i];
+          }
+          continue;
         }
-        continue;
+        const unsigned k = (unsigned)(j[i] - c0);
+        if (k >= (unsigned)cols) continue;
+        if ((k >> 5) != at) {
+          if (acc) atomicOr(&my[at], acc);
+          at = k >> 5;
+          acc = 0;
+        }
+        acc |= 1u << (k & 31);
       }
-      const unsigned k = (unsigned)(j - c0);
-      if (k < (unsigned)cols) atomicOr(&my[k >> 5], 1u << (k & 31));
+      if (acc) atomicOr(&my[at], acc);
     }
     __syncwarp();
     for (int w = lane; w < n; w += 32) bits[row * wq + (c0 >> 6) + w] = reinterpret_cast<const u64*>(my)[w];
@@ -71,16 +87,29 @@ __global__ void __launch_bounds__(kCsrWarps * 32) k_csr_to_bitmap(const int* __r
   }
 }
 
-// 32 x 32 bits transposed inside a warp (lane = row on entry, column on exit): five exchanges
-__device__ __forceinline__ unsigned transpose_bits32(unsigned x, int lane) {
-#pragma unroll
-  for (int j = 16; j; j >>= 1) {
-    const unsigned m = j == 16 ? 0x0000FFFFu : j == 8 ? 0x00FF00FFu : j == 4 ? 0x0F0F0F0Fu : j == 2 ? 0x33333333u : 0x55555555u;
-    const unsigned y = __shfl_xor_sync(0xffffffffu, x, j);
-    x = (lane & j) ? ((x & ~m) | ((y & ~m) >> j)) : ((x & m) | ((y & m) << j));
+// 32 x 32 bits transposed inside a warp (lane = row on entry, column on exit): five exchanges of half
+// the bits with the lane 16, 8, 4, 2, 1 away.  Bytes move by permutes, smaller pieces by a rotate and a
+// select; what depends on the lane is worked out once (Transposer).
+struct Transposer {
+  unsigned sel16, sel8, mask[3], rot[3];
+  __device__ __forceinline__ explicit Transposer(int lane) {
+    sel16 = lane & 16 ? 0x3276u : 0x5410u;
+    sel8 = lane & 8 ? 0x3715u : 0x6240u;
+    mask[0] = lane & 4 ? 0xF0F0F0F0u : 0x0F0F0F0Fu; rot[0] = lane & 4 ? 28 : 4;
+    mask[1] = lane & 2 ? 0xCCCCCCCCu : 0x33333333u; rot[1] = lane & 2 ? 30 : 2;
+    mask[2] = lane & 1 ? 0xAAAAAAAAu : 0x55555555u; rot[2] = lane & 1 ? 31 : 1;
   }
-  return x;
-}
+  __device__ __forceinline__ unsigned operator()(unsigned x) const {
+    x = __byte_perm(x, __shfl_xor_sync(0xffffffffu, x, 16), sel16);
+    x = __byte_perm(x, __shfl_xor_sync(0xffffffffu, x, 8), sel8);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const unsigned y = __shfl_xor_sync(0xffffffffu, x, 4 >> k);
+      x = (x & mask[k]) | (__funnelshift_l(y, y, rot[k]) & ~mask[k]);
+    }
+    return x;
+  }
+};
 
 // One pass over the mask: its bit transpose Mt[h][j][i>>6] bit (i&63) = M[h][i][j>>6] bit (j&63), the
 // column counts c = M^T 1 and the row counts n_i = M 1.
@@ -114,6 +143,7 @@ __global__ void __launch_bounds__(kStatThreads) k_mask_stats(const u64* __restri
     return;
   }
   const int jw = blockIdx.x, stride = 2 * wk + 1;                   // odd: the columns of a warp hit all banks
+  const Transposer transpose(lane);
   constexpr int kFly = 4;                                           // loads in flight
   for (int i0 = warp * 32; i0 < wk * 64; i0 += kFly * kStatThreads) {
     u64 w[kFly];
@@ -126,8 +156,8 @@ __global__ void __launch_bounds__(kStatThreads) k_mask_stats(const u64* __restri
     for (int k = 0; k < kFly; ++k) {
       const int i = i0 + k * kStatThreads;
       if (i >= wk * 64) break;
-      strip[lane * stride + (i >> 5)] = transpose_bits32((unsigned)w[k], lane);
-      strip[(lane + 32) * stride + (i >> 5)] = transpose_bits32((unsigned)(w[k] >> 32), lane);
+      strip[lane * stride + (i >> 5)] = transpose((unsigned)w[k]);
+      strip[(lane + 32) * stride + (i >> 5)] = transpose((unsigned)(w[k] >> 32));
     }
   }
   __syncthreads();
@@ -751,6 +781,7 @@ struct PlanParams {
   int ring_cut;         // open the angular ring at its largest gap instead of at -pi
   int csize;            // CTAs per head (thread-block cluster size)
   int mma;              // mask products on the integer matrix units (else: walk over the set bits)
+  int count_stage2;     // Stage 2 by counting inside the buckets (else: by a sort)
   int alias_yz;         // Y and Z share one buffer (two barriers more per iteration)
   int ksplit_y, ksplit_z, part_ints;
   unsigned off_items, off_part;     // bytes from the start of shared memory
@@ -1014,7 +1045,25 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
     return;
   }
   // ---- Stage 2: inside each bucket of `wave` consecutive positions, descending n_i, ties by
-  //      Stage-1 position: one sort on the key (bucket, max_count - n_i, position)
+  //      Stage-1 position
+  if (p.count_stage2) {
+    // small buckets: a row's place is the number of rows of its bucket that go before it, by a key of
+    // (n_b - n_i, position) in 32 bits.  The rows of a warp share a bucket, so the keys are read as broadcasts:
+    // ~2.5 instructions per comparison, against the ~600 an element takes in the merge sort.
+    unsigned* key = reinterpret_cast<unsigned*>(keys);
+    for (int i = tid; i < m_b; i += kPlanThreads) key[i] = (unsigned)(n_b - nnz[vals[i]]) << 14 | (unsigned)i;
+    __syncthreads();
+    for (int i = tid; i < m_b; i += kPlanThreads) {
+      const int b0 = i / p.wave * p.wave, b1 = min(b0 + p.wave, m_b);
+      const unsigned mine = key[i];
+      int at = b0;
+#pragma unroll 8
+      for (int j = b0; j < b1; ++j) at += key[j] < mine ? 1 : 0;
+      order_out[at] = vals[i];
+    }
+    return;
+  }
+  // otherwise one sort on the key (bucket, max_count - n_i, position)
   for (int i = tid; i < n_sort; i += kPlanThreads) {
     if (i < m_b) {
       u64 bucket = (u64)(i / p.wave);
@@ -1175,6 +1224,9 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
     s = cluster_size(dev, (int)H, L.mma ? groups : (groups < 4 ? groups : 4), &csize);
     if (s != WAVEAL_OK) return s;
   }
+  // counting costs 2.5 wave instructions a row, the merge sort ~550: kMaxSort = 2^14 positions, and
+  // n - n_i has to fit the other 18 bits
+  p.count_stage2 = p.wave <= 220 && n < (1u << 18);
   p.mma = L.mma; p.alias_yz = L.alias_yz; p.off_items = (unsigned)L.off_items;
   p.ksplit_y = p.ksplit_z = 1;
   int y_exp = 0;
