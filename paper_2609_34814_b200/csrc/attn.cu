@@ -8,12 +8,10 @@
 // SM, take tickets from a global counter, so a freed SM starts the next row of the list at
 // once - the streaming "wave" behaviour of Section 2.3 that the schedule is built for.
 //
-// Structure of one CTA (608 threads; 640 in the kernels of the 64-row blocks):
-//   warp 0      producer: takes tickets, publishes tasks, issues TMA loads of the Q tile and
-//               of the K and V tiles (128-byte-swizzled slabs) into two shared-memory rings
-//   warp 19     64-row blocks only: requests the V tiles instead of warp 0 (a tile of that shape
-//               takes two list entries and up to four boxes; one warp for both streams was the
-//               limit of the whole kernel there)
+// Structure of one CTA (640 threads):
+//   warp 0      producer: takes tickets, publishes tasks, issues TMA loads of the Q tile and of the K
+//               tiles (128-byte-swizzled slabs) into shared-memory rings, as far ahead as the rings allow
+//   warp 19     requests the V tiles (one warp for both streams was the limit of the 64-row kernels)
 //   warp 18     MMA issuer 1: S_j = Q K_j^T (operands in shared memory) into one of three S
 //               buffers in tensor memory, up to three blocks ahead of the softmax
 //   warp 1      MMA issuer 2: O += P_j V_j (P read from tensor memory, where it lies over the
@@ -21,7 +19,7 @@
 //               the waits and ring arithmetic of one run while the other's MMAs execute
 //   warps 2-17  softmax, two teams of eight warps that take the KV blocks of a task in turn;
 //               inside a team a row of S has two owners, one per half of its columns (row max
-//               in the blocks that take one, then exponentials and P in a second read of S,
+//               in the tiles that take one, then exponentials and P in a second read of S,
 //               32 columns at a time in a rolled loop).  On every scheduler two warps of each
 //               team are resident, the teams half a block apart, so one team's waits and loads
 //               hide behind the other's arithmetic.  The teams hand each other the running
@@ -29,10 +27,11 @@
 //               sum of its own columns; O in tensor memory is rescaled only when the max grew
 //               by more than 2^8; the epilogue adds the four partial sums of a row, normalises
 //               and stores O at the ORIGINAL row (no inverse permutation)
-// Two launches per call: in the first the row max is taken in blocks 0 and 1 of a task only and
-// the reference stays fixed afterwards (softmax does not depend on it short of overflow); a task
-// in which a block's sum of exponentials reaches 2^24 is listed in the workspace and computed
-// again by the second launch, which takes the max of every block.
+// Two launches per call: in the first the row max is taken in the first tile of a task only (64-row blocks:
+// the first two) and the reference stays fixed afterwards (softmax does not depend on it short of
+// overflow: P in bf16, the sums and O in fp32 have the same exponent range); a task in which a
+// tile's sum of exponentials reaches 2^60 is listed in the workspace and computed
+// again by the second launch, which takes the max of every tile.
 // Every wait on an mbarrier is bounded; when one runs out the CTA records
 // {WAVEAL_ERR_TIMEOUT, site} and all roles leave through the common teardown.
 #include <cuda.h>
@@ -43,14 +42,13 @@
 namespace {
 
 // 19 warps, and a 20th (the V tile loader) in the kernels of the 64-row blocks
-template <int BLOCK> constexpr int kThreadsOf = BLOCK == 64 ? 640 : 608;
+constexpr int kThreads = 640;
 constexpr int kProducerWarp = 0, kPvWarp = 1, kSoftmaxWarp0 = 2, kQkWarp = 18, kVLoadWarp = 19;
 constexpr long long kTimeoutCycles = 4000000000ll;   // ~2 s at boost clock
 constexpr long long kSelfTestCycles = 4000000ll;     // ~2 ms: wait limit under WAVEAL_ATTN_SELFTEST_LOST_TILE
-#ifndef WAVEAL_POLY_EVERY
-#define WAVEAL_POLY_EVERY 4
-#endif
-constexpr int kPolyEvery = WAVEAL_POLY_EVERY;          // n > 0: 1 pair of elements in n takes 2^x from the FMA pipe (0 = all from the transcendental unit)
+// 1 pair of elements in n takes 2^x from the FMA pipe, the others from the transcendental unit (dense 128-row
+// tiles, clk per tile: n = 3: 1,449, 4: 1,439, 5: 1,431)
+constexpr int kPolyEvery = 5;
 
 // ------------------------------------------------------------------ PTX wrappers
 
@@ -160,13 +158,13 @@ __device__ __forceinline__ void fadd2(float& d0, float& d1, float a0, float a1, 
 // confined to the window [kPolyLo, kPolyLo + 128] by a saturating multiply-add
 // (y = sat(x/128 - kPolyLo/128) in [0, 1]; x is taken back from y with an absolute error
 // below 2^-17), so that the exponent arithmetic below can neither wrap into the sign bit
-// (x >= 128.5 would) nor underflow: an x above the window comes out as 2^(kPolyLo+128) = 2^28,
+// (x >= 128.5 would) nor underflow: an x above the window comes out as 2^(kPolyLo+128) = 2^64,
 // far above the limit at which the fixed-reference pass hands a task to the second launch; an x
-// below it (a key that does not exist, -inf) as 2^-100.  x is then rounded to the nearest integer
+// below it (a key that does not exist, -inf) as 2^-64.  x is then rounded to the nearest integer
 // n with the 1.5*2^23 trick, a degree-3 polynomial gives 2^(x-n) on [-0.5, 0.5] (relative error
 // 7.5e-5, far below the bf16 cut of P), and n is added to the exponent field.
-constexpr float kPolyLo = -100.0f;
-constexpr float kRedoLimit = 16777216.0f;     // 2^24: block sums at or above it (or NaN) list the task
+constexpr float kPolyLo = -64.0f;
+constexpr float kRedoLimit = 1152921504606846976.0f;     // 2^60: tile sums at or above it (or NaN) list the task
 __device__ __forceinline__ float fma_sat(float a, float b, float c) {
   float d;
   asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
@@ -253,6 +251,12 @@ __device__ __forceinline__ void st_global_v8(void* ptr, const uint32_t* w) {
                : "memory");
 }
 
+__device__ __forceinline__ float fmax3(float a, float b, float c) {
+  float d;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -332,24 +336,30 @@ struct Geo {
   static constexpr int Q_BYTES = SLABS * 128 * 128;  // smem reserved for the 128 MMA rows
   static constexpr int TILE_BYTES = SLABS * BK * 128;
   static constexpr int KV_SLAB_BYTES = BK * 128;
-  static constexpr int NSTAGE_RAW = (200 * 1024 - Q_BYTES) / TILE_BYTES;
+  // Q tiles: with two, the next task's is requested while this one's is in use, for a K ring of two stages
+  // instead of three (128-row tiles of 8 tiles a task: 16.0k against 16.4k clk; 64-row tiles: 18.5 M against
+  // 18.2 M cycles on 8 heads of 1536 rows, their tasks are longer and their rings do the work)
+  static constexpr int NQ = KB == 1 ? 2 : 1;
+  static constexpr int NSTAGE_RAW = (200 * 1024 - NQ * Q_BYTES) / TILE_BYTES;
   static constexpr int NSTAGE = NSTAGE_RAW > 8 ? 8 : NSTAGE_RAW;
   static constexpr int NKS = (NSTAGE + 1) / 2;       // K tile ring
   static constexpr int NVS = NSTAGE / 2;             // V tile ring
+  // tiles of a task that take a row max in the first launch (one instead of two: 5.7k -> 4.6k clk a task beyond its
+  // tiles; the 64-row kernels, which keep only half of their warps busy, do not gain: +3 % cycles)
+  static constexpr int MAX_TILES = KB == 1 ? 1 : 2;
   static constexpr int NSBUF = 3;                    // S/P buffers in tensor memory
-  static constexpr bool SPLIT_LOADERS = KB == 2;     // K and V tiles requested by a warp each (else one warp, interleaved)
   static constexpr int HC = BK / 2;                  // S columns of a row one softmax thread owns (a row has two owners)
   static constexpr int CH = 32;                      // S columns a softmax thread holds at a time
   static constexpr int NCH = HC / CH;                // such chunks per thread and block
-  static constexpr int CO = D / 4;                   // O columns per epilogue thread
+  static constexpr int CO = D / 2;                   // O columns per epilogue thread
   static constexpr int OFF_Q = 0;
-  static constexpr int OFF_K = OFF_Q + Q_BYTES;
+  static constexpr int OFF_K = OFF_Q + NQ * Q_BYTES;
   static constexpr int OFF_V = OFF_K + NKS * TILE_BYTES;
   static constexpr int OFF_BAR = OFF_V + NVS * TILE_BYTES;
-  static constexpr int N_BAR = 4 + 2 + 2 * NKS + 2 * NVS + 4 * NSBUF + 2 + 2 + 8 + 4 + 8;
+  static constexpr int N_BAR = 4 + 4 + 2 * NKS + 2 * NVS + 4 * NSBUF + 2 + 2 + 16 + 16 + 8;
   static constexpr int OFF_TASK = OFF_BAR + ((N_BAR * 8 + 15) / 16) * 16;
   static constexpr int OFF_MX = OFF_TASK + 2 * (int)sizeof(Task);
-  static constexpr int OFF_MISC = OFF_MX + 4 * 128 * 4 + 2 * 2 * 2 * 128 * 4 + 2 * 4 * 128 * 8;
+  static constexpr int OFF_MISC = OFF_MX + 4 * 128 * 4 + 2 * 2 * 2 * 128 * 4 + 4 * 4 * 128 * 8;
   static constexpr int SMEM_BYTES = OFF_MISC + 32 + 1024;   // + slack for 1024-byte alignment
   // tensor memory: three S/P buffers of 128 columns, then the output accumulator
   static constexpr uint32_t S_STRIDE = 128, O_COL = 384, TMEM_COLS = 512;
@@ -373,9 +383,10 @@ __device__ __noinline__ void signal_abort(const Ctx& c, int site) {
   }
 }
 
-// bounded wait; false = gave up (this CTA is aborting)
-__device__ __forceinline__ bool mbar_wait(const Ctx& c, uint32_t bar, uint32_t parity, int site) {
-  if (mbar_try_wait(bar, parity)) return true;
+// bounded wait; false = gave up (this CTA is aborting).  The polling loop is one function for all the
+// waits of the kernel: inlined twenty times it cost 3 % of the cycles in instruction fetches (the softmax
+// loop and the waits around it have to stay in the schedulers' instruction caches).
+__device__ __noinline__ bool mbar_wait_slow(const Ctx& c, uint32_t bar, uint32_t parity, int site) {
   long long t0 = clock64();
   for (;;) {
 #pragma unroll 1
@@ -384,6 +395,10 @@ __device__ __forceinline__ bool mbar_wait(const Ctx& c, uint32_t bar, uint32_t p
     if (*c.abort_smem) return false;
     if (clock64() - t0 > c.limit) { signal_abort(c, site); return false; }
   }
+}
+
+__device__ __forceinline__ bool mbar_wait(const Ctx& c, uint32_t bar, uint32_t parity, int site) {
+  return mbar_try_wait(bar, parity) || mbar_wait_slow(c, bar, parity, site);
 }
 
 // same, with one answer for the whole warp (the roles use warp-collective instructions).  All
@@ -448,8 +463,25 @@ __device__ __forceinline__ bool load_kv_tile(const Ctx& ctx, const AttnParams& p
   return true;
 }
 
+// scores of a thread's own columns of a tile from column `valid` on become -inf (in tensor memory and out of
+// line, so that the two loops over the scores carry no code for the rare ragged tile)
+template <int NCH>
+__device__ __noinline__ void mask_scores(uint32_t s_addr, int valid) {
+#pragma unroll 1
+  for (int ch = 0; ch < NCH; ++ch) {
+    uint32_t sv[32];
+    WAVEAL_TMEM_LD32(s_addr + ch * 32, sv, 0);
+    WAVEAL_TMEM_WAIT_LD32(sv, 0);
+#pragma unroll
+    for (int c = 0; c < 32; ++c)
+      if (ch * 32 + c >= valid) sv[c] = __float_as_uint(-INFINITY);
+    WAVEAL_TMEM_ST32(s_addr + ch * 32, sv, 0);
+  }
+  tc_wait_st();
+}
+
 template <int BLOCK, int D, bool FAST>
-__global__ void __launch_bounds__(kThreadsOf<BLOCK>, 1)
+__global__ void __launch_bounds__(kThreads, 1)
 k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
              const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmK2,
              const __grid_constant__ CUtensorMap tmV2, const AttnParams p) {
@@ -467,27 +499,26 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 
   const uint32_t bar0 = sbase + G::OFF_BAR;
   auto BAR = [&](int i) { return bar0 + 8u * (uint32_t)i; };
-  constexpr int B_TASK_FULL = 0, B_TASK_EMPTY = 2, B_Q_FULL = 4, B_Q_EMPTY = 5, B_K_FULL = 6,
+  constexpr int B_TASK_FULL = 0, B_TASK_EMPTY = 2, B_Q_FULL = 4, B_Q_EMPTY = 6, B_K_FULL = 8,
                 B_K_EMPTY = B_K_FULL + G::NKS, B_V_FULL = B_K_EMPTY + G::NKS, B_V_EMPTY = B_V_FULL + G::NVS,
                 B_S_FULL = B_V_EMPTY + G::NVS, B_P_FULL = B_S_FULL + G::NSBUF, B_S_FREE = B_P_FULL + 2 * G::NSBUF,
                 B_O_FULL = B_S_FREE + G::NSBUF, B_O_FREE = B_O_FULL + 1, B_FINAL = B_O_FREE + 1, B_MX = B_FINAL + 2,
-                B_EX = B_MX + 8, B_HX = B_EX + 4;
+                B_EX = B_MX + 16, B_HX = B_EX + 16;
   static_assert(B_HX + 8 <= G::N_BAR, "barrier count");
   Task* tasks = reinterpret_cast<Task*>(smem + G::OFF_TASK);
-  volatile float* mpub = reinterpret_cast<volatile float*>(smem + G::OFF_MX);   // [block index mod 4][128] reference max after a block
+  volatile float* mpub = reinterpret_cast<volatile float*>(smem + G::OFF_MX);   // [tile count mod 4][128] reference max after a tile
   volatile float* mhalf = reinterpret_cast<volatile float*>(smem + G::OFF_MX + 4 * 128 * 4);   // [use parity][team][column half][128] max of a half row
-  float2* ex = reinterpret_cast<float2*>(smem + G::OFF_MX + 4 * 128 * 4 + 2 * 2 * 2 * 128 * 4);    // [task parity][team*2+half][128] (reference, sum)
+  float2* ex = reinterpret_cast<float2*>(smem + G::OFF_MX + 4 * 128 * 4 + 2 * 2 * 2 * 128 * 4);    // [task mod 4][tile parity*2+half][128] (reference, sum)
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + G::OFF_MISC);
   volatile int* abort_smem = reinterpret_cast<volatile int*>(smem + G::OFF_MISC + 4);
-  volatile int* redo_flag = reinterpret_cast<volatile int*>(smem + G::OFF_MISC + 8);   // [task parity]
+  volatile int* redo_flag = reinterpret_cast<volatile int*>(smem + G::OFF_MISC + 8);   // [task mod 4]
   Ctx ctx{bar0, abort_smem, p.ws, p.dev_status, p.wait_limit};
   const long long t_start = clock64();
 
   if (tid == 0) {
     // a task is read by the V loader, the two MMA issuers and the sixteen softmax warps
-    for (int i = 0; i < 2; ++i) { mbar_init(BAR(B_TASK_FULL + i), 1); mbar_init(BAR(B_TASK_EMPTY + i), G::SPLIT_LOADERS ? 19 : 18); }
-    mbar_init(BAR(B_Q_FULL), 1);
-    mbar_init(BAR(B_Q_EMPTY), 1);
+    for (int i = 0; i < 2; ++i) { mbar_init(BAR(B_TASK_FULL + i), 1); mbar_init(BAR(B_TASK_EMPTY + i), 19); }
+    for (int i = 0; i < 2; ++i) { mbar_init(BAR(B_Q_FULL + i), 1); mbar_init(BAR(B_Q_EMPTY + i), 1); }
     for (int i = 0; i < G::NKS; ++i) { mbar_init(BAR(B_K_FULL + i), 1); mbar_init(BAR(B_K_EMPTY + i), 1); }
     for (int i = 0; i < G::NVS; ++i) { mbar_init(BAR(B_V_FULL + i), 1); mbar_init(BAR(B_V_EMPTY + i), 1); }
     for (int i = 0; i < G::NSBUF; ++i) {
@@ -497,20 +528,19 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       mbar_init(BAR(B_S_FREE + i), 1);
     }
     mbar_init(BAR(B_O_FULL), 1);
-    mbar_init(BAR(B_O_FREE), 16);
+    mbar_init(BAR(B_O_FREE), 8);              // the team that runs the epilogue
     mbar_init(BAR(B_FINAL), 1);
     mbar_init(BAR(B_FINAL + 1), 1);
-    for (int i = 0; i < 8; ++i) mbar_init(BAR(B_MX + i), 1);
-    for (int i = 0; i < 4; ++i) mbar_init(BAR(B_EX + i), 4);    // the four warps of a lane quadrant, once per task
+    for (int i = 0; i < 16; ++i) mbar_init(BAR(B_MX + i), 1);   // (lane quadrant, tile count mod 4)
+    for (int i = 0; i < 16; ++i) mbar_init(BAR(B_EX + i), 4);   // (task mod 4, lane quadrant): its four warps, once per task
     for (int i = 0; i < 8; ++i) mbar_init(BAR(B_HX + i), 2);    // the two owners of a row (team, quadrant), once per max
     *abort_smem = 0;
-    redo_flag[0] = 0;
-    redo_flag[1] = 0;
+    for (int i = 0; i < 4; ++i) redo_flag[i] = 0;
     fence_mbar_init();
     fence_proxy_async();
   }
   // the MMA reads all 128 rows of the Q region even when a query block has 64 rows: clear it once
-  for (int i = tid; i < G::Q_BYTES / 16; i += kThreadsOf<BLOCK>) reinterpret_cast<uint4*>(smem + G::OFF_Q)[i] = make_uint4(0, 0, 0, 0);
+  for (int i = tid; i < G::NQ * G::Q_BYTES / 16; i += kThreads) reinterpret_cast<uint4*>(smem + G::OFF_Q)[i] = make_uint4(0, 0, 0, 0);
   fence_proxy_async();
   if (warp == kPvWarp) {
     tmem_alloc(smem_u32(tmem_holder), G::TMEM_COLS);
@@ -527,11 +557,11 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   if (warp == kProducerWarp) {
     // ============================================================== producer
     if (lane == 0) { prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmV); prefetch_tmap(&tmK2); prefetch_tmap(&tmV2); }
-    uint32_t task_it = 0, q_it = 0, k_it = 0, v_it = 0;
+    uint32_t task_it = 0, q_it = 0, k_it = 0;
     int n_tiles = 0, n_pairs = 0;        // words 7 and 6 of the workspace: KV tiles (128 rows x 128 keys) and shared tiles this call ran
     bool ok = true;
-    uint32_t k_armed = 0, k_parity = 0, v_armed = 0, v_parity = 0;   // per stage: parity of the last load armed on it
-    bool q_armed = false; uint32_t q_armed_parity = 0;
+    uint32_t k_armed = 0, k_parity = 0;   // per stage: parity of the last load armed on it
+    uint32_t q_armed = 0, q_parity = 0;
     // the next task: a ticket from the global counter and the task it stands for (n = -1: none left)
     auto draw = [&](long long& t_out) -> Task {
       for (;;) {
@@ -591,49 +621,30 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       n_tiles += tk.n;
       n_pairs += G::KB == 2 && tk.row2 >= 0;
       // Q tile
-      ok = warp_wait(ctx, BAR(B_Q_EMPTY), (q_it & 1) ^ 1, 2);
+      const uint32_t qb = G::NQ == 2 ? q_it & 1 : 0, q_ph = (G::NQ == 2 ? q_it >> 1 : q_it) & 1, q_smem = sbase + G::OFF_Q + qb * G::Q_BYTES;
+      ok = warp_wait(ctx, BAR(B_Q_EMPTY + qb), q_ph ^ 1, 2);
       if (!ok) break;
       if (lane == 0) {
         const bool two = G::KB == 2 && tk.row2 >= 0;
-        mbar_expect_tx(BAR(B_Q_FULL), (two ? 2 : 1) * G::SLABS * G::BQ * 128);
+        mbar_expect_tx(BAR(B_Q_FULL + qb), (two ? 2 : 1) * G::SLABS * G::BQ * 128);
 #pragma unroll
         for (int s = 0; s < G::SLABS; ++s)
-          tma_load_3d(sbase + G::OFF_Q + s * 128 * 128, &tmQ, s * 64, tk.row * G::BQ, tk.h, BAR(B_Q_FULL));
+          tma_load_3d(q_smem + s * 128 * 128, &tmQ, s * 64, tk.row * G::BQ, tk.h, BAR(B_Q_FULL + qb));
         if (two) {
           // the partner's 64 rows go to rows 64..127 of the tile
 #pragma unroll
           for (int s = 0; s < G::SLABS; ++s)
-            tma_load_3d(sbase + G::OFF_Q + s * 128 * 128 + 64 * 128, &tmQ, s * 64, tk.row2 * G::BQ, tk.h, BAR(B_Q_FULL));
+            tma_load_3d(q_smem + s * 128 * 128 + 64 * 128, &tmQ, s * 64, tk.row2 * G::BQ, tk.h, BAR(B_Q_FULL + qb));
         }
       }
-      q_armed = true; q_armed_parity = q_it & 1;
+      q_armed |= 1u << qb; q_parity = (q_parity & ~(1u << qb)) | q_ph << qb;
       ++q_it;
       int chunk_base = -64, my_idx = 0;
-      if constexpr (G::SPLIT_LOADERS) {
-        // all K tiles of the task, as fast as the ring takes them; the V tiles come from a warp of
-        // their own (64-row shapes: a tile takes twice the list entries and boxes, and one warp
-        // for both streams was the limit of the whole kernel: -27 % cycles with two)
-        for (int j = 0; j < tk.n && ok; ++j) {
-          if (!drawn && j >= tk.n - kDrawAhead) { tk_next = draw(t_next); drawn = true; }
-          ok = load_kv_tile<G, BLOCK, true>(ctx, p, tk, p.drop_tile && t == 0 && j == 0, j, lane, sbase, BAR(B_K_FULL),
-                                            BAR(B_K_EMPTY), &tmK, &tmK2, k_it, k_armed, k_parity, chunk_base, my_idx);
-        }
-      } else {
-        // K tiles run three tiles ahead of the V tiles, like the MMAs that consume them; one warp
-        // for both streams paces the start of the next task (128-row shapes: an earlier start of
-        // the next task's loads costs more than a second loader gains, +2 % cycles)
-        int v_chunk_base = -64, v_my_idx = 0;
-        for (int j = 0; j < G::NSBUF && j < tk.n && ok; ++j)
-          ok = load_kv_tile<G, BLOCK, true>(ctx, p, tk, p.drop_tile && t == 0 && j == 0, j, lane, sbase, BAR(B_K_FULL),
-                                            BAR(B_K_EMPTY), &tmK, &tmK2, k_it, k_armed, k_parity, chunk_base, my_idx);
-        for (int j = 0; j < tk.n && ok; ++j) {
-          if (!drawn && j >= tk.n - kDrawAhead) { tk_next = draw(t_next); drawn = true; }
-          ok = load_kv_tile<G, BLOCK, false>(ctx, p, tk, false, j, lane, sbase, BAR(B_V_FULL), BAR(B_V_EMPTY), &tmV, &tmV2,
-                                             v_it, v_armed, v_parity, v_chunk_base, v_my_idx);
-          if (ok && j + G::NSBUF < tk.n)
-            ok = load_kv_tile<G, BLOCK, true>(ctx, p, tk, false, j + G::NSBUF, lane, sbase, BAR(B_K_FULL), BAR(B_K_EMPTY),
-                                              &tmK, &tmK2, k_it, k_armed, k_parity, chunk_base, my_idx);
-        }
+      // all K tiles of the task, as fast as the ring takes them
+      for (int j = 0; j < tk.n && ok; ++j) {
+        if (!drawn && j >= tk.n - kDrawAhead) { tk_next = draw(t_next); drawn = true; }
+        ok = load_kv_tile<G, BLOCK, true>(ctx, p, tk, p.drop_tile && t == 0 && j == 0, j, lane, sbase, BAR(B_K_FULL),
+                                          BAR(B_K_EMPTY), &tmK, &tmK2, k_it, k_armed, k_parity, chunk_base, my_idx);
       }
     }
     if (lane == 0 && !p.redo_pass) {
@@ -647,18 +658,14 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           long long t0 = clock64();
           while (!mbar_try_wait(BAR(B_K_FULL + st), (k_parity >> st) & 1) && clock64() - t0 < p.wait_limit / 4) {}
         }
-      for (int st = 0; st < G::NVS; ++st)
-        if (v_armed & (1u << st)) {
+      for (int st = 0; st < G::NQ; ++st)
+        if (q_armed & (1u << st)) {
           long long t0 = clock64();
-          while (!mbar_try_wait(BAR(B_V_FULL + st), (v_parity >> st) & 1) && clock64() - t0 < p.wait_limit / 4) {}
+          while (!mbar_try_wait(BAR(B_Q_FULL + st), (q_parity >> st) & 1) && clock64() - t0 < p.wait_limit / 4) {}
         }
-      if (q_armed) {
-        long long t0 = clock64();
-        while (!mbar_try_wait(BAR(B_Q_FULL), q_armed_parity) && clock64() - t0 < p.wait_limit / 4) {}
-      }
     }
-  } else if (G::SPLIT_LOADERS && warp == kVLoadWarp) {
-    // ============================================================== V tile loader (64-row shapes)
+  } else if (warp == kVLoadWarp) {
+    // ============================================================== V tile loader
     uint32_t task_slot = 0, task_ph = 0, v_it = 0, v_armed = 0, v_parity = 0;
     bool ok = true;
     while (ok) {
@@ -692,7 +699,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     // Every operand of a tcgen05 instruction stays warp-uniform in the compiler's eyes
     // (shuffle-broadcast values, compare-and-reset ring positions).
     constexpr uint32_t IDESC_QK = make_idesc(128, G::BK, false);
-    uint32_t task_slot = 0, task_ph = 0, q_ph = 0, k_st = 0, k_ph = 0, sb = 0, free_bits = 0, first_uses = G::NSBUF;
+    uint32_t task_slot = 0, task_ph = 0, q_it = 0, k_st = 0, k_ph = 0, sb = 0, free_bits = 0, first_uses = G::NSBUF;
     const uint64_t qdesc0 = make_desc(sbase + G::OFF_Q, 16, 1024);
     const uint64_t kdesc0 = make_desc(sbase + G::OFF_K, 16, 1024);
     bool ok = true;
@@ -706,9 +713,11 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       task_ph ^= (task_slot == 0);
       if (n < 0) break;
       if (n == 0) continue;
-      ok = warp_wait(ctx, BAR(B_Q_FULL), q_ph, 11);
+      const uint32_t qb = G::NQ == 2 ? q_it & 1 : 0;
+      ok = warp_wait(ctx, BAR(B_Q_FULL + qb), (G::NQ == 2 ? q_it >> 1 : q_it) & 1, 11);
       if (!ok) break;
-      q_ph ^= 1;
+      ++q_it;
+      const uint64_t qdesc = qdesc0 + (uint64_t)(qb * (uint32_t)(G::Q_BYTES >> 4));
       for (int j = 0; j < n && ok; ++j) {
         ok = warp_wait(ctx, BAR(B_K_FULL + k_st), k_ph, 12);
         if (!ok) break;
@@ -728,12 +737,12 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           const uint32_t d_s = tmem_base + sb * G::S_STRIDE;
 #pragma unroll
           for (int k = 0; k < D / 16; ++k) {
-            umma_bf16(d_s, qdesc0 + (uint64_t)(((k / 4) * 128 * 128 + (k % 4) * 32) >> 4),
+            umma_bf16(d_s, qdesc + (uint64_t)(((k / 4) * 128 * 128 + (k % 4) * 32) >> 4),
                       kd + (uint64_t)(((k / 4) * G::KV_SLAB_BYTES + (k % 4) * 32) >> 4), IDESC_QK, k > 0);
           }
           tc_commit(BAR(B_K_EMPTY + k_st));
           tc_commit(BAR(B_S_FULL + sb));
-          if (j == n - 1) tc_commit(BAR(B_Q_EMPTY));
+          if (j == n - 1) tc_commit(BAR(B_Q_EMPTY + qb));
         }
         if (++k_st == (uint32_t)G::NKS) { k_st = 0; k_ph ^= 1; }
         if (++sb == (uint32_t)G::NSBUF) sb = 0;
@@ -830,13 +839,21 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     // epilogue adds the four partial sums of a row.
     const int sw = warp - kSoftmaxWarp0;       // 0..15
     const int quad = warp & 3;                 // tensor-memory lane quadrant this warp may access
-    const int team = (sw >> 2) & 1;            // owns blocks j with (j & 1) == team
-    const int half = sw >> 3;                  // column half of S; epilogue: quarter team*2+half of the O columns
+    const int team = (sw >> 2) & 1;            // owns the tiles whose number over the CTA's life has this parity
+    const int half = sw >> 3;                  // column half of S; epilogue: the same half of the O columns
     const int r = quad * 32 + lane;            // row of the 128-row MMA tile
     const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
     const uint32_t o_row = tmem_base + lane_addr + G::O_COL;
-    const int part = team * 2 + half;
-    uint32_t task_it = 0, s_phase = 0, o_it = 0, mx_phase = 0, hx_it = 0, sb = 0;   // s_phase bit b: parity of the uses of S[b] so far
+    // Tiles alternate between the teams across the boundary of two tasks: the team of a task's last tile
+    // runs its epilogue (waits for the last P V, reads O, stores it) while the other one is already at the
+    // next task's first tile, whose max pass, exponentials and P would otherwise come after all of that.
+    // (With both teams in the epilogue a task cost ~6,000 clk beyond its tiles.)  What a team leaves for
+    // the other (running reference, partial sums, redo flag) therefore lies in four slots each: three S
+    // buffers let a team run ahead of the other's epilogue by two of its own tiles, hence two tasks.
+    uint32_t task_it = 0, o_it = 0, mx_phase = 0, hx_it = 0;
+    uint32_t g0 = 0;                           // tiles before this task
+    uint32_t sb = (uint32_t)team, s_ph = 0;    // S buffer of this team's next tile and the parity of that use
+    auto next_buffer = [&]() { sb += 2; if (sb >= (uint32_t)G::NSBUF) { sb -= (uint32_t)G::NSBUF; s_ph ^= 1; } };
     bool ok = true;
     while (ok) {
       const uint32_t slot = task_it & 1, ph = (task_it >> 1) & 1;
@@ -845,8 +862,8 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       const Task tk = tasks[slot];
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR(B_TASK_EMPTY + slot));
-      float2* exb = ex + (task_it & 1) * 512;
-      const uint32_t rslot = task_it & 1;
+      float2* exb = ex + (o_it & 3) * 512;
+      const uint32_t rslot = o_it & 3, ex_bar = B_EX + quad + 4 * (o_it & 3), ex_ph = (o_it >> 2) & 1;
       ++task_it;
       if (tk.n < 0) break;
       // rows 64..127 of the tile belong to the partner block of a pair (64-row blocks only)
@@ -856,41 +873,41 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       // rows 64..127 of a tile that no second block shares hold nothing: their warps only keep
       // the barriers of the tile going (each output row of an MMA depends on its own row of S / P alone)
       const bool idle = G::KB == 2 && quad >= 2 && tk.row2 < 0;
-      __nv_bfloat16* o_ptr = p.O + (size_t)tk.h * p.o_stride_h + (size_t)q_tok * p.o_stride_t + part * G::CO;
+      __nv_bfloat16* o_ptr = p.O + (size_t)tk.h * p.o_stride_h + (size_t)q_tok * p.o_stride_t + half * G::CO;
       if (tk.n == 0) {
-        if (row_live) {
+        if (row_live && team == 0) {
 #pragma unroll
           for (int c = 0; c < G::CO / 8; ++c) reinterpret_cast<uint4*>(o_ptr)[c] = make_uint4(0, 0, 0, 0);
-          if (p.lse && part == 0) p.lse[(size_t)tk.h * p.seq_q + q_tok] = -INFINITY;
+          if (p.lse && half == 0) p.lse[(size_t)tk.h * p.seq_q + q_tok] = -INFINITY;
         }
         continue;
       }
       // l_run: sum over this thread's columns of this team's blocks, relative to the reference m_ref
       float m_ref = -INFINITY, l_run = 0.f;
-      for (int j = 0; j < tk.n && ok; ++j) {
-        const uint32_t par = (uint32_t)j & 1u;
-        if ((int)par == team) {
-          ok = warp_wait(ctx, BAR(B_S_FULL + sb), (s_phase >> sb) & 1u, 21);
-          if (!ok) break;
-          if (idle) {
-            if (lane == 0) mbar_arrive(BAR(B_P_FULL + sb * 2 + half));
-            s_phase ^= 1u << sb;
-            if (++sb == (uint32_t)G::NSBUF) sb = 0;
-            continue;
-          }
+      const int last = tk.n - 1;
+      for (int j = (int)((g0 ^ (uint32_t)team) & 1u); j < tk.n; j += 2) {
+        const uint32_t g = g0 + (uint32_t)j;
+        ok = warp_wait(ctx, BAR(B_S_FULL + sb), s_ph, 21);
+        if (!ok) break;
+        if (idle) {
+          if (lane == 0) mbar_arrive(BAR(B_P_FULL + sb * 2 + half));
+          next_buffer();
+          continue;
+        }
+        {
           tc_fence_after();
           const uint32_t s_addr = tmem_base + lane_addr + sb * G::S_STRIDE + half * G::HC;
-          const bool ragged = j == tk.n - 1 && tk.tail_valid < G::BK;
-          const int col0 = half * G::HC;       // first key of the block this thread looks at
+          const bool ragged = j == last && tk.tail_valid < G::BK;
+          if (ragged) mask_scores<G::NCH>(s_addr, tk.tail_valid - half * G::HC);   // keys beyond seq_kv (ragged last block) do not exist
           // ---- pass 1: row max (the values are loaded again for the exponentials: a second
           // tensor-memory load is cheaper than keeping them in registers)
-          // In the first pass over the tasks (FAST) only blocks 0 and 1 of a task take a max and
-          // may move the reference; from block 2 on both teams keep the reference of block 1.
+          // In the first pass over the tasks (FAST) only the first MAX_TILES tiles of a task take a max and
+          // may move the reference; both teams keep it from there on.
           // Any reference gives the same softmax as long as nothing overflows, so the later
-          // blocks only watch the sum of the exponentials they produce: if it ever reaches 2^24 the
+          // tiles only watch the sum of the exponentials they produce: if it ever reaches 2^60 the
           // task is put on a list and computed again by the second launch, which takes the
-          // max of every block (the rule of the paper's online softmax).
-          const bool fixed_ref = FAST && j >= 2;
+          // max of every tile (the rule of the paper's online softmax).
+          const bool fixed_ref = FAST && j >= G::MAX_TILES;
           float mloc = -INFINITY;
           if (!fixed_ref) {
 #pragma unroll 1
@@ -898,22 +915,17 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
               uint32_t sv[G::CH];
               WAVEAL_TMEM_LD32(s_addr + ch * G::CH, sv, 0);
               WAVEAL_TMEM_WAIT_LD32(sv, 0);
-              // scores of keys beyond seq_kv (ragged last block) do not exist
-              if (ragged) {
+              float mx4[4];
 #pragma unroll
-                for (int c = 0; c < G::CH; ++c)
-                  if (col0 + ch * G::CH + c >= tk.tail_valid) sv[c] = __float_as_uint(-INFINITY);
+              for (int i = 0; i < 4; ++i) mx4[i] = __uint_as_float(sv[i]);
+#pragma unroll
+              for (int c = 4; c < G::CH - 4; c += 8) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) mx4[i] = fmax3(mx4[i], __uint_as_float(sv[c + 2 * i]), __uint_as_float(sv[c + 2 * i + 1]));
               }
-              float mx8[8];
 #pragma unroll
-              for (int i = 0; i < 8; ++i) mx8[i] = __uint_as_float(sv[i]);
-#pragma unroll
-              for (int c = 8; c < G::CH; c += 8) {
-#pragma unroll
-                for (int i = 0; i < 8; ++i) mx8[i] = fmaxf(mx8[i], __uint_as_float(sv[c + i]));
-              }
-              mloc = fmaxf(mloc, fmaxf(fmaxf(fmaxf(mx8[0], mx8[1]), fmaxf(mx8[2], mx8[3])),
-                                       fmaxf(fmaxf(mx8[4], mx8[5]), fmaxf(mx8[6], mx8[7]))));
+              for (int i = 0; i < 4; ++i) mx4[i] = fmaxf(mx4[i], __uint_as_float(sv[G::CH - 4 + i]));
+              mloc = fmax3(fmax3(mx4[0], mx4[1], mx4[2]), mx4[3], mloc);
             }
             // the other owner of the row (same team and quadrant, other column half)
             // (two buffers by use parity: the partner's next value cannot land on one not yet read)
@@ -928,11 +940,13 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           }
           // ---- the row's reference after block j-1, from the other team
           float m_prev = m_ref;
-          if (j > 0 && (!fixed_ref || j == 2)) {
-            // that team's arrival for block j-1 is phase number (arrivals of that parity so far) - 1
-            ok = warp_wait(ctx, BAR(B_MX + quad * 2 + (par ^ 1u)), ((mx_phase >> (par ^ 1u)) & 1u) ^ 1u, 24);
+          if (j > 0 && !(FAST && j > G::MAX_TILES)) mx_phase ^= 1u << ((g - 1) & 3);   // the other team's arrival for tile g-1
+          if (j > 0 && (!fixed_ref || j == G::MAX_TILES)) {
+            // that team's arrival for tile g-1 is phase number (arrivals of that slot so far) - 1
+            const uint32_t mx = (g - 1) & 3;
+            ok = warp_wait(ctx, BAR(B_MX + quad * 4 + mx), ((mx_phase >> mx) & 1u) ^ 1u, 24);
             if (!ok) break;
-            m_prev = mpub[((j - 1) & 3) * 128 + r];
+            m_prev = mpub[((g - 1) & 3) * 128 + r];
           }
           const float m_cand = fmaxf(m_prev, mloc * p.sl2);
           // keep the stale reference unless it is exceeded by more than 2^8 (exact: the final
@@ -941,11 +955,11 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           const bool grow = !fixed_ref && __any_sync(0xffffffffu, m_cand > m_prev + 8.0f);
           const float m_new = grow ? m_cand : m_prev;
           if (!fixed_ref && half == 0) {
-            // (slot j mod 4: the owner of block j+4 cannot get there before both owners of block
-            // j+1 have read this one)
-            mpub[(j & 3) * 128 + r] = m_new;
+            // (slot and barrier g mod 4: the owner of tile g+4 cannot get there before both owners of
+            // tile g+1 have read this one, which its S buffer waits for)
+            mpub[(g & 3) * 128 + r] = m_new;
             __syncwarp();
-            if (lane == 0) mbar_arrive(BAR(B_MX + quad * 2 + par));
+            if (lane == 0) mbar_arrive(BAR(B_MX + quad * 4 + (g & 3)));
           }
           if (m_new != m_ref) {
             l_run *= (m_ref == -INFINITY) ? 0.f : ex2(m_ref - m_new);
@@ -958,7 +972,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           // the row's output columns.
           if (grow && j > 0) {
             const uint32_t sbp = sb == 0 ? (uint32_t)G::NSBUF - 1u : sb - 1u;
-            ok = warp_wait(ctx, BAR(B_S_FREE + sbp), ((s_phase >> sbp) & 1u) ^ 1u, 22);
+            ok = warp_wait(ctx, BAR(B_S_FREE + sbp), sb == 0 ? s_ph ^ 1u : s_ph, 22);
             if (!ok) break;
             tc_fence_after();
             const float alpha = ex2(m_prev - m_new);
@@ -987,16 +1001,11 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             uint32_t sv[G::CH];
             WAVEAL_TMEM_LD32(s_addr + ch * G::CH, sv, 0);
             WAVEAL_TMEM_WAIT_LD32(sv, 0);
-            if (ragged) {
-#pragma unroll
-              for (int c = 0; c < G::CH; ++c)
-                if (col0 + ch * G::CH + c >= tk.tail_valid) sv[c] = __float_as_uint(-INFINITY);
-            }
             uint32_t pk[G::CH / 2];
 #pragma unroll
             for (int c = 0; c < G::CH; c += 2) {
               float e0, e1;
-              if (kPolyEvery > 0 && ((c >> 1) % (kPolyEvery > 0 ? kPolyEvery : 1)) == (kPolyEvery > 0 ? kPolyEvery : 1) - 1) {
+              if ((c >> 1) % kPolyEvery == kPolyEvery - 1) {
                 ex2_fma2(e0, e1, __uint_as_float(sv[c]), __uint_as_float(sv[c + 1]), a128, b128);
               } else {
                 float x0, x1;
@@ -1011,7 +1020,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           const float l_blk = (ls4[0] + ls4[1]) + (ls4[2] + ls4[3]);
           l_run += l_blk;
           // all terms are positive (the transcendental unit returns +inf on overflow, the
-          // polynomial share saturates at 2^28), so a sum below 2^24 bounds every exponent it
+          // polynomial share saturates at 2^64), so a sum below 2^60 bounds every exponent it
           // covers; at or above it (or not a number) the fixed reference is too far off:
           // redo the task
           if (fixed_ref && __any_sync(0xffffffffu, !(l_blk < kRedoLimit))) redo_flag[rslot] = 1;
@@ -1020,27 +1029,41 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           __syncwarp();
           if (lane == 0) mbar_arrive(BAR(B_P_FULL + sb * 2 + half));
         }
-        // both teams count every block
-        s_phase ^= 1u << sb;
-        if (!(FAST && j >= 2) && !idle) mx_phase ^= 1u << par;   // one flip per arrival on that parity's barrier
-        if (++sb == (uint32_t)G::NSBUF) sb = 0;
+        if (!(FAST && j >= G::MAX_TILES)) mx_phase ^= 1u << (g & 3);                  // one flip per arrival on that slot's barrier
+        next_buffer();
       }
       if (!ok) break;
-      // ---- epilogue: O / l at the original row position; l = the four partial sums of the row
-      // brought to the final reference (the larger of the two teams', references never shrink)
-      // (the partial sums are final once the thread's last tile is done: publish them before the
-      // wait for the last P V, so that nothing but the load of O stands between that MMA and the
-      // first one of the next task)
-      exb[part * 128 + r] = make_float2(m_ref, l_run);
+      // ---- epilogue: O / l at the original row position; l = the four partial sums of the row (by parity of
+      // the tile in the task, so that the result does not depend on which team had which) brought to
+      // the final reference (the larger of the two parities', references never shrink)
+      // (a thread's partial sum is final once its last tile is done)
+      exb[(((team ^ (int)g0) & 1) * 2 + half) * 128 + r] = make_float2(m_ref, l_run);
       __syncwarp();
-      if (lane == 0) mbar_arrive(BAR(B_EX + quad));
-      ok = warp_wait(ctx, BAR(B_O_FULL), o_it & 1, 23);
-      if (!ok) break;
+      if (lane == 0) mbar_arrive(BAR(ex_bar));
+      const bool mine = (int)((g0 + (uint32_t)last) & 1u) == team;
+      if (!mine && !idle && !(FAST && last >= G::MAX_TILES)) mx_phase ^= 1u << ((g0 + (uint32_t)last) & 3);
+      g0 += (uint32_t)tk.n;
+      const uint32_t o_ph = o_it & 1;
       ++o_it;
+      if (!mine) continue;
+      // All four warps of this lane quadrant have left their sums; the other team's are there long
+      // before.  (This wait stands before the one for O: a team that has run ahead could otherwise
+      // take the completion of the task before the previous one for that of its own.)  Bounded
+      // like every other wait, so that a warp whose partners gave up does not stay behind.
+      ok = warp_wait(ctx, BAR(ex_bar), ex_ph, 25);
+      if (!ok) break;
+      const float2 e00 = exb[0 * 128 + r], e01 = exb[1 * 128 + r], e10 = exb[2 * 128 + r], e11 = exb[3 * 128 + r];
+      const float m0 = fmaxf(e00.x, e01.x), m1 = fmaxf(e10.x, e11.x);     // the two owners of a parity agree; a parity
+      const float m_all = fmaxf(m0, m1);                                   // without tiles (n == 1) has -inf
+      const float a0 = (m0 == -INFINITY) ? 0.f : ex2(m0 - m_all);
+      const float a1 = (m1 == -INFINITY) ? 0.f : ex2(m1 - m_all);
+      const float l_tot = a0 * (e00.y + e01.y) + a1 * (e10.y + e11.y);
+      const float inv_l = 1.0019531f / l_tot;    // the sums carry the centring factor 1 + 2^-9
+      ok = warp_wait(ctx, BAR(B_O_FULL), o_ph, 23);
+      if (!ok) break;
       tc_fence_after();
-      if (FAST && sw == 0 && lane == 0 && redo_flag[rslot]) {
-        // every warp's blocks of this task lie before O_FULL; the slot is used again two tasks
-        // later, after this warp's O_FREE arrival below
+      if (FAST && half == 0 && quad == 0 && lane == 0 && redo_flag[rslot]) {
+        // every warp's tiles of this task lie before O_FULL; the slot is used again four tasks later
         const int e = atomicAdd(&p.ws[2], (G::KB == 2 && tk.row2 >= 0) ? 2 : 1);
         p.ws[8 + 2 * e] = tk.h;
         p.ws[9 + 2 * e] = tk.row;
@@ -1048,23 +1071,14 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         redo_flag[rslot] = 0;
       }
       uint32_t ov[G::CO];
-      static_assert(G::CO == 32 || G::CO == 16, "a quarter of head_dim 128 or 64");
-      if constexpr (G::CO == 32) { WAVEAL_TMEM_LD32(o_row + part * G::CO, ov, 0); WAVEAL_TMEM_WAIT_LD32(ov, 0); }
-      else { WAVEAL_TMEM_LD16(o_row + part * G::CO, ov, 0); WAVEAL_TMEM_WAIT_LD16(ov, 0); }
+      static_assert(G::CO == 64 || G::CO == 32, "half of head_dim 128 or 64");
+      WAVEAL_TMEM_LD32(o_row + half * G::CO, ov, 0);
+      if constexpr (G::CO == 64) WAVEAL_TMEM_LD32(o_row + half * G::CO + 32, ov, 32);
+      WAVEAL_TMEM_WAIT_LD32(ov, 0);
+      if constexpr (G::CO == 64) WAVEAL_TMEM_WAIT_LD32(ov, 32);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR(B_O_FREE));
-      // the other three warps of this lane quadrant have written their parts: a bounded wait
-      // like every other, so that a warp whose partners gave up does not stay behind
-      ok = warp_wait(ctx, BAR(B_EX + quad), (o_it & 1) ^ 1, 25);
-      if (!ok) break;
-      const float2 e00 = exb[0 * 128 + r], e01 = exb[1 * 128 + r], e10 = exb[2 * 128 + r], e11 = exb[3 * 128 + r];
-      const float m0 = fmaxf(e00.x, e01.x), m1 = fmaxf(e10.x, e11.x);     // the two owners of a team agree; a team
-      const float m_all = fmaxf(m0, m1);                                   // without blocks (n == 1) has -inf
-      const float a0 = (m0 == -INFINITY) ? 0.f : ex2(m0 - m_all);
-      const float a1 = (m1 == -INFINITY) ? 0.f : ex2(m1 - m_all);
-      const float l_tot = a0 * (e00.y + e01.y) + a1 * (e10.y + e11.y);
-      const float inv_l = 1.0019531f / l_tot;    // the sums carry the centring factor 1 + 2^-9
       if (row_live) {
         // a thread holds a piece of one row, so a store instruction of a warp touches 32 rows:
         // its cost in the memory pipe is per row, not per byte.  32-byte stores halve the number
@@ -1083,7 +1097,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           for (int c = 0; c < G::CO / 2; c += 4)
             *reinterpret_cast<uint4*>(o_ptr + 2 * c) = make_uint4(w[c], w[c + 1], w[c + 2], w[c + 3]);
         }
-        if (p.lse && part == 0) p.lse[(size_t)tk.h * p.seq_q + q_tok] = (m_all + log2f(l_tot) - 0.0028150156f) * 0.6931471805599453f;
+        if (p.lse && half == 0) p.lse[(size_t)tk.h * p.seq_q + q_tok] = (m_all + log2f(l_tot) - 0.0028150156f) * 0.6931471805599453f;
       }
     }
   }
@@ -1353,7 +1367,7 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   WAVEAL_CUDA_OK(cudaGetLastError());
   if (d->flags & WAVEAL_ATTN_ONLINE_MAX_ONLY) {
     p.redo_pass = 0;
-    k_bsattn_fwd<BLOCK, D, false><<<(unsigned)grid, kThreadsOf<BLOCK>, G::SMEM_BYTES, st>>>(tq, tk, tv, tk2, tv2, p);
+    k_bsattn_fwd<BLOCK, D, false><<<(unsigned)grid, kThreads, G::SMEM_BYTES, st>>>(tq, tk, tv, tk2, tv2, p);
     WAVEAL_CUDA_OK(cudaGetLastError());
     waveal::launch_counter() = 2;
     return WAVEAL_OK;
@@ -1361,10 +1375,10 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   // first pass: reference fixed after the first two blocks of a task; second pass: the tasks the
   // first one listed (normally none: its CTAs leave at once), max of every block
   p.redo_pass = 0;
-  k_bsattn_fwd<BLOCK, D, true><<<(unsigned)grid, kThreadsOf<BLOCK>, G::SMEM_BYTES, st>>>(tq, tk, tv, tk2, tv2, p);
+  k_bsattn_fwd<BLOCK, D, true><<<(unsigned)grid, kThreads, G::SMEM_BYTES, st>>>(tq, tk, tv, tk2, tv2, p);
   WAVEAL_CUDA_OK(cudaGetLastError());
   p.redo_pass = 1;
-  k_bsattn_fwd<BLOCK, D, false><<<(unsigned)grid, kThreadsOf<BLOCK>, G::SMEM_BYTES, st>>>(tq, tk, tv, tk2, tv2, p);
+  k_bsattn_fwd<BLOCK, D, false><<<(unsigned)grid, kThreads, G::SMEM_BYTES, st>>>(tq, tk, tv, tk2, tv2, p);
   WAVEAL_CUDA_OK(cudaGetLastError());
   waveal::launch_counter() = 3;
   return WAVEAL_OK;
