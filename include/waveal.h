@@ -216,7 +216,8 @@ waveal_status waveal_bsattn_workspace_bytes(const waveal_attn_desc* desc /*host*
  * for query block i of head h, O = softmax(scale * Q_i K_sel^T) V_sel over the tokens of
  * the K/V blocks listed for (h, i), visited in the listed (ascending) order.
  * Persistent CTAs take (head, position) tickets in head-major order and process query
- * block row_order[h][position] (Algorithm 2 output; NULL = natural order); each output
+ * block row_order[h][position] (Algorithm 2 output; NULL = natural order; the last 1,024 tickets of a
+ * call, seven per SM, are handed out longest list first, so that no SM is left with a long row at the end); each output
  * tile is written at its original rows, so no inverse permutation pass exists.
  * Q, K, V, O: dev bf16, 16-byte aligned, strides multiples of 8 elements, head_dim
  * contiguous; query tokens >= seq_q are not written; keys >= seq_kv are ignored.

@@ -1154,16 +1154,73 @@ __device__ __forceinline__ void clear_counters(const AttnParams& p) {
   if (blockIdx.x == 0 && threadIdx.x < 8) p.ws[threadIdx.x] = 0;
 }
 
-__global__ void k_task_table(AttnParams p, int block_k, Task* table) {
+// The last kTailTasks tickets of a call are handed out longest first (1,024 = 7 per SM).  In the planned
+// or natural order a long row may start last and leave the other SMs waiting for it: the row lengths of
+// the masks in use spread over a factor of ten.  Calls of a few tasks per SM gain most (5 heads of 256
+// rows: 655k -> 501k cycles), the largest lose nothing: before the last 1,024 tickets the order is the
+// caller's, and no result depends on it.  A histogram of 1,024 lengths is enough (which of two tasks of
+// about the same length goes first makes no difference).
+constexpr int kTailTasks = 1024;
+__device__ __forceinline__ int tail_place(int n, bool live) {            // called by a block of kTailTasks threads
+  __shared__ int bins[kTailTasks], warp_sum[kTailTasks / 32], longest;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  bins[tid] = 0;
+  if (tid == 0) longest = 1;
+  __syncthreads();
+  const int w = __reduce_max_sync(0xffffffffu, live ? n : 0);
+  if (lane == 0) atomicMax(&longest, w);
+  __syncthreads();
+  // absorbed and empty tasks last
+  const int bin = kTailTasks - 1 - (n <= 0 ? 0 : (int)((long long)n * (kTailTasks - 1) / longest));
+  const int at = live ? atomicAdd(&bins[bin], 1) : 0;
+  __syncthreads();
+  const int c = bins[tid];
+  int incl = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  if (lane == 31) warp_sum[warp] = incl;
+  __syncthreads();
+  int before = 0;
+  for (int i = 0; i < warp; ++i) before += warp_sum[i];
+  bins[tid] = before + incl - c;
+  __syncthreads();
+  return bins[bin] + at;
+}
+
+__global__ void __launch_bounds__(kTailTasks) k_task_table(AttnParams p, int block_k, Task* table) {
   clear_counters(p);
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= p.total_tasks) return;
-  int h, pos;
-  if (p.interleaved) { pos = (int)(t / p.heads); h = (int)(t % p.heads); }
-  else { h = (int)(t / p.m_b); pos = (int)(t % p.m_b); }
-  Task tk = make_task(p, block_k, h, pos);
-  tk.pad2 = 0;
-  table[t] = tk;
+  // block 0: the last kTailTasks tickets (or all of them); the others the rest in order
+  const long long first_tail = p.total_tasks > kTailTasks ? p.total_tasks - kTailTasks : 0;
+  const long long t = blockIdx.x == 0 ? first_tail + threadIdx.x : (long long)(blockIdx.x - 1) * kTailTasks + threadIdx.x;
+  const bool live = blockIdx.x == 0 ? t < p.total_tasks : t < first_tail;
+  Task tk{};
+  if (live) {
+    int h, pos;
+    if (p.interleaved) { pos = (int)(t / p.heads); h = (int)(t % p.heads); }
+    else { h = (int)(t / p.m_b); pos = (int)(t % p.m_b); }
+    tk = make_task(p, block_k, h, pos);
+    tk.pad2 = 0;
+  }
+  if (blockIdx.x == 0) {
+    const int at = tail_place(tk.n, live);
+    if (live) table[first_tail + at] = tk;
+  } else if (live) {
+    table[t] = tk;
+  }
+}
+
+// the same for a table that is there already (64-row blocks: pairs are formed first)
+__global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* table) {
+  const long long first_tail = p.total_tasks > kTailTasks ? p.total_tasks - kTailTasks : 0;
+  const long long t = first_tail + threadIdx.x;
+  const bool live = t < p.total_tasks;
+  Task tk{};
+  if (live) tk = table[t];
+  const int at = tail_place(tk.n, live);
+  if (live) table[first_tail + at] = tk;
 }
 
 // The same for 64-row query blocks, where two blocks with the very same list share one 128-row tile.
@@ -1358,18 +1415,25 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   p.drop_tile = 0;
   if (d->flags & WAVEAL_ATTN_SELFTEST_LOST_TILE) { p.wait_limit = kSelfTestCycles; p.drop_tile = 1; }
   p.no_pairing = (d->flags & WAVEAL_ATTN_NO_ROW_PAIRING) ? 1 : 0;
+  int launches = 1;
   if (BLOCK == 64) {
     const int chunks = (p.m_b + kPairRows - 1) / kPairRows;
     k_task_table_pairs<<<(unsigned)((long long)p.heads * chunks), kPairThreads, 0, st>>>(p, table, chunks);
+    if (p.total_tasks > sms) {            // (else all tasks start at once)
+      WAVEAL_CUDA_OK(cudaGetLastError());
+      k_sort_tail<<<1, kTailTasks, 0, st>>>(p, table);
+      ++launches;
+    }
   } else {
-    k_task_table<<<(unsigned)((p.total_tasks + 255) / 256), 256, 0, st>>>(p, BLOCK, table);
+    const long long before_tail = p.total_tasks > kTailTasks ? p.total_tasks - kTailTasks : 0;
+    k_task_table<<<(unsigned)(1 + (before_tail + kTailTasks - 1) / kTailTasks), kTailTasks, 0, st>>>(p, BLOCK, table);
   }
   WAVEAL_CUDA_OK(cudaGetLastError());
   if (d->flags & WAVEAL_ATTN_ONLINE_MAX_ONLY) {
     p.redo_pass = 0;
     k_bsattn_fwd<BLOCK, D, false><<<(unsigned)grid, kThreads, G::SMEM_BYTES, st>>>(tq, tk, tv, tk2, tv2, p);
     WAVEAL_CUDA_OK(cudaGetLastError());
-    waveal::launch_counter() = 2;
+    waveal::launch_counter() = launches + 1;
     return WAVEAL_OK;
   }
   // first pass: reference fixed after the first two blocks of a task; second pass: the tasks the
@@ -1380,7 +1444,7 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   p.redo_pass = 1;
   k_bsattn_fwd<BLOCK, D, false><<<(unsigned)grid, kThreads, G::SMEM_BYTES, st>>>(tq, tk, tv, tk2, tv2, p);
   WAVEAL_CUDA_OK(cudaGetLastError());
-  waveal::launch_counter() = 3;
+  waveal::launch_counter() = launches + 2;
   return WAVEAL_OK;
 }
 
