@@ -493,6 +493,8 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   const uint32_t sbase = smem_u32(smem);
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // provably warp-uniform role index
+  waveal::let_next_kernel_start();
+  if (p.redo_pass) waveal::wait_for_previous_kernel();
 
   // second pass with nothing listed (or after an abort): leave before anything is set up
   if (p.redo_pass && (p.ws[2] == 0 || p.ws[1] != 0)) return;
@@ -550,6 +552,8 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_holder, 0);
+  // tickets, table and counters are the work of the kernel before this one
+  waveal::wait_for_previous_kernel();
 
   // Every role walks the same sequence of tasks (query blocks) and, inside a task, of KV blocks;
   // block number g (counted over the CTA's whole life) uses S buffer g mod 3, K stage g mod NKS
@@ -1170,9 +1174,12 @@ __device__ __forceinline__ int tail_place(int n, bool live) {            // call
   const int w = __reduce_max_sync(0xffffffffu, live ? n : 0);
   if (lane == 0) atomicMax(&longest, w);
   __syncthreads();
-  // absorbed and empty tasks last
+  // absorbed and empty tasks last.  One atomic per warp and length (rows of one length are common)
   const int bin = kTailTasks - 1 - (n <= 0 ? 0 : (int)((long long)n * (kTailTasks - 1) / longest));
-  const int at = live ? atomicAdd(&bins[bin], 1) : 0;
+  const unsigned same = __match_any_sync(0xffffffffu, live ? bin : -1 - lane);
+  int at = 0;
+  if (live && lane == __ffs(same) - 1) at = atomicAdd(&bins[bin], __popc(same));
+  at = __shfl_sync(0xffffffffu, at, __ffs(same) - 1) + __popc(same & ((1u << lane) - 1u));
   __syncthreads();
   const int c = bins[tid];
   int incl = c;
@@ -1183,14 +1190,14 @@ __device__ __forceinline__ int tail_place(int n, bool live) {            // call
   }
   if (lane == 31) warp_sum[warp] = incl;
   __syncthreads();
-  int before = 0;
-  for (int i = 0; i < warp; ++i) before += warp_sum[i];
+  const int before = __reduce_add_sync(0xffffffffu, lane < warp ? warp_sum[lane] : 0);
   bins[tid] = before + incl - c;
   __syncthreads();
   return bins[bin] + at;
 }
 
 __global__ void __launch_bounds__(kTailTasks) k_task_table(AttnParams p, int block_k, Task* table) {
+  waveal::let_next_kernel_start();
   clear_counters(p);
   // block 0: the last kTailTasks tickets (or all of them); the others the rest in order
   const long long first_tail = p.total_tasks > kTailTasks ? p.total_tasks - kTailTasks : 0;
@@ -1214,6 +1221,8 @@ __global__ void __launch_bounds__(kTailTasks) k_task_table(AttnParams p, int blo
 
 // the same for a table that is there already (64-row blocks: pairs are formed first)
 __global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* table) {
+  waveal::let_next_kernel_start();
+  waveal::wait_for_previous_kernel();
   const long long first_tail = p.total_tasks > kTailTasks ? p.total_tasks - kTailTasks : 0;
   const long long t = first_tail + threadIdx.x;
   const bool live = t < p.total_tasks;
@@ -1243,6 +1252,7 @@ __global__ void __launch_bounds__(kPairThreads) k_task_table_pairs(AttnParams p,
   __shared__ int s_mate_row[kPairRows], s_mate_pos[kPairRows], s_same[kPairRows];   // its row; its position here, -1: elsewhere
   __shared__ int s_full[kPairRows];                 // positions of the full rows of this block, in order
   __shared__ int s_before, s_prev, s_next, s_n_full;
+  waveal::let_next_kernel_start();
   clear_counters(p);
   const int h = blockIdx.x / chunks, c0 = (blockIdx.x - h * chunks) * kPairRows, tid = threadIdx.x;
   const int lane = tid & 31, warp = tid >> 5;
@@ -1421,7 +1431,7 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
     k_task_table_pairs<<<(unsigned)((long long)p.heads * chunks), kPairThreads, 0, st>>>(p, table, chunks);
     if (p.total_tasks > sms) {            // (else all tasks start at once)
       WAVEAL_CUDA_OK(cudaGetLastError());
-      k_sort_tail<<<1, kTailTasks, 0, st>>>(p, table);
+      WAVEAL_CUDA_OK(waveal::launch_chained(k_sort_tail, dim3(1), kTailTasks, 0, st, p, table));
       ++launches;
     }
   } else {
@@ -1431,19 +1441,16 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   WAVEAL_CUDA_OK(cudaGetLastError());
   if (d->flags & WAVEAL_ATTN_ONLINE_MAX_ONLY) {
     p.redo_pass = 0;
-    k_bsattn_fwd<BLOCK, D, false><<<(unsigned)grid, kThreads, G::SMEM_BYTES, st>>>(tq, tk, tv, tk2, tv2, p);
-    WAVEAL_CUDA_OK(cudaGetLastError());
+    WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, false>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, p));
     waveal::launch_counter() = launches + 1;
     return WAVEAL_OK;
   }
   // first pass: reference fixed after the first two blocks of a task; second pass: the tasks the
   // first one listed (normally none: its CTAs leave at once), max of every block
   p.redo_pass = 0;
-  k_bsattn_fwd<BLOCK, D, true><<<(unsigned)grid, kThreads, G::SMEM_BYTES, st>>>(tq, tk, tv, tk2, tv2, p);
-  WAVEAL_CUDA_OK(cudaGetLastError());
+  WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, true>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, p));
   p.redo_pass = 1;
-  k_bsattn_fwd<BLOCK, D, false><<<(unsigned)grid, kThreads, G::SMEM_BYTES, st>>>(tq, tk, tv, tk2, tv2, p);
-  WAVEAL_CUDA_OK(cudaGetLastError());
+  WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, false>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, p));
   waveal::launch_counter() = launches + 2;
   return WAVEAL_OK;
 }

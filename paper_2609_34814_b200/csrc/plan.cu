@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(kCsrWarps * 32) k_csr_to_bitmap(const int* __r
                                                                   u64* __restrict__ bits, long long n_rows, int wq, int n_kv,
                                                                   int m_b, int* dev_status) {
   __shared__ __align__(8) unsigned words[kCsrWarps][kCsrCols / 32];
+  waveal::let_next_kernel_start();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long row = (long long)blockIdx.x * kCsrWarps + warp;
   if (row >= n_rows) return;
@@ -122,6 +123,8 @@ __global__ void __launch_bounds__(kStatThreads) k_mask_stats(const u64* __restri
                                                              int wq, int wk, int* __restrict__ nnz, int* __restrict__ cnt,
                                                              int* __restrict__ nnz_out, int* __restrict__ cnt_out) {
   extern __shared__ unsigned strip[];
+  waveal::let_next_kernel_start();
+  waveal::wait_for_previous_kernel();
   const int h = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const u64* Mh = M + (size_t)h * m_b * wq;
   if ((int)blockIdx.x >= wq) {
@@ -207,6 +210,7 @@ __device__ __forceinline__ int list_sum(int v, int* part, int& before) {
 __global__ void __launch_bounds__(kListThreads) k_count_words(const u64* __restrict__ bits, long long n_words, int steps,
                                                               int* __restrict__ share) {
   __shared__ int part[kListThreads / 32];
+  waveal::let_next_kernel_start();
   const long long w0 = (long long)blockIdx.x * steps * kListThreads;
   int c = 0, ignored;
 #pragma unroll 4
@@ -230,6 +234,7 @@ __global__ void __launch_bounds__(kListThreads) k_fill_lists(const u64* __restri
   const long long w0 = (long long)blockIdx.x * steps * kListThreads;
   int base = 0, pos;
   if (share) {
+    waveal::wait_for_previous_kernel();
     for (int i = threadIdx.x; i < (int)blockIdx.x; i += kListThreads) base += share[i];
   } else {
 #pragma unroll 4
@@ -815,6 +820,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
   int* order_out = p.row_order + (size_t)h * m_b;
   int* order1_out = p.order1 ? p.order1 + (size_t)h * m_b : nullptr;
 
+  waveal::wait_for_previous_kernel();
   // (a CTA writes into another's shared memory only once that one runs: waited for below)
   if (csize > 1) cluster_arrive();
   // ---- guard statistics over natural-order waves (Section 4.5): selected pairs, and for the overlap
@@ -1199,8 +1205,14 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
   int* cnt = reinterpret_cast<int*>(w + L.off_cnt);
   const size_t strip_bytes = (size_t)64 * (2 * L.wk + 1) * 4;       // at most 131,328: wk <= kMaxSort / 64
   WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_mask_stats, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)strip_bytes));
-  k_mask_stats<<<dim3(L.wq + (unsigned)((m + kStatRows - 1) / kStatRows), (unsigned)H), kStatThreads, strip_bytes, st>>>(
-      M, Mt, (int)m, (int)n, L.wq, L.wk, nnz, cnt, out->row_nnz, out->col_count);
+  const dim3 stat_grid(L.wq + (unsigned)((m + kStatRows - 1) / kStatRows), (unsigned)H);
+  if (mask_bits) {
+    k_mask_stats<<<stat_grid, kStatThreads, strip_bytes, st>>>(M, Mt, (int)m, (int)n, L.wq, L.wk, nnz, cnt, out->row_nnz, out->col_count);
+    WAVEAL_CUDA_OK(cudaGetLastError());
+  } else {
+    WAVEAL_CUDA_OK(waveal::launch_chained(k_mask_stats, stat_grid, kStatThreads, strip_bytes, st, M, Mt, (int)m, (int)n, L.wq, L.wk,
+                                          nnz, cnt, out->row_nnz, out->col_count));
+  }
   ++launches;
   PlanParams p{};
   p.M = M; p.Mt = Mt; p.m_b = (int)m; p.n_b = (int)n; p.wq = L.wq; p.wk = L.wk;
@@ -1251,20 +1263,18 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
   }
   WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_plan_head, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   p.csize = csize;
-  if (csize == 1) {
-    k_plan_head<<<(unsigned)H, kPlanThreads, smem, st>>>(p);
-  } else {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(H * csize));
-    cfg.blockDim = dim3(kPlanThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)csize; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    WAVEAL_CUDA_OK(cudaLaunchKernelEx(&cfg, k_plan_head, p));
-  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(H * csize));
+  cfg.blockDim = dim3(kPlanThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)csize; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr; cfg.numAttrs = csize == 1 ? 1 : 2;
+  WAVEAL_CUDA_OK(cudaLaunchKernelEx(&cfg, k_plan_head, p));
   ++launches;
   WAVEAL_CUDA_OK(cudaGetLastError());
   waveal::launch_counter() = launches;
@@ -1335,8 +1345,12 @@ extern "C" waveal_status waveal_bitmap_to_csr(int32_t heads, int32_t n_q_blocks,
     k_count_words<<<blocks, kListThreads, 0, st>>>(bits, words, (int)steps, cnt);
     ++launches;
   }
-  k_fill_lists<<<blocks, kListThreads, 0, st>>>(bits, words, wq, (int)steps, direct ? nullptr : cnt, kv_row_ptr_out, rows,
-                                                kv_block_indices_out, capacity);
+  if (direct)
+    k_fill_lists<<<blocks, kListThreads, 0, st>>>(bits, words, wq, (int)steps, nullptr, kv_row_ptr_out, rows, kv_block_indices_out,
+                                                  capacity);
+  else
+    WAVEAL_CUDA_OK(waveal::launch_chained(k_fill_lists, dim3(blocks), kListThreads, 0, st, bits, words, wq, (int)steps, cnt,
+                                          kv_row_ptr_out, rows, kv_block_indices_out, capacity));
   ++launches;
   WAVEAL_CUDA_OK(cudaGetLastError());
   waveal::launch_counter() = launches;
