@@ -110,7 +110,8 @@ def _ptr(t) -> Optional[int]:
 def _stream(stream) -> Optional[int]:
     if stream is None:
         import torch
-        stream = torch.cuda.current_stream()
+        # the handle of the current stream without a Stream object around it (3.3 us each, three times a step)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) or None
     return stream.cuda_stream or None
 
 
@@ -143,14 +144,17 @@ class PlanResult:
         self.__dict__.update(kw)
 
 
-def _plan_outputs(desc: PlanDesc, device, debug: bool):
+def _plan_outputs(desc: PlanDesc, like, debug: bool):
     import torch
     H, M, N = desc.heads, desc.n_q_blocks, desc.n_kv_blocks
+    device = like.device
+    # two allocations: a tensor per output took more of the host's time than the call itself
+    buf = like.new_empty((2 * H * M + (H + 3) // 4,), dtype=torch.int32)
     res = PlanResult(
-        row_order=torch.empty((H, M), dtype=torch.int32, device=device),
-        row_nnz=torch.empty((H, M), dtype=torch.int32, device=device),
-        skip_flags=torch.empty((H,), dtype=torch.uint8, device=device),
-        dev_status=torch.zeros((4,), dtype=torch.int32, device=device),
+        row_order=buf.as_strided((H, M), (M, 1), 0),
+        row_nnz=buf.as_strided((H, M), (M, 1), H * M),
+        skip_flags=buf.view(torch.uint8).as_strided((H,), (1,), 8 * H * M),
+        dev_status=like.new_zeros((4,), dtype=torch.int32),
         col_count=None, order1=None, embedding=None, stats=None)
     if debug:
         res.col_count = torch.empty((H, N), dtype=torch.int32, device=device)
@@ -168,7 +172,7 @@ def plan_bitmap(desc: PlanDesc, mask_bits, workspace=None, debug: bool = False, 
     lib = load()
     if workspace is None:
         workspace = torch.empty((plan_workspace_bytes(desc) + 256,), dtype=torch.uint8, device=mask_bits.device)
-    res, out = _plan_outputs(desc, mask_bits.device, debug)
+    res, out = _plan_outputs(desc, mask_bits, debug)
     res.workspace = workspace
     _check(lib.waveal_plan_bitmap(ctypes.byref(desc), _ptr(mask_bits), _ptr(workspace), workspace.numel(),
                                   ctypes.byref(out), _stream(stream)))
@@ -181,7 +185,7 @@ def plan_csr(desc: PlanDesc, kv_row_ptr, kv_block_indices, workspace=None, debug
     lib = load()
     if workspace is None:
         workspace = torch.empty((plan_workspace_bytes(desc) + 256,), dtype=torch.uint8, device=kv_row_ptr.device)
-    res, out = _plan_outputs(desc, kv_row_ptr.device, debug)
+    res, out = _plan_outputs(desc, kv_row_ptr, debug)
     res.workspace = workspace
     _check(lib.waveal_plan_csr(ctypes.byref(desc), _ptr(kv_row_ptr), _ptr(kv_block_indices), _ptr(workspace),
                                workspace.numel(), ctypes.byref(out), _stream(stream)))
@@ -195,17 +199,18 @@ def bitmap_to_csr(mask_bits, n_kv_blocks: int, capacity: Optional[int] = None, s
     import torch
     lib = load()
     H, M, _ = mask_bits.shape
-    dev = mask_bits.device
-    ptr = torch.empty((H * M + 1,), dtype=torch.int32, device=dev)
-    ws = torch.empty(((H * M + 1) * 4,), dtype=torch.uint8, device=dev)
+    n = H * M + 1
     if capacity is None:
-        _check(lib.waveal_bitmap_to_csr(H, M, n_kv_blocks, _ptr(mask_bits), _ptr(ptr), None, 0, _ptr(ws), ws.numel(),
-                                        _stream(stream)))
-        capacity = int(ptr[-1].item())
-    idx = torch.empty((max(capacity, 1),), dtype=torch.int32, device=dev)
-    _check(lib.waveal_bitmap_to_csr(H, M, n_kv_blocks, _ptr(mask_bits), _ptr(ptr), _ptr(idx), capacity, _ptr(ws),
-                                    ws.numel(), _stream(stream)))
-    return ptr, idx[:capacity]
+        buf = mask_bits.new_empty((2 * n,), dtype=torch.int32)
+        at = buf.data_ptr()
+        _check(lib.waveal_bitmap_to_csr(H, M, n_kv_blocks, _ptr(mask_bits), at, None, 0, at + 4 * n, 4 * n, _stream(stream)))
+        capacity = int(buf[n - 1].item())
+    # row pointers, the call's workspace and the indices in one allocation
+    buf = mask_bits.new_empty((2 * n + max(capacity, 1),), dtype=torch.int32)
+    at = buf.data_ptr()
+    _check(lib.waveal_bitmap_to_csr(H, M, n_kv_blocks, _ptr(mask_bits), at, at + 8 * n, capacity, at + 4 * n, 4 * n,
+                                    _stream(stream)))
+    return buf.as_strided((n,), (1,), 0), buf.as_strided((capacity,), (1,), 2 * n)
 
 
 def noalloc_max_rows() -> int:
