@@ -1,0 +1,209 @@
+"""The branches that a call's sizes select, at the sizes where they change over: the plan's mask products
+(integer matrix units or walk over the set bits, one CTA or a cluster, Stage 2 by counting or by a sort),
+the list conversions, the pairing of 64-row blocks across blocks of positions, the longest-first tail of
+the tickets, tasks of zero to a few tiles back to back, and a captured call."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import waveal_oracle as wo
+from paper_2609_34814_b200 import binding as wb
+
+pytestmark = pytest.mark.gpu
+
+
+def _pack(mask):
+    """[heads, rows, columns] of bool on the GPU -> bitmap words."""
+    H, m, n = mask.shape
+    bits = torch.zeros((H, m, (n + 63) // 64 * 64), dtype=torch.int64, device="cuda")
+    bits[..., :n] = mask
+    return (bits.view(H, m, -1, 64) << torch.arange(64, device="cuda")).sum(3).contiguous()
+
+
+def _mask(H, m, n, density, seed):
+    g = torch.Generator("cuda")
+    g.manual_seed(seed)
+    x = torch.rand((H, m, n), generator=g, device="cuda") < density
+    x |= (torch.arange(m, device="cuda")[:, None] * n // m - torch.arange(n, device="cuda")[None]).abs() < 2
+    return x
+
+
+def _plan(mask, wave=148, mode=wb.FORCE_REORDER):
+    H, m, n = mask.shape
+    d = wb.plan_desc_default(heads=H, n_q_blocks=m, n_kv_blocks=n, wave_size=wave, mode=mode, seed=5)
+    return wb.plan_bitmap(d, _pack(mask), debug=True)
+
+
+# 256 / 257 rows: one CTA or a cluster; 255 / 256 / 257 columns: one 256-column chunk or two; wave 220 / 221: Stage 2 by
+# counting or by the sort; one row or one column
+@pytest.mark.parametrize("H,m,n,wave", [(2, 1, 1, 148), (2, 1, 300, 7), (2, 33, 1, 7), (3, 31, 255, 16), (2, 256, 256, 220),
+                                        (2, 257, 257, 221), (1, 600, 511, 148)])
+def test_plan_products_match_the_oracle(H, m, n, wave):
+    mask = _mask(H, m, n, 0.2, m + n)
+    r = _plan(mask, wave)
+    for h in range(H):
+        mk = mask[h].cpu().numpy()
+        u = wo.mfcsi(mk, 5, wo.start_block(5, h, m))
+        e = r.embedding[h].cpu().numpy()
+        # fp64 on both sides, entries below 1; ~n roundings of 1e-16 per sum and 12 sums in a row
+        assert np.abs(e - u).max() <= 12 * (m + n) * 2.3e-16 + 1e-15
+        order1 = r.order1[h].cpu().numpy().astype(np.int64)
+        assert np.array_equal(order1, wo.stage1_order(wo.polar_angles(e)))
+        assert np.array_equal(r.row_order[h].cpu().numpy(), wo.stage2_order(order1, mk.sum(1), wave))
+        st = wo.guard_stats(mk, wave)
+        assert r.stats[h].tolist()[:3] == [st["nnz"], st["ov_nat"], st["pair2"]]
+        assert np.array_equal(r.row_nnz[h].cpu().numpy(), mk.sum(1)) and np.array_equal(r.col_count[h].cpu().numpy(), mk.sum(0))
+
+
+# columns that select nothing change no product: the same mask with 10,000 of them goes through the walk over the
+# set bits, widened to 4,700 x 4,700 or 5,000 x 5,000 through the shared Y / Z buffer or the workspace
+@pytest.mark.parametrize("m,n,wide", [(100, 300, 10000), (4700, 300, 4700), (5000, 300, 5000)])
+def test_plan_products_agree_between_their_forms(m, n, wide):
+    mask = _mask(2, m, n, 0.1, 9)
+    padded = torch.zeros((2, m, wide), dtype=torch.bool, device="cuda")
+    padded[..., :n] = mask
+    a, b = _plan(mask), _plan(padded)
+    assert (a.embedding - b.embedding).abs().max().item() <= 12 * (m + n) * 2.3e-16 + 1e-15
+    assert torch.equal(a.order1, b.order1) and torch.equal(a.row_order, b.row_order)
+
+
+@pytest.mark.parametrize("m", [9600, 9601])       # the second sort buffer fits shared memory, or not
+def test_sorts_of_many_rows(m):
+    mask = _mask(1, m, 64, 0.3, m)
+    mask[0, 1::3] = mask[0, 0]                    # equal rows, equal angles: ties by row
+    r = _plan(mask, wave=500)
+    order1 = r.order1[0].cpu().numpy().astype(np.int64)
+    assert np.array_equal(order1, wo.stage1_order(wo.polar_angles(r.embedding[0].cpu().numpy())))
+    assert np.array_equal(r.row_order[0].cpu().numpy(), wo.stage2_order(order1, mask[0].sum(1).cpu().numpy(), 500))
+
+
+# 16,384 words: the last size without a counting launch; blocks of one step, then of more; a row of several blocks
+@pytest.mark.parametrize("H,m,n", [(1, 1, 1), (1, 16384, 64), (1, 16385, 64), (2, 8192, 64 * 32 + 1), (1, 3, 70001)])
+def test_list_conversions(H, m, n):
+    mask = _mask(H, m, n, 0.05, 3)
+    mask[:, 0] = True
+    mask[:, m // 2] = m == 1
+    bm = _pack(mask)
+    ptr, idx = wb.bitmap_to_csr(bm, n)
+    flat = mask.reshape(H * m, n)
+    assert torch.equal(ptr[1:].long(), flat.sum(1).cumsum(0)) and ptr[0].item() == 0
+    assert torch.equal(idx, flat.nonzero()[:, 1].int())
+    half, first = wb.bitmap_to_csr(bm, n, capacity=idx.numel() // 2)       # lists that end early: the rest is left out
+    assert torch.equal(half, ptr) and torch.equal(first, idx[:idx.numel() // 2])
+    if m <= 8192:                                                          # and back (8,192 columns at a time)
+        d = wb.plan_desc_default(heads=H, n_q_blocks=m, n_kv_blocks=n, wave_size=148, mode=wb.FORCE_NATURAL)
+        a, b = wb.plan_csr(d, ptr, idx, debug=True), wb.plan_bitmap(d, bm, debug=True)
+        assert torch.equal(a.col_count, b.col_count) and torch.equal(a.row_nnz, b.row_nnz) and a.dev_status.tolist() == [0] * 4
+
+
+def _attend(q, k, v, block, ptr, idx, T, order=None, flags=0):
+    o = torch.full_like(q, float("nan"))
+    lse = torch.full(q.shape[:2], float("nan"), device="cuda")
+    d = wb.attn_desc(q, k, v, o, T, T, block, flags=flags)
+    ws = torch.empty((wb.bsattn_workspace_bytes(d),), dtype=torch.uint8, device="cuda")
+    st = torch.zeros((4,), dtype=torch.int32, device="cuda")
+    wb.bsattn_fwd(d, q, k, v, o, ptr, idx, row_order=order, lse=lse, workspace=ws, dev_status=st)
+    torch.cuda.synchronize()
+    assert st.tolist() == [0] * 4
+    return o, lse, ws.view(torch.int32)[:8].tolist()
+
+
+def _inputs(H, T, D, seed):
+    g = torch.Generator("cuda")
+    g.manual_seed(seed)
+    return [torch.randn((H, T, D), generator=g, device="cuda").to(torch.bfloat16) for _ in range(3)]
+
+
+# tasks of 0 to 5 blocks one behind the other (1,023 to 1,025 of them: the tail takes the last 1,024), in natural and
+# reversed order, with a ragged last block
+@pytest.mark.parametrize("block,D", [(128, 128), (128, 64), (64, 128), (64, 64)])
+@pytest.mark.parametrize("tasks", [1, 150, 1023, 1025])
+def test_short_tasks_back_to_back(block, D, tasks):
+    T = tasks * block - 37 if tasks > 1 else 90 - block // 2
+    nb = (T + block - 1) // block
+    counts = torch.tensor([(1, 0, 2, 1, 1, 3, 0, 0, 5, 1, 2, 4)[i % 12] for i in range(nb)]).clamp(max=nb)
+    g = torch.Generator().manual_seed(tasks)
+    lists = [torch.randperm(nb, generator=g)[:c].sort().values for c in counts.tolist()]
+    ptr = torch.cat([torch.zeros(1, dtype=torch.long), counts.cumsum(0)]).int().cuda()
+    idx = torch.cat(lists).int().cuda()
+    q, k, v = _inputs(1, T, D, 1)
+    o, lse, _ = _attend(q, k, v, block, ptr, idx, T)
+    back, lse_back, _ = _attend(q, k, v, block, ptr, idx, T, order=torch.arange(nb - 1, -1, -1, device="cuda", dtype=torch.int32))
+    assert torch.equal(o, back) and torch.equal(lse, lse_back)
+    pad = torch.nn.functional.pad
+    qf, kf, vf, of = (pad(x[0].double(), (0, 0, 0, nb * block - T)).view(nb, block, D) for x in (q, k, v, o))
+    lf = pad(lse[0].double(), (0, nb * block - T)).view(nb, block)
+    exists = torch.arange(nb * block, device="cuda").view(nb, block) < T
+    for c in counts.unique().tolist():
+        rows = (counts == c).nonzero()[:, 0].cuda()
+        live, got, got_lse = exists[rows], of[rows], lf[rows]
+        if c == 0:
+            assert (got[live] == 0).all() and (got_lse[live] == -float("inf")).all()
+            continue
+        sel = torch.stack([lists[i] for i in rows.tolist()]).cuda()
+        K, V = kf[sel].flatten(1, 2), vf[sel].flatten(1, 2)
+        s = (qf[rows] @ K.transpose(1, 2) / D ** 0.5).masked_fill(~exists[sel].flatten(1)[:, None, :], -float("inf"))
+        p = s.softmax(-1)
+        ref = p @ V
+        # P is cut to bf16 (each weight within 2^-8 of itself) and O rounded to bf16
+        bound = 2.0 ** -8 * (p @ V.abs()) + 2.0 ** -8 * ref.abs() + 1e-6
+        assert ((got - ref).abs() <= bound)[live].all()
+        # the polynomial share of the exponentials is within 7.5e-5 of itself, fp32 scores and logarithm add a few 1e-6
+        assert ((got_lse - s.logsumexp(-1)).abs() <= 1.5e-4)[live].all()
+
+
+# rows that select everything stand in several blocks of 64 positions, an odd number of them, besides equal neighbours
+@pytest.mark.parametrize("nb,full", [(65, [0, 63, 64]), (150, [5, 63, 64, 66, 128, 130, 149]), (130, [70])])
+def test_pairs_across_blocks_of_positions(nb, full):
+    mask = _mask(2, nb, nb, 0.15, nb)
+    mask[:, full] = True
+    mask[0, 21] = mask[0, 20]
+    mask[1, 23] = mask[1, 22]
+    mask[1, 25] = mask[1, 24]
+    ptr, idx = wb.bitmap_to_csr(_pack(mask), nb)
+    q, k, v = _inputs(2, nb * 64, 64, 2)
+    order = torch.stack([torch.randperm(nb, generator=torch.Generator().manual_seed(h)) for h in range(2)]).int().cuda()
+    o, lse, w = _attend(q, k, v, 64, ptr, idx, nb * 64)
+    alone, lse_alone, w_alone = _attend(q, k, v, 64, ptr, idx, nb * 64, flags=wb.ATTN_NO_ROW_PAIRING)
+    mixed, lse_mixed, w_mixed = _attend(q, k, v, 64, ptr, idx, nb * 64, order=order)
+    assert torch.equal(o, alone) and torch.equal(lse, lse_alone) and torch.equal(o, mixed) and torch.equal(lse, lse_mixed)
+    tiles = int(((mask.sum(2) + 1) // 2).sum())
+    assert w_alone[6] == 0 and w_alone[7] == tiles
+    assert w[6] == 2 * (len(full) // 2) + 3 and w_mixed[6] >= 2 * (len(full) // 2)
+    shared = 2 * (len(full) // 2) * ((nb + 1) // 2) + sum(int((mask[h, i].sum() + 1) // 2) for h, i in ((0, 20), (1, 22), (1, 24)))
+    assert w[7] == tiles - shared
+
+
+@pytest.mark.parametrize("block", [64, 128])
+def test_a_captured_step_replays(block):
+    nb, D = 200, 64
+    mask = _mask(2, nb, nb, 0.1, 4)
+    bm, pairs = _pack(mask), int(mask.sum())
+    q, k, v = _inputs(2, nb * block, D, 3)
+    o = torch.zeros_like(q)
+    pd = wb.plan_desc_default(heads=2, n_q_blocks=nb, n_kv_blocks=nb, wave_size=148, mode=wb.FORCE_REORDER, seed=1)
+    pws = torch.empty((wb.plan_workspace_bytes(pd) + 256,), dtype=torch.uint8, device="cuda")
+    ad = wb.attn_desc(q, k, v, o, nb * block, nb * block, block)
+    aws = torch.empty((wb.bsattn_workspace_bytes(ad),), dtype=torch.uint8, device="cuda")
+
+    def step():
+        ptr, idx = wb.bitmap_to_csr(bm, nb, capacity=pairs)
+        plan = wb.plan_bitmap(pd, bm, workspace=pws)
+        wb.bsattn_fwd(ad, q, k, v, o, ptr, idx, row_order=plan.row_order, workspace=aws)
+        return plan.row_order
+
+    side = torch.cuda.Stream()
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        order = step().clone()
+    torch.cuda.synchronize()
+    ref = o.clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        replayed = step()
+    o.zero_()
+    graph.replay()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(o, ref) and torch.equal(replayed, order)
+    del graph
