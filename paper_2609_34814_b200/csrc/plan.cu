@@ -1229,11 +1229,14 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
   p.row_order = out->row_order; p.flags = out->skip_flags;
   p.order1 = out->order1; p.embedding = out->embedding; p.stats = reinterpret_cast<long long*>(out->stats);
   // CTAs per head: the largest cluster of which the device holds one per head at once, and no more than
-  // there are groups of 32 rows
+  // half as many CTAs as there are groups of 32 rows
   int csize = 1;
   {
     const int groups = (int)(((m > n ? m : n) + kUnitRows - 1) / kUnitRows);
-    s = cluster_size(dev, (int)H, L.mma ? groups : (groups < 4 ? groups : 4), &csize);
+    // (up to 256 rows one CTA is quickest: 73.8 us against 82.2 us with eight on 5 heads of 256 rows; above, two
+    // groups a CTA: 88.5 / 92.0 / 97.4 us with 7 / 4 / 2 CTAs on 12 heads of 400 rows)
+    const int limit = groups <= 8 ? 1 : (groups + 1) / 2;
+    s = cluster_size(dev, (int)H, L.mma ? limit : (groups < 4 ? groups : 4), &csize);
     if (s != WAVEAL_OK) return s;
   }
   // counting costs 2.5 wave instructions a row, the merge sort ~550: kMaxSort = 2^14 positions, and
