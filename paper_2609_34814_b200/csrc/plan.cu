@@ -7,18 +7,18 @@
 //   inside each bucket.
 //
 // Layout of the work: the mask is kept as a bitmap M and its bit transpose Mt (both stay
-// resident in L2; a bitmap is smaller than index lists once density exceeds 1/32).  A
-// thread-block cluster of 1 to 4 CTAs of 1024 threads (as many as the device holds at once
-// for the given number of heads) owns one head and runs every step for it, with the iteration
-// blocks X, Y, Z (fp64) in shared memory, so the whole plan is one launch after the transpose
-// and no step needs a grid-wide barrier.  The CTAs of a cluster keep identical copies of the
-// state: the cheap steps (counts, guard, QR, rotation) are done by each of them in the same
-// order, the two mask sweeps of an iteration - where the time goes - are split by rows and
-// each result is written into every copy through distributed shared memory; the lead CTA does
-// the sorts and writes the outputs.  All floating-point reductions use a fixed thread ->
-// element assignment and a fixed combination tree, and a row is summed by the same lanes in the
-// same order whichever CTA takes it, so a plan is reproducible bit for bit and does not
-// depend on the cluster size.
+// resident in L2; a bitmap is smaller than index lists once density exceeds 1/32).  One launch
+// transposes and counts; a second plans: a thread-block cluster of 1 to 16 CTAs of 1024 threads
+// (as many as the device holds at once for the given number of heads) owns one head and runs every
+// step for it, with the iteration blocks X, Y, Z (fp64) in shared memory, so no step needs a
+// grid-wide barrier.  The CTAs of a cluster keep identical copies of the state: the cheap steps
+// (QR, rotation) are done by each of them in the same order, the two mask products of an iteration
+// are split by rows and each result is written into every copy through distributed shared memory;
+// the lead CTA does the sorts and writes the outputs.  The products are exact integer sums on the
+// matrix units (multiply_rows), the floating-point reductions use a fixed thread -> element
+// assignment and a fixed combination tree, so a plan is reproducible bit for bit and does not
+// depend on the cluster size.  Shapes whose digits do not fit shared memory walk the set bits in fp64
+// instead (gather_rows), also in an order that does not depend on which CTA takes a row.
 #include <cfloat>
 #include <climits>
 #include <cmath>
@@ -286,39 +286,40 @@ __global__ void __launch_bounds__(kListThreads) k_fill_lists(const u64* __restri
 
 // ------------------------------------------------------------------ block-wide helpers
 
-// Sum of N doubles per thread over the CTA, same result in every thread; fixed tree
-// (lanes, then warps).  fp64 adds are scarce on this part, so the second level is one more
-// shuffle tree in warp 0, not a serial sum in every thread.
+// Sum of N <= 4 doubles per thread over the CTA, same result in every thread; fixed tree.  The lanes of a warp
+// first hand half of their values over (lane distance 16), then half of those (8), so that from there on
+// each lane sums one value: 6 exchanges instead of 5 N, which the shuffle unit (one warp a clock) would take 1,280
+// clk for with 32 warps and N = 4.  Warps without elements (`any` false) only leave zeros.
 template <int N>
-__device__ __forceinline__ void block_sum(double (&v)[N], double* scratch) {
-  int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ void block_sum(double (&v)[N], double* scratch, bool any) {
+  static_assert(N <= 4 && kPlanWarps == 32, "one quarter of a warp per value, one lane per four warps' partial sums");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double* part = scratch + 4;                 // [warp][4]; the results stand before them
+  const int k = (lane >> 3) & 3;              // the value this lane ends up with
+  double x = 0.0;
+  if (any) {
+    double u[4];
 #pragma unroll
-  for (int k = 0; k < N; ++k) {
+    for (int i = 0; i < 4; ++i) u[i] = i < N ? v[i < N ? i : 0] : 0.0;
+    const bool h16 = lane & 16, h8 = lane & 8;
+    const double p = (h16 ? u[2] : u[0]) + __shfl_xor_sync(0xffffffffu, h16 ? u[0] : u[2], 16);
+    const double q = (h16 ? u[3] : u[1]) + __shfl_xor_sync(0xffffffffu, h16 ? u[1] : u[3], 16);
+    x = (h8 ? q : p) + __shfl_xor_sync(0xffffffffu, h8 ? p : q, 8);
 #pragma unroll
-    for (int o = 16; o; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    for (int o = 4; o; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
   }
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < N; ++k) scratch[warp * N + k] = v[k];
-  }
+  if ((lane & 7) == 0) part[warp * 4 + k] = x;
   __syncthreads();
   if (warp == 0) {
-    double t[N];
+    const int val = lane & 3, grp = lane >> 2;
+    double y = (part[grp * 4 + val] + part[(grp + 8) * 4 + val]) + (part[(grp + 16) * 4 + val] + part[(grp + 24) * 4 + val]);
 #pragma unroll
-    for (int k = 0; k < N; ++k) {
-      t[k] = scratch[lane * N + k];           // kPlanWarps == 32: one partial per lane
-#pragma unroll
-      for (int o = 16; o; o >>= 1) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
-    }
-    if (lane == 0) {
-#pragma unroll
-      for (int k = 0; k < N; ++k) scratch[kPlanWarps * N + k] = t[k];
-    }
+    for (int o = 4; o < 32; o <<= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+    if (lane < 4) scratch[lane] = y;
   }
   __syncthreads();
 #pragma unroll
-  for (int k = 0; k < N; ++k) v[k] = scratch[kPlanWarps * N + k];
-  __syncthreads();
+  for (int i = 0; i < N; ++i) v[i] = scratch[i];
 }
 
 // the same for whole numbers
@@ -504,7 +505,8 @@ __device__ __forceinline__ Qr2 thin_qr2(const double2* z_in, int m, double* scra
   const int tid = threadIdx.x;
   double a[3] = {0, 0, 0};
   for (int i = tid; i < m; i += kPlanThreads) { const double2 z = z_in[i]; a[0] += z.x * z.x; a[1] += z.x * z.y; a[2] += z.y * z.y; }
-  block_sum<3>(a, scratch);
+  const bool any = (tid & ~31) < m;
+  block_sum<3>(a, scratch, any);
   Qr2 r;
   r.inv1 = a[0] > tiny_sq ? rsqrt(a[0]) : 0.0;
   r.d = a[1] * r.inv1;
@@ -514,7 +516,7 @@ __device__ __forceinline__ Qr2 thin_qr2(const double2* z_in, int m, double* scra
     const double q1 = z.x * r.inv1, y = z.y - r.d * q1;
     s[0] += q1 * y; s[1] += y * y; s[2] += q1; s[3] += y;
   }
-  block_sum<4>(s, scratch);
+  block_sum<4>(s, scratch, any);
   r.e = s[0];
   const double n2_sq = s[1] - r.e * r.e;         // dropped too: 1e-9 or less of the norm before the projection
   r.inv2 = n2_sq > tiny_sq && n2_sq > 1e-18 * a[2] ? rsqrt(n2_sq) : 0.0;
@@ -603,8 +605,8 @@ __device__ __forceinline__ void multiply_rows(const u64* __restrict__ bits, int 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
   const int units = (n_rows + kUnitRows - 1) / kUnitRows, chunks = (wpr + 3) >> 2;
   const int slots = kPlanWarps / ksplit, slot = warp / ksplit, kp = warp - slot * ksplit;
-  auto put = [&](int r, double x, double y) {
-    const double sc = cnt ? (double)cnt[r] : 1.0;
+  auto put = [&](int r, int c_r, double x, double y) {
+    const double sc = (double)c_r;
     const double2 v = make_double2(x * inv_scale - sc * corr.x, y * inv_scale - sc * corr.y);
     dst[r] = v;
     if (peers)
@@ -622,6 +624,7 @@ __device__ __forceinline__ void multiply_rows(const u64* __restrict__ bits, int 
 #pragma unroll
           for (int e = 0; e < 4; ++e) acc[i][c][e] = 0;
       const int r0 = u * kUnitRows + g;
+      const int c_mine = ksplit == 1 && cnt && r0 + t * 8 < n_rows ? cnt[r0 + t * 8] : 1;    // (loaded ahead of the products)
       for (int ch = kp * chunks / ksplit; ch < (kp + 1) * chunks / ksplit; ++ch) {
         u64 w[4];
 #pragma unroll
@@ -664,7 +667,7 @@ __device__ __forceinline__ void multiply_rows(const u64* __restrict__ bits, int 
         const double x = t == 0 ? val[0][0][0] : t == 1 ? val[0][1][0] : t == 2 ? val[1][0][0] : val[1][1][0];
         const double y = t == 0 ? val[0][0][1] : t == 1 ? val[0][1][1] : t == 2 ? val[1][0][1] : val[1][1][1];
         const int r = r0 + t * 8;
-        if (r < n_rows) put(r, x, y);
+        if (r < n_rows) put(r, c_mine, x, y);
       } else {
         int* pp = part + slot * (kUnitRows * 16);
 #pragma unroll
@@ -677,9 +680,12 @@ __device__ __forceinline__ void multiply_rows(const u64* __restrict__ bits, int 
       }
     }
     if (ksplit > 1) {
+      // (slots * 32 <= 512 rows: one a thread)
+      const int i = threadIdx.x, uu = u0 + (i / kUnitRows) * csize, r = uu * kUnitRows + i % kUnitRows;
+      const bool mine = i < slots * kUnitRows;
+      const int c_mine = mine && cnt && uu < units && r < n_rows ? cnt[r] : 1;
       __syncthreads();
-      for (int i = threadIdx.x; i < slots * kUnitRows; i += kPlanThreads) {
-        const int uu = u0 + (i / kUnitRows) * csize, r = uu * kUnitRows + i % kUnitRows;
+      if (mine) {
         if (uu < units && r < n_rows) {
           int4* pr = reinterpret_cast<int4*>(part + i * 16);
           double v[2];
@@ -689,7 +695,7 @@ __device__ __forceinline__ void multiply_rows(const u64* __restrict__ bits, int 
             v[c] = join_digits((long long)l.x + ((long long)l.y << 8) + ((long long)l.z << 16) + ((long long)l.w << 24),
                                (long long)h.x + ((long long)h.y << 8) + ((long long)h.z << 16) + ((long long)h.w << 24));
           }
-          put(r, v[0], v[1]);
+          put(r, c_mine, v[0], v[1]);
         }
         int4* pz = reinterpret_cast<int4*>(part + i * 16);
 #pragma unroll
@@ -933,7 +939,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
       double cy[2] = {0, 0};
       for (int j = tid; j < n_b; j += kPlanThreads) { double2 y = Y[j]; double c = (double)cnt[j]; cy[0] += c * y.x; cy[1] += c * y.y; }
       if (p.mma) pack_digits(items, n_b, y_scale, [&](int k, int col) { return col ? Y[k].y : Y[k].x; });
-      block_sum<2>(cy, scratch);
+      block_sum<2>(cy, scratch, (tid & ~31) < n_b);
       // Z = M Y - 1 (c^T Y)/m
       const double2 corr_z = make_double2(cy[0] * inv_m, cy[1] * inv_m);
       if (p.mma) {
@@ -953,9 +959,15 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
       double2 x = X[i], z = Z[i];
       b[0] += x.x * z.x; b[1] += x.x * z.y; b[2] += x.y * z.x; b[3] += x.y * z.y;
     }
-    block_sum<4>(b, scratch);
-    double th = 0.5 * atan2(2.0 * (0.5 * (b[1] + b[2])), b[0] - b[3]);
-    double cs = cos(th), sn = sin(th);
+    block_sum<4>(b, scratch, (tid & ~31) < m_b);
+    // (one warp works the angle out: 32 of them kept the fp64 units busy with it for 4,000 cycles)
+    if (tid < 32) {
+      const double th = 0.5 * atan2(2.0 * (0.5 * (b[1] + b[2])), b[0] - b[3]);
+      if (tid == 0) { scratch[4] = cos(th); scratch[5] = sin(th); }
+    }
+    __syncthreads();
+    const double cs = scratch[4], sn = scratch[5];
+    __syncthreads();
     double mx[2] = {0, 0};
     for (int i = tid; i < m_b; i += kPlanThreads) {
       double2 x = X[i];
