@@ -1161,7 +1161,7 @@ __device__ __forceinline__ void clear_counters(const AttnParams& p) {
 // The last kTailTasks tickets of a call are handed out longest first (1,024 = 7 per SM).  In the planned
 // or natural order a long row may start last and leave the other SMs waiting for it: the row lengths of
 // the masks in use spread over a factor of ten.  Calls of a few tasks per SM gain most (5 heads of 256
-// rows: 655k -> 501k cycles), the largest lose nothing: before the last 1,024 tickets the order is the
+// rows: 655k -> 494k cycles), the largest lose nothing: before the last 1,024 tickets the order is the
 // caller's, and no result depends on it.  A histogram of 1,024 lengths is enough (which of two tasks of
 // about the same length goes first makes no difference).
 constexpr int kTailTasks = 1024;
