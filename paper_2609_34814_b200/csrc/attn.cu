@@ -535,7 +535,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     mbar_init(BAR(B_FINAL + 1), 1);
     for (int i = 0; i < 16; ++i) mbar_init(BAR(B_MX + i), 1);   // (lane quadrant, tile count mod 4)
     for (int i = 0; i < 16; ++i) mbar_init(BAR(B_EX + i), 4);   // (task mod 4, lane quadrant): its four warps, once per task
-    for (int i = 0; i < 8; ++i) mbar_init(BAR(B_HX + i), 2);    // the two owners of a row (team, quadrant), once per max
+    for (int i = 0; i < 8; ++i) mbar_init(BAR(B_HX + i), 2);    // the two owners of a row (team, quadrant), once per max and once per rescale of O
     *abort_smem = 0;
     for (int i = 0; i < 4; ++i) redo_flag[i] = 0;
     fence_mbar_init();
@@ -972,8 +972,9 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           // rare: the reference grew, so O (blocks 0..j-1) is rescaled; its last MMA (block j-1)
           // must be complete: that is the latest phase of the barrier of the S buffer before
           // this one (the next P V on that buffer needs a P this team has not produced yet).
-          // Done before any part of P_j is released to the MMA warp; each owner takes half of
-          // the row's output columns.
+          // Each owner takes half of the row's output columns, and both halves are done before either half of
+          // P_j is released: the P V warp starts on the first half of P as soon as that one has arrived, and
+          // those MMAs add to all columns of O.  So the two meet once more (the decision to grow is the same in both).
           if (grow && j > 0) {
             const uint32_t sbp = sb == 0 ? (uint32_t)G::NSBUF - 1u : sb - 1u;
             ok = warp_wait(ctx, BAR(B_S_FREE + sbp), sb == 0 ? s_ph ^ 1u : s_ph, 22);
@@ -989,6 +990,14 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
               for (int c = 0; c < 32; ++c) ov[c] = __float_as_uint(__uint_as_float(ov[c]) * alpha);
               WAVEAL_TMEM_ST32(o_row + c0, ov, 0);
             }
+            tc_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(BAR(B_HX + team * 4 + quad));
+            ok = warp_wait(ctx, BAR(B_HX + team * 4 + quad), hx_it & 1u, 27);
+            if (!ok) break;
+            ++hx_it;
+            tc_fence_after();
           }
           // p' = 2^(s*scale*log2e - m + log2(1 + 2^-9)); P is p' cut to its top 16 bits (one byte
           // permute per pair instead of a conversion).  The extra factor centres the cut's error

@@ -226,6 +226,40 @@ def test_reference_growth_and_short_rows():
     assert np.abs(lse[0].cpu().numpy() - ref_lse).max() < 5e-3 * max(1.0, np.abs(ref_lse).max() / 10)
 
 
+@pytest.mark.parametrize("flags", [0, wb.ATTN_ONLINE_MAX_ONLY])
+@pytest.mark.parametrize("block,d", [(64, 128), (64, 64), (128, 128), (128, 64)])
+def test_scores_that_grow_in_every_tile(block, d, flags):
+    """The reference of a row grows by more than 2^8 from each tile to the next, so O is rescaled before
+    every P V: at tile 1 of the first launch (64-row blocks), at every tile of the second launch and
+    of the single one.  Each half of O's columns has to be rescaled before the products of either
+    half of P are added."""
+    cfg = dataclasses.replace(_small("wan480p", 2, 2), head_dim=d, block=block)
+    w = Workload(cfg)
+    nb = cfg.n_blocks
+    rng = np.random.default_rng(block + d)
+    w.masks = [rng.random((nb, nb)) < 0.5 for _ in range(2)]
+    ptr_np, idx_np = I.masks_to_csr(w.masks)
+    w.ptr, w.idx = torch.from_numpy(ptr_np).cuda(), torch.from_numpy(idx_np).cuda()
+    # scale 1: scores of block j have a spread of sqrt(d) (1 + j / 2); tiles are 128 keys of every second block,
+    # so the largest of a tile rises by 2.5 * sqrt(d) / 2 = 10 nats or more to the next one
+    grow = (1.0 + 0.5 * torch.arange(nb, device="cuda")).repeat_interleave(block)[:, None]
+    for h in range(2):
+        w.k[h].copy_((w.k[h].float() * grow[:w.k.shape[1]]).to(torch.bfloat16))
+    o = torch.full_like(w.o, float("nan"))
+    lse = torch.empty((2, cfg.seq), dtype=torch.float32, device="cuda")
+    st = torch.zeros(4, dtype=torch.int32, device="cuda")
+    desc = wb.attn_desc(w.q, w.k, w.v, o, cfg.seq, cfg.seq, block, flags=flags)
+    wb.bsattn_fwd(desc, w.q, w.k, w.v, o, w.ptr, w.idx, lse=lse, scale=1.0, dev_status=st)
+    torch.cuda.synchronize()
+    assert st.tolist() == [0, 0, 0, 0]
+    for h in range(2):
+        ref, ref_lse = wo.block_sparse_attention(w.head_f64("q", h), I.bf16_to_f64(w.k[h].cpu()), w.head_f64("v", h),
+                                                 w.masks[h], block, block, cfg.seq, cfg.seq, 1.0)
+        assert_parity(o[h, :cfg.seq].float().cpu().numpy(), ref, "growing in every tile", one_hot=True)
+        live = np.isfinite(ref_lse)
+        assert np.abs(lse[h].cpu().numpy() - ref_lse)[live].max() < 5e-3 * max(1.0, np.abs(ref_lse[live]).max() / 10)
+
+
 def test_second_launch_recomputes_tasks_whose_reference_was_too_low():
     """Keys that are far larger in one late KV block push the exponents of the fixed-reference
     pass over its limit: those tasks must be listed, computed again with the max of every
