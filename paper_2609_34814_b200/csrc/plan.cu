@@ -1228,7 +1228,9 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
   ++launches;
   PlanParams p{};
   p.M = M; p.Mt = Mt; p.m_b = (int)m; p.n_b = (int)n; p.wq = L.wq; p.wk = L.wk;
+  // (a wave longer than the head is the whole head; cut to it, row + wave stays far from the end of int)
   p.wave = d->wave_size > 0 ? d->wave_size : sms;
+  if (p.wave > (int)m) p.wave = (int)m;
   p.iters = d->svd_iters; p.mode = d->mode & ~WAVEAL_RING_CUT_LARGEST_GAP;
   p.ring_cut = (d->mode & WAVEAL_RING_CUT_LARGEST_GAP) ? 1 : 0; p.n_pow2 = L.n_pow2; p.state_in_smem = L.state_in_smem;
   p.seed = d->seed;

@@ -55,6 +55,20 @@ def test_plan_products_match_the_oracle(H, m, n, wave):
         assert np.array_equal(r.row_nnz[h].cpu().numpy(), mk.sum(1)) and np.array_equal(r.col_count[h].cpu().numpy(), mk.sum(0))
 
 
+# a wave of the head's length or more is one wave, up to the largest value the descriptor holds
+@pytest.mark.parametrize("m", [2, 100, 300, 9700])
+def test_waves_longer_than_the_head(m):
+    mask = _mask(2, m, 70, 0.2, m)
+    ref = _plan(mask, wave=m)
+    for wave in (m + 1, 2 ** 31 - m, 2 ** 31 - 1):
+        r = _plan(mask, wave=wave)
+        assert torch.equal(r.row_order, ref.row_order) and torch.equal(r.order1, ref.order1) and torch.equal(r.stats, ref.stats)
+    nnz = ref.row_nnz.long().gather(1, ref.row_order.long())
+    assert (nnz[:, :-1] >= nnz[:, 1:]).all()
+    st = wo.guard_stats(mask[0].cpu().numpy(), m)
+    assert ref.stats[0].tolist()[:3] == [st["nnz"], st["ov_nat"], st["pair2"]]
+
+
 # columns that select nothing change no product: the same mask with 10,000 of them goes through the walk over the
 # set bits, widened to 4,700 x 4,700 or 5,000 x 5,000 through the shared Y / Z buffer or the workspace
 @pytest.mark.parametrize("m,n,wide", [(100, 300, 10000), (4700, 300, 4700), (5000, 300, 5000)])
