@@ -119,6 +119,7 @@ struct Transposer {
 // the columns leave in whole lines and are counted on the way.  The other blocks count 32 rows each.
 // Counting here spreads what every CTA of a head's cluster used to do for itself over the whole chip.
 constexpr int kStatThreads = 256, kStatRows = 32;
+constexpr int kStripMax = 64 * (2 * (kMaxSort / 64) + 1) * 4;      // bytes of the longest strip: 131,328
 __global__ void __launch_bounds__(kStatThreads) k_mask_stats(const u64* __restrict__ M, u64* __restrict__ Mt, int m_b, int n_b,
                                                              int wq, int wk, int* __restrict__ nnz, int* __restrict__ cnt,
                                                              int* __restrict__ nnz_out, int* __restrict__ cnt_out) {
@@ -1168,7 +1169,6 @@ waveal_status cluster_size(int dev, int heads, int limit, int* out) {
   for (int c = limit < kMaxCluster ? limit : kMaxCluster; c > 1; --c) {
     if (!fit[dev][c]) {
       WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_plan_head, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-      WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_plan_head, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3((unsigned)c);
       cfg.blockDim = dim3(kPlanThreads);
@@ -1178,7 +1178,7 @@ waveal_status cluster_size(int dev, int heads, int limit, int* out) {
       attr[0].val.clusterDim.x = (unsigned)c; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
       cfg.attrs = attr; cfg.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, k_plan_head, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+      if (cudaOccupancyMaxActiveClusters(&n, k_plan_head, &cfg) != cudaSuccess) { cudaGetLastError(); continue; }
       fit[dev][c] = n + 1;
     }
     if (fit[dev][c] - 1 >= heads) { *out = c; return WAVEAL_OK; }
@@ -1215,8 +1215,11 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
   u64* Mt = reinterpret_cast<u64*>(w + L.off_mt);
   int* nnz = reinterpret_cast<int*>(w + L.off_nnz);
   int* cnt = reinterpret_cast<int*>(w + L.off_cnt);
-  const size_t strip_bytes = (size_t)64 * (2 * L.wk + 1) * 4;       // at most 131,328: wk <= kMaxSort / 64
-  WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_mask_stats, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)strip_bytes));
+  // The limits on dynamic shared memory belong to the process, and another host thread may stand between its own
+  // setting of them and its launch: every call sets the same values, the largest any shape takes.
+  const size_t strip_bytes = (size_t)64 * (2 * L.wk + 1) * 4;
+  WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_mask_stats, cudaFuncAttributeMaxDynamicSharedMemorySize, kStripMax));
+  WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_plan_head, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
   const dim3 stat_grid(L.wq + (unsigned)((m + kStatRows - 1) / kStatRows), (unsigned)H);
   if (mask_bits) {
     k_mask_stats<<<stat_grid, kStatThreads, strip_bytes, st>>>(M, Mt, (int)m, (int)n, L.wq, L.wk, nnz, cnt, out->row_nnz, out->col_count);
@@ -1278,7 +1281,6 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
     const size_t need = L.items_end + (size_t)ints * 4;
     smem = smem > need ? smem : need;
   }
-  WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_plan_head, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   p.csize = csize;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(H * csize));

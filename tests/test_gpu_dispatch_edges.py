@@ -2,6 +2,9 @@
 (integer matrix units or walk over the set bits, one CTA or a cluster, Stage 2 by counting or by a sort),
 the list conversions, the pairing of 64-row blocks across blocks of positions, the longest-first tail of
 the tickets, tasks of zero to a few tiles back to back, and a captured call."""
+import ctypes
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -108,6 +111,37 @@ def test_list_conversions(H, m, n):
         d = wb.plan_desc_default(heads=H, n_q_blocks=m, n_kv_blocks=n, wave_size=148, mode=wb.FORCE_NATURAL)
         a, b = wb.plan_csr(d, ptr, idx, debug=True), wb.plan_bitmap(d, bm, debug=True)
         assert torch.equal(a.col_count, b.col_count) and torch.equal(a.row_nnz, b.row_nnz) and a.dev_status.tolist() == [0] * 4
+
+
+def test_host_threads_plan_different_sizes():
+    """A small plan must not take from a large one, between that one's set-up and its launches, the shared
+    memory they need."""
+    lib, jobs, failed = wb.load(), [], []
+    for m, n in ((64, 64), (16384, 64), (128, 64), (4700, 300)):
+        mask = _mask(1, m, n, 0.1, m)
+        d = wb.plan_desc_default(heads=1, n_q_blocks=m, n_kv_blocks=n, wave_size=148, mode=wb.FORCE_NATURAL, seed=5)
+        ws = torch.empty((wb.plan_workspace_bytes(d) + 256,), dtype=torch.uint8, device="cuda")
+        jobs.append((d, _pack(mask), ws, wb.plan_bitmap(d, _pack(mask), workspace=ws), mask.sum(2), torch.cuda.Stream()))
+    torch.cuda.synchronize()
+
+    def work(d, bits, ws, res, nnz, stream):
+        out = wb.PlanOut(row_order=res.row_order.data_ptr(), row_nnz=res.row_nnz.data_ptr())
+        args = (ctypes.byref(d), bits.data_ptr(), ws.data_ptr(), ws.numel(), ctypes.byref(out), stream.cuda_stream)
+        for _ in range(4000):                     # (the library call alone: the threads run it side by side)
+            status = lib.waveal_plan_bitmap(*args)
+            if status != wb.OK:
+                failed.append((d.n_q_blocks, status, wb.last_error()))
+                return
+
+    threads = [threading.Thread(target=work, args=j) for j in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not failed, failed
+    for _, _, _, res, nnz, _ in jobs:
+        assert torch.equal(res.row_nnz.long(), nnz)
 
 
 def _attend(q, k, v, block, ptr, idx, T, order=None, flags=0):
