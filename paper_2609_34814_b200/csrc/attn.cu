@@ -360,7 +360,7 @@ struct Geo {
   static constexpr int OFF_TASK = OFF_BAR + ((N_BAR * 8 + 15) / 16) * 16;
   static constexpr int OFF_MX = OFF_TASK + 2 * (int)sizeof(Task);
   static constexpr int OFF_MISC = OFF_MX + 4 * 128 * 4 + 2 * 2 * 2 * 128 * 4 + 4 * 4 * 128 * 8;
-  static constexpr int SMEM_BYTES = OFF_MISC + 32 + 1024;   // + slack for 1024-byte alignment
+  static constexpr int SMEM_BYTES = OFF_MISC + 48 + 1024;   // + slack for 1024-byte alignment
   // tensor memory: three S/P buffers of 128 columns, then the output accumulator
   static constexpr uint32_t S_STRIDE = 128, O_COL = 384, TMEM_COLS = 512;
 };
@@ -513,7 +513,9 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   float2* ex = reinterpret_cast<float2*>(smem + G::OFF_MX + 4 * 128 * 4 + 2 * 2 * 2 * 128 * 4);    // [task mod 4][tile parity*2+half][128] (reference, sum)
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + G::OFF_MISC);
   volatile int* abort_smem = reinterpret_cast<volatile int*>(smem + G::OFF_MISC + 4);
-  volatile int* redo_flag = reinterpret_cast<volatile int*>(smem + G::OFF_MISC + 8);   // [task mod 4]
+  // by task mod 4: number (from 1) of the last task that a tile wants computed again, and of the last one listed for it
+  volatile int* redo_flag = reinterpret_cast<volatile int*>(smem + G::OFF_MISC + 8);
+  int* redo_listed = reinterpret_cast<int*>(smem + G::OFF_MISC + 24);
   Ctx ctx{bar0, abort_smem, p.ws, p.dev_status, p.wait_limit};
   const long long t_start = clock64();
 
@@ -537,7 +539,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     for (int i = 0; i < 16; ++i) mbar_init(BAR(B_EX + i), 4);   // (task mod 4, lane quadrant): its four warps, once per task
     for (int i = 0; i < 8; ++i) mbar_init(BAR(B_HX + i), 2);    // the two owners of a row (team, quadrant), once per max and once per rescale of O
     *abort_smem = 0;
-    for (int i = 0; i < 4; ++i) redo_flag[i] = 0;
+    for (int i = 0; i < 4; ++i) { redo_flag[i] = 0; redo_listed[i] = 0; }
     fence_mbar_init();
     fence_proxy_async();
   }
@@ -867,6 +869,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR(B_TASK_EMPTY + slot));
       float2* exb = ex + (o_it & 3) * 512;
+      const int task_no = (int)o_it + 1;
       const uint32_t rslot = o_it & 3, ex_bar = B_EX + quad + 4 * (o_it & 3), ex_ph = (o_it >> 2) & 1;
       ++task_it;
       if (tk.n < 0) break;
@@ -1036,7 +1039,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           // polynomial share saturates at 2^64), so a sum below 2^60 bounds every exponent it
           // covers; at or above it (or not a number) the fixed reference is too far off:
           // redo the task
-          if (fixed_ref && __any_sync(0xffffffffu, !(l_blk < kRedoLimit))) redo_flag[rslot] = 1;
+          if (fixed_ref && __any_sync(0xffffffffu, !(l_blk < kRedoLimit))) redo_flag[rslot] = task_no;
           tc_wait_st();
           tc_fence_before();
           __syncwarp();
@@ -1075,14 +1078,6 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       ok = warp_wait(ctx, BAR(B_O_FULL), o_ph, 23);
       if (!ok) break;
       tc_fence_after();
-      if (FAST && half == 0 && quad == 0 && lane == 0 && redo_flag[rslot]) {
-        // every warp's tiles of this task lie before O_FULL; the slot is used again four tasks later
-        const int e = atomicAdd(&p.ws[2], (G::KB == 2 && tk.row2 >= 0) ? 2 : 1);
-        p.ws[8 + 2 * e] = tk.h;
-        p.ws[9 + 2 * e] = tk.row;
-        if (G::KB == 2 && tk.row2 >= 0) { p.ws[10 + 2 * e] = tk.h; p.ws[11 + 2 * e] = tk.row2; }   // computed again one by one
-        redo_flag[rslot] = 0;
-      }
       uint32_t ov[G::CO];
       static_assert(G::CO == 64 || G::CO == 32, "half of head_dim 128 or 64");
       WAVEAL_TMEM_LD32(o_row + half * G::CO, ov, 0);
@@ -1092,16 +1087,21 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR(B_O_FREE));
+      bool bad = false;
       if (row_live) {
         // a thread holds a piece of one row, so a store instruction of a warp touches 32 rows:
         // its cost in the memory pipe is per row, not per byte.  32-byte stores halve the number
         // of instructions where the row piece is 32-byte aligned (else 16-byte stores)
         uint32_t w[G::CO / 2];
+        float z0 = 0.f, z1 = 0.f;          // stay 0 as long as every result is finite
 #pragma unroll
         for (int c = 0; c < G::CO; c += 2) {
-          __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(ov[c]) * inv_l, __uint_as_float(ov[c + 1]) * inv_l);
+          const float o0 = __uint_as_float(ov[c]) * inv_l, o1 = __uint_as_float(ov[c + 1]) * inv_l;
+          if (FAST) ffma2(z0, z1, o0, o1, 0.f, 0.f, z0, z1);
+          __nv_bfloat162 b2 = __floats2bfloat162_rn(o0, o1);
           w[c / 2] = *reinterpret_cast<uint32_t*>(&b2);
         }
+        bad = FAST && !(z0 + z1 == 0.f);
         if ((reinterpret_cast<uintptr_t>(o_ptr) & 31) == 0) {
 #pragma unroll
           for (int c = 0; c < G::CO / 2; c += 8) st_global_v8(o_ptr + 2 * c, w + c);
@@ -1111,6 +1111,17 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             *reinterpret_cast<uint4*>(o_ptr + 2 * c) = make_uint4(w[c], w[c + 1], w[c + 2], w[c + 3]);
         }
         if (p.lse && half == 0) p.lse[(size_t)tk.h * p.seq_q + q_tok] = (m_all + log2f(l_tot) - 0.0028150156f) * 0.6931471805599453f;
+      }
+      // The task goes to the second launch if the sum of a tile left the range (every warp's tiles of this task lie
+      // before O_FULL) or if a result is not finite: with sums of up to 2^60 O overflows from |V| = 2^67 on, and a
+      // first tile whose scores are all -inf leaves no reference.  (Where V itself holds an inf or NaN the second
+      // launch finds the same again.)  Whichever of the epilogue's warps sees it first writes the entry.
+      if (FAST && (__any_sync(0xffffffffu, bad) || redo_flag[rslot] == task_no) && lane == 0 &&
+          atomicExch(&redo_listed[rslot], task_no) != task_no) {
+        const int e = atomicAdd(&p.ws[2], (G::KB == 2 && tk.row2 >= 0) ? 2 : 1);
+        p.ws[8 + 2 * e] = tk.h;
+        p.ws[9 + 2 * e] = tk.row;
+        if (G::KB == 2 && tk.row2 >= 0) { p.ws[10 + 2 * e] = tk.h; p.ws[11 + 2 * e] = tk.row2; }   // computed again one by one
       }
     }
   }

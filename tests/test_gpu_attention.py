@@ -304,6 +304,49 @@ def test_second_launch_recomputes_tasks_whose_reference_was_too_low():
     assert_parity(o2[0, :cfg.seq].float().cpu().numpy(), ref, "max of every block", one_hot=True)
 
 
+@pytest.mark.parametrize("block,d", [(128, 128), (64, 64)])
+@pytest.mark.parametrize("what", ["large values", "no reference"])
+def test_results_out_of_the_first_launch_s_range_are_computed_again(block, d, what):
+    """What the sums of a tile do not show: (1) V of 2^90 with tile sums of up to 2^50 overflows the fp32
+    accumulator (128 bits of exponent), though the weighted mean of V does not; (2) a first tile (64-row blocks:
+    the first two) whose scores are all -inf leaves the row without a reference."""
+    cfg = dataclasses.replace(_small("wan480p", 2, 1), head_dim=d, block=block)
+    w = Workload(cfg)
+    nb, rows = cfg.n_blocks, torch.arange(cfg.seq_pad, device="cuda") // block
+    w.masks = [np.ones((nb, nb), dtype=bool)]
+    ptr_np, idx_np = I.masks_to_csr(w.masks)
+    w.ptr, w.idx = torch.from_numpy(ptr_np).cuda(), torch.from_numpy(idx_np).cuda()
+    up = 1.0
+    if what == "large values":
+        # block 12: scores of +-28 nats = 2^+-40 (five standard deviations of 8 / sqrt(d) * sqrt(d) = 8)
+        w.k[0].mul_(torch.where(rows == 12, 8.0, 1.0)[:, None])
+        up = 2.0 ** 90
+        w.v.mul_(up)
+    else:
+        w.q.abs_()
+        w.k[0].copy_(torch.where((rows * block < 128 * (128 // block))[:, None], -3e38, w.k[0].float()).to(torch.bfloat16))
+    o = torch.full_like(w.o, float("nan"))
+    lse = torch.empty((1, cfg.seq), dtype=torch.float32, device="cuda")
+    st = torch.zeros(4, dtype=torch.int32, device="cuda")
+    desc = wb.attn_desc(w.q, w.k, w.v, o, cfg.seq, cfg.seq, block)
+    ws = torch.zeros((wb.bsattn_workspace_bytes(desc),), dtype=torch.uint8, device="cuda")
+    wb.bsattn_fwd(desc, w.q, w.k, w.v, o, w.ptr, w.idx, lse=lse, workspace=ws, dev_status=st)
+    torch.cuda.synchronize()
+    assert st.tolist() == [0, 0, 0, 0]
+    n_redo = ws.view(torch.int32)[2].item()
+    listed = sorted(ws.view(torch.int32)[8:8 + 2 * n_redo].view(-1, 2)[:, 1].tolist())
+    assert n_redo > 0 and len(set(listed)) == n_redo                # every task once
+    Q, K, V = (I.bf16_to_f64(x[0].cpu()) for x in (w.q, w.k, w.v))
+    if what == "no reference":
+        assert n_redo == nb                                         # every row selects those blocks
+        K[K < -1e37] = -1e30                                        # (the oracle's scores stay finite; these weigh exp(-1e30))
+    ref, ref_lse = wo.block_sparse_attention(Q, K, V / up, w.masks[0], block, block, cfg.seq, cfg.seq)
+    g = o[0, :cfg.seq].double().cpu().numpy() / up
+    assert np.isfinite(g).all()
+    assert_parity(g, ref, what, one_hot=True)
+    assert np.abs(lse[0].cpu().numpy() - ref_lse).max() < 5e-3 * max(1.0, np.abs(ref_lse).max() / 10)
+
+
 def test_isolated_huge_key_in_a_polynomial_slot_is_recomputed():
     """One key far above everything else, in a late KV block and at a column whose exponential is
     taken from the polynomial: the fixed-reference launch must notice (its polynomial saturates
