@@ -205,12 +205,14 @@ def bitmap_to_csr(mask_bits, n_kv_blocks: int, capacity: Optional[int] = None, s
         at = buf.data_ptr()
         _check(lib.waveal_bitmap_to_csr(H, M, n_kv_blocks, _ptr(mask_bits), at, None, 0, at + 4 * n, 4 * n, _stream(stream)))
         capacity = int(buf[n - 1].item())
-    # row pointers, the call's workspace and the indices in one allocation
-    buf = mask_bits.new_empty((2 * n + max(capacity, 1),), dtype=torch.int32)
+    # the call's workspace behind the row pointers; the indices by themselves: a caller that keeps the row
+    # pointers alone does not keep the lists
+    buf = mask_bits.new_empty((2 * n,), dtype=torch.int32)
+    idx = mask_bits.new_empty((max(capacity, 1),), dtype=torch.int32)
     at = buf.data_ptr()
-    _check(lib.waveal_bitmap_to_csr(H, M, n_kv_blocks, _ptr(mask_bits), at, at + 8 * n, capacity, at + 4 * n, 4 * n,
+    _check(lib.waveal_bitmap_to_csr(H, M, n_kv_blocks, _ptr(mask_bits), at, idx.data_ptr(), capacity, at + 4 * n, 4 * n,
                                     _stream(stream)))
-    return buf.as_strided((n,), (1,), 0), buf.as_strided((capacity,), (1,), 2 * n)
+    return buf.as_strided((n,), (1,), 0), idx if capacity > 0 else idx[:0]
 
 
 def noalloc_max_rows() -> int:

@@ -105,6 +105,8 @@ def test_list_conversions(H, m, n):
     flat = mask.reshape(H * m, n)
     assert torch.equal(ptr[1:].long(), flat.sum(1).cumsum(0)) and ptr[0].item() == 0
     assert torch.equal(idx, flat.nonzero()[:, 1].int())
+    # either can be kept without the other
+    assert ptr.untyped_storage().nbytes() <= 8 * ptr.numel() and idx.untyped_storage().nbytes() == 4 * max(1, idx.numel())
     half, first = wb.bitmap_to_csr(bm, n, capacity=idx.numel() // 2)       # lists that end early: the rest is left out
     assert torch.equal(half, ptr) and torch.equal(first, idx[:idx.numel() // 2])
     if m <= 8192:                                                          # and back (8,192 columns at a time)
