@@ -797,7 +797,6 @@ struct PlanParams {
   int alias_yz;         // Y and Z share one buffer (two barriers more per iteration)
   int ksplit_y, ksplit_z, part_ints;
   unsigned off_items, off_part;     // bytes from the start of shared memory
-  double y_scale;       // power of two: |y| y_scale < 2^62
   u64 seed;
   long long kv_bytes, l2_bytes, min_nnz;
   int fit_num, fit_den, min_ppm, loc_num, loc_den;
@@ -907,7 +906,22 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
     double2* Y = p.alias_yz ? Z : Z + m_b;
     uint4* items = reinterpret_cast<uint4*>(smem + p.off_items);
     int* part = reinterpret_cast<int*>(smem + p.off_part);
-    const double y_scale = p.y_scale, x_scale = 4611686018427387904.0;     // 2^62: |x| <= 1
+    const double x_scale = 4611686018427387904.0;     // 2^62: |x| <= 1
+    double y_scale = 1.0;
+    if (p.mma) {
+      // |y_j| <= sqrt(c_j (m - c_j) / m), the norm of a centred 0/1 column: the largest column count gives a power of
+      // two 2^e >= |y|, and y_scale = 2^(62 - e).  (sqrt(m) / 2, which holds for any mask, is far above what columns of a
+      // few blocks reach and quantises coarser than fp64 rounds: 14,336 rows of one block each, one sweep, embedding
+      // against 80-bit arithmetic: 3.7e-16 with it, 1.3e-16 so and with fp64 sums.)
+      int c_mine = 0;
+      for (int j = tid; j < n_b; j += kPlanThreads) c_mine = max(c_mine, cnt[j]);
+      double c_max[1] = {(double)c_mine};
+      block_max<1>(c_max, scratch);
+      const long long c = min((int)c_max[0], m_b / 2);
+      int e = 0;
+      while (((long long)m_b << (2 * e)) < c * (m_b - c)) ++e;
+      y_scale = __longlong_as_double((long long)(1023 + 62 - e) << 52);
+    }
     const bool peers = csize > 1 && p.state_in_smem;
     auto sync_head = [&]() { if (csize > 1) cluster_sync_all(); else __syncthreads(); };
     if (p.mma)
@@ -1261,9 +1275,6 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
   p.count_stage2 = p.wave <= 220 && n < (1u << 18);
   p.mma = L.mma; p.alias_yz = L.alias_yz; p.off_items = (unsigned)L.off_items;
   p.ksplit_y = p.ksplit_z = 1;
-  int y_exp = 0;
-  while ((1ll << (2 * y_exp)) < (long long)m) ++y_exp;       // 2^y_exp >= sqrt(m) >= 2 |y| (rows of X have norm 1 by column)
-  p.y_scale = ldexp(1.0, 63 - y_exp);
   size_t smem = L.smem;
   if (L.mma) {
     // fewer groups of rows than warps: the warps of a CTA share the columns of a group

@@ -84,6 +84,47 @@ def test_plan_products_agree_between_their_forms(m, n, wide):
     assert torch.equal(a.order1, b.order1) and torch.equal(a.row_order, b.row_order)
 
 
+def _first_sweep(rows, cols, m, n, real):
+    """Q factor after one sweep of Algorithm 1 over the sorted (row, column) pairs, in NumPy at the precision `real`."""
+    def product(out, src, size, x):               # sums of x[src] over equal, ascending `out`
+        at = np.flatnonzero(np.r_[True, out[1:] != out[:-1]])
+        y = np.zeros((size, 2), real)
+        y[out[at]] = np.add.reduceat(x[src], at, axis=0)
+        return y
+
+    def qr(z):
+        q1 = z[:, 0] / np.sqrt((z[:, 0] ** 2).sum())
+        y = z[:, 1] - (q1 * z[:, 1]).sum() * q1
+        y = y - (q1 * y).sum() * q1
+        return np.stack([q1, y / np.sqrt((y * y).sum())], 1)
+
+    c = np.bincount(cols, minlength=n).astype(real)[:, None]
+    by_col = np.argsort(cols, kind="stable")
+    x = qr(wo.start_block(5, 0, m).astype(real))
+    y = product(cols[by_col], rows[by_col], n, x) - c * (x.sum(0) / m)
+    return qr(product(rows, cols, m, y) - (c * y).sum(0) / m)
+
+
+# rows of one or two blocks: the entries of a sweep are far below what a mask of that size can reach
+@pytest.mark.parametrize("m,blocks", [(14336, 1), (14336, 2), (2841, 1), (300, 2)])
+def test_products_of_sparse_masks_are_as_close_as_fp64_sums(m, blocks):
+    rng = np.random.default_rng(3)
+    mask = torch.zeros((1, m, m), dtype=torch.bool, device="cuda")
+    mask[0, torch.arange(m, device="cuda").repeat_interleave(blocks), torch.from_numpy(rng.integers(0, m, m * blocks)).cuda()] = True
+    rows, cols = (x.cpu().numpy() for x in mask[0].nonzero(as_tuple=True))
+    d = wb.plan_desc_default(heads=1, n_q_blocks=m, n_kv_blocks=m, wave_size=148, mode=wb.FORCE_REORDER, seed=5, svd_iters=1)
+    e = wb.plan_bitmap(d, _pack(mask), debug=True).embedding[0].cpu().numpy()
+    exact = _first_sweep(rows, cols, m, m, np.longdouble)
+
+    def off(u):                                   # part of u outside the exact plane (rotation, sign and scale drop out)
+        u = u.astype(np.longdouble)
+        r = u - exact @ (exact.T @ u)
+        return float(np.sqrt((r * r).sum() / (u * u).sum()))
+
+    # (the last QR step's own rounding is in both; 1.5: the kernel's sums are not NumPy's)
+    assert off(e) <= 1.5 * off(_first_sweep(rows, cols, m, m, np.float64))
+
+
 @pytest.mark.parametrize("m", [9600, 9601])       # the second sort buffer fits shared memory, or not
 def test_sorts_of_many_rows(m):
     mask = _mask(1, m, 64, 0.3, m)
