@@ -517,7 +517,6 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   volatile int* redo_flag = reinterpret_cast<volatile int*>(smem + G::OFF_MISC + 8);
   int* redo_listed = reinterpret_cast<int*>(smem + G::OFF_MISC + 24);
   Ctx ctx{bar0, abort_smem, p.ws, p.dev_status, p.wait_limit};
-  const long long t_start = clock64();
 
   if (tid == 0) {
     // a task is read by the V loader, the two MMA issuers and the sixteen softmax warps
@@ -556,6 +555,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_holder, 0);
   // tickets, table and counters are the work of the kernel before this one
   waveal::wait_for_previous_kernel();
+  const long long t_start = clock64();          // (that kernel's time is not this launch's)
 
   // Every role walks the same sequence of tasks (query blocks) and, inside a task, of KV blocks;
   // block number g (counted over the CTA's whole life) uses S buffer g mod 3, K stage g mod NKS
@@ -1133,7 +1133,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     tc_fence_after();
     tmem_dealloc(tmem_base, G::TMEM_COLS);
   }
-  // SM cycles this CTA was alive: the largest over the grid is the launch's length in cycles,
+  // SM cycles since the launch before this one ended: the largest over the grid is the launch's length in cycles,
   // a figure that does not depend on the clock the GPU happened to run at
   if (tid == 0) {
     const long long dt = clock64() - t_start;
