@@ -165,6 +165,7 @@ __device__ __forceinline__ void fadd2(float& d0, float& d1, float a0, float a1, 
 // 7.5e-5, far below the bf16 cut of P), and n is added to the exponent field.
 constexpr float kPolyLo = -64.0f;
 constexpr float kRedoLimit = 1152921504606846976.0f;     // 2^60: tile sums at or above it (or NaN) list the task
+constexpr float kCheckSum = 16777216.0f;                 // 2^24: rows with a sum at or above it are looked over for results that are not finite
 __device__ __forceinline__ float fma_sat(float a, float b, float c) {
   float d;
   asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
@@ -480,6 +481,20 @@ __device__ __noinline__ void mask_scores(uint32_t s_addr, int valid) {
   tc_wait_st();
 }
 
+// a task for the second launch, unless another warp has listed it already; the blocks of a pair are computed again one by one
+// (out of line for 64-row blocks, 18.75 M -> 18.35 M cycles on 8 heads of 1536 rows; for 128-row blocks in line, 521 k -> 506 k
+// on 5 heads of 256 rows: a call there makes the compiler spill)
+__device__ __forceinline__ void list_task(int* ws, int* listed, int task_no, int h, int row, int row2) {
+  if (atomicExch(listed, task_no) == task_no) return;
+  const int e = atomicAdd(&ws[2], row2 >= 0 ? 2 : 1);
+  ws[8 + 2 * e] = h;
+  ws[9 + 2 * e] = row;
+  if (row2 >= 0) { ws[10 + 2 * e] = h; ws[11 + 2 * e] = row2; }
+}
+__device__ __noinline__ void list_task_call(int* ws, int* listed, int task_no, int h, int row, int row2) {
+  list_task(ws, listed, task_no, h, row, row2);
+}
+
 template <int BLOCK, int D, bool FAST>
 __global__ void __launch_bounds__(kThreads, 1)
 k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
@@ -536,7 +551,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     mbar_init(BAR(B_FINAL + 1), 1);
     for (int i = 0; i < 16; ++i) mbar_init(BAR(B_MX + i), 1);   // (lane quadrant, tile count mod 4)
     for (int i = 0; i < 16; ++i) mbar_init(BAR(B_EX + i), 4);   // (task mod 4, lane quadrant): its four warps, once per task
-    for (int i = 0; i < 8; ++i) mbar_init(BAR(B_HX + i), 2);    // the two owners of a row (team, quadrant), once per max and once per rescale of O
+    for (int i = 0; i < 8; ++i) mbar_init(BAR(B_HX + i), 2);    // the two owners of a row (team, quadrant), once per max
     *abort_smem = 0;
     for (int i = 0; i < 4; ++i) { redo_flag[i] = 0; redo_listed[i] = 0; }
     fence_mbar_init();
@@ -859,6 +874,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     uint32_t task_it = 0, o_it = 0, mx_phase = 0, hx_it = 0;
     uint32_t g0 = 0;                           // tiles before this task
     uint32_t sb = (uint32_t)team, s_ph = 0;    // S buffer of this team's next tile and the parity of that use
+    constexpr bool kRescales = !FAST || G::MAX_TILES > 1;     // (a reference that is taken once never grows)
     auto next_buffer = [&]() { sb += 2; if (sb >= (uint32_t)G::NSBUF) { sb -= (uint32_t)G::NSBUF; s_ph ^= 1; } };
     bool ok = true;
     while (ok) {
@@ -975,17 +991,17 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           // rare: the reference grew, so O (blocks 0..j-1) is rescaled; its last MMA (block j-1)
           // must be complete: that is the latest phase of the barrier of the S buffer before
           // this one (the next P V on that buffer needs a P this team has not produced yet).
-          // Each owner takes half of the row's output columns, and both halves are done before either half of
-          // P_j is released: the P V warp starts on the first half of P as soon as that one has arrived, and
-          // those MMAs add to all columns of O.  So the two meet once more (the decision to grow is the same in both).
-          if (grow && j > 0) {
+          // The owner of the first half of P does it for all columns of O before it releases that half: the P V
+          // warp starts on the first half as soon as it has arrived, its MMAs add to all columns, and those on the
+          // second half come behind.  (Split between the two owners, each would have to wait for the other.)
+          if (kRescales && grow && j > 0 && half == 0) {
             const uint32_t sbp = sb == 0 ? (uint32_t)G::NSBUF - 1u : sb - 1u;
             ok = warp_wait(ctx, BAR(B_S_FREE + sbp), sb == 0 ? s_ph ^ 1u : s_ph, 22);
             if (!ok) break;
             tc_fence_after();
             const float alpha = ex2(m_prev - m_new);
 #pragma unroll 1
-            for (int c0 = half * (D / 2); c0 < (half + 1) * (D / 2); c0 += 32) {
+            for (int c0 = 0; c0 < D; c0 += 32) {
               uint32_t ov[32];
               WAVEAL_TMEM_LD32(o_row + c0, ov, 0);
               WAVEAL_TMEM_WAIT_LD32(ov, 0);
@@ -993,14 +1009,6 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
               for (int c = 0; c < 32; ++c) ov[c] = __float_as_uint(__uint_as_float(ov[c]) * alpha);
               WAVEAL_TMEM_ST32(o_row + c0, ov, 0);
             }
-            tc_wait_st();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(BAR(B_HX + team * 4 + quad));
-            ok = warp_wait(ctx, BAR(B_HX + team * 4 + quad), hx_it & 1u, 27);
-            if (!ok) break;
-            ++hx_it;
-            tc_fence_after();
           }
           // p' = 2^(s*scale*log2e - m + log2(1 + 2^-9)); P is p' cut to its top 16 bits (one byte
           // permute per pair instead of a conversion).  The extra factor centres the cut's error
@@ -1093,15 +1101,18 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         // its cost in the memory pipe is per row, not per byte.  32-byte stores halve the number
         // of instructions where the row piece is 32-byte aligned (else 16-byte stores)
         uint32_t w[G::CO / 2];
-        float z0 = 0.f, z1 = 0.f;          // stay 0 as long as every result is finite
 #pragma unroll
         for (int c = 0; c < G::CO; c += 2) {
-          const float o0 = __uint_as_float(ov[c]) * inv_l, o1 = __uint_as_float(ov[c + 1]) * inv_l;
-          if (FAST) ffma2(z0, z1, o0, o1, 0.f, 0.f, z0, z1);
-          __nv_bfloat162 b2 = __floats2bfloat162_rn(o0, o1);
+          __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(ov[c]) * inv_l, __uint_as_float(ov[c + 1]) * inv_l);
           w[c / 2] = *reinterpret_cast<uint32_t*>(&b2);
         }
-        bad = FAST && !(z0 + z1 == 0.f);
+        // |O| <= l_tot max|V|: only a large sum (or none) can have led out of fp32's range
+        if (FAST && !(l_tot > 0.f && l_tot < kCheckSum)) {
+          uint32_t top = 0;                // an exponent field of ones in either half of a pair carries into its top bit
+#pragma unroll
+          for (int c = 0; c < G::CO / 2; ++c) top |= (w[c] & 0x7F807F80u) + 0x00800080u;
+          bad = (top & 0x80008000u) != 0;
+        }
         if ((reinterpret_cast<uintptr_t>(o_ptr) & 31) == 0) {
 #pragma unroll
           for (int c = 0; c < G::CO / 2; c += 8) st_global_v8(o_ptr + 2 * c, w + c);
@@ -1116,12 +1127,9 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       // before O_FULL) or if a result is not finite: with sums of up to 2^60 O overflows from |V| = 2^67 on, and a
       // first tile whose scores are all -inf leaves no reference.  (Where V itself holds an inf or NaN the second
       // launch finds the same again.)  Whichever of the epilogue's warps sees it first writes the entry.
-      if (FAST && (__any_sync(0xffffffffu, bad) || redo_flag[rslot] == task_no) && lane == 0 &&
-          atomicExch(&redo_listed[rslot], task_no) != task_no) {
-        const int e = atomicAdd(&p.ws[2], (G::KB == 2 && tk.row2 >= 0) ? 2 : 1);
-        p.ws[8 + 2 * e] = tk.h;
-        p.ws[9 + 2 * e] = tk.row;
-        if (G::KB == 2 && tk.row2 >= 0) { p.ws[10 + 2 * e] = tk.h; p.ws[11 + 2 * e] = tk.row2; }   // computed again one by one
+      if (FAST && (__any_sync(0xffffffffu, bad) || redo_flag[rslot] == task_no) && lane == 0) {
+        if constexpr (G::KB == 2) list_task_call(p.ws, &redo_listed[rslot], task_no, tk.h, tk.row, tk.row2);
+        else list_task(p.ws, &redo_listed[rslot], task_no, tk.h, tk.row, -1);
       }
     }
   }
