@@ -278,7 +278,7 @@ def test_second_launch_recomputes_tasks_whose_reference_was_too_low():
     k = w.k[0].float()
     k[jb * b:(jb + 1) * b] *= 40.0
     w.k[0].copy_(k.to(torch.bfloat16))
-    hit = [i for i in range(nb) if w.masks[0][i, jb] and np.nonzero(w.masks[0][i])[0].tolist().index(jb) >= 2]
+    hit = [i for i in range(nb) if w.masks[0][i, jb] and np.nonzero(w.masks[0][i])[0].tolist().index(jb) >= 1]
     assert len(hit) >= 3
     o = torch.full_like(w.o, float("nan"))
     ws.zero_()
@@ -347,36 +347,50 @@ def test_results_out_of_the_first_launch_s_range_are_computed_again(block, d, wh
     assert np.abs(lse[0].cpu().numpy() - ref_lse).max() < 5e-3 * max(1.0, np.abs(ref_lse).max() / 10)
 
 
-def test_isolated_huge_key_in_a_polynomial_slot_is_recomputed():
-    """One key far above everything else, in a late KV block and at a column whose exponential is
-    taken from the polynomial: the fixed-reference launch must notice (its polynomial saturates
-    instead of wrapping around), list the task, and the second launch must match the oracle."""
-    cfg = _small("wan480p", 3, 1)
+# a pair of neighbouring columns in five takes the polynomial: columns 8, 9, 18, 19, 28 and 29 of every 32 (0 and 70 do not)
+@pytest.mark.parametrize("block,d,first_fixed", [(128, 128, 1), (64, 64, 2)])      # tile from which the reference stays
+@pytest.mark.parametrize("col", [0, 8, 19, 28, 70, 64 + 40, 64 + 61])
+def test_isolated_huge_key_is_recomputed(block, d, first_fixed, col):
+    """One key far above everything else, in a late tile, at a column whose exponential is taken from the polynomial
+    or the transcendental unit: above 2^60 the fixed-reference launch must notice (its polynomial saturates at 2^64
+    instead of wrapping around), list the task, and the second launch must match the oracle; below, the
+    task stays with the first launch and matches it too."""
+    cfg = dataclasses.replace(_small("wan480p", 2, 1), head_dim=d, block=block)
     w = Workload(cfg)
-    b, nb = cfg.block, cfg.n_blocks
-    jb = 20
-    for col in (0, 2, 3, 70):             # 2, 3 and 70 = 64 + 6 are polynomial slots of a 64-column chunk, 0 is not
-        w2 = Workload(cfg)
-        k = w2.k[0].float()
-        k[jb * b + col] *= 300.0          # scores of about +-300 nats on this key
-        w2.k[0].copy_(k.to(torch.bfloat16))
-        d = wb.attn_desc(w2.q, w2.k, w2.v, w2.o, cfg.seq, cfg.seq, b)
-        ws = torch.zeros((wb.bsattn_workspace_bytes(d),), dtype=torch.uint8, device="cuda")
+    nb, per = cfg.n_blocks, 128 // block
+    rng = np.random.default_rng(7)
+    mask = rng.random((nb, nb)) < 0.6
+    ib = 3 * nb // 4 // 2 * 2                     # 64-row blocks: a pair of blocks, so that `col` is a column of one tile
+    mask[:, ib:ib + per] = (rng.random(nb) < 0.7)[:, None]
+    if per == 2:                                  # an even number of blocks in front of it
+        for i in range(nb):
+            if mask[i, :ib].sum() % 2:
+                mask[i, 0] ^= True
+    w.masks = [mask]
+    ptr_np, idx_np = I.masks_to_csr(w.masks)
+    w.ptr, w.idx = torch.from_numpy(ptr_np).cuda(), torch.from_numpy(idx_np).cuda()
+    # dimension 0 of Q is 8 and of K 0 but for the one key, which has nothing else: its score is the same for all queries
+    w.q[..., 0] = 8.0
+    w.k[..., 0] = 0.0
+    hit = [i for i in range(nb) if mask[i, ib] and mask[i, :ib].sum() // per >= first_fixed]
+    assert 3 <= len(hit) < nb
+    # nats of the key: exponents of about 2^(43 - 6), 2^(87 - 6) and 2^(288 - 6) above a reference of 2 to 6 nats
+    for nats, listed_then in ((30.0, []), (60.0, hit), (200.0, hit)):
+        w.k[0, ib * block + col] = 0.0
+        w.k[0, ib * block + col, 0] = nats * math.sqrt(d) / 8.0
+        desc = wb.attn_desc(w.q, w.k, w.v, w.o, cfg.seq, cfg.seq, block, flags=wb.ATTN_NO_ROW_PAIRING)
+        ws = torch.zeros((wb.bsattn_workspace_bytes(desc),), dtype=torch.uint8, device="cuda")
         st = torch.zeros(4, dtype=torch.int32, device="cuda")
-        o = torch.full_like(w2.o, float("nan"))
-        wb.bsattn_fwd(d, w2.q, w2.k, w2.v, o, w2.ptr, w2.idx, workspace=ws, dev_status=st)
+        w.o.fill_(float("nan"))
+        wb.bsattn_fwd(desc, w.q, w.k, w.v, w.o, w.ptr, w.idx, workspace=ws, dev_status=st)
         torch.cuda.synchronize()
         assert st.tolist() == [0, 0, 0, 0]
-        hit = [i for i in range(nb) if w2.masks[0][i, jb] and np.nonzero(w2.masks[0][i])[0].tolist().index(jb) >= 2]
         n_redo = ws.view(torch.int32)[2].item()
         listed = sorted(ws.view(torch.int32)[8:8 + 2 * n_redo].view(-1, 2)[:, 1].tolist())
-        assert len(hit) >= 3 and listed == hit, (col, listed, hit)
-        K64 = I.bf16_to_f64(w2.k[0].cpu())
-        ref, _ = wo.block_sparse_attention(w2.head_f64("q", 0), K64, w2.head_f64("v", 0), w2.masks[0], b, b,
-                                           cfg.seq, cfg.seq)
-        g = o[0, :cfg.seq].float().cpu().numpy()
-        assert np.isfinite(g).all()
-        assert_parity(g, ref, f"huge key at column {col}", one_hot=True)
+        assert listed == listed_then, (nats, listed, listed_then)
+        Q, K = (I.bf16_to_f64(x[0].cpu()) for x in (w.q, w.k))
+        ref, _ = wo.block_sparse_attention(Q, K, w.head_f64("v", 0), mask, block, block, cfg.seq, cfg.seq)
+        assert_parity(w.o[0, :cfg.seq].float().cpu().numpy(), ref, f"{nats} nats at column {col}", one_hot=True)
 
 
 MASKS = ["dense", "random20"]

@@ -38,9 +38,11 @@ def _plan(mask, wave=148, mode=wb.FORCE_REORDER):
 
 
 # 256 / 257 rows: one CTA or a cluster; 255 / 256 / 257 columns: one 256-column chunk or two; wave 220 / 221: Stage 2 by
-# counting or by the sort; one row or one column
+# counting or by the sort; one row or one column; 14,336 / 14,337 rows: digits in shared memory and the state in the workspace, or
+# the walk by a cluster over that state; 16,384 rows: the most the plan takes, and the longest strip of the transpose
 @pytest.mark.parametrize("H,m,n,wave", [(2, 1, 1, 148), (2, 1, 300, 7), (2, 33, 1, 7), (3, 31, 255, 16), (2, 256, 256, 220),
-                                        (2, 257, 257, 221), (1, 600, 511, 148)])
+                                        (2, 257, 257, 221), (1, 600, 511, 148),
+                                        (2, 14336, 200, 148), (2, 14337, 200, 148), (1, 16384, 200, 148)])
 def test_plan_products_match_the_oracle(H, m, n, wave):
     mask = _mask(H, m, n, 0.2, m + n)
     r = _plan(mask, wave)
@@ -74,7 +76,9 @@ def test_waves_longer_than_the_head(m):
 
 # columns that select nothing change no product: the same mask with 10,000 of them goes through the walk over the
 # set bits, widened to 4,700 x 4,700 or 5,000 x 5,000 through the shared Y / Z buffer or the workspace
-@pytest.mark.parametrize("m,n,wide", [(100, 300, 10000), (4700, 300, 4700), (5000, 300, 5000)])
+# (4,768: the last square whose digits fit beside the state; then the walk; columns beyond 14,336: the walk over the workspace)
+@pytest.mark.parametrize("m,n,wide", [(100, 300, 10000), (4700, 300, 4700), (4768, 300, 4768), (4769, 300, 4769),
+                                      (5000, 300, 5000), (2000, 300, 14336), (2000, 300, 14400)])
 def test_plan_products_agree_between_their_forms(m, n, wide):
     mask = _mask(2, m, n, 0.1, 9)
     padded = torch.zeros((2, m, wide), dtype=torch.bool, device="cuda")
@@ -187,10 +191,10 @@ def test_host_threads_plan_different_sizes():
         assert torch.equal(res.row_nnz.long(), nnz)
 
 
-def _attend(q, k, v, block, ptr, idx, T, order=None, flags=0):
+def _attend(q, k, v, block, ptr, idx, T, order=None, flags=0, interleaved=False):
     o = torch.full_like(q, float("nan"))
     lse = torch.full(q.shape[:2], float("nan"), device="cuda")
-    d = wb.attn_desc(q, k, v, o, T, T, block, flags=flags)
+    d = wb.attn_desc(q, k, v, o, T, T, block, interleaved, flags=flags)
     ws = torch.empty((wb.bsattn_workspace_bytes(d),), dtype=torch.uint8, device="cuda")
     st = torch.zeros((4,), dtype=torch.int32, device="cuda")
     wb.bsattn_fwd(d, q, k, v, o, ptr, idx, row_order=order, lse=lse, workspace=ws, dev_status=st)
@@ -241,6 +245,35 @@ def test_short_tasks_back_to_back(block, D, tasks):
         assert ((got - ref).abs() <= bound)[live].all()
         # the polynomial share of the exponentials is within 7.5e-5 of itself, fp32 scores and logarithm add a few 1e-6
         assert ((got_lse - s.logsumexp(-1)).abs() <= 1.5e-4)[live].all()
+
+
+# heads of unequal row lengths, more tickets than the sorted tail: no order of heads or rows shows in the results
+@pytest.mark.parametrize("block,nb", [(128, 420), (64, 420), (128, 300)])
+def test_tail_over_several_heads(block, nb):
+    H = 3
+    mask = torch.cat([_mask(1, nb, nb, dens, nb + i) for i, dens in enumerate((0.01, 0.08, 0.03))])
+    mask[1, 5] = True
+    mask[2, 9] = False
+    ptr, idx = wb.bitmap_to_csr(_pack(mask), nb)
+    T = nb * block - 11
+    q, k, v = _inputs(H, T, 64, 6)
+    order = torch.stack([torch.randperm(nb, generator=torch.Generator().manual_seed(h)) for h in range(H)]).int().cuda()
+    o, lse, w = _attend(q, k, v, block, ptr, idx, T)
+    for order_i in (None, order):
+        for interleaved in (False, True):
+            o2, lse2, w2 = _attend(q, k, v, block, ptr, idx, T, order=order_i, interleaved=interleaved)
+            assert torch.equal(o, o2) and torch.equal(lse, lse2)
+            assert w2[0] >= H * nb
+    assert (o[2, 9 * block:10 * block] == 0).all() and not torch.isnan(o).any()
+    for h, i in ((0, 0), (1, 5), (2, nb - 1)):
+        blocks = mask[h, i].nonzero()[:, 0]
+        sel = (blocks[:, None] * block + torch.arange(block, device="cuda")).flatten()
+        sel = sel[sel < T]
+        s = q[h, i * block:(i + 1) * block].double() @ k[h, sel].double().T / 8.0
+        p = s.softmax(-1)
+        ref = p @ v[h, sel].double()
+        bound = 2.0 ** -8 * (p @ v[h, sel].double().abs()) + 2.0 ** -8 * ref.abs() + 1e-6      # as in the test above
+        assert ((o[h, i * block:(i + 1) * block].double() - ref).abs() <= bound).all()
 
 
 # rows that select everything stand in several blocks of 64 positions, an odd number of them, besides equal neighbours
