@@ -168,10 +168,10 @@ size_t waveal_noalloc_max_rows(void);
 
 /* waveal_attn_desc.flags: take the row max of every KV block (the online-softmax rule as the
  * paper's backends apply it) in a single launch.  Without the flag the kernel fixes each row's
- * reference after the first two blocks of a task - softmax does not depend on the reference as
- * long as nothing overflows - watches the size of every block's sum, lists the tasks where a
- * sum reached 2^24 and computes those again, with the max of every block, in a second launch
- * on the same stream.  Results agree to rounding; the flag exists for comparison runs. */
+ * reference after the first 128 keys of a task (64-row blocks: the first 256) - softmax does not depend on the
+ * reference as long as nothing overflows - watches the size of every later sum and, where a row's sum is large, its
+ * results, lists the tasks where a sum reached 2^60 or a result is not finite and computes those again, with the max of
+ * every block, in a second launch on the same stream.  Results agree to rounding; the flag exists for comparison runs. */
 #define WAVEAL_ATTN_ONLINE_MAX_ONLY 1
 /* Self-test of the kernel's failure handling, never set in production: the loader leaves out
  * the first K tile of the first task and every bounded wait gives up after about 2 ms instead
@@ -216,8 +216,9 @@ waveal_status waveal_bsattn_workspace_bytes(const waveal_attn_desc* desc /*host*
  * for query block i of head h, O = softmax(scale * Q_i K_sel^T) V_sel over the tokens of
  * the K/V blocks listed for (h, i), visited in the listed (ascending) order.
  * Persistent CTAs take (head, position) tickets in head-major order and process query
- * block row_order[h][position] (Algorithm 2 output; NULL = natural order; the last 1,024 tickets of a
- * call, seven per SM, are handed out longest list first, so that no SM is left with a long row at the end); each output
+ * block row_order[h][position] (Algorithm 2 output; NULL = natural order); the last 1,024 tickets of a
+ * call, seven per SM, are handed out longest list first, so that no SM is left with a long row at the end (a call of no
+ * more blocks than that runs in this order alone, whatever row_order and order_heads_interleaved say); each output
  * tile is written at its original rows, so no inverse permutation pass exists.
  * Q, K, V, O: dev bf16, 16-byte aligned, strides multiples of 8 elements, head_dim
  * contiguous; query tokens >= seq_q are not written; keys >= seq_kv are ignored.

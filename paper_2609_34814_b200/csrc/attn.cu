@@ -30,7 +30,7 @@
 // Two launches per call: in the first the row max is taken in the first tile of a task only (64-row blocks:
 // the first two) and the reference stays fixed afterwards (softmax does not depend on it short of
 // overflow: P in bf16, the sums and O in fp32 have the same exponent range); a task in which a
-// tile's sum of exponentials reaches 2^60 is listed in the workspace and computed
+// tile's sum of exponentials reaches 2^60 or a result is not finite is listed in the workspace and computed
 // again by the second launch, which takes the max of every tile.
 // Every wait on an mbarrier is bounded; when one runs out the CTA records
 // {WAVEAL_ERR_TIMEOUT, site} and all roles leave through the common teardown.
@@ -41,7 +41,7 @@
 
 namespace {
 
-// 19 warps, and a 20th (the V tile loader) in the kernels of the 64-row blocks
+// 20 warps: producer, two MMA issuers, sixteen softmax warps, V tile loader
 constexpr int kThreads = 640;
 constexpr int kProducerWarp = 0, kPvWarp = 1, kSoftmaxWarp0 = 2, kQkWarp = 18, kVLoadWarp = 19;
 constexpr long long kTimeoutCycles = 4000000000ll;   // ~2 s at boost clock
@@ -165,7 +165,7 @@ __device__ __forceinline__ void fadd2(float& d0, float& d1, float a0, float a1, 
 // 7.5e-5, far below the bf16 cut of P), and n is added to the exponent field.
 constexpr float kPolyLo = -64.0f;
 constexpr float kRedoLimit = 1152921504606846976.0f;     // 2^60: tile sums at or above it (or NaN) list the task
-constexpr float kCheckSum = 16777216.0f;                 // 2^24: rows with a sum at or above it are looked over for results that are not finite
+constexpr float kCheckSum = 16777216.0f;                 // 2^24: results of rows with a sum at or above it are checked for being finite
 __device__ __forceinline__ float fma_sat(float a, float b, float c) {
   float d;
   asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
@@ -1190,7 +1190,9 @@ __device__ __forceinline__ void clear_counters(const AttnParams& p) {
 // or natural order a long row may start last and leave the other SMs waiting for it: the row lengths of
 // the masks in use spread over a factor of ten.  Calls of a few tasks per SM gain most (5 heads of 256
 // rows: 655k -> 494k cycles), the largest lose nothing: before the last 1,024 tickets the order is the
-// caller's, and no result depends on it.  A histogram of 1,024 lengths is enough (which of two tasks of
+// caller's, and no result depends on it.  The tail reads K and V more often than the planned order would (8 heads of 591
+// rows: 0.88 GB against 0.58 GB), which costs less than the balance brings also where a head's K+V exceed L2: 1 / 2 / 5
+// heads of 2,841 planned rows 2.38 / 5.25 / 13.25 ms, without the tail 3.18 / 5.74 / 13.63 ms.  A histogram of 1,024 lengths is enough (which of two tasks of
 // about the same length goes first makes no difference).
 constexpr int kTailTasks = 1024;
 __device__ __forceinline__ int tail_place(int n, bool live) {            // called by a block of kTailTasks threads
@@ -1473,7 +1475,7 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
     waveal::launch_counter() = launches + 1;
     return WAVEAL_OK;
   }
-  // first pass: reference fixed after the first two blocks of a task; second pass: the tasks the
+  // first pass: reference fixed after the first tile of a task (64-row blocks: the first two); second pass: the tasks the
   // first one listed (normally none: its CTAs leave at once), max of every block
   p.redo_pass = 0;
   WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, true>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, p));

@@ -1081,7 +1081,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
   //      Stage-1 position
   if (p.count_stage2) {
     // small buckets: a row's place is the number of rows of its bucket that go before it, by a key of
-    // (n_b - n_i, position) in 32 bits.  The rows of a warp share a bucket, so the keys are read as broadcasts:
+    // (n_b - n_i, position) in 32 bits.  Most warps lie in one bucket, whose keys they read as broadcasts:
     // ~2.5 instructions per comparison, against the ~600 an element takes in the merge sort.
     unsigned* key = reinterpret_cast<unsigned*>(keys);
     for (int i = tid; i < m_b; i += kPlanThreads) key[i] = (unsigned)(n_b - nnz[vals[i]]) << 14 | (unsigned)i;
