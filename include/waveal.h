@@ -168,7 +168,7 @@ size_t waveal_noalloc_max_rows(void);
 
 /* waveal_attn_desc.flags: take the row max of every KV block (the online-softmax rule as the
  * paper's backends apply it) in a single launch.  Without the flag the kernel fixes each row's
- * reference after the first 128 keys of a task (64-row blocks: the first 256) - softmax does not depend on the
+ * reference after the first 128 keys of a task - softmax does not depend on the
  * reference as long as nothing overflows - watches the size of every later sum and, where a row's sum is large, its
  * results, lists the tasks where a sum reached 2^60 or a result is not finite and computes those again, with the max of
  * every block, in a second launch on the same stream.  Results agree to rounding; the flag exists for comparison runs. */

@@ -27,8 +27,8 @@
 //               sum of its own columns; O in tensor memory is rescaled only when the max grew
 //               by more than 2^8; the epilogue adds the four partial sums of a row, normalises
 //               and stores O at the ORIGINAL row (no inverse permutation)
-// Two launches per call: in the first the row max is taken in the first tile of a task only (64-row blocks:
-// the first two) and the reference stays fixed afterwards (softmax does not depend on it short of
+// Two launches per call: in the first the row max is taken in the first tile of a task only
+// and the reference stays fixed afterwards (softmax does not depend on it short of
 // overflow: P in bf16, the sums and O in fp32 have the same exponent range); a task in which a
 // tile's sum of exponentials reaches 2^60 or a result is not finite is listed in the workspace and computed
 // again by the second launch, which takes the max of every tile.
@@ -264,6 +264,21 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
+// largest of 32 scores
+__device__ __forceinline__ float row_max32(const uint32_t (&sv)[32]) {
+  float mx4[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) mx4[i] = __uint_as_float(sv[i]);
+#pragma unroll
+  for (int c = 4; c < 28; c += 8) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) mx4[i] = fmax3(mx4[i], __uint_as_float(sv[c + 2 * i]), __uint_as_float(sv[c + 2 * i + 1]));
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) mx4[i] = fmaxf(mx4[i], __uint_as_float(sv[28 + i]));
+  return fmaxf(fmax3(mx4[0], mx4[1], mx4[2]), mx4[3]);
+}
+
 // shared-memory matrix descriptor, 128-byte swizzle, Blackwell version field
 __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
   uint64_t d = 0;
@@ -345,9 +360,6 @@ struct Geo {
   static constexpr int NSTAGE = NSTAGE_RAW > 8 ? 8 : NSTAGE_RAW;
   static constexpr int NKS = (NSTAGE + 1) / 2;       // K tile ring
   static constexpr int NVS = NSTAGE / 2;             // V tile ring
-  // tiles of a task that take a row max in the first launch (one instead of two: 5.7k -> 4.6k clk a task beyond its
-  // tiles; the 64-row kernels, which keep only half of their warps busy, do not gain: +3 % cycles)
-  static constexpr int MAX_TILES = KB == 1 ? 1 : 2;
   static constexpr int NSBUF = 3;                    // S/P buffers in tensor memory
   static constexpr int HC = BK / 2;                  // S columns of a row one softmax thread owns (a row has two owners)
   static constexpr int CH = 32;                      // S columns a softmax thread holds at a time
@@ -523,7 +535,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                 B_EX = B_MX + 16, B_HX = B_EX + 16;
   static_assert(B_HX + 8 <= G::N_BAR, "barrier count");
   Task* tasks = reinterpret_cast<Task*>(smem + G::OFF_TASK);
-  volatile float* mpub = reinterpret_cast<volatile float*>(smem + G::OFF_MX);   // [tile count mod 4][128] reference max after a tile
+  volatile float* mpub = reinterpret_cast<volatile float*>(smem + G::OFF_MX);   // [tile count mod 4][128] reference max after a tile; FAST: [tile count mod 4][column half][128], over mhalf too
   volatile float* mhalf = reinterpret_cast<volatile float*>(smem + G::OFF_MX + 4 * 128 * 4);   // [use parity][team][column half][128] max of a half row
   float2* ex = reinterpret_cast<float2*>(smem + G::OFF_MX + 4 * 128 * 4 + 2 * 2 * 2 * 128 * 4);    // [task mod 4][tile parity*2+half][128] (reference, sum)
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + G::OFF_MISC);
@@ -549,7 +561,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     mbar_init(BAR(B_O_FREE), 8);              // the team that runs the epilogue
     mbar_init(BAR(B_FINAL), 1);
     mbar_init(BAR(B_FINAL + 1), 1);
-    for (int i = 0; i < 16; ++i) mbar_init(BAR(B_MX + i), 1);   // (lane quadrant, tile count mod 4)
+    for (int i = 0; i < 16; ++i) mbar_init(BAR(B_MX + i), FAST ? 2 : 1);   // (lane quadrant, tile count mod 4)
     for (int i = 0; i < 16; ++i) mbar_init(BAR(B_EX + i), 4);   // (task mod 4, lane quadrant): its four warps, once per task
     for (int i = 0; i < 8; ++i) mbar_init(BAR(B_HX + i), 2);    // the two owners of a row (team, quadrant), once per max
     *abort_smem = 0;
@@ -874,7 +886,6 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     uint32_t task_it = 0, o_it = 0, mx_phase = 0, hx_it = 0;
     uint32_t g0 = 0;                           // tiles before this task
     uint32_t sb = (uint32_t)team, s_ph = 0;    // S buffer of this team's next tile and the parity of that use
-    constexpr bool kRescales = !FAST || G::MAX_TILES > 1;     // (a reference that is taken once never grows)
     auto next_buffer = [&]() { sb += 2; if (sb >= (uint32_t)G::NSBUF) { sb -= (uint32_t)G::NSBUF; s_ph ^= 1; } };
     bool ok = true;
     while (ok) {
@@ -924,31 +935,51 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           if (ragged) mask_scores<G::NCH>(s_addr, tk.tail_valid - half * G::HC);   // keys beyond seq_kv (ragged last block) do not exist
           // ---- pass 1: row max (the values are loaded again for the exponentials: a second
           // tensor-memory load is cheaper than keeping them in registers)
-          // In the first pass over the tasks (FAST) only the first MAX_TILES tiles of a task take a max and
-          // may move the reference; both teams keep it from there on.
-          // Any reference gives the same softmax as long as nothing overflows, so the later
-          // tiles only watch the sum of the exponentials they produce: if it ever reaches 2^60 the
-          // task is put on a list and computed again by the second launch, which takes the
-          // max of every tile (the rule of the paper's online softmax).
-          const bool fixed_ref = FAST && j >= G::MAX_TILES;
+          // In the first pass over the tasks (FAST) only the first tile of a task takes a max; both teams keep it as
+          // their reference.  Any reference gives the same softmax as long as nothing overflows, so all tiles watch the
+          // sum of the exponentials they produce: if it ever reaches 2^60 the task is put on a list and computed again
+          // by the second launch, which takes the max of every tile (the rule of the paper's online softmax).
+          // One tile and one meeting of all who need its max, and nothing of the rule for a max that grows in this kernel
+          // (no rescale of O, no hand-over from tile to tile): against the code with both in it, and two such tiles for
+          // 64-row blocks, 64x128 rows of 64 / 256 blocks 1,485 -> 1,383 / 1,359 -> 1,290 clk a tile, 64x64 1,326 -> 1,260,
+          // 128x128 tasks of 38 / 256 tiles 1,520 -> 1,492 / 1,385 -> 1,363, 128x64 1,311 -> 1,272.  A max over 32 keys only
+          // would save another 1-4 %, but scores that spread by 40 nats inside a tile then need the second launch.
+          float m_new;
+          if constexpr (FAST) {
+            // The two owners of the row in the first tile leave the largest of their own scores; they and, at its first tile,
+            // the other team take the larger of the two.  (Slot and barrier by tile count mod 4: a later task's first tile
+            // that uses the slot again waits for its S buffer, hence for the P V of this task's second tile.)
+            if (j <= 1) {
+              const uint32_t mx = (g - (uint32_t)j) & 3;
+              volatile float* mh = mpub + mx * 256;
+              if (j == 0) {
+                float mloc = -INFINITY;
+#pragma unroll 1
+                for (int ch = 0; ch < G::NCH; ++ch) {
+                  uint32_t sv[G::CH];
+                  WAVEAL_TMEM_LD32(s_addr + ch * G::CH, sv, 0);
+                  WAVEAL_TMEM_WAIT_LD32(sv, 0);
+                  mloc = fmaxf(mloc, row_max32(sv));
+                }
+                mh[half * 128 + r] = mloc;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(BAR(B_MX + quad * 4 + mx));
+              }
+              ok = warp_wait(ctx, BAR(B_MX + quad * 4 + mx), (mx_phase >> mx) & 1u, 24);
+              if (!ok) break;
+              mx_phase ^= 1u << mx;
+              m_ref = fmaxf(mh[r], mh[128 + r]) * p.sl2;
+            }
+            m_new = m_ref;
+          } else {
           float mloc = -INFINITY;
-          if (!fixed_ref) {
+          {
 #pragma unroll 1
             for (int ch = 0; ch < G::NCH; ++ch) {
               uint32_t sv[G::CH];
               WAVEAL_TMEM_LD32(s_addr + ch * G::CH, sv, 0);
               WAVEAL_TMEM_WAIT_LD32(sv, 0);
-              float mx4[4];
-#pragma unroll
-              for (int i = 0; i < 4; ++i) mx4[i] = __uint_as_float(sv[i]);
-#pragma unroll
-              for (int c = 4; c < G::CH - 4; c += 8) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) mx4[i] = fmax3(mx4[i], __uint_as_float(sv[c + 2 * i]), __uint_as_float(sv[c + 2 * i + 1]));
-              }
-#pragma unroll
-              for (int i = 0; i < 4; ++i) mx4[i] = fmaxf(mx4[i], __uint_as_float(sv[G::CH - 4 + i]));
-              mloc = fmax3(fmax3(mx4[0], mx4[1], mx4[2]), mx4[3], mloc);
+              mloc = fmaxf(mloc, row_max32(sv));
             }
             // the other owner of the row (same team and quadrant, other column half)
             // (two buffers by use parity: the partner's next value cannot land on one not yet read)
@@ -963,8 +994,8 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           }
           // ---- the row's reference after block j-1, from the other team
           float m_prev = m_ref;
-          if (j > 0 && !(FAST && j > G::MAX_TILES)) mx_phase ^= 1u << ((g - 1) & 3);   // the other team's arrival for tile g-1
-          if (j > 0 && (!fixed_ref || j == G::MAX_TILES)) {
+          if (j > 0) {
+            mx_phase ^= 1u << ((g - 1) & 3);                   // the other team's arrival for tile g-1
             // that team's arrival for tile g-1 is phase number (arrivals of that slot so far) - 1
             const uint32_t mx = (g - 1) & 3;
             ok = warp_wait(ctx, BAR(B_MX + quad * 4 + mx), ((mx_phase >> mx) & 1u) ^ 1u, 24);
@@ -975,9 +1006,9 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           // keep the stale reference unless it is exceeded by more than 2^8 (exact: the final
           // normalisation divides by a sum taken with the same reference); both owners of a row
           // see the same values and take the same decision
-          const bool grow = !fixed_ref && __any_sync(0xffffffffu, m_cand > m_prev + 8.0f);
-          const float m_new = grow ? m_cand : m_prev;
-          if (!fixed_ref && half == 0) {
+          const bool grow = __any_sync(0xffffffffu, m_cand > m_prev + 8.0f);
+          m_new = grow ? m_cand : m_prev;
+          if (half == 0) {
             // (slot and barrier g mod 4: the owner of tile g+4 cannot get there before both owners of
             // tile g+1 have read this one, which its S buffer waits for)
             mpub[(g & 3) * 128 + r] = m_new;
@@ -994,7 +1025,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           // The owner of the first half of P does it for all columns of O before it releases that half: the P V
           // warp starts on the first half as soon as it has arrived, its MMAs add to all columns, and those on the
           // second half come behind.  (Split between the two owners, each would have to wait for the other.)
-          if (kRescales && grow && j > 0 && half == 0) {
+          if (grow && j > 0 && half == 0) {
             const uint32_t sbp = sb == 0 ? (uint32_t)G::NSBUF - 1u : sb - 1u;
             ok = warp_wait(ctx, BAR(B_S_FREE + sbp), sb == 0 ? s_ph ^ 1u : s_ph, 22);
             if (!ok) break;
@@ -1009,6 +1040,8 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
               for (int c = 0; c < 32; ++c) ov[c] = __float_as_uint(__uint_as_float(ov[c]) * alpha);
               WAVEAL_TMEM_ST32(o_row + c0, ov, 0);
             }
+          }
+          mx_phase ^= 1u << (g & 3);                           // one flip per arrival on that slot's barrier
           }
           // p' = 2^(s*scale*log2e - m + log2(1 + 2^-9)); P is p' cut to its top 16 bits (one byte
           // permute per pair instead of a conversion).  The extra factor centres the cut's error
@@ -1047,13 +1080,12 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           // polynomial share saturates at 2^64), so a sum below 2^60 bounds every exponent it
           // covers; at or above it (or not a number) the fixed reference is too far off:
           // redo the task
-          if (fixed_ref && __any_sync(0xffffffffu, !(l_blk < kRedoLimit))) redo_flag[rslot] = task_no;
+          if (FAST && __any_sync(0xffffffffu, !(l_blk < kRedoLimit))) redo_flag[rslot] = task_no;
           tc_wait_st();
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(BAR(B_P_FULL + sb * 2 + half));
         }
-        if (!(FAST && j >= G::MAX_TILES)) mx_phase ^= 1u << (g & 3);                  // one flip per arrival on that slot's barrier
         next_buffer();
       }
       if (!ok) break;
@@ -1065,7 +1097,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR(ex_bar));
       const bool mine = (int)((g0 + (uint32_t)last) & 1u) == team;
-      if (!mine && !idle && !(FAST && last >= G::MAX_TILES)) mx_phase ^= 1u << ((g0 + (uint32_t)last) & 3);
+      if (!mine && !idle && !(FAST && last > 0)) mx_phase ^= 1u << ((g0 + (uint32_t)last) & 3);
       g0 += (uint32_t)tk.n;
       const uint32_t o_ph = o_it & 1;
       ++o_it;
@@ -1475,7 +1507,7 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
     waveal::launch_counter() = launches + 1;
     return WAVEAL_OK;
   }
-  // first pass: reference fixed after the first tile of a task (64-row blocks: the first two); second pass: the tasks the
+  // first pass: reference fixed after the first tile of a task; second pass: the tasks the
   // first one listed (normally none: its CTAs leave at once), max of every block
   p.redo_pass = 0;
   WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, true>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, p));
