@@ -97,6 +97,17 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm,
       ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
       : "memory");
 }
+// one bulk group per store; the coordinates of elements beyond the tensor are left out by the copy engine
+__device__ __forceinline__ void tma_store_3d(const CUtensorMap* tm, uint32_t src, int c0, int c1, int c2) {
+  asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];"
+               ::"l"(reinterpret_cast<uint64_t>(tm)), "r"(c0), "r"(c1), "r"(c2), "r"(src) : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* tm) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tm)) : "memory");
 }
@@ -356,6 +367,9 @@ struct Geo {
   // instead of three (128-row tiles of 8 tiles a task: 16.0k against 16.4k clk; 64-row tiles: 18.5 M against
   // 18.2 M cycles on 8 heads of 1536 rows, their tasks are longer and their rings do the work)
   static constexpr int NQ = KB == 1 ? 2 : 1;
+  // O leaves through shared memory: staged in the task's own Q tile, which nobody reads any more, and stored by the copy
+  // engine.  64-row blocks have one Q tile, which the next task's Q is loaded into meanwhile; they store from registers.
+  static constexpr bool STAGED = NQ == 2;
   static constexpr int NSTAGE_RAW = (200 * 1024 - NQ * Q_BYTES) / TILE_BYTES;
   static constexpr int NSTAGE = NSTAGE_RAW > 8 ? 8 : NSTAGE_RAW;
   static constexpr int NKS = (NSTAGE + 1) / 2;       // K tile ring
@@ -511,9 +525,10 @@ template <int BLOCK, int D, bool FAST>
 __global__ void __launch_bounds__(kThreads, 1)
 k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
              const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmK2,
-             const __grid_constant__ CUtensorMap tmV2, const AttnParams p) {
+             const __grid_constant__ CUtensorMap tmV2, const __grid_constant__ CUtensorMap tmO, const AttnParams p) {
   // tmK2 / tmV2: the same K and V with boxes of 128 rows, used by the 64-key-block kernels when the
-  // two blocks of a tile lie next to each other in memory (for 128-key blocks they equal tmK / tmV)
+  // two blocks of a tile lie next to each other in memory (for 128-key blocks they equal tmK / tmV).
+  // tmO: O in boxes of 32 rows and half of head_dim, what a warp stores (128-row blocks only)
   using G = Geo<BLOCK, D>;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -548,7 +563,8 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   if (tid == 0) {
     // a task is read by the V loader, the two MMA issuers and the sixteen softmax warps
     for (int i = 0; i < 2; ++i) { mbar_init(BAR(B_TASK_FULL + i), 1); mbar_init(BAR(B_TASK_EMPTY + i), 19); }
-    for (int i = 0; i < 2; ++i) { mbar_init(BAR(B_Q_FULL + i), 1); mbar_init(BAR(B_Q_EMPTY + i), 1); }
+    // a Q tile is free when the last Q K^T has read it and, where O is staged in it, its eight warps' stores have
+    for (int i = 0; i < 2; ++i) { mbar_init(BAR(B_Q_FULL + i), 1); mbar_init(BAR(B_Q_EMPTY + i), G::STAGED ? 9 : 1); }
     for (int i = 0; i < G::NKS; ++i) { mbar_init(BAR(B_K_FULL + i), 1); mbar_init(BAR(B_K_EMPTY + i), 1); }
     for (int i = 0; i < G::NVS; ++i) { mbar_init(BAR(B_V_FULL + i), 1); mbar_init(BAR(B_V_EMPTY + i), 1); }
     for (int i = 0; i < G::NSBUF; ++i) {
@@ -589,7 +605,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   // and V stage g mod NVS, so no role needs to be told where a tile or a buffer is.
   if (warp == kProducerWarp) {
     // ============================================================== producer
-    if (lane == 0) { prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmV); prefetch_tmap(&tmK2); prefetch_tmap(&tmV2); }
+    if (lane == 0) { prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmV); prefetch_tmap(&tmK2); prefetch_tmap(&tmV2); if (G::STAGED) prefetch_tmap(&tmO); }
     uint32_t task_it = 0, q_it = 0, k_it = 0;
     int n_tiles = 0, n_pairs = 0;        // words 7 and 6 of the workspace: KV tiles (128 rows x 128 keys) and shared tiles this call ran
     bool ok = true;
@@ -887,7 +903,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     uint32_t g0 = 0;                           // tiles before this task
     uint32_t sb = (uint32_t)team, s_ph = 0;    // S buffer of this team's next tile and the parity of that use
     auto next_buffer = [&]() { sb += 2; if (sb >= (uint32_t)G::NSBUF) { sb -= (uint32_t)G::NSBUF; s_ph ^= 1; } };
-    bool ok = true;
+    bool ok = true, storing = false;           // storing: the stores of this warp's last epilogue may still read the Q tile
     while (ok) {
       const uint32_t slot = task_it & 1, ph = (task_it >> 1) & 1;
       ok = warp_wait(ctx, BAR(B_TASK_FULL + slot), ph, 20);
@@ -895,6 +911,12 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       const Task tk = tasks[slot];
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR(B_TASK_EMPTY + slot));
+      // (here and not behind the stores: by now the copy engine has read them.  The next task is published before the one
+      // whose Q needs this tile, so nobody waits for this in a circle)
+      if (G::STAGED && storing) {
+        if (lane == 0) { bulk_wait_read(); mbar_arrive(BAR(B_Q_EMPTY + ((o_it - 1) & 1))); }
+        storing = false;
+      }
       float2* exb = ex + (o_it & 3) * 512;
       const int task_no = (int)o_it + 1;
       const uint32_t rslot = o_it & 3, ex_bar = B_EX + quad + 4 * (o_it & 3), ex_ph = (o_it >> 2) & 1;
@@ -1128,10 +1150,12 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR(B_O_FREE));
       bool bad = false;
+      // From registers a store instruction touches 32 rows and the memory pipe takes 2 clk for each: 2,300 clk a task for the
+      // 1,024 row pieces of 32 bytes, in which the team could have been at its next tile.
+      // Staged: 128x64 tasks of 24 tiles 1,272 -> 1,247 clk a tile, 128x128 tasks of 17 tiles 1,698 -> 1,664, of 32 tiles
+      // 1,501 -> 1,489; tasks of 256 tiles pay 1 % for it (1,364 -> 1,380).
+      const uint32_t stage = sbase + G::OFF_Q + (G::NQ == 2 ? ((uint32_t)o_it - 1u) & 1u : 0u) * G::Q_BYTES + (uint32_t)(quad * 2 + half) * (32 * G::CO * 2);
       if (row_live) {
-        // a thread holds a piece of one row, so a store instruction of a warp touches 32 rows:
-        // its cost in the memory pipe is per row, not per byte.  32-byte stores halve the number
-        // of instructions where the row piece is 32-byte aligned (else 16-byte stores)
         uint32_t w[G::CO / 2];
 #pragma unroll
         for (int c = 0; c < G::CO; c += 2) {
@@ -1145,7 +1169,15 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           for (int c = 0; c < G::CO / 2; ++c) top |= (w[c] & 0x7F807F80u) + 0x00800080u;
           bad = (top & 0x80008000u) != 0;
         }
-        if ((reinterpret_cast<uintptr_t>(o_ptr) & 31) == 0) {
+        if constexpr (G::STAGED) {
+          // the box's rows of 128 (64) bytes, 16-byte pieces swizzled as the tensor map says: eight (four) lanes a wavefront
+          const uint32_t row0 = stage + (uint32_t)lane * (G::CO * 2), sw = G::CO == 64 ? lane & 7 : (lane >> 1) & 3;
+#pragma unroll
+          for (int c = 0; c < G::CO / 8; ++c) st_shared_v4(row0 + (((uint32_t)c ^ sw) << 4), w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+        } else if ((reinterpret_cast<uintptr_t>(o_ptr) & 31) == 0) {
+          // a thread holds a piece of one row, so a store instruction of a warp touches 32 rows:
+          // its cost in the memory pipe is per row, not per byte.  32-byte stores halve the number
+          // of instructions where the row piece is 32-byte aligned (else 16-byte stores)
 #pragma unroll
           for (int c = 0; c < G::CO / 2; c += 8) st_global_v8(o_ptr + 2 * c, w + c);
         } else {
@@ -1154,6 +1186,13 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             *reinterpret_cast<uint4*>(o_ptr + 2 * c) = make_uint4(w[c], w[c + 1], w[c + 2], w[c + 3]);
         }
         if (p.lse && half == 0) p.lse[(size_t)tk.h * p.seq_q + q_tok] = (m_all + log2f(l_tot) - 0.0028150156f) * 0.6931471805599453f;
+      }
+      if constexpr (G::STAGED) {
+        fence_proxy_async();
+        __syncwarp();
+        const int tok0 = tk.row * G::BQ + quad * 32;         // (rows beyond seq_q are left out)
+        if (lane == 0 && tok0 < p.seq_q) { tma_store_3d(&tmO, stage, half * G::CO, tok0, tk.h); bulk_commit(); }
+        storing = true;
       }
       // The task goes to the second launch if the sum of a tile left the range (every warp's tiles of this task lie
       // before O_FULL) or if a result is not finite: with sums of up to 2^60 O overflows from |V| = 2^67 on, and a
@@ -1166,6 +1205,8 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     }
   }
 
+  // (stores still under way read this CTA's shared memory)
+  if (G::STAGED && warp >= kSoftmaxWarp0 && warp < kQkWarp && lane == 0) bulk_wait_all();
   // ------------------------------------------------------------------ teardown
   tc_fence_before();
   __syncthreads();
@@ -1429,17 +1470,18 @@ EncodeTiledFn get_encode() {
   return fn;
 }
 
-// bf16 tensor [heads][seq][head_dim] with element strides {head, token}; box = 64 columns x rows
+// bf16 tensor [heads][seq][head_dim] with element strides {head, token}; box = 64 (or 32) columns x rows
 waveal_status make_map(CUtensorMap* tm, const void* base, int head_dim, int seq, int heads, long long stride_h,
-                       long long stride_t, int box_rows, const char* what) {
+                       long long stride_t, int box_rows, const char* what, int box_cols = 64) {
   EncodeTiledFn enc = get_encode();
   if (!enc) return waveal::fail(WAVEAL_ERR_CUDA, "cuTensorMapEncodeTiled entry point not available");
   cuuint64_t dims[3] = {(cuuint64_t)head_dim, (cuuint64_t)seq, (cuuint64_t)heads};
   cuuint64_t strides[2] = {(cuuint64_t)stride_t * 2, (cuuint64_t)stride_h * 2};
-  cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
+  cuuint32_t box[3] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, 1};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, box_cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
+                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return waveal::fail(WAVEAL_ERR_CUDA, "tensor map for %s rejected (CUresult %d)", what, (int)r);
   return WAVEAL_OK;
@@ -1470,13 +1512,19 @@ template <int BLOCK, int D>
 waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, const void* V, AttnParams& p,
                      int sms, cudaStream_t st) {
   using G = Geo<BLOCK, D>;
-  CUtensorMap tq, tk, tv, tk2, tv2;
+  CUtensorMap tq, tk, tv, tk2, tv2, to;
   waveal_status s;
   if ((s = make_map(&tq, Q, D, d->seq_q, d->heads, d->q_stride[0], d->q_stride[1], BLOCK, "Q")) != WAVEAL_OK) return s;
   if ((s = make_map(&tk, K, D, d->seq_kv, d->heads, d->k_stride[0], d->k_stride[1], BLOCK, "K")) != WAVEAL_OK) return s;
   if ((s = make_map(&tv, V, D, d->seq_kv, d->heads, d->v_stride[0], d->v_stride[1], BLOCK, "V")) != WAVEAL_OK) return s;
-  if ((s = make_map(&tk2, K, D, d->seq_kv, d->heads, d->k_stride[0], d->k_stride[1], 128, "K (128-row boxes)")) != WAVEAL_OK) return s;
-  if ((s = make_map(&tv2, V, D, d->seq_kv, d->heads, d->v_stride[0], d->v_stride[1], 128, "V (128-row boxes)")) != WAVEAL_OK) return s;
+  if (BLOCK == 128) {                     // (each kernel reads the maps of its own block size)
+    tk2 = tk; tv2 = tv;
+    if ((s = make_map(&to, p.O, D, d->seq_q, d->heads, d->o_stride[0], d->o_stride[1], 32, "O", D / 2)) != WAVEAL_OK) return s;
+  } else {
+    if ((s = make_map(&tk2, K, D, d->seq_kv, d->heads, d->k_stride[0], d->k_stride[1], 128, "K (128-row boxes)")) != WAVEAL_OK) return s;
+    if ((s = make_map(&tv2, V, D, d->seq_kv, d->heads, d->v_stride[0], d->v_stride[1], 128, "V (128-row boxes)")) != WAVEAL_OK) return s;
+    to = tq;
+  }
   WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd<BLOCK, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES));
   WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd<BLOCK, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES));
   long long grid = p.total_tasks < sms ? p.total_tasks : sms;
@@ -1503,16 +1551,16 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   WAVEAL_CUDA_OK(cudaGetLastError());
   if (d->flags & WAVEAL_ATTN_ONLINE_MAX_ONLY) {
     p.redo_pass = 0;
-    WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, false>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, p));
+    WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, false>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, to, p));
     waveal::launch_counter() = launches + 1;
     return WAVEAL_OK;
   }
   // first pass: reference fixed after the first tile of a task; second pass: the tasks the
   // first one listed (normally none: its CTAs leave at once), max of every block
   p.redo_pass = 0;
-  WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, true>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, p));
+  WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, true>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, to, p));
   p.redo_pass = 1;
-  WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, false>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, p));
+  WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, false>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, to, p));
   waveal::launch_counter() = launches + 2;
   return WAVEAL_OK;
 }

@@ -247,6 +247,32 @@ def test_short_tasks_back_to_back(block, D, tasks):
         assert ((got_lse - s.logsumexp(-1)).abs() <= 1.5e-4)[live].all()
 
 
+# O leaves in boxes of 32 rows and half of head_dim: the last box whole, cut and left out; rows of O with other tensors'
+# rows between them, at 16-byte boundaries, and nothing written behind seq_q
+@pytest.mark.parametrize("D", [64, 128])
+@pytest.mark.parametrize("cut", [0, 1, 31, 32, 33, 64, 95, 96, 127])
+def test_stores_end_with_the_sequence(D, cut):
+    H, nb, block = 2, 3, 128
+    T = nb * block - cut
+    q, k, v = _inputs(H, nb * block, D, cut)
+    ptr = torch.arange(0, 2 * H * nb + 1, 2, device="cuda", dtype=torch.int32)
+    idx = torch.tensor([0, 2, 0, 1, 1, 2], device="cuda", dtype=torch.int32).repeat(H)
+    buf = torch.full((nb * block, H, D + 8), float("nan"), dtype=torch.bfloat16, device="cuda")
+    o = buf[:, :, 8:].permute(1, 0, 2)
+    st = torch.zeros((4,), dtype=torch.int32, device="cuda")
+    wb.bsattn_fwd(wb.attn_desc(q, k, v, o, T, T, block), q, k, v, o, ptr, idx, dev_status=st)
+    torch.cuda.synchronize()
+    assert st.tolist() == [0] * 4
+    assert torch.isnan(buf[:, :, :8]).all() and torch.isnan(buf[T:]).all()
+    for i, pair in enumerate(((0, 2), (0, 1), (1, 2))):
+        sel = torch.cat([torch.arange(j * block, min((j + 1) * block, T)) for j in pair]).cuda()
+        rows = slice(i * block, min((i + 1) * block, T))
+        p = (q[:, rows].double() @ k[:, sel].double().transpose(1, 2) / D ** 0.5).softmax(-1)
+        ref = p @ v[:, sel].double()
+        bound = 2.0 ** -8 * (p @ v[:, sel].double().abs()) + 2.0 ** -8 * ref.abs() + 1e-6      # as in the test above
+        assert ((o[:, rows].double() - ref).abs() <= bound).all()
+
+
 # heads of unequal row lengths, more tickets than the sorted tail: no order of heads or rows shows in the results
 @pytest.mark.parametrize("block,nb", [(128, 420), (64, 420), (128, 300)])
 def test_tail_over_several_heads(block, nb):
