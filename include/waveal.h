@@ -205,7 +205,7 @@ typedef struct waveal_attn_desc {
 /* Bytes of device workspace waveal_bsattn_fwd needs: 32 bytes of counters (int32 words: ticket
  * counter, abort flag, number of tasks computed twice, ticket counter of the second launch,
  * length of the first and of the second launch in SM cycles = the longest that a thread block ran
- * after the launch before it had ended, number of query-block pairs that shared a tile, number of 128-row x 128-key tiles the call runs),
+ * after its first task could start, number of query-block pairs that shared a tile, number of 128-row x 128-key tiles the call runs),
  * 8 bytes per (head, query block) for the list of tasks to compute again and
  * 32 bytes per (head, query block) for the table that maps a ticket to its task.  The counters
  * are live state of the call (tickets are drawn from them): calls that may overlap on the GPU
@@ -218,7 +218,8 @@ waveal_status waveal_bsattn_workspace_bytes(const waveal_attn_desc* desc /*host*
  * Persistent CTAs take (head, position) tickets in head-major order and process query
  * block row_order[h][position] (Algorithm 2 output; NULL = natural order); the last 1,024 tickets of a
  * call, seven per SM, are handed out longest list first, so that no SM is left with a long row at the end (a call of no
- * more blocks than that runs in this order alone, whatever row_order and order_heads_interleaved say); each output
+ * more blocks than that runs in this order alone, whatever row_order and order_heads_interleaved say, but for the first
+ * ticket of every SM with 128-row blocks and at least two blocks an SM); each output
  * tile is written at its original rows, so no inverse permutation pass exists.
  * Q, K, V, O: dev bf16, 16-byte aligned, strides multiples of 8 elements, head_dim
  * contiguous; query tokens >= seq_q are not written; keys >= seq_kv are ignored.

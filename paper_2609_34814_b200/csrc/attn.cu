@@ -341,6 +341,8 @@ struct AttnParams {
                       // the redo pass, [8 + 2i], [9 + 2i] = (head, query block) of redo entry i
   int redo_pass;      // 0: all tasks by ticket; 1: only the tasks the first pass listed
   const Task* table;         // task of every ticket of the first pass (k_task_table)
+  int direct;         // CTAs that take the ticket of their own number before the table is there (0: none, else the grid)
+  long long first_tail;      // tickets before this one are in the caller's order, the rest longest first
   int* dev_status;
   long long o_stride_h, o_stride_t;
   int heads, m_b, n_b, seq_q, seq_kv, interleaved;
@@ -351,6 +353,45 @@ struct AttnParams {
   float sl2;          // scale * log2(e)
 };
 
+
+// Task of every ticket (head-major or position-major over the planned order), so that the
+// persistent CTAs need one load behind a ticket instead of a chain through row_order, the row
+// pointers and the index list.
+// The inputs are checked on the way (a thread per task, so it costs nothing): an entry of
+// row_order outside [0, M_B), a row-pointer pair that is negative, decreasing or beyond the end
+// of the index list, or a last index outside [0, N_B) is reported as
+// {WAVEAL_ERR_BAD_MASK, site, head, offending value} and the task is given an empty list
+// (its output rows become 0) instead of reading out of range.
+__device__ __forceinline__ Task make_task(const AttnParams& p, int block_k, int h, int pos) {
+  auto report = [&](int site, int value) {
+    if (p.dev_status && atomicCAS(p.dev_status, 0, WAVEAL_ERR_BAD_MASK) == 0) {
+      p.dev_status[1] = site; p.dev_status[2] = h; p.dev_status[3] = value;
+    }
+  };
+  int row = p.row_order ? p.row_order[(size_t)h * p.m_b + pos] : pos;
+  bool bad = false;
+  if (row < 0 || row >= p.m_b) { report(31, row); row = pos; bad = true; }
+  const long long nnz = p.row_ptr[p.total_tasks];
+  const int lo = p.row_ptr[(size_t)h * p.m_b + row], hi = p.row_ptr[(size_t)h * p.m_b + row + 1];
+  if (lo < 0 || hi < lo || (long long)hi > nnz) { report(32, lo < 0 ? lo : hi); bad = true; }
+  Task tk{};
+  tk.h = h; tk.row = row; tk.lo = bad ? 0 : lo; tk.row2 = -1;
+  int len = bad ? 0 : hi - lo, last = 0;
+  if (len > 0) {
+    last = p.kv_idx[hi - 1];
+    if (last < 0 || last >= p.n_b) { report(33, last); len = 0; }
+  }
+  fill_tiles(tk, len, block_k, last, p.n_b, p.seq_kv);
+  if (bad) tk.pad2 = 1;                             // takes no part in pairing
+  return tk;
+}
+
+__device__ __forceinline__ Task task_of_ticket(const AttnParams& p, int block_k, long long t) {
+  const int h = p.interleaved ? (int)(t % p.heads) : (int)(t / p.m_b), pos = p.interleaved ? (int)(t / p.heads) : (int)(t % p.m_b);
+  Task tk = make_task(p, block_k, h, pos);
+  tk.pad2 = 0;
+  return tk;
+}
 
 template <int BLOCK, int D>
 struct Geo {
@@ -402,6 +443,7 @@ struct Ctx {
 
 __device__ __noinline__ void signal_abort(const Ctx& c, int site) {
   *c.abort_smem = 1;
+  waveal::wait_for_previous_kernel();      // (which clears the flag)
   atomicExch(&c.ws[1], 1);
   if (c.dev_status && atomicCAS(c.dev_status, 0, WAVEAL_ERR_TIMEOUT) == 0) {
     c.dev_status[1] = site;
@@ -512,6 +554,7 @@ __device__ __noinline__ void mask_scores(uint32_t s_addr, int valid) {
 // on 5 heads of 256 rows: a call there makes the compiler spill)
 __device__ __forceinline__ void list_task(int* ws, int* listed, int task_no, int h, int row, int row2) {
   if (atomicExch(listed, task_no) == task_no) return;
+  waveal::wait_for_previous_kernel();      // (which clears the count: a first task may end before it)
   const int e = atomicAdd(&ws[2], row2 >= 0 ? 2 : 1);
   ws[8 + 2 * e] = h;
   ws[9 + 2 * e] = row;
@@ -596,8 +639,10 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_holder, 0);
-  // tickets, table and counters are the work of the kernel before this one
-  waveal::wait_for_previous_kernel();
+  // Tickets, table and counters are the work of the kernel before this one.  It was launched the ordinary way, so all that
+  // came before it (the lists, Q, K, V) is there by now: a CTA with a first task of its own (p.direct) begins, and whoever
+  // touches the counters or the table waits there.
+  if (!p.direct) waveal::wait_for_previous_kernel();
   const long long t_start = clock64();          // (that kernel's time is not this launch's)
 
   // Every role walks the same sequence of tasks (query blocks) and, inside a task, of KV blocks;
@@ -613,6 +658,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     uint32_t q_armed = 0, q_parity = 0;
     // the next task: a ticket from the global counter and the task it stands for (n = -1: none left)
     auto draw = [&](long long& t_out) -> Task {
+      if (p.direct) waveal::wait_for_previous_kernel();
       for (;;) {
         long long t = 0, n_tasks = p.total_tasks;
         if (lane == 0) {
@@ -650,8 +696,10 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     // counter and of the table entry (~2,000 cycles) then no longer stand between the end of a
     // task and the request for the next Q tile.
     constexpr int kDrawAhead = 3;
-    long long t = 0, t_next = 0;
-    Task tk_next = draw(t_next);
+    long long t = 0, t_next = blockIdx.x;
+    Task tk_next;
+    if (FAST && G::KB == 1 && p.direct) tk_next = task_of_ticket(p, BLOCK, t_next);
+    else tk_next = draw(t_next);
     while (ok) {
       Task tk = tk_next;
       t = t_next;
@@ -696,6 +744,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                                           BAR(B_K_EMPTY), &tmK, &tmK2, k_it, k_armed, k_parity, chunk_base, my_idx);
       }
     }
+    if (p.direct) waveal::wait_for_previous_kernel();       // (after an abort: the counters below are cleared by it)
     if (lane == 0 && !p.redo_pass) {
       if (n_tiles) atomicAdd(&p.ws[7], n_tiles);
       if (n_pairs) atomicAdd(&p.ws[6], n_pairs);
@@ -1222,41 +1271,10 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   }
 }
 
-// Task of every ticket (head-major or position-major over the planned order), so that the
-// persistent CTAs need one load behind a ticket instead of a chain through row_order, the row
-// pointers and the index list.
-// The inputs are checked on the way (a thread per task, so it costs nothing): an entry of
-// row_order outside [0, M_B), a row-pointer pair that is negative, decreasing or beyond the end
-// of the index list, or a last index outside [0, N_B) is reported as
-// {WAVEAL_ERR_BAD_MASK, site, head, offending value} and the task is given an empty list
-// (its output rows become 0) instead of reading out of range.
-// It also clears the call's counters (the launch before it on the stream has ended).
-__device__ __forceinline__ Task make_task(const AttnParams& p, int block_k, int h, int pos) {
-  auto report = [&](int site, int value) {
-    if (p.dev_status && atomicCAS(p.dev_status, 0, WAVEAL_ERR_BAD_MASK) == 0) {
-      p.dev_status[1] = site; p.dev_status[2] = h; p.dev_status[3] = value;
-    }
-  };
-  int row = p.row_order ? p.row_order[(size_t)h * p.m_b + pos] : pos;
-  bool bad = false;
-  if (row < 0 || row >= p.m_b) { report(31, row); row = pos; bad = true; }
-  const long long nnz = p.row_ptr[p.total_tasks];
-  const int lo = p.row_ptr[(size_t)h * p.m_b + row], hi = p.row_ptr[(size_t)h * p.m_b + row + 1];
-  if (lo < 0 || hi < lo || (long long)hi > nnz) { report(32, lo < 0 ? lo : hi); bad = true; }
-  Task tk{};
-  tk.h = h; tk.row = row; tk.lo = bad ? 0 : lo; tk.row2 = -1;
-  int len = bad ? 0 : hi - lo, last = 0;
-  if (len > 0) {
-    last = p.kv_idx[hi - 1];
-    if (last < 0 || last >= p.n_b) { report(33, last); len = 0; }
-  }
-  fill_tiles(tk, len, block_k, last, p.n_b, p.seq_kv);
-  if (bad) tk.pad2 = 1;                             // takes no part in pairing
-  return tk;
-}
-
+// The kernel that makes the table also clears the call's counters (the launch before it on the stream has ended);
+// tickets are counted from behind those that the CTAs have without asking.
 __device__ __forceinline__ void clear_counters(const AttnParams& p) {
-  if (blockIdx.x == 0 && threadIdx.x < 8) p.ws[threadIdx.x] = 0;
+  if (blockIdx.x == 0 && threadIdx.x < 8) p.ws[threadIdx.x] = threadIdx.x == 0 ? p.direct : 0;
 }
 
 // The last kTailTasks tickets of a call are handed out longest first (1,024 = 7 per SM).  In the planned
@@ -1303,20 +1321,13 @@ __global__ void __launch_bounds__(kTailTasks) k_task_table(AttnParams p, int blo
   waveal::let_next_kernel_start();
   clear_counters(p);
   // block 0: the last kTailTasks tickets (or all of them); the others the rest in order
-  const long long first_tail = p.total_tasks > kTailTasks ? p.total_tasks - kTailTasks : 0;
-  const long long t = blockIdx.x == 0 ? first_tail + threadIdx.x : (long long)(blockIdx.x - 1) * kTailTasks + threadIdx.x;
-  const bool live = blockIdx.x == 0 ? t < p.total_tasks : t < first_tail;
+  const long long t = blockIdx.x == 0 ? p.first_tail + threadIdx.x : (long long)(blockIdx.x - 1) * kTailTasks + threadIdx.x;
+  const bool live = blockIdx.x == 0 ? t < p.total_tasks : t < p.first_tail;
   Task tk{};
-  if (live) {
-    int h, pos;
-    if (p.interleaved) { pos = (int)(t / p.heads); h = (int)(t % p.heads); }
-    else { h = (int)(t / p.m_b); pos = (int)(t % p.m_b); }
-    tk = make_task(p, block_k, h, pos);
-    tk.pad2 = 0;
-  }
+  if (live) tk = task_of_ticket(p, block_k, t);
   if (blockIdx.x == 0) {
     const int at = tail_place(tk.n, live);
-    if (live) table[first_tail + at] = tk;
+    if (live) table[p.first_tail + at] = tk;
   } else if (live) {
     table[t] = tk;
   }
@@ -1326,13 +1337,12 @@ __global__ void __launch_bounds__(kTailTasks) k_task_table(AttnParams p, int blo
 __global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* table) {
   waveal::let_next_kernel_start();
   waveal::wait_for_previous_kernel();
-  const long long first_tail = p.total_tasks > kTailTasks ? p.total_tasks - kTailTasks : 0;
-  const long long t = first_tail + threadIdx.x;
+  const long long t = p.first_tail + threadIdx.x;
   const bool live = t < p.total_tasks;
   Task tk{};
   if (live) tk = table[t];
   const int at = tail_place(tk.n, live);
-  if (live) table[first_tail + at] = tk;
+  if (live) table[p.first_tail + at] = tk;
 }
 
 // The same for 64-row query blocks, where two blocks with the very same list share one 128-row tile.
@@ -1535,6 +1545,14 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   p.drop_tile = 0;
   if (d->flags & WAVEAL_ATTN_SELFTEST_LOST_TILE) { p.wait_limit = kSelfTestCycles; p.drop_tile = 1; }
   p.no_pairing = (d->flags & WAVEAL_ATTN_NO_ROW_PAIRING) ? 1 : 0;
+  // From two tasks an SM on, the first task of every CTA is the ticket of its own number: it runs while the table is made
+  // (10 us: 1,320 tasks of 17 tiles 196.7 -> 187.2 us a call, 1,280 of 38 386 -> 373, 3,816 of 24 at head_dim 64 501 -> 494).  Those tickets stay out of the sorted tail.  (64-row blocks: which blocks share a tile is known from the table only.)
+  p.first_tail = p.total_tasks > kTailTasks ? p.total_tasks - kTailTasks : 0;
+  p.direct = 0;
+  if (BLOCK == 128 && p.total_tasks >= 2 * sms && !(d->flags & WAVEAL_ATTN_ONLINE_MAX_ONLY)) {
+    p.direct = (int)grid;
+    if (p.first_tail < grid) p.first_tail = grid;
+  }
   int launches = 1;
   if (BLOCK == 64) {
     const int chunks = (p.m_b + kPairRows - 1) / kPairRows;
@@ -1545,8 +1563,7 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
       ++launches;
     }
   } else {
-    const long long before_tail = p.total_tasks > kTailTasks ? p.total_tasks - kTailTasks : 0;
-    k_task_table<<<(unsigned)(1 + (before_tail + kTailTasks - 1) / kTailTasks), kTailTasks, 0, st>>>(p, BLOCK, table);
+    k_task_table<<<(unsigned)(1 + (p.first_tail + kTailTasks - 1) / kTailTasks), kTailTasks, 0, st>>>(p, BLOCK, table);
   }
   WAVEAL_CUDA_OK(cudaGetLastError());
   if (d->flags & WAVEAL_ATTN_ONLINE_MAX_ONLY) {
@@ -1560,6 +1577,7 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   p.redo_pass = 0;
   WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, true>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, to, p));
   p.redo_pass = 1;
+  p.direct = 0;
   WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, false>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, to, p));
   waveal::launch_counter() = launches + 2;
   return WAVEAL_OK;
