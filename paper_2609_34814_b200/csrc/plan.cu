@@ -400,15 +400,22 @@ __device__ __forceinline__ void store_peer(const long long* local_ptr, unsigned 
   asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(raddr), "l"(v) : "memory");
 }
 
-// number of set bits with index in [lo, hi) of a bit row
+// number of set bits with index in [lo, hi) of a bit row; four words in flight (a wave of 148 rows lies in at most
+// four; one load after the other, a head's statistics took 18,200 clk instead of 14,400 on 32 heads of 1,536 blocks)
 __device__ __forceinline__ int popcount_range(const u64* __restrict__ words, int lo, int hi) {
   if (hi <= lo) return 0;
-  int w0 = lo >> 6, w1 = (hi - 1) >> 6, c = 0;
-  for (int w = w0; w <= w1; ++w) {
-    u64 x = words[w];
-    if (w == w0) x &= ~0ull << (lo & 63);
-    if (w == w1 && (hi & 63)) x &= (1ull << (hi & 63)) - 1ull;
-    c += __popcll(x);
+  const int w0 = lo >> 6, w1 = (hi - 1) >> 6;
+  int c = 0;
+  for (int w = w0; w <= w1; w += 4) {
+    u64 x[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = w + k <= w1 ? words[w + k] : 0ull;
+    if (w == w0) x[0] &= ~0ull << (lo & 63);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (w + k == w1 && (hi & 63)) x[k] &= (1ull << (hi & 63)) - 1ull;
+      c += __popcll(x[k]);
+    }
   }
   return c;
 }
@@ -766,6 +773,101 @@ __device__ __forceinline__ int merge_sort(u64* k0, int* v0, u64* k1, int* v1, in
   return at;
 }
 
+// Exclusive prefix sums of n ints in shared memory, in place.  part: 32 ints.  Ends with a barrier.
+__device__ __forceinline__ void exclusive_scan(int* a, int n, int* part) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per = (n + kPlanThreads - 1) / kPlanThreads, i0 = min((int)threadIdx.x * per, n), i1 = min(i0 + per, n);
+  int mine = 0;
+  for (int i = i0; i < i1; ++i) mine += a[i];
+  int incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  if (lane == 31) part[warp] = incl;
+  __syncthreads();
+  int at = __reduce_add_sync(0xffffffffu, lane < warp ? part[lane] : 0) + incl - mine;
+  for (int i = i0; i < i1; ++i) { const int v = a[i]; a[i] = at; at += v; }
+  __syncthreads();
+}
+
+// Ascending sort of n pairs (key, val) with distinct pairs, ties of the key by val, through bins that are themselves in
+// ascending order: `bin(key)` < n_bins never falls as the key grows.  Counts per bin, prefix sums, a scatter, and every
+// element counts the elements of its own bin that go before it: the work per element is the size of its bin, where the
+// merge sort walks log2(n) binary searches.  43,800 -> 11,200 clk for 2,841 rows of a video mask, 10,400 -> 8,500 for 591; where a
+// sixth of the rows have one angle (rows that select everything) as long as the merge sort, 24,000 for 1,536.  (Bins cut at
+// the quantiles of a sample of the keys: 41,700 for the 2,841 rows, their bins of 22 and more are walked for longer.)
+// The sorted values go to v0.  False, with the pairs as they were, if a bin holds more than kBinMax.  (The order inside a
+// bin before the count depends on the atomics, the result does not.)
+constexpr int kBinMax = 192;
+template <class Bin>
+__device__ __forceinline__ bool bin_sort(const u64* k0, int* v0, u64* k1, int* v1, int n, int* bins, int n_bins, int* part, Bin bin) {
+  for (int i = threadIdx.x; i < n_bins; i += kPlanThreads) bins[i] = 0;
+  __syncthreads();
+  bool big = false;
+  for (int i = threadIdx.x; i < n; i += kPlanThreads) big |= atomicAdd(&bins[bin(k0[i])], 1) >= kBinMax;
+  if (__syncthreads_or(big)) return false;
+  exclusive_scan(bins, n_bins, part);
+  for (int i = threadIdx.x; i < n; i += kPlanThreads) {
+    const u64 key = k0[i];
+    const int at = atomicAdd(&bins[bin(key)], 1);          // leaves the end of every bin
+    k1[at] = key;
+    v1[at] = v0[i];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += kPlanThreads) {
+    const u64 key = k1[i];
+    const int val = v1[i], b = bin(key), from = b ? bins[b - 1] : 0, to = bins[b];
+    int at = from;
+#pragma unroll 4
+    for (int j = from; j < to; ++j) {
+      const u64 kj = k1[j];
+      at += (kj < key || (kj == key && v1[j] < val)) ? 1 : 0;
+    }
+    v0[at] = val;
+  }
+  __syncthreads();
+  return true;
+}
+
+// 256 keys ascending, eight neighbours a lane: a bitonic network in registers (steps inside a lane by min and max, the others by
+// a shuffle).  In a descending stretch the keys are complemented instead of the comparisons turned around.
+__device__ __forceinline__ void warp_sort256(unsigned (&a)[8]) {
+  const unsigned lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 2; k <= 256; k <<= 1) {
+    // (stretches of up to eight keys lie inside a lane, where the direction is known while compiling)
+    const unsigned flip = k >= 8 && k < 256 && (lane & (k >> 3)) ? ~0u : 0u;
+    if (k >= 8)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) a[e] ^= flip;
+#pragma unroll
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      if (j >= 8) {
+        const bool upper = lane & (j >> 3);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const unsigned b = __shfl_xor_sync(0xffffffffu, a[e], j >> 3);
+          a[e] = upper ? max(a[e], b) : min(a[e], b);
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+          if ((e & j) == 0) {
+            const unsigned lo = min(a[e], a[e | j]), hi = max(a[e], a[e | j]);
+            const bool up = k >= 8 || (e & k) == 0;
+            a[e] = up ? lo : hi;
+            a[e | j] = up ? hi : lo;
+          }
+      }
+    }
+    if (k >= 8)
+#pragma unroll
+      for (int e = 0; e < 8; ++e) a[e] ^= flip;
+  }
+}
+
 // ascending bitonic sort of (key, val) pairs, ties by val; n is a power of two (row counts whose
 // second buffer does not fit shared memory)
 __device__ __forceinline__ void bitonic_sort(u64* keys, int* vals, int n) {
@@ -794,6 +896,8 @@ struct PlanParams {
   int csize;            // CTAs per head (thread-block cluster size)
   int mma;              // mask products on the integer matrix units (else: walk over the set bits)
   int count_stage2;     // Stage 2 by counting inside the buckets (else: by a sort)
+  int warp_stage2;      // Stage 2 by a warp per bucket
+  int bins;             // bins of the angular sort (0: by merging)
   int alias_yz;         // Y and Z share one buffer (two barriers more per iteration)
   int ksplit_y, ksplit_z, part_ints;
   unsigned off_items, off_part;     // bytes from the start of shared memory
@@ -806,6 +910,10 @@ struct PlanParams {
   int* row_order; unsigned char* flags; int* order1;
   double* embedding; long long* stats;
 };
+
+// (one copy of the function, in a rolled loop: sixteen in line were fetched one behind the other, 17,700 clk for 1,536
+// rows against 4,500)
+__device__ __noinline__ double polar_angle(double y, double x) { return atan2(y, x); }
 
 __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -891,6 +999,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
   u64* keys2 = keys + (merging ? m_b : 0);
   int* vals = reinterpret_cast<int*>(keys + (merging ? 2 * m_b : p.n_pow2));
   int* vals2 = vals + m_b;
+  int* bins = vals2 + m_b;
   auto sort_pairs = [&]() {
     if (!merging) { bitonic_sort(keys, vals, p.n_pow2); return; }
     if (merge_sort(keys, vals, keys2, vals2, m_b)) {
@@ -977,7 +1086,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
     block_sum<4>(b, scratch, (tid & ~31) < m_b);
     // (one warp works the angle out: 32 of them kept the fp64 units busy with it for 4,000 cycles)
     if (tid < 32) {
-      const double th = 0.5 * atan2(2.0 * (0.5 * (b[1] + b[2])), b[0] - b[3]);
+      const double th = 0.5 * polar_angle(2.0 * (0.5 * (b[1] + b[2])), b[0] - b[3]);
       if (tid == 0) { scratch[4] = cos(th); scratch[5] = sin(th); }
     }
     __syncthreads();
@@ -1003,32 +1112,41 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
     double s1 = (f[0] != INT_MAX && X[f[0]].x < 0.0) ? -1.0 : 1.0;
     double s2 = (f[1] != INT_MAX && X[f[1]].y < 0.0) ? -1.0 : 1.0;
     __syncthreads();
-    // ---- polar angle a_i = atan2(u_2[i], u_1[i]) (Eq. 4); kept in registers across the
-    //      re-use of the shared region by the sort
+    // ---- polar angle a_i = atan2(u_2[i], u_1[i]) (Eq. 4), as a sort key in the place of u_1; the keys
+    //      go through registers into the shared region, where they overwrite X
+#pragma unroll 1
+    for (int i = tid; i < m_b; i += kPlanThreads) {
+      const double2 u = X[i];
+      const double u1 = s1 * u.x + 0.0, u2 = s2 * u.y + 0.0;
+      if (p.embedding) { p.embedding[((size_t)h * m_b + i) * 2] = u1; p.embedding[((size_t)h * m_b + i) * 2 + 1] = u2; }
+      X[i].x = __longlong_as_double((long long)sortable(polar_angle(u2, u1) + 0.0));
+    }
     constexpr int kPer = (kMaxSort + kPlanThreads - 1) / kPlanThreads;
-    double ang[kPer];
+    u64 ang[kPer];
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
-      int i = tid + k * kPlanThreads;
-      ang[k] = 0.0;
-      if (i < m_b) {
-        double2 u = X[i];
-        double u1 = s1 * u.x + 0.0, u2 = s2 * u.y + 0.0;
-        if (p.embedding) { p.embedding[((size_t)h * m_b + i) * 2] = u1; p.embedding[((size_t)h * m_b + i) * 2 + 1] = u2; }
-        ang[k] = atan2(u2, u1) + 0.0;
-      }
+      const int i = tid + k * kPlanThreads;
+      ang[k] = i < m_b ? (u64)__double_as_longlong(X[i].x) : ~0ull;
     }
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < kPer; ++k) {
-      int i = tid + k * kPlanThreads;
+      const int i = tid + k * kPlanThreads;
       if (i < n_sort) {
-        keys[i] = i < m_b ? sortable(ang[k]) : ~0ull;
+        keys[i] = ang[k];
         vals[i] = i < m_b ? i : INT_MAX;
       }
     }
     __syncthreads();
-    sort_pairs();                           // Stage 1: rows by ascending angle, ties by row index
+    // Stage 1: rows by ascending angle, ties by row index.  Bins of equal width over the circle (the
+    // map is monotone: every rounding in it is)
+    const double per_bin = (double)p.bins * 0.15915494309189535;       // bins / (2 pi)
+    auto angle_bin = [&](u64 k) {
+      const double a = __longlong_as_double((long long)((k >> 63) ? (k & 0x7FFFFFFFFFFFFFFFull) : ~k));
+      return min(max((int)((a + 3.14159265358979323846) * per_bin), 0), p.bins - 1);
+    };
+    if (p.bins == 0 || p.ring_cut || !bin_sort(keys, vals, keys2, vals2, m_b, bins, p.bins, reinterpret_cast<int*>(scratch), angle_bin))
+      sort_pairs();
     if (p.ring_cut && m_b >= 2) {
       // Variant: the sorted rows form a ring (Section 4.3.1); open it at the largest gap between
       // neighbouring angles (the gap around the back, first + 2 pi - last, included; the first
@@ -1079,6 +1197,27 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
   }
   // ---- Stage 2: inside each bucket of `wave` consecutive positions, descending n_i, ties by
   //      Stage-1 position
+  if (p.warp_stage2) {
+    // a warp per bucket: keys (n_b - n_i, position) in 32 bits, sorted in registers.  21,000 -> 7,200 clk for
+    // 2,841 rows, 14,600 -> 12,000 for 1,536
+    const int lane = tid & 31;
+    for (int b0 = (tid >> 5) * p.wave; b0 < m_b; b0 += kPlanWarps * p.wave) {
+      const int b1 = min(b0 + p.wave, m_b);
+      unsigned a[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {                    // (any order will do to begin with: neighbouring lanes, neighbouring rows)
+        const int i = b0 + e * 32 + lane;
+        a[e] = i < b1 ? (unsigned)(n_b - nnz[vals[i]]) << 14 | (unsigned)i : UINT_MAX;
+      }
+      warp_sort256(a);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) {
+        const int at = b0 + lane * 8 + e;
+        if (at < b1) order_out[at] = vals[a[e] & (kMaxSort - 1)];
+      }
+    }
+    return;
+  }
   if (p.count_stage2) {
     // small buckets: a row's place is the number of rows of its bucket that go before it, by a key of
     // (n_b - n_i, position) in 32 bits.  Most warps lie in one bucket, whose keys they read as broadcasts:
@@ -1115,7 +1254,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
 
 struct PlanLayout {
   size_t off_bitmap, off_mt, off_nnz, off_cnt, off_state, total;
-  int wq, wk, n_pow2, state_in_smem;
+  int wq, wk, n_pow2, state_in_smem, bins;
   size_t smem;
   // shared memory of the matrix-unit form: does it fit, the iteration blocks behind `region`, the
   // digits behind them (the partial sums of the column split come last, launch_shape() adds them)
@@ -1148,7 +1287,11 @@ waveal_status plan_layout(const waveal_plan_desc* d, PlanLayout* L) {
   L->n_pow2 = p2;
   size_t sort_bytes = (size_t)p2 * 12, state_bytes = (2 * m + n) * 16;
   L->state_in_smem = 2048 + (state_bytes > sort_bytes ? state_bytes : sort_bytes) <= kSmemMax;
+  // angular sort by two bins a row from 513 rows on (below, the merge sort has few passes), as far as they fit behind its buffers
+  // (7,200 rows)
+  L->bins = 0;
   if (m <= (size_t)kMaxMerge) sort_bytes = m * 24;
+  if (m > 512 && 2048 + m * 32 <= kSmemMax) { L->bins = (int)(2 * m); sort_bytes = m * 32; }
   L->smem = 2048 + (L->state_in_smem ? (state_bytes > sort_bytes ? state_bytes : sort_bytes) : sort_bytes);
   // The matrix-unit form also keeps the digits of one block, 16 bytes an entry.  On square masks it
   // fits up to ~3,580 blocks as it is, up to ~4,730 with Y and Z in one buffer and up to 14,336
@@ -1273,6 +1416,10 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
   // counting costs 2.5 wave instructions a row, the merge sort ~550: kMaxSort = 2^14 positions, and
   // n - n_i has to fit the other 18 bits
   p.count_stage2 = p.wave <= 220 && n < (1u << 18);
+  // a warp sorts up to 256 rows.  Counting is quicker where a thread has one row to place (591 rows: 8,200 clk against
+  // 10,500) and where the buckets are short
+  p.warp_stage2 = p.count_stage2 && p.wave >= 64 && m > kPlanThreads;
+  p.bins = L.bins;
   p.mma = L.mma; p.alias_yz = L.alias_yz; p.off_items = (unsigned)L.off_items;
   p.ksplit_y = p.ksplit_z = 1;
   size_t smem = L.smem;

@@ -88,6 +88,28 @@ def test_plan_products_agree_between_their_forms(m, n, wide):
     assert torch.equal(a.order1, b.order1) and torch.equal(a.row_order, b.row_order)
 
 
+# 512 / 513 rows: angles by merging or by bins; 150 / 250 equal rows: a full bin, or one too many for it; 1,024 / 1,025 rows:
+# Stage 2 by counting or a warp per bucket, buckets of 63 / 64 / 219 / 220 rows and of what is left
+@pytest.mark.parametrize("m,wave,equal", [(512, 148, 0), (513, 148, 0), (700, 148, 150), (700, 148, 250), (1024, 64, 0), (1025, 63, 0),
+                                          (1025, 64, 20), (1300, 219, 0), (1500, 220, 700), (2841, 148, 0), (7168, 148, 300)])
+def test_sorts_of_the_plan(m, wave, equal):
+    mask = _mask(2, m, 300, 0.1, m + wave)
+    mask[0, torch.randperm(m, generator=torch.Generator().manual_seed(m))[:equal].cuda()] = True
+    r = _plan(mask, wave)
+    nnz = mask.sum(2).cpu().numpy()
+    for h in range(2):
+        first, order = r.order1[h].cpu().numpy(), r.row_order[h].cpu().numpy()
+        u = r.embedding[h].cpu().numpy()[first]
+        a = np.arctan2(u[:, 1], u[:, 0])
+        assert np.array_equal(np.sort(first), np.arange(m))
+        assert (np.diff(a) > -1e-14).all()                 # (NumPy's and the device's arctangents are an ulp or two apart)
+        same = (np.diff(u, axis=0) == 0).all(1)
+        assert (np.diff(first)[same] > 0).all()
+        for lo in range(0, m, wave):
+            bucket = first[lo:lo + wave]
+            assert np.array_equal(order[lo:lo + wave], bucket[np.argsort(-nnz[h][bucket], kind="stable")])
+
+
 def _first_sweep(rows, cols, m, n, real):
     """Q factor after one sweep of Algorithm 1 over the sorted (row, column) pairs, in NumPy at the precision `real`."""
     def product(out, src, size, x):               # sums of x[src] over equal, ascending `out`
