@@ -595,7 +595,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   Task* tasks = reinterpret_cast<Task*>(smem + G::OFF_TASK);
   volatile float* mpub = reinterpret_cast<volatile float*>(smem + G::OFF_MX);   // [tile count mod 4][128] reference max after a tile; FAST: [tile count mod 4][column half][128], over mhalf too
   volatile float* mhalf = reinterpret_cast<volatile float*>(smem + G::OFF_MX + 4 * 128 * 4);   // [use parity][team][column half][128] max of a half row
-  float2* ex = reinterpret_cast<float2*>(smem + G::OFF_MX + 4 * 128 * 4 + 2 * 2 * 2 * 128 * 4);    // [task mod 4][tile parity*2+half][128] (reference, sum)
+  float2* ex = reinterpret_cast<float2*>(smem + G::OFF_MX + 4 * 128 * 4 + 2 * 2 * 2 * 128 * 4);    // [task mod 4][role*2+half][128] (reference, sum); role 0: the team of the task's first tile
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + G::OFF_MISC);
   volatile int* abort_smem = reinterpret_cast<volatile int*>(smem + G::OFF_MISC + 4);
   // by task mod 4: number (from 1) of the last task that a tile wants computed again, and of the last one listed for it
@@ -937,7 +937,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     // epilogue adds the four partial sums of a row.
     const int sw = warp - kSoftmaxWarp0;       // 0..15
     const int quad = warp & 3;                 // tensor-memory lane quadrant this warp may access
-    const int team = (sw >> 2) & 1;            // owns the tiles whose number over the CTA's life has this parity
+    const int team = (sw >> 2) & 1;            // owns every second tile (by the tile's number over the CTA's life, or as kTwoFirst says)
     const int half = sw >> 3;                  // column half of S; epilogue: the same half of the O columns
     const int r = quad * 32 + lane;            // row of the 128-row MMA tile
     const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
@@ -949,9 +949,17 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     // the other (running reference, partial sums, redo flag) therefore lies in four slots each: three S
     // buffers let a team run ahead of the other's epilogue by two of its own tiles, hence two tasks.
     uint32_t task_it = 0, o_it = 0, mx_phase = 0, hx_it = 0;
+    // kTwoFirst: the team that is not in the epilogue of the task before takes the first two tiles, then they alternate: 0 1 3 5 ...
+    // and 2 4 6 ...  By turns from the first tile on, the second one's P waits for the end of that epilogue, and the P V of
+    // the third, long ready, for it.  First launch of 128-row blocks at head_dim 64: tasks of 16 / 24 / 256 tiles 1,292 -> 1,266 /
+    // 1,246 -> 1,228 / 1,160 -> 1,151 clk a tile.  (At head_dim 128 tasks of 17 tiles gained 2 %, but every form of it made the
+    // compiler's code for the loop over the tiles slower, 1,366 -> 1,404 clk a tile of long tasks, and so it did for 64x64
+    // blocks, 1,257 -> 1,297.  The second launch hands a reference on from tile to tile.)
+    constexpr bool kTwoFirst = FAST && D == 64 && G::KB == 1;
     uint32_t g0 = 0;                           // tiles before this task
+    int first_team = 0;                        // kTwoFirst: the team of the task's first tile
     uint32_t sb = (uint32_t)team, s_ph = 0;    // S buffer of this team's next tile and the parity of that use
-    auto next_buffer = [&]() { sb += 2; if (sb >= (uint32_t)G::NSBUF) { sb -= (uint32_t)G::NSBUF; s_ph ^= 1; } };
+    auto next_buffer = [&](int j) { sb += kTwoFirst && j == 0 ? 1 : 2; if (sb >= (uint32_t)G::NSBUF) { sb -= (uint32_t)G::NSBUF; s_ph ^= 1; } };
     bool ok = true, storing = false;           // storing: the stores of this warp's last epilogue may still read the Q tile
     while (ok) {
       const uint32_t slot = task_it & 1, ph = (task_it >> 1) & 1;
@@ -990,13 +998,16 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       // l_run: sum over this thread's columns of this team's blocks, relative to the reference m_ref
       float m_ref = -INFINITY, l_run = 0.f;
       const int last = tk.n - 1;
-      for (int j = (int)((g0 ^ (uint32_t)team) & 1u); j < tk.n; j += 2) {
+      const int role = kTwoFirst ? (team == first_team ? 0 : 1) : (int)((g0 ^ (uint32_t)team) & 1u);       // 0: has the first tile
+      const int j0 = kTwoFirst ? 2 * role : role;
+      if (kTwoFirst) { sb = (g0 + (uint32_t)j0) % G::NSBUF; s_ph = ((g0 + (uint32_t)j0) / G::NSBUF) & 1u; }
+      for (int j = j0; j < tk.n; j += kTwoFirst && j == 0 ? 1 : 2) {
         const uint32_t g = g0 + (uint32_t)j;
         ok = warp_wait(ctx, BAR(B_S_FULL + sb), s_ph, 21);
         if (!ok) break;
         if (idle) {
           if (lane == 0) mbar_arrive(BAR(B_P_FULL + sb * 2 + half));
-          next_buffer();
+          next_buffer(j);
           continue;
         }
         {
@@ -1019,9 +1030,12 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           if constexpr (FAST) {
             // The two owners of the row in the first tile leave the largest of their own scores; they and, at its first tile,
             // the other team take the larger of the two.  (Slot and barrier by tile count mod 4: a later task's first tile
-            // that uses the slot again waits for its S buffer, hence for the P V of this task's second tile.)
-            if (j <= 1) {
-              const uint32_t mx = (g - (uint32_t)j) & 3;
+            // that uses the slot again waits for its S buffer, hence for the P V of this task's second tile.  kTwoFirst, where the other
+            // team comes to it in the task's third tile: by task count mod 4, so that the first tile that uses the slot again lies
+            // six tiles or more behind this one, four if the task has no third tile; it waits for the P V of the tile
+            // three before it.)
+            if (kTwoFirst ? j == j0 : j <= 1) {
+              const uint32_t mx = kTwoFirst ? o_it & 3 : (g - (uint32_t)j) & 3;
               volatile float* mh = mpub + mx * 256;
               if (j == 0) {
                 float mloc = -INFINITY;
@@ -1157,18 +1171,24 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           __syncwarp();
           if (lane == 0) mbar_arrive(BAR(B_P_FULL + sb * 2 + half));
         }
-        next_buffer();
+        next_buffer(j);
       }
       if (!ok) break;
-      // ---- epilogue: O / l at the original row position; l = the four partial sums of the row (by parity of
-      // the tile in the task, so that the result does not depend on which team had which) brought to
-      // the final reference (the larger of the two parities', references never shrink)
+      // ---- epilogue: O / l at the original row position; l = the four partial sums of the row (by whether
+      // the team had the task's first tile, so that the result does not depend on which team had which) brought to
+      // the final reference (the larger of the two teams', references never shrink)
       // (a thread's partial sum is final once its last tile is done)
-      exb[(((team ^ (int)g0) & 1) * 2 + half) * 128 + r] = make_float2(m_ref, l_run);
+      exb[(role * 2 + half) * 128 + r] = make_float2(m_ref, l_run);
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR(ex_bar));
-      const bool mine = (int)((g0 + (uint32_t)last) & 1u) == team;
-      if (!mine && !idle && !(FAST && last > 0)) mx_phase ^= 1u << ((g0 + (uint32_t)last) & 3);
+      // (the team of the last tile; at least one of the first two is the first team's)
+      const bool mine = kTwoFirst ? (role == 0) == (last == 0 || (last & 1)) : (int)((g0 + (uint32_t)last) & 1u) == team;
+      if (kTwoFirst) {
+        if (j0 >= tk.n && !idle) mx_phase ^= 1u << (o_it & 3);
+        first_team = mine ? team ^ 1 : team;
+      } else if (!mine && !idle && !(FAST && last > 0)) {
+        mx_phase ^= 1u << ((g0 + (uint32_t)last) & 3);
+      }
       g0 += (uint32_t)tk.n;
       const uint32_t o_ph = o_it & 1;
       ++o_it;
@@ -1180,7 +1200,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       ok = warp_wait(ctx, BAR(ex_bar), ex_ph, 25);
       if (!ok) break;
       const float2 e00 = exb[0 * 128 + r], e01 = exb[1 * 128 + r], e10 = exb[2 * 128 + r], e11 = exb[3 * 128 + r];
-      const float m0 = fmaxf(e00.x, e01.x), m1 = fmaxf(e10.x, e11.x);     // the two owners of a parity agree; a parity
+      const float m0 = fmaxf(e00.x, e01.x), m1 = fmaxf(e10.x, e11.x);     // the two owners of a team's rows agree; a team
       const float m_all = fmaxf(m0, m1);                                   // without tiles (n == 1) has -inf
       const float a0 = (m0 == -INFINITY) ? 0.f : ex2(m0 - m_all);
       const float a1 = (m1 == -INFINITY) ? 0.f : ex2(m1 - m_all);
