@@ -419,6 +419,7 @@ struct Geo {
   static constexpr int HC = BK / 2;                  // S columns of a row one softmax thread owns (a row has two owners)
   static constexpr int CH = 32;                      // S columns a softmax thread holds at a time
   static constexpr int NCH = HC / CH;                // such chunks per thread and block
+  static constexpr int LAG = KB == 1 && D == 64 ? 0 : 4;   // pairs of exponentials under way before the first is used
   static constexpr int CO = D / 2;                   // O columns per epilogue thread
   static constexpr int OFF_Q = 0;
   static constexpr int OFF_K = OFF_Q + NQ * Q_BYTES;
@@ -1144,19 +1145,25 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             WAVEAL_TMEM_LD32(s_addr + ch * G::CH, sv, 0);
             WAVEAL_TMEM_WAIT_LD32(sv, 0);
             uint32_t pk[G::CH / 2];
+            // a pair's results are used LAG pairs later (written so, the compiler keeps more exponentials under way: 1,366 -> 1,347
+            // clk a tile of 128x128 tasks of 256 tiles, 64x64 1,195 -> 1,186; 128x64 blocks lost 0.6 % and use them at once)
+            float x[G::CH];
+            auto use = [&](int c) {
+              fadd2(ls4[c & 2], ls4[(c & 2) + 1], ls4[c & 2], ls4[(c & 2) + 1], x[c], x[c + 1]);
+              pk[c / 2] = __byte_perm(__float_as_uint(x[c]), __float_as_uint(x[c + 1]), 0x7632);
+            };
 #pragma unroll
             for (int c = 0; c < G::CH; c += 2) {
-              float e0, e1;
               if ((c >> 1) % kPolyEvery == kPolyEvery - 1) {
-                ex2_fma2(e0, e1, __uint_as_float(sv[c]), __uint_as_float(sv[c + 1]), a128, b128);
+                ex2_fma2(x[c], x[c + 1], __uint_as_float(sv[c]), __uint_as_float(sv[c + 1]), a128, b128);
               } else {
-                float x0, x1;
-                ffma2(x0, x1, __uint_as_float(sv[c]), __uint_as_float(sv[c + 1]), p.sl2, p.sl2, neg_m, neg_m);
-                e0 = ex2(x0); e1 = ex2(x1);
+                ffma2(x[c], x[c + 1], __uint_as_float(sv[c]), __uint_as_float(sv[c + 1]), p.sl2, p.sl2, neg_m, neg_m);
+                x[c] = ex2(x[c]); x[c + 1] = ex2(x[c + 1]);
               }
-              fadd2(ls4[c & 2], ls4[(c & 2) + 1], ls4[c & 2], ls4[(c & 2) + 1], e0, e1);
-              pk[c / 2] = __byte_perm(__float_as_uint(e0), __float_as_uint(e1), 0x7632);
+              if (c >= 2 * G::LAG) use(c - 2 * G::LAG);
             }
+#pragma unroll
+            for (int c = G::CH - 2 * G::LAG; c < G::CH; c += 2) use(c);
             WAVEAL_TMEM_ST16(s_addr + ch * 16, pk, 0);
           }
           const float l_blk = (ls4[0] + ls4[1]) + (ls4[2] + ls4[3]);
