@@ -419,6 +419,9 @@ struct Geo {
   static constexpr int HC = BK / 2;                  // S columns of a row one softmax thread owns (a row has two owners)
   static constexpr int CH = 32;                      // S columns a softmax thread holds at a time
   static constexpr int NCH = HC / CH;                // such chunks per thread and block
+  // chunks of the exponential loop in line: both at head_dim 64 (128x64 blocks 1,229 -> 1,212 clk a tile, 64x64 1,182 -> 1,150 and
+  // 1,248 -> 1,218 for lists of 256 / 64 blocks), one at head_dim 128 (both: 1,346 -> 1,368 and 1,292 -> 1,302)
+  static constexpr int UNROLL = D == 64 ? NCH : 1;
   static constexpr int LAG = KB == 1 && D == 64 ? 0 : 4;   // pairs of exponentials under way before the first is used
   static constexpr int CO = D / 2;                   // O columns per epilogue thread
   static constexpr int OFF_Q = 0;
@@ -1137,9 +1140,9 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           const float a128 = p.sl2 * 0.0078125f, b128 = (neg_m - kPolyLo) * 0.0078125f;   // polynomial share
           float ls4[4] = {0.f, 0.f, 0.f, 0.f};
           // ---- pass 2: exponentials; P (bf16 pairs) goes over the first half of the thread's own
-          // S columns, each chunk after its S values have been read.  A rolled loop over
-          // 32-column chunks: the body stays small enough for the instruction cache.
-#pragma unroll 1
+          // S columns, each chunk after its S values have been read.  A loop over
+          // 32-column chunks, rolled at head_dim 128.
+#pragma unroll G::UNROLL
           for (int ch = 0; ch < G::NCH; ++ch) {
             uint32_t sv[G::CH];
             WAVEAL_TMEM_LD32(s_addr + ch * G::CH, sv, 0);
