@@ -20,13 +20,13 @@
 //   warps 2-17  softmax, two teams of eight warps that take the KV blocks of a task in turn;
 //               inside a team a row of S has two owners, one per half of its columns (row max
 //               in the tiles that take one, then exponentials and P in a second read of S,
-//               32 columns at a time in a rolled loop).  On every scheduler two warps of each
+//               32 columns at a time).  On every scheduler two warps of each
 //               team are resident, the teams half a block apart, so one team's waits and loads
-//               hide behind the other's arithmetic.  The teams hand each other the running
+//               hide behind the other's arithmetic.  The teams hand each other the
 //               reference max of every row through shared memory; every thread keeps the row
-//               sum of its own columns; O in tensor memory is rescaled only when the max grew
-//               by more than 2^8; the epilogue adds the four partial sums of a row, normalises
-//               and stores O at the ORIGINAL row (no inverse permutation)
+//               sum of its own columns; O in tensor memory is rescaled only in the second launch, when the
+//               max grew by more than 2^8; the epilogue adds the four partial sums of a row, normalises
+//               and stores O at the ORIGINAL row (no inverse permutation; 128-row blocks through shared memory)
 // Two launches per call: in the first the row max is taken in the first tile of a task only
 // and the reference stays fixed afterwards (softmax does not depend on it short of
 // overflow: P in bf16, the sums and O in fp32 have the same exponent range); a task in which a
@@ -1151,9 +1151,9 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             // a pair's results are used LAG pairs later (written so, the compiler keeps more exponentials under way: 1,366 -> 1,347
             // clk a tile of 128x128 tasks of 256 tiles, 64x64 1,195 -> 1,186; 128x64 blocks lost 0.6 % and use them at once)
             float x[G::CH];
-            auto use = [&](int c) {
-              fadd2(ls4[c & 2], ls4[(c & 2) + 1], ls4[c & 2], ls4[(c & 2) + 1], x[c], x[c + 1]);
-              pk[c / 2] = __byte_perm(__float_as_uint(x[c]), __float_as_uint(x[c + 1]), 0x7632);
+            auto use = [&](int c, float e0, float e1) {
+              fadd2(ls4[c & 2], ls4[(c & 2) + 1], ls4[c & 2], ls4[(c & 2) + 1], e0, e1);
+              pk[c / 2] = __byte_perm(__float_as_uint(e0), __float_as_uint(e1), 0x7632);
             };
 #pragma unroll
             for (int c = 0; c < G::CH; c += 2) {
@@ -1163,10 +1163,10 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                 ffma2(x[c], x[c + 1], __uint_as_float(sv[c]), __uint_as_float(sv[c + 1]), p.sl2, p.sl2, neg_m, neg_m);
                 x[c] = ex2(x[c]); x[c + 1] = ex2(x[c + 1]);
               }
-              if (c >= 2 * G::LAG) use(c - 2 * G::LAG);
+              if (c >= 2 * G::LAG) use(c - 2 * G::LAG, x[c - 2 * G::LAG], x[c + 1 - 2 * G::LAG]);
             }
 #pragma unroll
-            for (int c = G::CH - 2 * G::LAG; c < G::CH; c += 2) use(c);
+            for (int c = G::CH - 2 * G::LAG; c < G::CH; c += 2) use(c, x[c], x[c + 1]);
             WAVEAL_TMEM_ST16(s_addr + ch * 16, pk, 0);
           }
           const float l_blk = (ls4[0] + ls4[1]) + (ls4[2] + ls4[3]);
