@@ -143,45 +143,47 @@ class PlanResult:
     def __init__(self, **kw):
         self.__dict__.update(kw)
 
-    def __getattr__(self, name):
-        # A plan from a bitmap has nothing to report from the device: its status is zeros, and is made for those who look
-        # at it (clearing four words at every call was a launch between two others, 6 us of the host's 22)
-        if name != "dev_status":
-            raise AttributeError(name)
-        self.dev_status = self.row_order.new_zeros((4,))
-        return self.dev_status
 
-
-def _plan_outputs(desc: PlanDesc, like, debug: bool, reports: bool):
+def _plan_outputs(desc: PlanDesc, like, debug: bool, stream):
     import torch
     H, M, N = desc.heads, desc.n_q_blocks, desc.n_kv_blocks
     device = like.device
-    # two allocations: a tensor per output took more of the host's time than the call itself
-    buf = like.new_empty((2 * H * M + (H + 3) // 4,), dtype=torch.int32)
+    # one allocation: a tensor per output took more of the host's time than the call itself
+    at_flags, at_status = 2 * H * M, 2 * H * M + (H + 3) // 4
+    buf = like.new_empty((at_status + 4,), dtype=torch.int32)
     res = PlanResult(
         row_order=buf.as_strided((H, M), (M, 1), 0),
         row_nnz=buf.as_strided((H, M), (M, 1), H * M),
-        skip_flags=buf.view(torch.uint8).as_strided((H,), (1,), 8 * H * M),
+        skip_flags=buf.view(torch.uint8).as_strided((H,), (1,), 4 * at_flags),
+        dev_status=buf.as_strided((4,), (1,), at_status),
         col_count=None, order1=None, embedding=None, stats=None)
-    if reports:
-        res.dev_status = like.new_zeros((4,), dtype=torch.int32)
+    # cleared on the call's own stream: ordered before the kernels that may report something, and for whoever
+    # reads the words behind them
+    if stream is None:
+        res.dev_status.zero_()
+    else:
+        if not isinstance(stream, torch.cuda.Stream):
+            stream = torch.cuda.ExternalStream(stream.cuda_stream, device)
+        with torch.cuda.stream(stream):
+            res.dev_status.zero_()
     if debug:
         res.col_count = torch.empty((H, N), dtype=torch.int32, device=device)
         res.order1 = torch.empty((H, M), dtype=torch.int32, device=device)
         res.embedding = torch.empty((H, M, 2), dtype=torch.float64, device=device)
         res.stats = torch.empty((H, 4), dtype=torch.int64, device=device)
     out = PlanOut(_ptr(res.row_order), _ptr(res.row_nnz), _ptr(res.skip_flags), _ptr(res.col_count),
-                  _ptr(res.order1), _ptr(res.embedding), _ptr(res.stats), _ptr(res.dev_status) if reports else None)
+                  _ptr(res.order1), _ptr(res.embedding), _ptr(res.stats), _ptr(res.dev_status))
     return res, out
 
 
 def plan_bitmap(desc: PlanDesc, mask_bits, workspace=None, debug: bool = False, stream=None) -> PlanResult:
-    """waveal_plan_bitmap.  mask_bits: cuda tensor of 64-bit words [heads, M_B, ceil(N_B/64)]."""
+    """waveal_plan_bitmap.  mask_bits: cuda tensor of 64-bit words [heads, M_B, ceil(N_B/64)].  A bitmap holds
+    nothing that could be malformed: the result's dev_status stays zero."""
     import torch
     lib = load()
     if workspace is None:
         workspace = torch.empty((plan_workspace_bytes(desc) + 256,), dtype=torch.uint8, device=mask_bits.device)
-    res, out = _plan_outputs(desc, mask_bits, debug, reports=False)
+    res, out = _plan_outputs(desc, mask_bits, debug, stream)
     res.workspace = workspace
     _check(lib.waveal_plan_bitmap(ctypes.byref(desc), _ptr(mask_bits), _ptr(workspace), workspace.numel(),
                                   ctypes.byref(out), _stream(stream)))
@@ -189,12 +191,12 @@ def plan_bitmap(desc: PlanDesc, mask_bits, workspace=None, debug: bool = False, 
 
 
 def plan_csr(desc: PlanDesc, kv_row_ptr, kv_block_indices, workspace=None, debug: bool = False, stream=None) -> PlanResult:
-    """waveal_plan_csr."""
+    """waveal_plan_csr.  dev_status reports an index out of range."""
     import torch
     lib = load()
     if workspace is None:
         workspace = torch.empty((plan_workspace_bytes(desc) + 256,), dtype=torch.uint8, device=kv_row_ptr.device)
-    res, out = _plan_outputs(desc, kv_row_ptr, debug, reports=True)      # (an index out of range)
+    res, out = _plan_outputs(desc, kv_row_ptr, debug, stream)
     res.workspace = workspace
     _check(lib.waveal_plan_csr(ctypes.byref(desc), _ptr(kv_row_ptr), _ptr(kv_block_indices), _ptr(workspace),
                                workspace.numel(), ctypes.byref(out), _stream(stream)))

@@ -6,6 +6,7 @@ import os
 import re
 
 import pytest
+import torch
 
 from paper_2609_34814_b200 import binding as wb
 from paper_2609_34814_b200 import build as wbuild
@@ -97,6 +98,35 @@ def test_attention_host_errors_before_any_launch(lib):
     d.q_stride[1] = 100
     assert call() == wb.ERR_INVALID_ARG
     assert wb.status_string(wb.ERR_TIMEOUT) == "device-side wait timed out"
+
+
+@pytest.mark.parametrize("lists", [False, True])
+def test_a_plan_s_status_words_are_cleared_by_the_call(monkeypatch, lists):
+    """Not when they are first looked at: that could be inside a graph capture or on another stream."""
+    handed = []
+
+    class Lib:
+        def waveal_plan_bitmap(self, desc, bits, ws, n, out, stream):
+            handed.append(out._obj.dev_status)
+            return wb.OK
+
+        def waveal_plan_csr(self, desc, ptr, idx, ws, n, out, stream):
+            handed.append(out._obj.dev_status)
+            return wb.OK
+
+    monkeypatch.setattr(wb, "load", lambda: Lib())
+    monkeypatch.setattr(wb, "_stream", lambda s: None)
+    desc = wb.PlanDesc(heads=3, n_q_blocks=5, n_kv_blocks=70)
+    ws = torch.empty((64,), dtype=torch.uint8)
+    if lists:
+        res = wb.plan_csr(desc, torch.zeros((16,), dtype=torch.int32), torch.zeros((1,), dtype=torch.int32), workspace=ws)
+    else:
+        res = wb.plan_bitmap(desc, torch.zeros((3, 5, 2), dtype=torch.int64), workspace=ws)
+    assert vars(res)["dev_status"].tolist() == [0] * 4 and res.dev_status.dtype == torch.int32
+    assert handed == [res.dev_status.data_ptr()]
+    for name in ("row_order", "row_nnz", "skip_flags"):      # (they share an allocation)
+        getattr(res, name).fill_(77)
+    assert res.dev_status.tolist() == [0] * 4 and (res.row_order == 77).all() and (res.row_nnz == 77).all()
 
 
 def test_missing_library_fails_loudly(monkeypatch, tmp_path):

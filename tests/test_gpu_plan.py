@@ -185,6 +185,31 @@ def test_plan_out_of_range_index_is_reported_not_faulted():
     assert _np(res.row_nnz[0]).tolist() == [1, 1]       # the bad entry was skipped
 
 
+@pytest.mark.parametrize("lists", [False, True])
+def test_status_words_are_cleared_on_the_plan_s_own_stream(lists):
+    """The caller's current stream is busy while the plan runs on another one: what is read behind it there is zero,
+    and its reports are not cleared afterwards."""
+    H, m = 2, 300
+    mask = torch.rand((H, m, m), generator=torch.Generator().manual_seed(1)) < 0.1
+    bm = _bitmap_dev([x.numpy() for x in mask])
+    ptr, idx = wb.bitmap_to_csr(bm, m)
+    idx[idx.numel() - 1] = m + 5                            # (reported, not followed)
+    d = wb.plan_desc_default(heads=H, n_q_blocks=m, n_kv_blocks=m, wave_size=16, mode=wb.FORCE_REORDER)
+    ws = torch.empty((wb.plan_workspace_bytes(d) + 256,), dtype=torch.uint8, device="cuda")
+    used = [torch.full((2 * H * m + k,), 7, dtype=torch.int32, device="cuda") for k in (1, 5) for _ in range(16)]
+    used += [torch.full((4,), 7, dtype=torch.int32, device="cuda") for _ in range(16)]
+    torch.cuda.synchronize()
+    del used                                                # memory that does not happen to hold zeros
+    side = torch.cuda.Stream()
+    torch.cuda._sleep(200_000_000)                          # 0.1 s on the current stream
+    res = wb.plan_csr(d, ptr, idx, workspace=ws, stream=side) if lists else wb.plan_bitmap(d, bm, workspace=ws, stream=side)
+    with torch.cuda.stream(side):
+        st = res.dev_status.tolist()
+    assert st == ([wb.ERR_BAD_MASK, 1, H - 1, m + 5] if lists else [0] * 4)
+    torch.cuda.synchronize()
+    assert res.dev_status.tolist() == st
+
+
 @pytest.mark.parametrize("shape", [(1, 5), (7, 200), (130, 40), (64, 64)])
 def test_plan_degenerate_and_rectangular(shape):
     m, n = shape
