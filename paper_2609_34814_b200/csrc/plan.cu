@@ -805,15 +805,14 @@ __device__ __forceinline__ void exclusive_scan(int* a, int n, int* part) {
 // merge sort walks log2(n) binary searches.  43,800 -> 11,200 clk for 2,841 rows of a video mask, 10,400 -> 8,500 for 591; where a
 // sixth of the rows have one angle (rows that select everything) as long as the merge sort, 24,000 for 1,536.  (Bins cut at
 // the quantiles of a sample of the keys: 41,700 for the 2,841 rows, their bins of 22 and more are walked for longer.)
-// The sorted values go to v0.  False, with the pairs as they were, if a bin holds more than kBinMax.  (The order inside a
+// The sorted values go to v0.  False, with the pairs as they were, if a bin holds more than `most`.  (The order inside a
 // bin before the count depends on the atomics, the result does not.)
-constexpr int kBinMax = 192;
 template <class Bin>
-__device__ __forceinline__ bool bin_sort(const u64* k0, int* v0, u64* k1, int* v1, int n, int* bins, int n_bins, int* part, Bin bin) {
+__device__ __forceinline__ bool bin_sort(const u64* k0, int* v0, u64* k1, int* v1, int n, int* bins, int n_bins, int most, int* part, Bin bin) {
   for (int i = threadIdx.x; i < n_bins; i += kPlanThreads) bins[i] = 0;
   __syncthreads();
   bool big = false;
-  for (int i = threadIdx.x; i < n; i += kPlanThreads) big |= atomicAdd(&bins[bin(k0[i])], 1) >= kBinMax;
+  for (int i = threadIdx.x; i < n; i += kPlanThreads) big |= atomicAdd(&bins[bin(k0[i])], 1) >= most;
   if (__syncthreads_or(big)) return false;
   exclusive_scan(bins, n_bins, part);
   for (int i = threadIdx.x; i < n; i += kPlanThreads) {
@@ -904,7 +903,7 @@ struct PlanParams {
   int mma;              // mask products on the integer matrix units (else: walk over the set bits)
   int count_stage2;     // Stage 2 by counting inside the buckets (else: by a sort)
   int warp_stage2;      // Stage 2 by a warp per bucket
-  int bins;             // bins of the angular sort (0: by merging)
+  int bins, bin_max;    // bins of the angular sort (0: by merging) and the most rows one may hold
   int alias_yz;         // Y and Z share one buffer (two barriers more per iteration)
   int ksplit_y, ksplit_z, part_ints;
   unsigned off_items, off_part;     // bytes from the start of shared memory
@@ -1152,7 +1151,7 @@ __global__ void __launch_bounds__(kPlanThreads, 1) k_plan_head(PlanParams p) {
       const double a = __longlong_as_double((long long)((k >> 63) ? (k & 0x7FFFFFFFFFFFFFFFull) : ~k));
       return min(max((int)((a + 3.14159265358979323846) * per_bin), 0), p.bins - 1);
     };
-    if (p.bins == 0 || p.ring_cut || !bin_sort(keys, vals, keys2, vals2, m_b, bins, p.bins, reinterpret_cast<int*>(scratch), angle_bin))
+    if (p.bins == 0 || p.ring_cut || !bin_sort(keys, vals, keys2, vals2, m_b, bins, p.bins, p.bin_max, reinterpret_cast<int*>(scratch), angle_bin))
       sort_pairs();
     if (p.ring_cut && m_b >= 2) {
       // Variant: the sorted rows form a ring (Section 4.3.1); open it at the largest gap between
@@ -1427,6 +1426,11 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
   // 10,500) and where the buckets are short
   p.warp_stage2 = p.count_stage2 && p.wave >= 64 && m > kPlanThreads;
   p.bins = L.bins;
+  // Equal rows share a bin, which each of them walks.  It takes as long as the merge sort from 64 rows on where a thread has one row
+  // (plan of 5 heads, us, by bins / by merging: 591 rows with 33 equal ones 87 / 89, 64: 89 / 89, 128: 93 / 89, 191: 95 / 89; 1,000 rows
+  // with 64: 99 / 99, 191: 105 / 99), from an eighth of the rows on above (1,200 with 150: 112 / 112; 1,536 with 128: 120 / 122, 191: 122 / 122).
+  // Finding that a bin is too full costs up to 2 us.
+  p.bin_max = m <= kPlanThreads ? 64 : m / 8 < 192 ? (int)(m / 8) : 192;
   p.mma = L.mma; p.alias_yz = L.alias_yz; p.off_items = (unsigned)L.off_items;
   p.ksplit_y = p.ksplit_z = 1;
   size_t smem = L.smem;

@@ -88,10 +88,13 @@ def test_plan_products_agree_between_their_forms(m, n, wide):
     assert torch.equal(a.order1, b.order1) and torch.equal(a.row_order, b.row_order)
 
 
-# 512 / 513 rows: angles by merging or by bins; 150 / 250 equal rows: a full bin, or one too many for it; 1,024 / 1,025 rows:
+# 512 / 513 rows: angles by merging or by bins; equal rows that fill a bin, or are too many for it (64 up to 1,024 rows, an
+# eighth of the rows up to 192 above); 1,024 / 1,025 rows:
 # Stage 2 by counting or a warp per bucket, buckets of 63 / 64 / 219 / 220 rows and of what is left
 @pytest.mark.parametrize("m,wave,equal", [(512, 148, 0), (513, 148, 0), (700, 148, 150), (700, 148, 250), (1024, 64, 0), (1025, 63, 0),
-                                          (1025, 64, 20), (1300, 219, 0), (1500, 220, 700), (2841, 148, 0), (7168, 148, 300)])
+                                          (1025, 64, 20), (1300, 219, 0), (1500, 220, 700), (2841, 148, 0), (7168, 148, 300),
+                                          (700, 148, 64), (700, 148, 65), (1024, 64, 64), (1024, 64, 65), (1025, 64, 127), (1025, 64, 129),
+                                          (1536, 148, 192), (1536, 148, 193), (2841, 148, 193)])
 def test_sorts_of_the_plan(m, wave, equal):
     mask = _mask(2, m, 300, 0.1, m + wave)
     mask[0, torch.randperm(m, generator=torch.Generator().manual_seed(m))[:equal].cuda()] = True
@@ -108,6 +111,30 @@ def test_sorts_of_the_plan(m, wave, equal):
         for lo in range(0, m, wave):
             bucket = first[lo:lo + wave]
             assert np.array_equal(order[lo:lo + wave], bucket[np.argsort(-nnz[h][bucket], kind="stable")])
+
+
+# a head with many rows of one angle is planned as fast as by the merge sort alone (walked as one bin of 190: 4.5 to 7 % slower)
+@pytest.mark.parametrize("m", [520, 700])
+def test_equal_rows_do_not_slow_a_plan(m):
+    def best(equal):
+        mask = _mask(5, m, m, 0.1, m)
+        mask[:, torch.randperm(m, generator=torch.Generator().manual_seed(m))[:equal].cuda()] = True
+        bits = _pack(mask)
+        d = wb.plan_desc_default(heads=5, n_q_blocks=m, n_kv_blocks=m, wave_size=148, mode=wb.FORCE_REORDER, seed=5)
+        ws = torch.empty((wb.plan_workspace_bytes(d) + 256,), dtype=torch.uint8, device="cuda")
+        out = []
+        for _ in range(10):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda._sleep(4_000_000)             # the calls are queued before the first one starts
+            a.record()
+            for _ in range(20):
+                wb.plan_bitmap(d, bits, workspace=ws)
+            b.record()
+            torch.cuda.synchronize()
+            out.append(a.elapsed_time(b))
+        return min(out)
+
+    assert best(190) <= 1.02 * best(m // 2)          # (half of the rows go through the merge sort)
 
 
 def _first_sweep(rows, cols, m, n, real):
