@@ -71,6 +71,12 @@ typedef enum {
  * and keeps a tight group of rows that straddles +-pi in one piece. */
 #define WAVEAL_RING_CUT_LARGEST_GAP 16
 
+/* Optional bit, OR-ed into waveal_plan_desc.mode of waveal_plan_bitmap: the call's first kernel writes zeros to
+ * out->dev_status, so that a caller who hands over fresh memory needs no launch of its own to clear it (a bitmap plan
+ * reports nothing).  Without the bit the words are left as they are.  waveal_plan_csr refuses it: its first kernel
+ * is the one that reports. */
+#define WAVEAL_PLAN_CLEAR_STATUS 32
+
 /* skip_flags bits */
 #define WAVEAL_FLAG_SKIPPED 1u        /* this head's row_order is the identity (skip applied) */
 #define WAVEAL_FLAG_SHORT_SEQ 2u      /* one head's K+V fit the L2 budget (Section 4.5, case 1) */
@@ -83,7 +89,7 @@ typedef struct waveal_plan_desc {
   int32_t n_kv_blocks;    /* N_B                                                              */
   int32_t wave_size;      /* W = SMs x resident CTAs (Section 6.1); 0 = this device's SM count */
   int32_t svd_iters;      /* T of Algorithm 1 (paper: 5-15; library default 5)                */
-  int32_t mode;           /* waveal_mode, optionally | WAVEAL_RING_CUT_LARGEST_GAP            */
+  int32_t mode;           /* waveal_mode, optionally | WAVEAL_RING_CUT_LARGEST_GAP | WAVEAL_PLAN_CLEAR_STATUS */
   uint64_t seed;          /* seed of the start block of Algorithm 1                           */
   /* guard thresholds, all integer comparisons (the "offline profile" of Section 4.5):       */
   int64_t kv_bytes_per_head; /* bytes of K plus V of one head; 0 disables the short-seq test */

@@ -144,7 +144,7 @@ class PlanResult:
         self.__dict__.update(kw)
 
 
-def _plan_outputs(desc: PlanDesc, like, debug: bool, stream):
+def _plan_outputs(desc: PlanDesc, like, debug: bool):
     import torch
     H, M, N = desc.heads, desc.n_q_blocks, desc.n_kv_blocks
     device = like.device
@@ -157,15 +157,6 @@ def _plan_outputs(desc: PlanDesc, like, debug: bool, stream):
         skip_flags=buf.view(torch.uint8).as_strided((H,), (1,), 4 * at_flags),
         dev_status=buf.as_strided((4,), (1,), at_status),
         col_count=None, order1=None, embedding=None, stats=None)
-    # cleared on the call's own stream: ordered before the kernels that may report something, and for whoever
-    # reads the words behind them
-    if stream is None:
-        res.dev_status.zero_()
-    else:
-        if not isinstance(stream, torch.cuda.Stream):
-            stream = torch.cuda.ExternalStream(stream.cuda_stream, device)
-        with torch.cuda.stream(stream):
-            res.dev_status.zero_()
     if debug:
         res.col_count = torch.empty((H, N), dtype=torch.int32, device=device)
         res.order1 = torch.empty((H, M), dtype=torch.int32, device=device)
@@ -178,14 +169,17 @@ def _plan_outputs(desc: PlanDesc, like, debug: bool, stream):
 
 def plan_bitmap(desc: PlanDesc, mask_bits, workspace=None, debug: bool = False, stream=None) -> PlanResult:
     """waveal_plan_bitmap.  mask_bits: cuda tensor of 64-bit words [heads, M_B, ceil(N_B/64)].  A bitmap holds
-    nothing that could be malformed: the result's dev_status stays zero."""
+    nothing that could be malformed: the result's dev_status is zero (cleared by the call's first kernel: a launch
+    of its own for four words took 7 of the smallest step's 47 us)."""
     import torch
     lib = load()
     if workspace is None:
         workspace = torch.empty((plan_workspace_bytes(desc) + 256,), dtype=torch.uint8, device=mask_bits.device)
-    res, out = _plan_outputs(desc, mask_bits, debug, stream)
+    res, out = _plan_outputs(desc, mask_bits, debug)
     res.workspace = workspace
-    _check(lib.waveal_plan_bitmap(ctypes.byref(desc), _ptr(mask_bits), _ptr(workspace), workspace.numel(),
+    own = PlanDesc.from_buffer_copy(desc)            # (the caller's may serve several threads)
+    own.mode |= PLAN_CLEAR_STATUS
+    _check(lib.waveal_plan_bitmap(ctypes.byref(own), _ptr(mask_bits), _ptr(workspace), workspace.numel(),
                                   ctypes.byref(out), _stream(stream)))
     return res
 
@@ -196,8 +190,15 @@ def plan_csr(desc: PlanDesc, kv_row_ptr, kv_block_indices, workspace=None, debug
     lib = load()
     if workspace is None:
         workspace = torch.empty((plan_workspace_bytes(desc) + 256,), dtype=torch.uint8, device=kv_row_ptr.device)
-    res, out = _plan_outputs(desc, kv_row_ptr, debug, stream)
+    res, out = _plan_outputs(desc, kv_row_ptr, debug)
     res.workspace = workspace
+    # cleared on the call's own stream: ordered before the kernels that may report something
+    if stream is None:
+        res.dev_status.zero_()
+    else:
+        own = stream if isinstance(stream, torch.cuda.Stream) else torch.cuda.ExternalStream(stream.cuda_stream, kv_row_ptr.device)
+        with torch.cuda.stream(own):
+            res.dev_status.zero_()
     _check(lib.waveal_plan_csr(ctypes.byref(desc), _ptr(kv_row_ptr), _ptr(kv_block_indices), _ptr(workspace),
                                workspace.numel(), ctypes.byref(out), _stream(stream)))
     return res
@@ -264,6 +265,7 @@ def scatter_rows(src, dst, row_order, block: int, stream=None):
 
 
 RING_CUT_LARGEST_GAP = 16
+PLAN_CLEAR_STATUS = 32
 ATTN_ONLINE_MAX_ONLY = 1
 ATTN_SELFTEST_LOST_TILE = 256
 ATTN_NO_ROW_PAIRING = 2

@@ -122,10 +122,12 @@ constexpr int kStatThreads = 256, kStatRows = 32;
 constexpr int kStripMax = 64 * (2 * (kMaxSort / 64) + 1) * 4;      // bytes of the longest strip: 131,328
 __global__ void __launch_bounds__(kStatThreads) k_mask_stats(const u64* __restrict__ M, u64* __restrict__ Mt, int m_b, int n_b,
                                                              int wq, int wk, int* __restrict__ nnz, int* __restrict__ cnt,
-                                                             int* __restrict__ nnz_out, int* __restrict__ cnt_out) {
+                                                             int* __restrict__ nnz_out, int* __restrict__ cnt_out,
+                                                             int* __restrict__ status_out) {
   extern __shared__ unsigned strip[];
   waveal::let_next_kernel_start();
   waveal::wait_for_previous_kernel();
+  if (status_out && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 4) status_out[threadIdx.x] = 0;
   const int h = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const u64* Mh = M + (size_t)h * m_b * wq;
   if ((int)blockIdx.x >= wq) {
@@ -1276,7 +1278,7 @@ waveal_status plan_layout(const waveal_plan_desc* d, PlanLayout* L) {
     return waveal::fail(WAVEAL_ERR_INVALID_ARG, "heads, n_q_blocks and n_kv_blocks must be positive");
   if (d->wave_size < 0 || d->svd_iters < 0 || d->svd_iters > 1000)
     return waveal::fail(WAVEAL_ERR_INVALID_ARG, "wave_size must be >= 0 and svd_iters in [0, 1000]");
-  const int base_mode = d->mode & ~WAVEAL_RING_CUT_LARGEST_GAP;
+  const int base_mode = d->mode & ~(WAVEAL_RING_CUT_LARGEST_GAP | WAVEAL_PLAN_CLEAR_STATUS);
   if (base_mode < WAVEAL_AUTO || base_mode > WAVEAL_STAGE2_ONLY)
     return waveal::fail(WAVEAL_ERR_INVALID_ARG, "unknown mode %d", d->mode);
   if (d->l2_fit_den <= 0 || d->local_den <= 0 || d->l2_fit_num < 0 || d->local_num < 0 || d->min_density_ppm < 0)
@@ -1385,11 +1387,12 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
   WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_plan_head, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
   const dim3 stat_grid(L.wq + (unsigned)((m + kStatRows - 1) / kStatRows), (unsigned)H);
   if (mask_bits) {
-    k_mask_stats<<<stat_grid, kStatThreads, strip_bytes, st>>>(M, Mt, (int)m, (int)n, L.wq, L.wk, nnz, cnt, out->row_nnz, out->col_count);
+    k_mask_stats<<<stat_grid, kStatThreads, strip_bytes, st>>>(M, Mt, (int)m, (int)n, L.wq, L.wk, nnz, cnt, out->row_nnz, out->col_count,
+                                                              (d->mode & WAVEAL_PLAN_CLEAR_STATUS) ? out->dev_status : nullptr);
     WAVEAL_CUDA_OK(cudaGetLastError());
   } else {
     WAVEAL_CUDA_OK(waveal::launch_chained(k_mask_stats, stat_grid, kStatThreads, strip_bytes, st, M, Mt, (int)m, (int)n, L.wq, L.wk,
-                                          nnz, cnt, out->row_nnz, out->col_count));
+                                          nnz, cnt, out->row_nnz, out->col_count, nullptr));
   }
   ++launches;
   PlanParams p{};
@@ -1397,7 +1400,7 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
   // (a wave longer than the head is the whole head; cut to it, row + wave stays far from the end of int)
   p.wave = d->wave_size > 0 ? d->wave_size : sms;
   if (p.wave > (int)m) p.wave = (int)m;
-  p.iters = d->svd_iters; p.mode = d->mode & ~WAVEAL_RING_CUT_LARGEST_GAP;
+  p.iters = d->svd_iters; p.mode = d->mode & ~(WAVEAL_RING_CUT_LARGEST_GAP | WAVEAL_PLAN_CLEAR_STATUS);
   p.ring_cut = (d->mode & WAVEAL_RING_CUT_LARGEST_GAP) ? 1 : 0; p.n_pow2 = L.n_pow2; p.state_in_smem = L.state_in_smem;
   p.seed = d->seed;
   p.kv_bytes = d->kv_bytes_per_head; p.l2_bytes = d->l2_bytes > 0 ? d->l2_bytes : (long long)l2;
@@ -1502,6 +1505,7 @@ extern "C" waveal_status waveal_plan_csr(const waveal_plan_desc* desc, const int
                                          const int32_t* kv_block_indices, void* ws, size_t ws_bytes,
                                          const waveal_plan_out* out, void* cuda_stream) {
   if (!kv_row_ptr || !kv_block_indices) return waveal::fail(WAVEAL_ERR_INVALID_ARG, "index lists are NULL");
+  if (desc && (desc->mode & WAVEAL_PLAN_CLEAR_STATUS)) return waveal::fail(WAVEAL_ERR_INVALID_ARG, "unknown mode %d", desc->mode);
   return plan_common(desc, nullptr, kv_row_ptr, kv_block_indices, ws, ws_bytes, out,
                      static_cast<cudaStream_t>(cuda_stream));
 }

@@ -53,6 +53,14 @@ def test_defaults_and_workspace_query(lib):
     d.n_q_blocks, d.mode = 100, 9
     with pytest.raises(wb.WavealError):
         wb.plan_workspace_bytes(d)
+    for mode in (9 | wb.PLAN_CLEAR_STATUS, 64, -1):
+        d.mode = mode
+        with pytest.raises(wb.WavealError):
+            wb.plan_workspace_bytes(d)
+    d.mode = wb.STAGE1_ONLY | wb.PLAN_CLEAR_STATUS
+    assert wb.plan_workspace_bytes(d) == n
+    assert lib.waveal_plan_csr(ctypes.byref(d), 0x1000, 0x2000, 0x3000, n, ctypes.byref(wb.PlanOut(row_order=0x4000)),
+                               None) == wb.ERR_INVALID_ARG and "mode" in wb.last_error()
 
 
 def test_plan_host_errors_before_any_launch(lib):
@@ -103,11 +111,14 @@ def test_attention_host_errors_before_any_launch(lib):
 @pytest.mark.parametrize("lists", [False, True])
 def test_a_plan_s_status_words_are_cleared_by_the_call(monkeypatch, lists):
     """Not when they are first looked at: that could be inside a graph capture or on another stream."""
-    handed = []
+    handed, modes = [], []
 
     class Lib:
         def waveal_plan_bitmap(self, desc, bits, ws, n, out, stream):
             handed.append(out._obj.dev_status)
+            modes.append(desc._obj.mode)
+            if desc._obj.mode & wb.PLAN_CLEAR_STATUS:
+                ctypes.memset(out._obj.dev_status, 0, 16)
             return wb.OK
 
         def waveal_plan_csr(self, desc, ptr, idx, ws, n, out, stream):
@@ -116,14 +127,15 @@ def test_a_plan_s_status_words_are_cleared_by_the_call(monkeypatch, lists):
 
     monkeypatch.setattr(wb, "load", lambda: Lib())
     monkeypatch.setattr(wb, "_stream", lambda s: None)
-    desc = wb.PlanDesc(heads=3, n_q_blocks=5, n_kv_blocks=70)
+    desc = wb.PlanDesc(heads=3, n_q_blocks=5, n_kv_blocks=70, mode=wb.STAGE2_ONLY | wb.RING_CUT_LARGEST_GAP)
     ws = torch.empty((64,), dtype=torch.uint8)
     if lists:
         res = wb.plan_csr(desc, torch.zeros((16,), dtype=torch.int32), torch.zeros((1,), dtype=torch.int32), workspace=ws)
     else:
         res = wb.plan_bitmap(desc, torch.zeros((3, 5, 2), dtype=torch.int64), workspace=ws)
     assert vars(res)["dev_status"].tolist() == [0] * 4 and res.dev_status.dtype == torch.int32
-    assert handed == [res.dev_status.data_ptr()]
+    assert handed == [res.dev_status.data_ptr()] and desc.mode == wb.STAGE2_ONLY | wb.RING_CUT_LARGEST_GAP
+    assert modes == ([] if lists else [desc.mode | wb.PLAN_CLEAR_STATUS])
     for name in ("row_order", "row_nnz", "skip_flags"):      # (they share an allocation)
         getattr(res, name).fill_(77)
     assert res.dev_status.tolist() == [0] * 4 and (res.row_order == 77).all() and (res.row_nnz == 77).all()

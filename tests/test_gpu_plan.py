@@ -196,18 +196,23 @@ def test_status_words_are_cleared_on_the_plan_s_own_stream(lists):
     idx[idx.numel() - 1] = m + 5                            # (reported, not followed)
     d = wb.plan_desc_default(heads=H, n_q_blocks=m, n_kv_blocks=m, wave_size=16, mode=wb.FORCE_REORDER)
     ws = torch.empty((wb.plan_workspace_bytes(d) + 256,), dtype=torch.uint8, device="cuda")
-    used = [torch.full((2 * H * m + k,), 7, dtype=torch.int32, device="cuda") for k in (1, 5) for _ in range(16)]
-    used += [torch.full((4,), 7, dtype=torch.int32, device="cuda") for _ in range(16)]
+    side = torch.cuda.Stream()
+    plan = (lambda: wb.plan_csr(d, ptr, idx, workspace=ws, stream=side)) if lists else \
+        (lambda: wb.plan_bitmap(d, bm, workspace=ws, stream=side))
+    first = plan()                                          # (loads the kernels, which would wait for the busy stream)
+    used = [torch.full((128,), 7, dtype=torch.int32, device="cuda") for _ in range(8192)]
     torch.cuda.synchronize()
     del used                                                # memory that does not happen to hold zeros
-    side = torch.cuda.Stream()
-    torch.cuda._sleep(200_000_000)                          # 0.1 s on the current stream
-    res = wb.plan_csr(d, ptr, idx, workspace=ws, stream=side) if lists else wb.plan_bitmap(d, bm, workspace=ws, stream=side)
+    done = torch.cuda.Event()
+    torch.cuda._sleep(400_000_000)                          # 0.2 s on the current stream
+    done.record()
+    res = plan()
     with torch.cuda.stream(side):
         st = res.dev_status.tolist()
+    assert not done.query()
     assert st == ([wb.ERR_BAD_MASK, 1, H - 1, m + 5] if lists else [0] * 4)
     torch.cuda.synchronize()
-    assert res.dev_status.tolist() == st
+    assert res.dev_status.tolist() == st and torch.equal(res.row_order, first.row_order)
 
 
 @pytest.mark.parametrize("shape", [(1, 5), (7, 200), (130, 40), (64, 64)])
