@@ -1130,7 +1130,6 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
               WAVEAL_TMEM_ST32(o_row + c0, ov, 0);
             }
           }
-          mx_phase ^= 1u << (g & 3);                           // one flip per arrival on that slot's barrier
           }
           // p' = 2^(s*scale*log2e - m + log2(1 + 2^-9)); P is p' cut to its top 16 bits (one byte
           // permute per pair instead of a conversion).  The extra factor centres the cut's error
@@ -1149,8 +1148,10 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             WAVEAL_TMEM_WAIT_LD32(sv, 0);
             uint32_t pk[G::CH / 2];
             // a pair's results are used LAG pairs later (written so, the compiler keeps more exponentials under way: 1,366 -> 1,347
-            // clk a tile of 128x128 tasks of 256 tiles, 64x64 1,195 -> 1,186; 128x64 blocks lost 0.6 % and use them at once)
+            // clk a tile of 128x128 tasks of 256 tiles, 64x64 1,195 -> 1,186; 128x64 blocks lost 0.6 % and use them at once, and so
+            // does the second launch: four pairs later 64x128 and 64x64 blocks took 0.6 % longer there)
             float x[G::CH];
+            constexpr int kLag = FAST ? G::LAG : 0;
             auto use = [&](int c, float e0, float e1) {
               fadd2(ls4[c & 2], ls4[(c & 2) + 1], ls4[c & 2], ls4[(c & 2) + 1], e0, e1);
               pk[c / 2] = __byte_perm(__float_as_uint(e0), __float_as_uint(e1), 0x7632);
@@ -1163,10 +1164,10 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
                 ffma2(x[c], x[c + 1], __uint_as_float(sv[c]), __uint_as_float(sv[c + 1]), p.sl2, p.sl2, neg_m, neg_m);
                 x[c] = ex2(x[c]); x[c + 1] = ex2(x[c + 1]);
               }
-              if (c >= 2 * G::LAG) use(c - 2 * G::LAG, x[c - 2 * G::LAG], x[c + 1 - 2 * G::LAG]);
+              if (c >= 2 * kLag) use(c - 2 * kLag, x[c - 2 * kLag], x[c + 1 - 2 * kLag]);
             }
 #pragma unroll
-            for (int c = G::CH - 2 * G::LAG; c < G::CH; c += 2) use(c, x[c], x[c + 1]);
+            for (int c = G::CH - 2 * kLag; c < G::CH; c += 2) use(c, x[c], x[c + 1]);
             WAVEAL_TMEM_ST16(s_addr + ch * 16, pk, 0);
           }
           const float l_blk = (ls4[0] + ls4[1]) + (ls4[2] + ls4[3]);
@@ -1181,6 +1182,8 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           __syncwarp();
           if (lane == 0) mbar_arrive(BAR(B_P_FULL + sb * 2 + half));
         }
+        // one flip per arrival on that slot's barrier (before the exponentials it cost 64x128 blocks 2-3 % of the cycles)
+        if (!FAST) mx_phase ^= 1u << (g & 3);
         next_buffer(j);
       }
       if (!ok) break;
