@@ -17,14 +17,15 @@
 //   warp 1      MMA issuer 2: O += P_j V_j (P read from tensor memory, where it lies over the
 //               columns S_j came from), fp32 accumulator in tensor memory.  Two issuing warps:
 //               the waits and ring arithmetic of one run while the other's MMAs execute
-//   warps 2-17  softmax, two teams of eight warps that take the KV blocks of a task in turn;
+//   warps 2-17  softmax, two teams of eight warps that share the KV tiles of a task (by turns, but for the first two
+//               in one kernel);
 //               inside a team a row of S has two owners, one per half of its columns (row max
 //               in the tiles that take one, then exponentials and P in a second read of S,
 //               32 columns at a time).  On every scheduler two warps of each
 //               team are resident, the teams half a block apart, so one team's waits and loads
-//               hide behind the other's arithmetic.  The teams hand each other the
-//               reference max of every row through shared memory; every thread keeps the row
-//               sum of its own columns; O in tensor memory is rescaled only in the second launch, when the
+//               hide behind the other's arithmetic.  Both teams have the reference max of a row
+//               from shared memory, in the first launch once a task, in the second from tile to
+//               tile; every thread keeps the row sum of its own columns; O in tensor memory is rescaled only in the second launch, when the
 //               max grew by more than 2^8; the epilogue adds the four partial sums of a row, normalises
 //               and stores O at the ORIGINAL row (no inverse permutation; 128-row blocks through shared memory)
 // Two launches per call: in the first the row max is taken in the first tile of a task only
@@ -420,7 +421,9 @@ struct Geo {
   static constexpr int CH = 32;                      // S columns a softmax thread holds at a time
   static constexpr int NCH = HC / CH;                // such chunks per thread and block
   // chunks of the exponential loop in line: both at head_dim 64 (128x64 blocks 1,229 -> 1,212 clk a tile, 64x64 1,182 -> 1,150 and
-  // 1,248 -> 1,218 for lists of 256 / 64 blocks), one at head_dim 128 (both: 1,346 -> 1,368 and 1,292 -> 1,302)
+  // 1,248 -> 1,218 for lists of 256 / 64 blocks), one at head_dim 128 (both: 1,346 -> 1,368 and 1,292 -> 1,302).  In line the
+  // kernels spill a few words at the 96 registers there are (28 to 48 bytes stored, 32 to 56 loaded; rolled none), in these
+  // figures too; the second launch's, 4 heads of 256 dense rows, rolled and in line: 128x64 2,606 k and 2,508 k cycles, 64x64 1,324 k and 1,294 k
   static constexpr int UNROLL = D == 64 ? NCH : 1;
   static constexpr int LAG = KB == 1 && D == 64 ? 0 : 4;   // pairs of exponentials under way before the first is used
   static constexpr int CO = D / 2;                   // O columns per epilogue thread
@@ -647,7 +650,9 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   // came before it (the lists, Q, K, V) is there by now: a CTA with a first task of its own (p.direct) begins, and whoever
   // touches the counters or the table waits there.
   if (!p.direct) waveal::wait_for_previous_kernel();
-  const long long t_start = clock64();          // (that kernel's time is not this launch's)
+  // (without a first task of its own that kernel's time is not this launch's; with one the count starts here, and what the
+  // CTA still waits for that kernel is in it)
+  const long long t_start = clock64();
 
   // Every role walks the same sequence of tasks (query blocks) and, inside a task, of KV blocks;
   // block number g (counted over the CTA's whole life) uses S buffer g mod 3, K stage g mod NKS
@@ -928,17 +933,19 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     }
   } else {
     // ============================================================== softmax / epilogue
-    // Sixteen warps: two teams take the KV blocks of a task in turn (team = block index mod 2),
-    // and inside a team a row of S has two owners, one per half of its columns (a warp can reach
+    // Sixteen warps: two teams share the KV tiles of a task (which tile is whose: below), and
+    // inside a team a row of S has two owners, one per half of its columns (a warp can reach
     // only the 32 tensor-memory lanes of its quadrant, so the two owners of a row sit in warps
     // four apart).  Four softmax warps per scheduler instead of two: the loop is bound by
-    // instruction issue and latency, and twice the warps hide twice the latency.  The owners
-    // of a row share its reference max (exchanged through shared memory in the blocks that
-    // take one); each keeps the sum of its own columns; P of a column half is written over the
-    // first columns of that half's own S columns and released with its own barrier.  The two
-    // teams hand each other the running reference of each row (shared memory + one mbarrier
-    // per lane quadrant and block parity), because both accumulate into the same O.  The
-    // epilogue adds the four partial sums of a row.
+    // instruction issue and latency, and twice the warps hide twice the latency.  Each owner
+    // keeps the sum of its own columns; P of a column half is written over the first columns of
+    // that half's own S columns and released with its own barrier.  Both teams accumulate into the
+    // same O, so they need the same reference max of a row.  First launch: the two owners of the row in
+    // the task's first tile leave the maxima of their halves in shared memory, and they and the
+    // other team, at its first tile, wait at one mbarrier (a lane quadrant's, four slots).  Second launch:
+    // the two owners of a row exchange their maxima in every tile, and the team of a tile leaves the
+    // running reference for that of the next (an mbarrier per lane quadrant and tile count mod 4).
+    // The epilogue adds the four partial sums of a row.
     const int sw = warp - kSoftmaxWarp0;       // 0..15
     const int quad = warp & 3;                 // tensor-memory lane quadrant this warp may access
     const int team = (sw >> 2) & 1;            // owns every second tile (by the tile's number over the CTA's life, or as kTwoFirst says)
@@ -972,8 +979,9 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       const Task tk = tasks[slot];
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR(B_TASK_EMPTY + slot));
-      // (here and not behind the stores: by now the copy engine has read them.  The next task is published before the one
-      // whose Q needs this tile, so nobody waits for this in a circle)
+      // (here and not behind the stores: what came after them, the second launch's list, does not wait for the copy engine.  The
+      // next task is mostly published by then, so lane 0 waits for the rest of its reads.  It is published before the
+      // one whose Q needs this tile, so nobody waits for this in a circle)
       if (G::STAGED && storing) {
         if (lane == 0) { bulk_wait_read(); mbar_arrive(BAR(B_Q_EMPTY + ((o_it - 1) & 1))); }
         storing = false;
@@ -1296,8 +1304,8 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     tc_fence_after();
     tmem_dealloc(tmem_base, G::TMEM_COLS);
   }
-  // SM cycles since the launch before this one ended: the largest over the grid is the launch's length in cycles,
-  // a figure that does not depend on the clock the GPU happened to run at
+  // SM cycles since the CTA's first task could start (t_start): the largest over the grid is the launch's length in
+  // cycles, a figure that does not depend on the clock the GPU happened to run at
   if (tid == 0) {
     const long long dt = clock64() - t_start;
     atomicMax(&p.ws[p.redo_pass ? 5 : 4], (int)(dt > 0x7fffffffll ? 0x7fffffffll : dt));
