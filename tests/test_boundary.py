@@ -133,7 +133,8 @@ def test_a_plan_s_status_words_are_cleared_by_the_call(monkeypatch, lists):
         res = wb.plan_csr(desc, torch.zeros((16,), dtype=torch.int32), torch.zeros((1,), dtype=torch.int32), workspace=ws)
     else:
         res = wb.plan_bitmap(desc, torch.zeros((3, 5, 2), dtype=torch.int64), workspace=ws)
-    assert vars(res)["dev_status"].tolist() == [0] * 4 and res.dev_status.dtype == torch.int32
+    assert handed[0] is not None and ctypes.string_at(handed[0], 16) == bytes(16)          # (before anyone looks)
+    assert res.dev_status.tolist() == [0] * 4 and res.dev_status.dtype == torch.int32
     assert handed == [res.dev_status.data_ptr()] and desc.mode == wb.STAGE2_ONLY | wb.RING_CUT_LARGEST_GAP
     assert modes == ([] if lists else [desc.mode | wb.PLAN_CLEAR_STATUS])
     for name in ("row_order", "row_nnz", "skip_flags"):      # (they share an allocation)
