@@ -190,12 +190,12 @@ size_t waveal_noalloc_max_rows(void);
  * through the common exit (no trap, no fault, the context stays usable); O is then undefined.
  * The next call on the same workspace works as usual. */
 #define WAVEAL_ATTN_SELFTEST_LOST_TILE 256
-/* 64-row query blocks run in a 128-row tensor-core tile.  By default two query blocks of a head
- * with the very same list of KV blocks share one tile, which halves their cost: rows that select
+/* 64-row query blocks: by default two of a head with the very same list of KV blocks share the K and V
+ * tiles of that list, which are loaded once for both: rows that select
  * every KV block pair up wherever they stand in the execution order (1st with 2nd, 3rd with 4th
  * such row; the pair runs at the position of its first row), other rows when they stand at
  * positions 2i and 2i+1 (Stage 2 of the plan puts rows of equal count side by side).  The results
- * are the same bits as without sharing (the two blocks never interact: a row of the tile only
+ * are the same bits as without sharing (the two blocks never interact: a row only
  * sees its own row of Q).  This flag switches the sharing off (comparison runs). */
 #define WAVEAL_ATTN_NO_ROW_PAIRING 2
 
@@ -213,7 +213,8 @@ typedef struct waveal_attn_desc {
 /* Bytes of device workspace waveal_bsattn_fwd needs: 32 bytes of counters (int32 words: ticket
  * counter, abort flag, number of tasks computed twice, ticket counter of the second launch,
  * length of the first and of the second launch in SM cycles = the longest that a thread block ran
- * after its first task could start, number of query-block pairs that shared a tile, number of 128-row x 128-key tiles the call runs),
+ * after its first task could start, number of query-block pairs that shared their tiles, number of 128-key tiles of K and V that the
+ * call went through, those of a pair counted once),
  * 8 bytes per (head, query block) for the list of tasks to compute again and
  * 32 bytes per (head, query block) for the table that maps a ticket to its task.  The counters
  * are live state of the call (tickets are drawn from them): calls that may overlap on the GPU

@@ -8,10 +8,10 @@
 // SM, take tickets from a global counter, so a freed SM starts the next row of the list at
 // once - the streaming "wave" behaviour of Section 2.3 that the schedule is built for.
 //
-// Structure of one CTA (640 threads):
+// Structure of one CTA (640 threads; the first launch of 64-row blocks has a kernel of its own, k_bsattn_fwd_rows64):
 //   warp 0      producer: takes tickets, publishes tasks, issues TMA loads of the Q tile and of the K
 //               tiles (128-byte-swizzled slabs) into shared-memory rings, as far ahead as the rings allow
-//   warp 19     requests the V tiles (one warp for both streams was the limit of the 64-row kernels)
+//   warp 19     requests the V tiles (a box costs the warp that requests it ~150 clk)
 //   warp 18     MMA issuer 1: S_j = Q K_j^T (operands in shared memory) into one of three S
 //               buffers in tensor memory, up to three blocks ahead of the softmax
 //   warp 1      MMA issuer 2: O += P_j V_j (P read from tensor memory, where it lies over the
@@ -38,6 +38,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cmath>
+#include <type_traits>
 #include "host_common.h"
 
 namespace {
@@ -150,6 +151,44 @@ __device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, u
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
       ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
+}
+
+// D[tmem] (+)= A[smem] * B[smem] for 64 rows of A: row m of D lies in lanes m and 64 + m, the first half of the N columns in the
+// lower lanes, the second half in the upper ones
+// N (4 or 8) of them along K, then the commit of all that this thread has issued.  A and B are a step further each time, and a
+// jump further from the fifth on.  One election for all: with one for each, the issuing warp's own instructions took
+// longer than the products.
+template <int N, int A_STEP, int A_JUMP, int B_STEP, int B_JUMP>
+__device__ __forceinline__ void umma_ws_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate, uint32_t bar) {
+  static_assert(N == 4 || N == 8, "four products or eight");
+#define WAVEAL_WS(a, b, p) "@e tcgen05.mma.ws.cta_group::1.kind::f16 [%0], " a ", " b ", %3, " p ";\n\t"
+  if constexpr (N == 8)
+    asm volatile(
+        "{\n\t.reg .b32 rx;\n\t.reg .pred e, p, t;\n\t.reg .b64 a, b;\n\t"
+        "elect.sync rx|e, 0xFFFFFFFF;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 t, %3, %3;\n\t"
+        WAVEAL_WS("%1", "%2", "p")
+        "add.s64 a, %1, %6;\n\tadd.s64 b, %2, %8;\n\t" WAVEAL_WS("a", "b", "t")
+        "add.s64 a, %1, 2 * %6;\n\tadd.s64 b, %2, 2 * %8;\n\t" WAVEAL_WS("a", "b", "t")
+        "add.s64 a, %1, 3 * %6;\n\tadd.s64 b, %2, 3 * %8;\n\t" WAVEAL_WS("a", "b", "t")
+        "add.s64 a, %1, %7;\n\tadd.s64 b, %2, %9;\n\t" WAVEAL_WS("a", "b", "t")
+        "add.s64 a, %1, %7 + %6;\n\tadd.s64 b, %2, %9 + %8;\n\t" WAVEAL_WS("a", "b", "t")
+        "add.s64 a, %1, %7 + 2 * %6;\n\tadd.s64 b, %2, %9 + 2 * %8;\n\t" WAVEAL_WS("a", "b", "t")
+        "add.s64 a, %1, %7 + 3 * %6;\n\tadd.s64 b, %2, %9 + 3 * %8;\n\t" WAVEAL_WS("a", "b", "t")
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(bar), "n"(A_STEP >> 4), "n"(A_JUMP >> 4), "n"(B_STEP >> 4), "n"(B_JUMP >> 4)
+        : "memory");
+  else
+    asm volatile(
+        "{\n\t.reg .b32 rx;\n\t.reg .pred e, p, t;\n\t.reg .b64 a, b;\n\t"
+        "elect.sync rx|e, 0xFFFFFFFF;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 t, %3, %3;\n\t"
+        WAVEAL_WS("%1", "%2", "p")
+        "add.s64 a, %1, %6;\n\tadd.s64 b, %2, %7;\n\t" WAVEAL_WS("a", "b", "t")
+        "add.s64 a, %1, 2 * %6;\n\tadd.s64 b, %2, 2 * %7;\n\t" WAVEAL_WS("a", "b", "t")
+        "add.s64 a, %1, 3 * %6;\n\tadd.s64 b, %2, 3 * %7;\n\t" WAVEAL_WS("a", "b", "t")
+        "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%5];\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "r"(bar), "n"(A_STEP >> 4), "n"(B_STEP >> 4)
+        : "memory");
+#undef WAVEAL_WS
 }
 
 // two fp32 operations per instruction (register pairs)
@@ -420,10 +459,10 @@ struct Geo {
   static constexpr int HC = BK / 2;                  // S columns of a row one softmax thread owns (a row has two owners)
   static constexpr int CH = 32;                      // S columns a softmax thread holds at a time
   static constexpr int NCH = HC / CH;                // such chunks per thread and block
-  // chunks of the exponential loop in line: both at head_dim 64 (128x64 blocks 1,229 -> 1,212 clk a tile, 64x64 1,182 -> 1,150 and
-  // 1,248 -> 1,218 for lists of 256 / 64 blocks), one at head_dim 128 (both: 1,346 -> 1,368 and 1,292 -> 1,302).  In line the
-  // kernels spill a few words at the 96 registers there are (28 to 48 bytes stored, 32 to 56 loaded; rolled none), in these
-  // figures too; the second launch's, 4 heads of 256 dense rows, rolled and in line: 128x64 2,606 k and 2,508 k cycles, 64x64 1,324 k and 1,294 k
+  // chunks of the exponential loop in line: both at head_dim 64 (128x64 blocks 1,229 -> 1,212 clk a tile), one at head_dim 128
+  // (both: 1,346 -> 1,368).  In line the kernels spill a few words at the 96 registers there are (28 to 48 bytes stored, 32 to
+  // 56 loaded; rolled none), in these figures too; the second launch's, 4 heads of 256 dense rows, rolled and in line: 128x64
+  // 2,606 k and 2,508 k cycles, 64x64 1,324 k and 1,294 k
   static constexpr int UNROLL = D == 64 ? NCH : 1;
   static constexpr int LAG = KB == 1 && D == 64 ? 0 : 4;   // pairs of exponentials under way before the first is used
   static constexpr int CO = D / 2;                   // O columns per epilogue thread
@@ -557,8 +596,7 @@ __device__ __noinline__ void mask_scores(uint32_t s_addr, int valid) {
 }
 
 // a task for the second launch, unless another warp has listed it already; the blocks of a pair are computed again one by one
-// (out of line for 64-row blocks, 18.75 M -> 18.35 M cycles on 8 heads of 1536 rows; for 128-row blocks in line, 521 k -> 506 k
-// on 5 heads of 256 rows: a call there makes the compiler spill)
+// (in line for 128-row blocks: 521 k -> 506 k cycles on 5 heads of 256 rows, a call there makes the compiler spill)
 __device__ __forceinline__ void list_task(int* ws, int* listed, int task_no, int h, int row, int row2) {
   if (atomicExch(listed, task_no) == task_no) return;
   waveal::wait_for_previous_kernel();      // (which clears the count: a first task may end before it)
@@ -566,9 +604,6 @@ __device__ __forceinline__ void list_task(int* ws, int* listed, int task_no, int
   ws[8 + 2 * e] = h;
   ws[9 + 2 * e] = row;
   if (row2 >= 0) { ws[10 + 2 * e] = h; ws[11 + 2 * e] = row2; }
-}
-__device__ __noinline__ void list_task_call(int* ws, int* listed, int task_no, int h, int row, int row2) {
-  list_task(ws, listed, task_no, h, row, row2);
 }
 
 template <int BLOCK, int D, bool FAST>
@@ -580,6 +615,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   // two blocks of a tile lie next to each other in memory (for 128-key blocks they equal tmK / tmV).
   // tmO: O in boxes of 32 rows and half of head_dim, what a warp stores (128-row blocks only)
   using G = Geo<BLOCK, D>;
+  static_assert(BLOCK == 128 || !FAST, "the first launch of 64-row blocks is k_bsattn_fwd_rows64");
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = smem_u32(smem);
@@ -964,8 +1000,8 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     // and 2 4 6 ...  By turns from the first tile on, the second one's P waits for the end of that epilogue, and the P V of
     // the third, long ready, for it.  First launch of 128-row blocks at head_dim 64: tasks of 16 / 24 / 256 tiles 1,292 -> 1,266 /
     // 1,246 -> 1,228 / 1,160 -> 1,151 clk a tile.  (At head_dim 128 tasks of 17 tiles gained 2 %, but every form of it made the
-    // compiler's code for the loop over the tiles slower, 1,366 -> 1,404 clk a tile of long tasks, and so it did for 64x64
-    // blocks, 1,257 -> 1,297.  The second launch hands a reference on from tile to tile.)
+    // compiler's code for the loop over the tiles slower, 1,366 -> 1,404 clk a tile of long tasks.  The second launch hands a
+    // reference on from tile to tile.)
     constexpr bool kTwoFirst = FAST && D == 64 && G::KB == 1;
     uint32_t g0 = 0;                           // tiles before this task
     int first_team = 0;                        // kTwoFirst: the team of the task's first tile
@@ -1034,9 +1070,8 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           // sum of the exponentials they produce: if it ever reaches 2^60 the task is put on a list and computed again
           // by the second launch, which takes the max of every tile (the rule of the paper's online softmax).
           // One tile and one meeting of all who need its max, and nothing of the rule for a max that grows in this kernel
-          // (no rescale of O, no hand-over from tile to tile): against the code with both in it, and two such tiles for
-          // 64-row blocks, 64x128 rows of 64 / 256 blocks 1,485 -> 1,383 / 1,359 -> 1,290 clk a tile, 64x64 1,326 -> 1,260,
-          // 128x128 tasks of 38 / 256 tiles 1,520 -> 1,492 / 1,385 -> 1,363, 128x64 1,311 -> 1,272.  A max over 32 keys only
+          // (no rescale of O, no hand-over from tile to tile): against the code with both in it 128x128 tasks of 38 / 256
+          // tiles 1,520 -> 1,492 / 1,385 -> 1,363 clk a tile, 128x64 1,311 -> 1,272.  A max over 32 keys only
           // would save another 1-4 %, but scores that spread by 40 nats inside a tile then need the second launch.
           float m_new;
           if constexpr (FAST) {
@@ -1156,7 +1191,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
             WAVEAL_TMEM_WAIT_LD32(sv, 0);
             uint32_t pk[G::CH / 2];
             // a pair's results are used LAG pairs later (written so, the compiler keeps more exponentials under way: 1,366 -> 1,347
-            // clk a tile of 128x128 tasks of 256 tiles, 64x64 1,195 -> 1,186; 128x64 blocks lost 0.6 % and use them at once, and so
+            // clk a tile of 128x128 tasks of 256 tiles; 128x64 blocks lost 0.6 % and use them at once, and so
             // does the second launch: four pairs later 64x128 and 64x64 blocks took 0.6 % longer there)
             float x[G::CH];
             constexpr int kLag = FAST ? G::LAG : 0;
@@ -1288,10 +1323,8 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       // before O_FULL) or if a result is not finite: with sums of up to 2^60 O overflows from |V| = 2^67 on, and a
       // first tile whose scores are all -inf leaves no reference.  (Where V itself holds an inf or NaN the second
       // launch finds the same again.)  Whichever of the epilogue's warps sees it first writes the entry.
-      if (FAST && (__any_sync(0xffffffffu, bad) || redo_flag[rslot] == task_no) && lane == 0) {
-        if constexpr (G::KB == 2) list_task_call(p.ws, &redo_listed[rslot], task_no, tk.h, tk.row, tk.row2);
-        else list_task(p.ws, &redo_listed[rslot], task_no, tk.h, tk.row, -1);
-      }
+      if (FAST && (__any_sync(0xffffffffu, bad) || redo_flag[rslot] == task_no) && lane == 0)
+        list_task(p.ws, &redo_listed[rslot], task_no, tk.h, tk.row, -1);
     }
   }
 
@@ -1309,6 +1342,620 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   if (tid == 0) {
     const long long dt = clock64() - t_start;
     atomicMax(&p.ws[p.redo_pass ? 5 : 4], (int)(dt > 0x7fffffffll ? 0x7fffffffll : dt));
+  }
+}
+
+// ------------------------------------------------------------------ 64-row query blocks, first launch
+//
+// A lone 64-row block leaves half of a 128-row product empty, and an ordinary product of 64 rows takes as long as one of 128
+// (64 clk for N = 128, K = 16).  tcgen05.mma.ws with M = 64 takes 48.7 clk: it lays row m of the result over lanes m and 64 + m,
+// half of the columns in each, so that all of tensor memory's lanes work and the softmax has 64 columns a lane.  What bounds
+// it is shared memory: A and B are read anew for every product, 6 KB at 128 bytes a clock (N = 256 takes 80).  One item, a block of
+// 64 rows against a tile of 128 keys, is 8 + 8 products = 779 clk at head_dim 128 and 4 + 8 = 484 at 64; P goes through
+// shared memory too (as an operand in tensor memory it would have to lie in both halves of the lanes).  64 KB of K and V an item are
+// 850 clk at the 77 bytes per clock and SM that all SMs draw from L2 together at the full clock.
+// Against the 128-row products (which a lone block half filled) with the same softmax: 8 heads of 1,536 rows of the LTX recipe, head_dim 128,
+// 1,319 -> 1,110 clk a tile (907 an item; two blocks that share the tiles of one list take two items each), 11.2 -> 9.4 ms;
+// 8 heads of 768 rows, head_dim 64, 1,165 -> 990; 8 heads of 317 rows of 9 or 10 tiles 1,773 -> 1,400, 241 -> 150 us.
+//
+// At this pace the issuing warps' and the loaders' own instructions count (~10 clk each beside four softmax warps a scheduler):
+//  - an item has ONE barrier on which its product waits (the tile's bytes and the softmax group's arrivals together) and ONE that it
+//    completes, by item number mod 8; loaders and softmax look at the same ones.  With barriers by ring stage and by buffer (two
+//    waits and two commits a product) an item took 1,020 clk instead of 919;
+//  - the products of an item are one block of instructions under one election (one for each: 1,286 -> 1,076);
+//  - four loaders, every second K and every second V tile each: a box of 64 rows costs its warp ~150 clk to request, a
+//    tile of two blocks is four (two loaders: 1,076, four: 1,020).
+//
+// Softmax: four groups of four warps; item q (counted over the CTA's life) belongs to group and S buffer q mod 4 and P buffer
+// q mod 3.  A lane has 64 columns of one row, lanes m and 64 + m the two halves of a tile.  The S buffer is free as soon as its scores are
+// in registers.  The accumulator has two copies, by task, so that the next task's products do not wait for this one's epilogue,
+// which the group of a block's last item runs while the others go on.
+// Pairs: two blocks with the very same list are items 2 i and 2 i + 1 of tile i, each with an accumulator of its own.  Everything a row
+// sees is as it would be alone: the products in the same order, a reference from the same first 128 keys, and the same
+// sums, which a lone block has by tile mod 4 (its groups) and a pair's groups keep two of.
+constexpr int kThreads64 = 704, kLoadWarps64 = 20;   // 22 warps: those of the kernel above and two more loaders
+
+template <int D>
+struct Geo64 {
+  static constexpr int BQ = 64, BK = 128;            // a KV tile is 128 keys: two consecutive entries of the row's list
+  static constexpr int SLABS = D / 64;               // 128-byte column slabs of a Q/K/V tile
+  static constexpr int Q_BYTES = SLABS * BQ * 128;   // one query block
+  static constexpr int KV_SLAB_BYTES = BK * 128;
+  static constexpr int TILE_BYTES = SLABS * KV_SLAB_BYTES;     // K tile
+  static constexpr int P_PANEL_BYTES = BQ * 128;     // P of 64 rows and 64 keys
+  static constexpr int P_BYTES = 2 * P_PANEL_BYTES;
+  static constexpr int NQ = 2;                       // query blocks: two of a pair, or this task's and the next one's
+  static constexpr int NP = 3;                       // P buffers
+  static constexpr int NKS = D == 128 ? 2 : 4;       // K tiles
+  static constexpr int NVS = NKS;                    // V tiles
+  static constexpr int NG = 4;                       // softmax groups of four warps, each with its own S buffer
+  static constexpr int CO = D / 2;                   // O columns per epilogue thread
+  static constexpr int LAG = 4;
+  static constexpr int NSL = 3;                      // slots by task for what the groups leave each other
+  static constexpr int OFF_Q = 0;
+  static constexpr int OFF_P = OFF_Q + NQ * Q_BYTES;
+  static constexpr int OFF_K = OFF_P + NP * P_BYTES;
+  static constexpr int OFF_V = OFF_K + NKS * TILE_BYTES;
+  static constexpr int OFF_BAR = OFF_V + NVS * TILE_BYTES;
+  static constexpr int N_BAR = 4 + 2 * NQ + 4 * 8 + 4 + 4 + 2 + NSL * 4 + NSL * 2;
+  static constexpr int OFF_TASK = OFF_BAR + ((N_BAR * 8 + 15) / 16) * 16;
+  static constexpr int OFF_MX = OFF_TASK + 2 * (int)sizeof(Task);             // [slot][block][128] largest score of a half row
+  static constexpr int OFF_EX = OFF_MX + NSL * 2 * 128 * 4;                   // [slot][block][tile mod 4][128] sums
+  static constexpr int OFF_MISC = OFF_EX + NSL * 2 * 4 * 128 * 4;
+  static constexpr int SMEM_BYTES = OFF_MISC + 48 + 1024;   // + slack for 1024-byte alignment
+  static_assert(SMEM_BYTES <= 232448, "shared memory of a CTA");
+  // tensor memory: an S buffer of 64 columns per softmax group, then two sets of output accumulators (by task) for two blocks
+  static constexpr uint32_t S_STRIDE = 64, O_COL = NG * 64, O_STRIDE = 64, TMEM_COLS = 512;
+};
+
+// One K or V tile of a task into its ring stage (called by a whole warp); see load_kv_tile.  done: the product that read the
+// stage's tile before this one (an item, or -1); item: the first that reads this one, of `blocks`.
+template <class G, bool IS_K>
+__device__ __forceinline__ bool load_tile64(const Ctx& ctx, const AttnParams& p, const Task& tk, bool dropped, int j, int lane,
+                                            uint32_t sbase, uint32_t stage, uint32_t bar_ready0, uint32_t bar_done0, int done,
+                                            int item, int blocks, const CUtensorMap* tm, const CUtensorMap* tm2, int& chunk_base,
+                                            int& my_idx) {
+  if (2 * j >= chunk_base + 32) {
+    chunk_base = (2 * j) & ~31;
+    my_idx = chunk_base + lane < tk.len ? p.kv_idx[tk.lo + chunk_base + lane] : 0;
+    if (my_idx < 0 || my_idx >= p.n_b) {             // malformed list: report it and stay in range
+      if (IS_K && p.dev_status && atomicCAS(p.dev_status, 0, WAVEAL_ERR_BAD_MASK) == 0) {
+        p.dev_status[1] = 30; p.dev_status[2] = tk.h; p.dev_status[3] = my_idx;
+      }
+      my_idx = 0;
+    }
+  }
+  const int sl = lane % G::SLABS, e = lane / G::SLABS, nblk = min(2, tk.len - 2 * j);
+  const int blk0 = __shfl_sync(0xffffffffu, my_idx, 2 * j - chunk_base), blk1 = __shfl_sync(0xffffffffu, my_idx, 2 * j + 1 - chunk_base);
+  if (done >= 0 && !warp_wait(ctx, bar_done0 + 8u * (done & 7), (done >> 3) & 1, IS_K ? 3 : 4)) return false;
+  if (dropped) return true;
+  const uint32_t b_ready = bar_ready0 + 8u * (item & 7);
+  if (lane == 0) {
+    mbar_expect_tx(b_ready, (uint32_t)nblk * G::SLABS * 64 * 128);
+    if (blocks == 2) mbar_arrive(bar_ready0 + 8u * ((item + 1) & 7));      // (of a pair; its two products are issued in order)
+  }
+  __syncwarp();
+  // one lane per box: lane e*SLABS + s requests slab s of block e; two blocks that follow each other in memory come as one box
+  const uint32_t dst = sbase + (IS_K ? G::OFF_K : G::OFF_V) + stage * G::TILE_BYTES + sl * G::KV_SLAB_BYTES;
+  if (nblk == 2 && blk1 == blk0 + 1) {
+    if (e == 0) tma_load_3d(dst, tm2, sl * 64, blk0 * 64, tk.h, b_ready);
+  } else if (e < nblk) {
+    tma_load_3d(dst + e * 64 * 128, tm, sl * 64, (e ? blk1 : blk0) * 64, tk.h, b_ready);
+  }
+  return true;
+}
+
+// Every second tile of all tasks, by the tile's number over the CTA's life
+template <class G, bool IS_K>
+struct TileLoader {
+  static constexpr int NST = IS_K ? G::NKS : G::NVS, NOWN = NST / 2;       // stages in all, and of this warp
+  uint32_t odd, base = 0;                            // tiles before this task
+  int q0 = 0;                                        // items before this task
+  int item[NOWN], done[NOWN];                        // of the tiles in this warp's stages, oldest first: first and last item
+  __device__ __forceinline__ explicit TileLoader(uint32_t o) : odd(o) {
+#pragma unroll
+    for (int i = 0; i < NOWN; ++i) item[i] = done[i] = -1;
+  }
+  template <class F>
+  __device__ __forceinline__ bool task(const Ctx& ctx, const AttnParams& p, const Task& tk, int lane, uint32_t sbase, uint32_t bar_ready0,
+                                       uint32_t bar_done0, const CUtensorMap* tm, const CUtensorMap* tm2, bool drop_first, F before) {
+    const int blocks = tk.row2 >= 0 ? 2 : 1;
+    int chunk_base = -64, my_idx = 0;
+#pragma unroll 1
+    for (int j = (int)((base ^ odd) & 1); j < tk.n; j += 2) {
+      before(j);
+      const int it = q0 + j * blocks;
+      if (!load_tile64<G, IS_K>(ctx, p, tk, drop_first && j == 0, j, lane, sbase, (base + (uint32_t)j) % NST, bar_ready0, bar_done0,
+                                done[0], it, blocks, tm, tm2, chunk_base, my_idx))
+        return false;
+#pragma unroll
+      for (int i = 0; i + 1 < NOWN; ++i) { item[i] = item[i + 1]; done[i] = done[i + 1]; }
+      item[NOWN - 1] = it;
+      done[NOWN - 1] = it + blocks - 1;
+    }
+    if (tk.n > 0) { base += (uint32_t)tk.n; q0 += tk.n * blocks; }
+    return true;
+  }
+  // leave no bulk copy in flight into this CTA's shared memory (bounded)
+  __device__ __forceinline__ void drain(const AttnParams& p, uint32_t bar_ready0) const {
+#pragma unroll
+    for (int i = 0; i < NOWN; ++i)
+      if (item[i] >= 0) {
+        const long long t0 = clock64();
+        while (!mbar_try_wait(bar_ready0 + 8u * (item[i] & 7), (item[i] >> 3) & 1) && clock64() - t0 < p.wait_limit / 4) {}
+      }
+  }
+};
+
+template <int D>
+__global__ void __launch_bounds__(kThreads64, 1)
+k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                    const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmK2,
+                    const __grid_constant__ CUtensorMap tmV2, const AttnParams p) {
+  // tmK2 / tmV2: K and V in boxes of 128 rows, for two blocks of a tile that lie next to each other in memory
+  using G = Geo64<D>;
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  const uint32_t sbase = smem_u32(smem);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // provably warp-uniform role index
+  waveal::let_next_kernel_start();
+
+  const uint32_t bar0 = sbase + G::OFF_BAR;
+  auto BAR = [&](int i) { return bar0 + 8u * (uint32_t)i; };
+  constexpr int B_TASK_FULL = 0, B_TASK_EMPTY = 2, B_Q_FULL = 4, B_Q_EMPTY = B_Q_FULL + G::NQ, B_QK_READY = B_Q_EMPTY + G::NQ,
+                B_QK_DONE = B_QK_READY + 8, B_PV_READY = B_QK_DONE + 8, B_PV_DONE = B_PV_READY + 8, B_O_FULL = B_PV_DONE + 8,
+                B_O_FREE = B_O_FULL + 4, B_FINAL = B_O_FREE + 4,
+                B_MX = B_FINAL + 2, B_EX = B_MX + G::NSL * 4;
+  static_assert(B_EX + G::NSL * 2 <= G::N_BAR, "barrier count");
+  Task* tasks = reinterpret_cast<Task*>(smem + G::OFF_TASK);
+  volatile float* mx = reinterpret_cast<volatile float*>(smem + G::OFF_MX);
+  float* ex = reinterpret_cast<float*>(smem + G::OFF_EX);
+  uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(smem + G::OFF_MISC);
+  volatile int* abort_smem = reinterpret_cast<volatile int*>(smem + G::OFF_MISC + 4);
+  // [slot]: number (from 1) of the last task that a tile wants computed again, and of the last one listed for it
+  volatile int* redo_flag = reinterpret_cast<volatile int*>(smem + G::OFF_MISC + 8);
+  int* redo_listed = reinterpret_cast<int*>(smem + G::OFF_MISC + 8 + G::NSL * 4);
+  Ctx ctx{bar0, abort_smem, p.ws, p.dev_status, p.wait_limit};
+
+  if (tid == 0) {
+    // a task is read by the three other loaders, the two MMA issuers and the sixteen softmax warps
+    for (int i = 0; i < 2; ++i) { mbar_init(BAR(B_TASK_FULL + i), 1); mbar_init(BAR(B_TASK_EMPTY + i), 21); }
+    for (int i = B_Q_FULL; i < B_QK_READY; ++i) mbar_init(BAR(i), 1);       // one load, one commit
+    for (int i = 0; i < 8; ++i) {
+      mbar_init(BAR(B_QK_READY + i), 5);                                    // the K tile, and the group's four warps have read their S buffer
+      mbar_init(BAR(B_PV_READY + i), 5);                                    // the V tile, and P by the group's four warps
+      mbar_init(BAR(B_QK_DONE + i), 1);
+      mbar_init(BAR(B_PV_DONE + i), 1);
+    }
+    for (int i = 0; i < 4; ++i) { mbar_init(BAR(B_O_FULL + i), 1); mbar_init(BAR(B_O_FREE + i), 4); }
+    for (int i = 0; i < 2; ++i) mbar_init(BAR(B_FINAL + i), 1);
+    for (int i = 0; i < G::NSL * 4; ++i) mbar_init(BAR(B_MX + i), 2);       // the two warps that have a row's first tile
+    for (int i = 0; i < G::NSL * 2; ++i) mbar_init(BAR(B_EX + i), 8);       // all warps that have sums of a row
+    *abort_smem = 0;
+    for (int i = 0; i < G::NSL; ++i) { redo_flag[i] = 0; redo_listed[i] = 0; }
+    fence_mbar_init();
+    fence_proxy_async();
+  }
+  if (warp == kPvWarp) {
+    tmem_alloc(smem_u32(tmem_holder), G::TMEM_COLS);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_holder, 0);
+  waveal::wait_for_previous_kernel();
+  const long long t_start = clock64();
+
+  // every role walks the same sequence of tasks and, inside a task, of items
+  if (warp == kProducerWarp) {
+    // ============================================================== producer: tickets, Q, every second K tile
+    if (lane == 0) { prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmV); prefetch_tmap(&tmK2); prefetch_tmap(&tmV2); }
+    uint32_t task_it = 0, q_it = 0, q_armed = 0, q_parity = 0;
+    TileLoader<G, true> k_tiles{0};
+    int n_tiles = 0, n_pairs = 0;        // words 7 and 6 of the workspace
+    bool ok = true;
+    auto draw = [&](long long& t_out) -> Task {
+      for (;;) {
+        long long t = 0;
+        if (lane == 0)                   // (volatile: another SM raises the flag while this kernel runs)
+          t = (*reinterpret_cast<volatile int*>(&p.ws[1]) != 0) ? p.total_tasks : (long long)(unsigned)atomicAdd(&p.ws[0], 1);
+        t = __shfl_sync(0xffffffffu, t, 0);
+        t_out = t;
+        Task tk{};
+        if (t >= p.total_tasks) { tk.n = -1; return tk; }
+        const uint4* e = reinterpret_cast<const uint4*>(p.table + t);
+        const uint4 a = e[0], b = e[1];
+        tk.h = (int)a.x; tk.row = (int)a.y; tk.lo = (int)a.z; tk.n = (int)a.w; tk.tail_valid = (int)b.x; tk.len = (int)b.y;
+        tk.row2 = (int)b.z;
+        if (tk.n != kAbsorbed) return tk;             // (else the second block of a pair: computed with its partner)
+      }
+    };
+    constexpr int kDrawAhead = 3;        // tiles before the task's last K loads: the round trips of the ticket hide behind the ring
+    long long t = 0, t_next = 0;
+    Task tk_next = draw(t_next);
+    while (ok) {
+      const Task tk = tk_next;
+      t = t_next;
+      bool drawn = false;
+      const uint32_t slot = task_it & 1, ph = (task_it >> 1) & 1;
+      ok = warp_wait(ctx, BAR(B_TASK_EMPTY + slot), ph ^ 1, 1);
+      if (!ok) break;
+      if (lane == 0) {
+        tasks[slot] = tk;
+        mbar_arrive(BAR(B_TASK_FULL + slot));
+      }
+      ++task_it;
+      if (tk.n < 0) break;
+      if (tk.n <= kDrawAhead) { tk_next = draw(t_next); drawn = true; }
+      if (tk.n == 0) continue;
+      const int blocks = tk.row2 >= 0 ? 2 : 1;
+      n_tiles += tk.n;
+      n_pairs += blocks - 1;
+      for (int b = 0; b < blocks && ok; ++b, ++q_it) {
+        const uint32_t qb = q_it % G::NQ, q_ph = (q_it / G::NQ) & 1;
+        ok = warp_wait(ctx, BAR(B_Q_EMPTY + qb), q_ph ^ 1, 2);
+        if (!ok) break;
+        if (lane == 0) {
+          mbar_expect_tx(BAR(B_Q_FULL + qb), G::Q_BYTES);
+#pragma unroll
+          for (int s = 0; s < G::SLABS; ++s)
+            tma_load_3d(sbase + G::OFF_Q + qb * G::Q_BYTES + s * G::BQ * 128, &tmQ, s * 64, (b ? tk.row2 : tk.row) * G::BQ, tk.h, BAR(B_Q_FULL + qb));
+        }
+        q_armed |= 1u << qb; q_parity = (q_parity & ~(1u << qb)) | q_ph << qb;
+      }
+      ok = ok && k_tiles.task(ctx, p, tk, lane, sbase, BAR(B_QK_READY), BAR(B_QK_DONE), &tmK, &tmK2, p.drop_tile && t == 0, [&](int j) {
+        if (!drawn && j >= tk.n - kDrawAhead) { tk_next = draw(t_next); drawn = true; }
+      });
+    }
+    if (lane == 0) {
+      if (n_tiles) atomicAdd(&p.ws[7], n_tiles);
+      if (n_pairs) atomicAdd(&p.ws[6], n_pairs);
+    }
+    if (*abort_smem) {
+      // leave no bulk copy in flight into this CTA's shared memory (bounded)
+      k_tiles.drain(p, BAR(B_QK_READY));
+      for (int st = 0; st < G::NQ; ++st)
+        if (q_armed & (1u << st)) {
+          long long t0 = clock64();
+          while (!mbar_try_wait(BAR(B_Q_FULL + st), (q_parity >> st) & 1) && clock64() - t0 < p.wait_limit / 4) {}
+        }
+    }
+  } else if (warp == kVLoadWarp || warp >= kLoadWarps64) {
+    // ============================================================== loaders of V and of the other K tiles
+    auto load_tiles = [&](auto tiles, uint32_t bar_ready0, uint32_t bar_done0, const CUtensorMap* tm, const CUtensorMap* tm2) {
+      uint32_t task_slot = 0, task_ph = 0;
+      bool ok = true;
+      while (ok) {
+        ok = warp_wait(ctx, BAR(B_TASK_FULL + task_slot), task_ph, 10);
+        if (!ok) break;
+        const Task tk = tasks[task_slot];
+        __syncwarp();
+        if (lane == 0) mbar_arrive(BAR(B_TASK_EMPTY + task_slot));
+        task_slot ^= 1;
+        task_ph ^= (task_slot == 0);
+        if (tk.n < 0) break;
+        ok = tiles.task(ctx, p, tk, lane, sbase, bar_ready0, bar_done0, tm, tm2, false, [](int) {});
+      }
+      if (*abort_smem) tiles.drain(p, bar_ready0);
+    };
+    if (warp == kLoadWarps64) load_tiles(TileLoader<G, true>{1}, BAR(B_QK_READY), BAR(B_QK_DONE), &tmK, &tmK2);
+    else load_tiles(TileLoader<G, false>{warp == kVLoadWarp ? 0u : 1u}, BAR(B_PV_READY), BAR(B_PV_DONE), &tmV, &tmV2);
+  } else if (warp == kQkWarp) {
+    // ============================================================== MMA issuer 1: S = Q K^T
+    constexpr uint32_t IDESC_QK = make_idesc(64, G::BK, false);
+    uint32_t task_slot = 0, task_ph = 0, q_it = 0, k_st = 0, it = 0;
+    const uint64_t qdesc0 = make_desc(sbase + G::OFF_Q, 16, 1024);
+    const uint64_t kdesc0 = make_desc(sbase + G::OFF_K, 16, 1024);
+    bool ok = true;
+    while (ok) {
+      ok = warp_wait(ctx, BAR(B_TASK_FULL + task_slot), task_ph, 10);
+      if (!ok) break;
+      const int n = __shfl_sync(0xffffffffu, tasks[task_slot].n, 0);
+      const int blocks = __shfl_sync(0xffffffffu, tasks[task_slot].row2, 0) >= 0 ? 2 : 1;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(BAR(B_TASK_EMPTY + task_slot));
+      task_slot ^= 1;
+      task_ph ^= (task_slot == 0);
+      if (n < 0) break;
+      if (n == 0) continue;
+      for (int b = 0; b < blocks && ok; ++b)
+        ok = warp_wait(ctx, BAR(B_Q_FULL + ((q_it + b) % G::NQ)), ((q_it + b) / G::NQ) & 1, 11);
+      for (int j = 0; j < n && ok; ++j) {
+        const uint64_t kd = kdesc0 + (uint64_t)(k_st * (uint32_t)(G::TILE_BYTES >> 4));
+#pragma unroll 1
+        for (int b = 0; b < blocks; ++b) {
+          const uint32_t qb = (q_it + b) % G::NQ;
+          const uint64_t qd = qdesc0 + (uint64_t)(qb * (uint32_t)(G::Q_BYTES >> 4));
+          const uint32_t d_s = tmem_base + (it % G::NG) * G::S_STRIDE;
+          // the K tile is there, and the group has read the scores of its item before this one
+          ok = warp_wait(ctx, BAR(B_QK_READY + (it & 7)), (it >> 3) & 1, 12);
+          if (!ok) break;
+          tc_fence_after();
+          umma_ws_bf16<D / 16, 32, G::BQ * 128, 32, G::KV_SLAB_BYTES>(d_s, qd, kd, IDESC_QK, 0, BAR(B_QK_DONE + (it & 7)));
+          if (j == n - 1) tc_commit(BAR(B_Q_EMPTY + qb));
+          ++it;
+        }
+        if (++k_st == (uint32_t)G::NKS) k_st = 0;
+      }
+      q_it += (uint32_t)blocks;
+    }
+    // none of this thread's MMAs is still running when tensor memory is released
+    tc_commit(BAR(B_FINAL + 1));
+    __syncwarp();
+    {
+      long long t0 = clock64();
+      while (!mbar_try_wait(BAR(B_FINAL + 1), 0) && clock64() - t0 < p.wait_limit / 4) {}
+    }
+  } else if (warp == kPvWarp) {
+    // ============================================================== MMA issuer 2: O += P V
+    constexpr uint32_t IDESC_PV = make_idesc(64, D, true);
+    uint32_t task_slot = 0, task_ph = 0, o_it = 0, o_free = 0xFu, v_st = 0, pb = 0, it = 0;
+    const uint64_t pdesc0 = make_desc(sbase + G::OFF_P, 16, 1024);
+    const uint64_t vdesc0 = make_desc(sbase + G::OFF_V, G::KV_SLAB_BYTES, 1024);
+    bool ok = true;
+    while (ok) {
+      ok = warp_wait(ctx, BAR(B_TASK_FULL + task_slot), task_ph, 10);
+      if (!ok) break;
+      const int n = __shfl_sync(0xffffffffu, tasks[task_slot].n, 0);
+      const int blocks = __shfl_sync(0xffffffffu, tasks[task_slot].row2, 0) >= 0 ? 2 : 1;
+      const bool half_tail = __shfl_sync(0xffffffffu, tasks[task_slot].tail_valid, 0) <= 64;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(BAR(B_TASK_EMPTY + task_slot));
+      task_slot ^= 1;
+      task_ph ^= (task_slot == 0);
+      if (n < 0) break;
+      if (n == 0) continue;
+      // the accumulators of the task before the previous one have been read by the epilogue
+      const uint32_t ob = (o_it & 1) * 2;
+      ++o_it;
+      for (int b = 0; b < blocks && ok; ++b) {
+        ok = warp_wait(ctx, BAR(B_O_FREE + ob + b), (o_free >> (ob + b)) & 1u, 16);
+        o_free ^= 1u << (ob + b);
+      }
+      for (int j = 0; j < n && ok; ++j) {
+        const bool half = j == n - 1 && half_tail;     // (the second half of a half tile has no keys: nothing was loaded for it)
+        const uint64_t vd = vdesc0 + (uint64_t)(v_st * (uint32_t)(G::TILE_BYTES >> 4));
+#pragma unroll 1
+        for (int b = 0; b < blocks; ++b) {
+          const uint64_t pd = pdesc0 + (uint64_t)(pb * (uint32_t)(G::P_BYTES >> 4));
+          const uint32_t d_o = tmem_base + G::O_COL + (ob + b) * G::O_STRIDE;
+          ok = warp_wait(ctx, BAR(B_PV_READY + (it & 7)), (it >> 3) & 1, 14);
+          if (!ok) break;
+          tc_fence_after();
+          // V tile as the N x K operand with N (head_dim) contiguous: 16 keys = 2048 bytes per MMA, the next 64 columns
+          // of head_dim one slab further
+          if (half) umma_ws_bf16<4, 32, 0, 16 * 128, 0>(d_o, pd, vd, IDESC_PV, j > 0, BAR(B_PV_DONE + (it & 7)));
+          else umma_ws_bf16<8, 32, G::P_PANEL_BYTES, 16 * 128, 64 * 128>(d_o, pd, vd, IDESC_PV, j > 0, BAR(B_PV_DONE + (it & 7)));
+          if (j == n - 1) tc_commit(BAR(B_O_FULL + ob + b));
+          ++it;
+          if (++pb == (uint32_t)G::NP) pb = 0;
+        }
+        if (++v_st == (uint32_t)G::NVS) v_st = 0;
+      }
+    }
+    tc_commit(BAR(B_FINAL));
+    __syncwarp();
+    {
+      long long t0 = clock64();
+      while (!mbar_try_wait(BAR(B_FINAL), 0) && clock64() - t0 < p.wait_limit / 4) {}
+    }
+  } else {
+    // ============================================================== softmax / epilogue (see the kernel above for what is the same)
+    const int quad = warp & 3;                          // tensor-memory lane quadrant this warp may access
+    const uint32_t group = (uint32_t)(warp - kSoftmaxWarp0) >> 2;
+    const int half = quad >> 1;                         // keys 64 half .. of a tile; epilogue: half of O's columns
+    const int rp = quad & 1, r = rp * 32 + lane;        // row of the query block
+    const uint32_t lane_addr = (uint32_t)(quad * 32) << 16;
+    const uint32_t s_addr = tmem_base + lane_addr + group * G::S_STRIDE;
+    uint32_t task_it = 0, o_it = 0, slot3 = 0, slot3_ph = 0, q0 = 0, mx1_bits = 0, of_bits = 0;
+    if (lane == 0) mbar_arrive(BAR(B_QK_READY + group));        // (the buffers are free)
+    bool ok = true;
+    while (ok) {
+      const uint32_t slot = task_it & 1, ph = (task_it >> 1) & 1;
+      ok = warp_wait(ctx, BAR(B_TASK_FULL + slot), ph, 20);
+      if (!ok) break;
+      const Task tk = tasks[slot];
+      __syncwarp();
+      if (lane == 0) mbar_arrive(BAR(B_TASK_EMPTY + slot));
+      ++task_it;
+      if (tk.n < 0) break;
+      if (tk.n == 0) {
+        const long long q_tok = (long long)tk.row * G::BQ + r;
+        if (group == 0 && q_tok < p.seq_q) {
+          uint4* o = reinterpret_cast<uint4*>(p.O + (size_t)tk.h * p.o_stride_h + (size_t)q_tok * p.o_stride_t + half * G::CO);
+#pragma unroll
+          for (int c = 0; c < G::CO / 8; ++c) o[c] = make_uint4(0, 0, 0, 0);
+          if (p.lse && half == 0) p.lse[(size_t)tk.h * p.seq_q + q_tok] = -INFINITY;
+        }
+        continue;
+      }
+      const bool pair = tk.row2 >= 0;
+      const int n_items = pair ? 2 * tk.n : tk.n, i0 = (int)((group - q0) & 3u);      // this group's first item of the task
+      const int blk = pair ? i0 & 1 : 0;                // its query block (the same in all its items: four items are two tiles further)
+      const int task_no = (int)o_it + 1;
+      const uint32_t mslot = slot3 * 2 + blk, mx_bar = BAR(B_MX + (slot3 * 2 + blk) * 2 + rp);
+      // sums of this thread's columns of its tiles; of a pair, two tiles apart, l_run and l_other take turns: one sum for the tiles of
+      // equal number mod 4, as the group of a block on its own has it
+      float m_ref = -INFINITY, l_run = 0.f, l_other = 0.f;
+      for (int i = i0; i < n_items; i += 4) {
+        const uint32_t q = q0 + (uint32_t)i;
+        const int tile = pair ? i >> 1 : i;
+        ok = warp_wait(ctx, BAR(B_QK_DONE + (q & 7)), (q >> 3) & 1, 21);
+        if (!ok) break;
+        tc_fence_after();
+        const int valid = tile == tk.n - 1 ? tk.tail_valid - half * 64 : 64;
+        if (valid < 64 && valid > 0) mask_scores<2>(s_addr, valid);      // keys beyond seq_kv (ragged last block) do not exist
+        if (i == i0) {
+          if (tile == 0) {
+            float mloc = -INFINITY;
+            if (valid > 0) {
+#pragma unroll 1
+              for (int ch = 0; ch < 2; ++ch) {
+                uint32_t sv[32];
+                WAVEAL_TMEM_LD32(s_addr + ch * 32, sv, 0);
+                WAVEAL_TMEM_WAIT_LD32(sv, 0);
+                mloc = fmaxf(mloc, row_max32(sv));
+              }
+            }
+            mx[mslot * 128 + half * 64 + r] = mloc;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(mx_bar);
+          }
+          ok = warp_wait(ctx, mx_bar, blk ? (mx1_bits >> slot3) & 1u : slot3_ph, 24);
+          if (!ok) break;
+          m_ref = fmaxf(mx[mslot * 128 + r], mx[mslot * 128 + 64 + r]) * p.sl2;
+        }
+        if (valid > 0) {
+          const float neg_m = ((m_ref == -INFINITY) ? 0.f : -m_ref) + 0.0028150156f;
+          const float a128 = p.sl2 * 0.0078125f, b128 = (neg_m - kPolyLo) * 0.0078125f;   // polynomial share
+          float ls4[4] = {0.f, 0.f, 0.f, 0.f};
+          const uint32_t p_row = sbase + G::OFF_P + (q % G::NP) * G::P_BYTES + half * G::P_PANEL_BYTES + (uint32_t)r * 128;
+#pragma unroll
+          for (int ch = 0; ch < 2; ++ch) {
+            uint32_t sv[32], pk[16];
+            WAVEAL_TMEM_LD32(s_addr + ch * 32, sv, 0);
+            WAVEAL_TMEM_WAIT_LD32(sv, 0);
+            if (ch == 1) {                              // the scores are read: the group's next product may begin
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(BAR(B_QK_READY + ((q + 4) & 7)));
+            }
+            float x[32];
+            auto use = [&](int c, float e0, float e1) {
+              fadd2(ls4[c & 2], ls4[(c & 2) + 1], ls4[c & 2], ls4[(c & 2) + 1], e0, e1);
+              pk[c / 2] = __byte_perm(__float_as_uint(e0), __float_as_uint(e1), 0x7632);
+            };
+#pragma unroll
+            for (int c = 0; c < 32; c += 2) {
+              if ((c >> 1) % kPolyEvery == kPolyEvery - 1) {
+                ex2_fma2(x[c], x[c + 1], __uint_as_float(sv[c]), __uint_as_float(sv[c + 1]), a128, b128);
+              } else {
+                ffma2(x[c], x[c + 1], __uint_as_float(sv[c]), __uint_as_float(sv[c + 1]), p.sl2, p.sl2, neg_m, neg_m);
+                x[c] = ex2(x[c]); x[c + 1] = ex2(x[c + 1]);
+              }
+              if (c >= 2 * G::LAG) use(c - 2 * G::LAG, x[c - 2 * G::LAG], x[c + 1 - 2 * G::LAG]);
+            }
+#pragma unroll
+            for (int c = 32 - 2 * G::LAG; c < 32; c += 2) use(c, x[c], x[c + 1]);
+            if (ch == 0) {
+              // the product of the buffer's item before this one has completed
+              ok = q < G::NP || warp_wait(ctx, BAR(B_PV_DONE + ((q - G::NP) & 7)), ((q - G::NP) >> 3) & 1, 22);
+              if (!ok) break;
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+              st_shared_v4(p_row + ((((uint32_t)(ch * 4 + c)) ^ (uint32_t)(r & 7)) << 4), pk[4 * c], pk[4 * c + 1], pk[4 * c + 2], pk[4 * c + 3]);
+          }
+          if (!ok) break;
+          const float l_blk = (ls4[0] + ls4[1]) + (ls4[2] + ls4[3]);
+          l_run += l_blk;
+          // all terms are positive, so a sum below 2^60 bounds every exponent it covers; at or above it (or not a number) the
+          // fixed reference is too far off: redo the task
+          if (__any_sync(0xffffffffu, !(l_blk < kRedoLimit))) redo_flag[slot3] = task_no;
+          fence_proxy_async();
+        } else {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(BAR(B_QK_READY + ((q + 4) & 7)));
+          ok = q < G::NP || warp_wait(ctx, BAR(B_PV_DONE + ((q - G::NP) & 7)), ((q - G::NP) >> 3) & 1, 22);
+          if (!ok) break;
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(BAR(B_PV_READY + (q & 7)));
+        if (pair) { const float t = l_run; l_run = l_other; l_other = t; }
+      }
+      if (!ok) break;
+      // ---- epilogue: the four sums of a row and its two halves of every tile, in an order that does not depend on which group had which
+      {
+        const int steps = i0 < n_items ? (n_items - i0 + 3) >> 2 : 0;       // this group's items
+        if (pair && (steps & 1)) { const float t = l_run; l_run = l_other; l_other = t; }
+        const int role = pair ? i0 >> 1 : i0;
+        float* e = ex + (mslot * 4 + role) * 128 + half * 64 + r;
+        e[0] = l_run;
+        if (pair) e[2 * 128] = l_other;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(BAR(B_EX + slot3 * 2 + rp));
+      }
+      // the group of a block's last item has its epilogue
+      const uint32_t last_group = (q0 + (uint32_t)n_items - 1u) & 3u;
+      const bool mine = group == last_group || (pair && group == ((last_group - 1u) & 3u));
+      const int my_blk = pair && group == last_group ? 1 : 0;
+      const uint32_t ob = (o_it & 1) * 2 + my_blk, of_ph = (of_bits >> ob) & 1u, ex_ph = slot3_ph;
+      const uint32_t tslot = slot3, es = slot3 * 2 + my_blk, ex_bar = BAR(B_EX + slot3 * 2 + rp);
+      of_bits ^= (pair ? 3u : 1u) << ((o_it & 1) * 2);
+      if (pair) mx1_bits ^= 1u << slot3;
+      if (++slot3 == (uint32_t)G::NSL) { slot3 = 0; slot3_ph ^= 1; }
+      q0 += (uint32_t)n_items;
+      ++o_it;
+      if (!mine) continue;
+      ok = warp_wait(ctx, ex_bar, ex_ph, 25);
+      if (!ok) break;
+      float l_tot;
+      {
+        const float* e = ex + es * 512 + r;
+        l_tot = ((e[0] + e[64]) + (e[128] + e[192])) + ((e[256] + e[320]) + (e[384] + e[448]));
+      }
+      const float m_all = fmaxf(mx[es * 128 + r], mx[es * 128 + 64 + r]) * p.sl2;
+      if (m_all == -INFINITY) l_tot = 0.f;       // no reference: a result that is not finite, for the second launch
+      const float inv_l = 1.0019531f / l_tot;    // the sums carry the centring factor 1 + 2^-9
+      const long long q_tok = (long long)(my_blk ? tk.row2 : tk.row) * G::BQ + r;
+      __nv_bfloat16* o_ptr = p.O + (size_t)tk.h * p.o_stride_h + (size_t)q_tok * p.o_stride_t + half * G::CO;
+      ok = warp_wait(ctx, BAR(B_O_FULL + ob), of_ph, 23);
+      if (!ok) break;
+      tc_fence_after();
+      uint32_t ov[G::CO];
+      const uint32_t o_addr = tmem_base + lane_addr + G::O_COL + ob * G::O_STRIDE;
+      WAVEAL_TMEM_LD32(o_addr, ov, 0);
+      if constexpr (G::CO == 64) WAVEAL_TMEM_LD32(o_addr + 32, ov, 32);
+      WAVEAL_TMEM_WAIT_LD32(ov, 0);
+      if constexpr (G::CO == 64) WAVEAL_TMEM_WAIT_LD32(ov, 32);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(BAR(B_O_FREE + ob));
+      bool bad = false;
+      if (q_tok < p.seq_q) {
+        uint32_t w[G::CO / 2];
+#pragma unroll
+        for (int c = 0; c < G::CO; c += 2) {
+          __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(ov[c]) * inv_l, __uint_as_float(ov[c + 1]) * inv_l);
+          w[c / 2] = *reinterpret_cast<uint32_t*>(&b2);
+        }
+        // |O| <= l_tot max|V|: only a large sum (or none) can have led out of fp32's range
+        if (!(l_tot > 0.f && l_tot < kCheckSum)) {
+          uint32_t top = 0;                // an exponent field of ones in either half of a pair carries into its top bit
+#pragma unroll
+          for (int c = 0; c < G::CO / 2; ++c) top |= (w[c] & 0x7F807F80u) + 0x00800080u;
+          bad = (top & 0x80008000u) != 0;
+        }
+        if ((reinterpret_cast<uintptr_t>(o_ptr) & 31) == 0) {
+          // (a store instruction of a warp touches 32 rows and costs the memory pipe per row, not per byte)
+#pragma unroll
+          for (int c = 0; c < G::CO / 2; c += 8) st_global_v8(o_ptr + 2 * c, w + c);
+        } else {
+#pragma unroll
+          for (int c = 0; c < G::CO / 2; c += 4)
+            *reinterpret_cast<uint4*>(o_ptr + 2 * c) = make_uint4(w[c], w[c + 1], w[c + 2], w[c + 3]);
+        }
+        if (p.lse && half == 0) p.lse[(size_t)tk.h * p.seq_q + q_tok] = (m_all + log2f(l_tot) - 0.0028150156f) * 0.6931471805599453f;
+      }
+      // to the second launch if the sum of a tile left the range (all items' flags were set before B_EX) or a result is not finite
+      if ((__any_sync(0xffffffffu, bad) || redo_flag[tslot] == task_no) && lane == 0)
+        list_task(p.ws, &redo_listed[tslot], task_no, tk.h, tk.row, tk.row2);
+    }
+  }
+
+  // ------------------------------------------------------------------ teardown
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kPvWarp) {
+    tc_fence_after();
+    tmem_dealloc(tmem_base, G::TMEM_COLS);
+  }
+  if (tid == 0) {
+    const long long dt = clock64() - t_start;
+    atomicMax(&p.ws[4], (int)(dt > 0x7fffffffll ? 0x7fffffffll : dt));
   }
 }
 
@@ -1382,7 +2029,7 @@ __global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* ta
   const bool live = t < p.total_tasks;
   Task tk{};
   if (live) tk = table[t];
-  const int at = tail_place(tk.n, live);
+  const int at = tail_place(tk.row2 >= 0 ? 2 * tk.n : tk.n, live);      // (a pair: two items a tile)
   if (live) table[p.first_tail + at] = tk;
 }
 
@@ -1576,7 +2223,10 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
     if ((s = make_map(&tv2, V, D, d->seq_kv, d->heads, d->v_stride[0], d->v_stride[1], 128, "V (128-row boxes)")) != WAVEAL_OK) return s;
     to = tq;
   }
-  WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd<BLOCK, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES));
+  if constexpr (BLOCK == 64)
+    WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd_rows64<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Geo64<D>::SMEM_BYTES));
+  else
+    WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd<BLOCK, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES));
   WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd<BLOCK, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES));
   long long grid = p.total_tasks < sms ? p.total_tasks : sms;
   Task* table = reinterpret_cast<Task*>(reinterpret_cast<char*>(p.ws) + table_offset(p.total_tasks));
@@ -1616,7 +2266,10 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   // first pass: reference fixed after the first tile of a task; second pass: the tasks the
   // first one listed (normally none: its CTAs leave at once), max of every block
   p.redo_pass = 0;
-  WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, true>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, to, p));
+  if constexpr (BLOCK == 64)
+    WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd_rows64<D>, dim3((unsigned)grid), kThreads64, Geo64<D>::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, p));
+  else
+    WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, true>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, to, p));
   p.redo_pass = 1;
   p.direct = 0;
   WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, false>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, to, p));
