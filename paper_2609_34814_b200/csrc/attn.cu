@@ -1356,7 +1356,8 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 // 850 clk at the 77 bytes per clock and SM that all SMs draw from L2 together at the full clock.
 // Against the 128-row products (which a lone block half filled) with the same softmax: 8 heads of 1,536 rows of the LTX recipe, head_dim 128,
 // 1,319 -> 1,110 clk a tile (907 an item; two blocks that share the tiles of one list take two items each), 11.2 -> 9.4 ms;
-// 8 heads of 768 rows, head_dim 64, 1,165 -> 990; 8 heads of 317 rows of 9 or 10 tiles 1,773 -> 1,400, 241 -> 150 us.
+// 8 heads of 768 rows, head_dim 64, 1,165 -> 930, 2.17 -> 1.70 ms; 8 heads of 317 rows of 9 or 10 tiles 1,773 -> 1,330, 241 -> 144 us.
+// Pairs as ordinary products of 128 rows (the same bits): 1,170, the code for both slows a lone block's softmax.
 //
 // At this pace the issuing warps' and the loaders' own instructions count (~10 clk each beside four softmax warps a scheduler):
 //  - an item has ONE barrier on which its product waits (the tile's bytes and the softmax group's arrivals together) and ONE that it
@@ -1390,7 +1391,6 @@ struct Geo64 {
   static constexpr int NVS = NKS;                    // V tiles
   static constexpr int NG = 4;                       // softmax groups of four warps, each with its own S buffer
   static constexpr int CO = D / 2;                   // O columns per epilogue thread
-  static constexpr int LAG = 4;
   static constexpr int NSL = 3;                      // slots by task for what the groups leave each other
   static constexpr int OFF_Q = 0;
   static constexpr int OFF_P = OFF_Q + NQ * Q_BYTES;
@@ -1399,7 +1399,7 @@ struct Geo64 {
   static constexpr int OFF_BAR = OFF_V + NVS * TILE_BYTES;
   static constexpr int N_BAR = 4 + 2 * NQ + 4 * 8 + 4 + 4 + 2 + NSL * 4 + NSL * 2;
   static constexpr int OFF_TASK = OFF_BAR + ((N_BAR * 8 + 15) / 16) * 16;
-  static constexpr int OFF_MX = OFF_TASK + 2 * (int)sizeof(Task);             // [slot][block][128] largest score of a half row
+  static constexpr int OFF_MX = OFF_TASK + 4 * (int)sizeof(Task);             // [slot][block][128] largest score of a half row
   static constexpr int OFF_EX = OFF_MX + NSL * 2 * 128 * 4;                   // [slot][block][tile mod 4][128] sums
   static constexpr int OFF_MISC = OFF_EX + NSL * 2 * 4 * 128 * 4;
   static constexpr int SMEM_BYTES = OFF_MISC + 48 + 1024;   // + slack for 1024-byte alignment
@@ -1583,7 +1583,7 @@ k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       ok = warp_wait(ctx, BAR(B_TASK_EMPTY + slot), ph ^ 1, 1);
       if (!ok) break;
       if (lane == 0) {
-        tasks[slot] = tk;
+        tasks[task_it & 3] = tk;           // (four places: an epilogue looks a task up when the next two may be there)
         mbar_arrive(BAR(B_TASK_FULL + slot));
       }
       ++task_it;
@@ -1630,7 +1630,7 @@ k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       while (ok) {
         ok = warp_wait(ctx, BAR(B_TASK_FULL + task_slot), task_ph, 10);
         if (!ok) break;
-        const Task tk = tasks[task_slot];
+        const Task tk = tasks[task_slot + 2 * task_ph];
         __syncwarp();
         if (lane == 0) mbar_arrive(BAR(B_TASK_EMPTY + task_slot));
         task_slot ^= 1;
@@ -1652,8 +1652,8 @@ k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     while (ok) {
       ok = warp_wait(ctx, BAR(B_TASK_FULL + task_slot), task_ph, 10);
       if (!ok) break;
-      const int n = __shfl_sync(0xffffffffu, tasks[task_slot].n, 0);
-      const int blocks = __shfl_sync(0xffffffffu, tasks[task_slot].row2, 0) >= 0 ? 2 : 1;
+      const int n = __shfl_sync(0xffffffffu, tasks[task_slot + 2 * task_ph].n, 0);
+      const int blocks = __shfl_sync(0xffffffffu, tasks[task_slot + 2 * task_ph].row2, 0) >= 0 ? 2 : 1;
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR(B_TASK_EMPTY + task_slot));
       task_slot ^= 1;
@@ -1698,9 +1698,9 @@ k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     while (ok) {
       ok = warp_wait(ctx, BAR(B_TASK_FULL + task_slot), task_ph, 10);
       if (!ok) break;
-      const int n = __shfl_sync(0xffffffffu, tasks[task_slot].n, 0);
-      const int blocks = __shfl_sync(0xffffffffu, tasks[task_slot].row2, 0) >= 0 ? 2 : 1;
-      const bool half_tail = __shfl_sync(0xffffffffu, tasks[task_slot].tail_valid, 0) <= 64;
+      const int n = __shfl_sync(0xffffffffu, tasks[task_slot + 2 * task_ph].n, 0);
+      const int blocks = __shfl_sync(0xffffffffu, tasks[task_slot + 2 * task_ph].row2, 0) >= 0 ? 2 : 1;
+      const bool half_tail = __shfl_sync(0xffffffffu, tasks[task_slot + 2 * task_ph].tail_valid, 0) <= 64;
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR(B_TASK_EMPTY + task_slot));
       task_slot ^= 1;
@@ -1756,23 +1756,24 @@ k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       const uint32_t slot = task_it & 1, ph = (task_it >> 1) & 1;
       ok = warp_wait(ctx, BAR(B_TASK_FULL + slot), ph, 20);
       if (!ok) break;
-      const Task tk = tasks[slot];
+      const volatile Task* tk = tasks + (task_it & 3);  // (what the epilogue needs of it is not kept in registers meanwhile)
+      const int n = tk->n, tail_valid = tk->tail_valid;
+      const bool pair = tk->row2 >= 0;
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR(B_TASK_EMPTY + slot));
       ++task_it;
-      if (tk.n < 0) break;
-      if (tk.n == 0) {
-        const long long q_tok = (long long)tk.row * G::BQ + r;
+      if (n < 0) break;
+      if (n == 0) {
+        const long long q_tok = (long long)tk->row * G::BQ + r;
         if (group == 0 && q_tok < p.seq_q) {
-          uint4* o = reinterpret_cast<uint4*>(p.O + (size_t)tk.h * p.o_stride_h + (size_t)q_tok * p.o_stride_t + half * G::CO);
-#pragma unroll
+          uint4* o = reinterpret_cast<uint4*>(p.O + (size_t)tk->h * p.o_stride_h + (size_t)q_tok * p.o_stride_t + half * G::CO);
+#pragma unroll 1
           for (int c = 0; c < G::CO / 8; ++c) o[c] = make_uint4(0, 0, 0, 0);
-          if (p.lse && half == 0) p.lse[(size_t)tk.h * p.seq_q + q_tok] = -INFINITY;
+          if (p.lse && half == 0) p.lse[(size_t)tk->h * p.seq_q + q_tok] = -INFINITY;
         }
         continue;
       }
-      const bool pair = tk.row2 >= 0;
-      const int n_items = pair ? 2 * tk.n : tk.n, i0 = (int)((group - q0) & 3u);      // this group's first item of the task
+      const int n_items = pair ? 2 * n : n, i0 = (int)((group - q0) & 3u);      // this group's first item of the task
       const int blk = pair ? i0 & 1 : 0;                // its query block (the same in all its items: four items are two tiles further)
       const int task_no = (int)o_it + 1;
       const uint32_t mslot = slot3 * 2 + blk, mx_bar = BAR(B_MX + (slot3 * 2 + blk) * 2 + rp);
@@ -1785,7 +1786,7 @@ k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
         ok = warp_wait(ctx, BAR(B_QK_DONE + (q & 7)), (q >> 3) & 1, 21);
         if (!ok) break;
         tc_fence_after();
-        const int valid = tile == tk.n - 1 ? tk.tail_valid - half * 64 : 64;
+        const int valid = tile == n - 1 ? tail_valid - half * 64 : 64;
         if (valid < 64 && valid > 0) mask_scores<2>(s_addr, valid);      // keys beyond seq_kv (ragged last block) do not exist
         if (i == i0) {
           if (tile == 0) {
@@ -1812,6 +1813,8 @@ k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           const float a128 = p.sl2 * 0.0078125f, b128 = (neg_m - kPolyLo) * 0.0078125f;   // polynomial share
           float ls4[4] = {0.f, 0.f, 0.f, 0.f};
           const uint32_t p_row = sbase + G::OFF_P + (q % G::NP) * G::P_BYTES + half * G::P_PANEL_BYTES + (uint32_t)r * 128;
+          // (both chunks in line: 1,141 -> 1,113 clk a tile, 1,055 -> 930 at head_dim 64; a pair's results used four pairs later, as in the
+          // kernel above: +0.4 .. +0.7 %)
 #pragma unroll
           for (int ch = 0; ch < 2; ++ch) {
             uint32_t sv[32], pk[16];
@@ -1822,23 +1825,18 @@ k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
               __syncwarp();
               if (lane == 0) mbar_arrive(BAR(B_QK_READY + ((q + 4) & 7)));
             }
-            float x[32];
-            auto use = [&](int c, float e0, float e1) {
-              fadd2(ls4[c & 2], ls4[(c & 2) + 1], ls4[c & 2], ls4[(c & 2) + 1], e0, e1);
-              pk[c / 2] = __byte_perm(__float_as_uint(e0), __float_as_uint(e1), 0x7632);
-            };
 #pragma unroll
             for (int c = 0; c < 32; c += 2) {
+              float e0, e1;
               if ((c >> 1) % kPolyEvery == kPolyEvery - 1) {
-                ex2_fma2(x[c], x[c + 1], __uint_as_float(sv[c]), __uint_as_float(sv[c + 1]), a128, b128);
+                ex2_fma2(e0, e1, __uint_as_float(sv[c]), __uint_as_float(sv[c + 1]), a128, b128);
               } else {
-                ffma2(x[c], x[c + 1], __uint_as_float(sv[c]), __uint_as_float(sv[c + 1]), p.sl2, p.sl2, neg_m, neg_m);
-                x[c] = ex2(x[c]); x[c + 1] = ex2(x[c + 1]);
+                ffma2(e0, e1, __uint_as_float(sv[c]), __uint_as_float(sv[c + 1]), p.sl2, p.sl2, neg_m, neg_m);
+                e0 = ex2(e0); e1 = ex2(e1);
               }
-              if (c >= 2 * G::LAG) use(c - 2 * G::LAG, x[c - 2 * G::LAG], x[c + 1 - 2 * G::LAG]);
+              fadd2(ls4[c & 2], ls4[(c & 2) + 1], ls4[c & 2], ls4[(c & 2) + 1], e0, e1);
+              pk[c / 2] = __byte_perm(__float_as_uint(e0), __float_as_uint(e1), 0x7632);
             }
-#pragma unroll
-            for (int c = 32 - 2 * G::LAG; c < 32; c += 2) use(c, x[c], x[c + 1]);
             if (ch == 0) {
               // the product of the buffer's item before this one has completed
               ok = q < G::NP || warp_wait(ctx, BAR(B_PV_DONE + ((q - G::NP) & 7)), ((q - G::NP) >> 3) & 1, 22);
@@ -1900,49 +1898,55 @@ k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       const float m_all = fmaxf(mx[es * 128 + r], mx[es * 128 + 64 + r]) * p.sl2;
       if (m_all == -INFINITY) l_tot = 0.f;       // no reference: a result that is not finite, for the second launch
       const float inv_l = 1.0019531f / l_tot;    // the sums carry the centring factor 1 + 2^-9
-      const long long q_tok = (long long)(my_blk ? tk.row2 : tk.row) * G::BQ + r;
-      __nv_bfloat16* o_ptr = p.O + (size_t)tk.h * p.o_stride_h + (size_t)q_tok * p.o_stride_t + half * G::CO;
+      const int h = tk->h;
+      const long long q_tok = (long long)(my_blk ? tk->row2 : tk->row) * G::BQ + r;
+      __nv_bfloat16* o_ptr = p.O + (size_t)h * p.o_stride_h + (size_t)q_tok * p.o_stride_t + half * G::CO;
       ok = warp_wait(ctx, BAR(B_O_FULL + ob), of_ph, 23);
       if (!ok) break;
       tc_fence_after();
-      uint32_t ov[G::CO];
       const uint32_t o_addr = tmem_base + lane_addr + G::O_COL + ob * G::O_STRIDE;
-      WAVEAL_TMEM_LD32(o_addr, ov, 0);
-      if constexpr (G::CO == 64) WAVEAL_TMEM_LD32(o_addr + 32, ov, 32);
-      WAVEAL_TMEM_WAIT_LD32(ov, 0);
-      if constexpr (G::CO == 64) WAVEAL_TMEM_WAIT_LD32(ov, 32);
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(BAR(B_O_FREE + ob));
       bool bad = false;
-      if (q_tok < p.seq_q) {
-        uint32_t w[G::CO / 2];
-#pragma unroll
-        for (int c = 0; c < G::CO; c += 2) {
-          __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(ov[c]) * inv_l, __uint_as_float(ov[c + 1]) * inv_l);
-          w[c / 2] = *reinterpret_cast<uint32_t*>(&b2);
+      // (all 64 columns at once do not fit the 80 registers that six warps a scheduler leave: with them, and the task held in registers,
+      // 930 -> 994 clk a tile at head_dim 64, 1,333 -> 1,409 for the short rows)
+#pragma unroll 1
+      for (int c0 = 0; c0 < G::CO; c0 += 32) {
+        uint32_t ov[32];
+        WAVEAL_TMEM_LD32(o_addr + c0, ov, 0);
+        WAVEAL_TMEM_WAIT_LD32(ov, 0);
+        if (c0 == G::CO - 32) {
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(BAR(B_O_FREE + ob));
         }
-        // |O| <= l_tot max|V|: only a large sum (or none) can have led out of fp32's range
-        if (!(l_tot > 0.f && l_tot < kCheckSum)) {
-          uint32_t top = 0;                // an exponent field of ones in either half of a pair carries into its top bit
+        if (q_tok < p.seq_q) {
+          uint32_t w[16];
 #pragma unroll
-          for (int c = 0; c < G::CO / 2; ++c) top |= (w[c] & 0x7F807F80u) + 0x00800080u;
-          bad = (top & 0x80008000u) != 0;
+          for (int c = 0; c < 32; c += 2) {
+            __nv_bfloat162 b2 = __floats2bfloat162_rn(__uint_as_float(ov[c]) * inv_l, __uint_as_float(ov[c + 1]) * inv_l);
+            w[c / 2] = *reinterpret_cast<uint32_t*>(&b2);
+          }
+          // |O| <= l_tot max|V|: only a large sum (or none) can have led out of fp32's range
+          if (!(l_tot > 0.f && l_tot < kCheckSum)) {
+            uint32_t top = 0;              // an exponent field of ones in either half of a pair carries into its top bit
+#pragma unroll
+            for (int c = 0; c < 16; ++c) top |= (w[c] & 0x7F807F80u) + 0x00800080u;
+            bad |= (top & 0x80008000u) != 0;
+          }
+          if ((reinterpret_cast<uintptr_t>(o_ptr) & 31) == 0) {
+            // (a store instruction of a warp touches 32 rows and costs the memory pipe per row, not per byte)
+#pragma unroll
+            for (int c = 0; c < 16; c += 8) st_global_v8(o_ptr + c0 + 2 * c, w + c);
+          } else {
+#pragma unroll
+            for (int c = 0; c < 16; c += 4)
+              *reinterpret_cast<uint4*>(o_ptr + c0 + 2 * c) = make_uint4(w[c], w[c + 1], w[c + 2], w[c + 3]);
+          }
         }
-        if ((reinterpret_cast<uintptr_t>(o_ptr) & 31) == 0) {
-          // (a store instruction of a warp touches 32 rows and costs the memory pipe per row, not per byte)
-#pragma unroll
-          for (int c = 0; c < G::CO / 2; c += 8) st_global_v8(o_ptr + 2 * c, w + c);
-        } else {
-#pragma unroll
-          for (int c = 0; c < G::CO / 2; c += 4)
-            *reinterpret_cast<uint4*>(o_ptr + 2 * c) = make_uint4(w[c], w[c + 1], w[c + 2], w[c + 3]);
-        }
-        if (p.lse && half == 0) p.lse[(size_t)tk.h * p.seq_q + q_tok] = (m_all + log2f(l_tot) - 0.0028150156f) * 0.6931471805599453f;
       }
+      if (p.lse && half == 0 && q_tok < p.seq_q) p.lse[(size_t)h * p.seq_q + q_tok] = (m_all + log2f(l_tot) - 0.0028150156f) * 0.6931471805599453f;
       // to the second launch if the sum of a tile left the range (all items' flags were set before B_EX) or a result is not finite
       if ((__any_sync(0xffffffffu, bad) || redo_flag[tslot] == task_no) && lane == 0)
-        list_task(p.ws, &redo_listed[tslot], task_no, tk.h, tk.row, tk.row2);
+        list_task(p.ws, &redo_listed[tslot], task_no, h, tk->row, tk->row2);
     }
   }
 
