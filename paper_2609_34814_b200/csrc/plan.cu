@@ -831,8 +831,8 @@ __device__ __forceinline__ void exclusive_scan(int* a, int n, int* part) {
 // Ascending sort of n pairs (key, val) with distinct pairs, ties of the key by val, through bins that are themselves in
 // ascending order: `bin(key)` < n_bins never falls as the key grows.  Counts per bin, prefix sums, a scatter, and every
 // element counts the elements of its own bin that go before it: the work per element is the size of its bin, where the
-// merge sort walks log2(n) binary searches.  43,800 -> 11,200 clk for 2,841 rows of a video mask, 10,400 -> 8,500 for 591; where a
-// sixth of the rows have one angle (rows that select everything) as long as the merge sort, 24,000 for 1,536.  (Bins cut at
+// merge sort walks log2(n) binary searches.  43,800 -> 9,100 clk for 2,841 rows of a video mask, 10,400 -> 8,100 for 591, 24,000 ->
+// 12,400 for 1,536 of which a tenth have one angle (rows that select everything).  (Bins cut at
 // the quantiles of a sample of the keys: 41,700 for the 2,841 rows, their bins of 22 and more are walked for longer.)
 // The sorted values go to v0.  False, with the pairs as they were, if a bin holds more than `most`.  (The order inside a
 // bin before the count depends on the atomics, the result does not.)
@@ -856,9 +856,10 @@ __device__ __forceinline__ bool bin_sort(const u64* k0, int* v0, u64* k1, int* v
     const int val = v1[i], b = bin(key), from = b ? bins[b - 1] : 0, to = bins[b];
     int at = from;
 #pragma unroll 4
-    for (int j = from; j < to; ++j) {
+    for (int j = from; j < to; ++j) {                      // (both are always read, several rows under way)
       const u64 kj = k1[j];
-      at += (kj < key || (kj == key && v1[j] < val)) ? 1 : 0;
+      const int vj = v1[j];
+      at += (int)(kj < key) | ((int)(kj == key) & (int)(vj < val));
     }
     v0[at] = val;
   }
