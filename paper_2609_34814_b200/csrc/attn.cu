@@ -394,6 +394,10 @@ struct AttnParams {
 };
 
 
+// 64-row blocks, behind the table: [0] 1: products of 128 rows for this call, 0: of 64 (k_sort_tail); [2 + 2i], [3 + 2i]: tiles in all
+// and of pairs in block i of k_task_table_pairs
+__device__ __forceinline__ const int* pick_word(const AttnParams& p) { return reinterpret_cast<const int*>(p.table + p.total_tasks); }
+
 // Task of every ticket (head-major or position-major over the planned order), so that the
 // persistent CTAs need one load behind a ticket instead of a chain through row_order, the row
 // pointers and the index list.
@@ -596,7 +600,8 @@ __device__ __noinline__ void mask_scores(uint32_t s_addr, int valid) {
 }
 
 // a task for the second launch, unless another warp has listed it already; the blocks of a pair are computed again one by one
-// (in line for 128-row blocks: 521 k -> 506 k cycles on 5 heads of 256 rows, a call there makes the compiler spill)
+// (in line for 128-row blocks: 521 k -> 506 k cycles on 5 heads of 256 rows, a call there makes the compiler spill; out of line
+// for 64-row blocks in products of 128 rows, 18.75 M -> 18.35 M on 8 heads of 1536 rows)
 __device__ __forceinline__ void list_task(int* ws, int* listed, int task_no, int h, int row, int row2) {
   if (atomicExch(listed, task_no) == task_no) return;
   waveal::wait_for_previous_kernel();      // (which clears the count: a first task may end before it)
@@ -605,8 +610,13 @@ __device__ __forceinline__ void list_task(int* ws, int* listed, int task_no, int
   ws[9 + 2 * e] = row;
   if (row2 >= 0) { ws[10 + 2 * e] = h; ws[11 + 2 * e] = row2; }
 }
+__device__ __noinline__ void list_task_call(int* ws, int* listed, int task_no, int h, int row, int row2) {
+  list_task(ws, listed, task_no, h, row, row2);
+}
 
-template <int BLOCK, int D, bool FAST>
+// MOD4 (64-row blocks, first launch): the row sums by tile mod 4, as k_bsattn_fwd_rows64 has them, whose place this kernel takes in
+// calls of many pairs: the same bits, whichever of the two runs
+template <int BLOCK, int D, bool FAST, bool MOD4 = false>
 __global__ void __launch_bounds__(kThreads, 1)
 k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
              const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmK2,
@@ -615,7 +625,6 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   // two blocks of a tile lie next to each other in memory (for 128-key blocks they equal tmK / tmV).
   // tmO: O in boxes of 32 rows and half of head_dim, what a warp stores (128-row blocks only)
   using G = Geo<BLOCK, D>;
-  static_assert(BLOCK == 128 || !FAST, "the first launch of 64-row blocks is k_bsattn_fwd_rows64");
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = smem_u32(smem);
@@ -626,6 +635,11 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 
   // second pass with nothing listed (or after an abort): leave before anything is set up
   if (p.redo_pass && (p.ws[2] == 0 || p.ws[1] != 0)) return;
+  // 64-row blocks of a call that k_bsattn_fwd_rows64 has done
+  if (MOD4) {
+    waveal::wait_for_previous_kernel();
+    if (*pick_word(p) == 0 || p.ws[1] != 0) return;
+  }
 
   const uint32_t bar0 = sbase + G::OFF_BAR;
   auto BAR = [&](int i) { return bar0 + 8u * (uint32_t)i; };
@@ -1044,7 +1058,8 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
         continue;
       }
       // l_run: sum over this thread's columns of this team's blocks, relative to the reference m_ref
-      float m_ref = -INFINITY, l_run = 0.f;
+      // (MOD4: l_other that of the tiles two further or before)
+      float m_ref = -INFINITY, l_run = 0.f, l_other = 0.f;
       const int last = tk.n - 1;
       const int role = kTwoFirst ? (team == first_team ? 0 : 1) : (int)((g0 ^ (uint32_t)team) & 1u);       // 0: has the first tile
       const int j0 = kTwoFirst ? 2 * role : role;
@@ -1215,6 +1230,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           }
           const float l_blk = (ls4[0] + ls4[1]) + (ls4[2] + ls4[3]);
           l_run += l_blk;
+          if (MOD4) { const float t = l_run; l_run = l_other; l_other = t; }
           // all terms are positive (the transcendental unit returns +inf on overflow, the
           // polynomial share saturates at 2^64), so a sum below 2^60 bounds every exponent it
           // covers; at or above it (or not a number) the fixed reference is too far off:
@@ -1234,7 +1250,8 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       // the team had the task's first tile, so that the result does not depend on which team had which) brought to
       // the final reference (the larger of the two teams', references never shrink)
       // (a thread's partial sum is final once its last tile is done)
-      exb[(role * 2 + half) * 128 + r] = make_float2(m_ref, l_run);
+      if (MOD4 && (((tk.n - role + 1) >> 1) & 1)) { const float t = l_run; l_run = l_other; l_other = t; }
+      exb[(role * 2 + half) * 128 + r] = MOD4 ? make_float2(l_run, l_other) : make_float2(m_ref, l_run);
       __syncwarp();
       if (lane == 0) mbar_arrive(BAR(ex_bar));
       // (the team of the last tile; at least one of the first two is the first team's)
@@ -1256,11 +1273,17 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       ok = warp_wait(ctx, BAR(ex_bar), ex_ph, 25);
       if (!ok) break;
       const float2 e00 = exb[0 * 128 + r], e01 = exb[1 * 128 + r], e10 = exb[2 * 128 + r], e11 = exb[3 * 128 + r];
-      const float m0 = fmaxf(e00.x, e01.x), m1 = fmaxf(e10.x, e11.x);     // the two owners of a team's rows agree; a team
-      const float m_all = fmaxf(m0, m1);                                   // without tiles (n == 1) has -inf
-      const float a0 = (m0 == -INFINITY) ? 0.f : ex2(m0 - m_all);
-      const float a1 = (m1 == -INFINITY) ? 0.f : ex2(m1 - m_all);
-      const float l_tot = a0 * (e00.y + e01.y) + a1 * (e10.y + e11.y);
+      float m_all, l_tot;
+      if constexpr (MOD4) {
+        m_all = m_ref;                                                     // (the same for all; no reference: for the second launch)
+        l_tot = m_ref == -INFINITY ? 0.f : ((e00.x + e01.x) + (e10.x + e11.x)) + ((e00.y + e01.y) + (e10.y + e11.y));
+      } else {
+        const float m0 = fmaxf(e00.x, e01.x), m1 = fmaxf(e10.x, e11.x);   // the two owners of a team's rows agree; a team
+        m_all = fmaxf(m0, m1);                                             // without tiles (n == 1) has -inf
+        const float a0 = (m0 == -INFINITY) ? 0.f : ex2(m0 - m_all);
+        const float a1 = (m1 == -INFINITY) ? 0.f : ex2(m1 - m_all);
+        l_tot = a0 * (e00.y + e01.y) + a1 * (e10.y + e11.y);
+      }
       const float inv_l = 1.0019531f / l_tot;    // the sums carry the centring factor 1 + 2^-9
       ok = warp_wait(ctx, BAR(B_O_FULL), o_ph, 23);
       if (!ok) break;
@@ -1323,8 +1346,10 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
       // before O_FULL) or if a result is not finite: with sums of up to 2^60 O overflows from |V| = 2^67 on, and a
       // first tile whose scores are all -inf leaves no reference.  (Where V itself holds an inf or NaN the second
       // launch finds the same again.)  Whichever of the epilogue's warps sees it first writes the entry.
-      if (FAST && (__any_sync(0xffffffffu, bad) || redo_flag[rslot] == task_no) && lane == 0)
-        list_task(p.ws, &redo_listed[rslot], task_no, tk.h, tk.row, -1);
+      if (FAST && (__any_sync(0xffffffffu, bad) || redo_flag[rslot] == task_no) && lane == 0) {
+        if constexpr (G::KB == 2) list_task_call(p.ws, &redo_listed[rslot], task_no, tk.h, tk.row, tk.row2);
+        else list_task(p.ws, &redo_listed[rslot], task_no, tk.h, tk.row, -1);
+      }
     }
   }
 
@@ -1356,7 +1381,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 // 850 clk at the 77 bytes per clock and SM that all SMs draw from L2 together at the full clock.
 // Against the 128-row products (which a lone block half filled) with the same softmax: 8 heads of 1,536 rows of the LTX recipe, head_dim 128,
 // 1,319 -> 1,110 clk a tile (907 an item; two blocks that share the tiles of one list take two items each), 11.2 -> 9.4 ms;
-// 8 heads of 768 rows, head_dim 64, 1,165 -> 930, 2.17 -> 1.70 ms; 8 heads of 317 rows of 9 or 10 tiles 1,773 -> 1,330, 241 -> 144 us.
+// 8 heads of 768 rows, head_dim 64, 1,165 -> 930, 2.17 -> 1.70 ms; 8 heads of 317 rows of 9 or 10 tiles 1,773 -> 1,330, 185 -> 144 us.
 // Pairs as ordinary products of 128 rows (the same bits): 1,170, the code for both slows a lone block's softmax.
 //
 // At this pace the issuing warps' and the loaders' own instructions count (~10 clk each beside four softmax warps a scheduler):
@@ -1371,6 +1396,11 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 // q mod 3.  A lane has 64 columns of one row, lanes m and 64 + m the two halves of a tile.  The S buffer is free as soon as its scores are
 // in registers.  The accumulator has two copies, by task, so that the next task's products do not wait for this one's epilogue,
 // which the group of a block's last item runs while the others go on.
+// Which kernel a call takes: two blocks that share their tiles (a pair) fill a product of 128 rows, which takes 1,327 clk a tile
+// (1,140 at head_dim 64) against their two items' 1,770 (1,370), a lone block's tile as long against its item's 886
+// (735): products of 64 rows are quicker until pairs have 47 % (64 %) of the tiles.  k_sort_tail, which has the counts, picks; the kernel not
+// picked leaves at once (~3 us).  (8 heads of the LTX recipe, a quarter: 11.2 -> 9.3 ms; 2 dense heads of 512 rows, all: 892 us with the
+// one, 1,100 with the other.)  Calls of no more tasks than SMs last as long as their longest task and stay with products of 128 rows.
 // Pairs: two blocks with the very same list are items 2 i and 2 i + 1 of tile i, each with an accumulator of its own.  Everything a row
 // sees is as it would be alone: the products in the same order, a reference from the same first 128 keys, and the same
 // sums, which a lone block has by tile mod 4 (its groups) and a pair's groups keep two of.
@@ -1556,11 +1586,12 @@ k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     TileLoader<G, true> k_tiles{0};
     int n_tiles = 0, n_pairs = 0;        // words 7 and 6 of the workspace
     bool ok = true;
+    const bool mine = *pick_word(p) == 0;
     auto draw = [&](long long& t_out) -> Task {
       for (;;) {
         long long t = 0;
         if (lane == 0)                   // (volatile: another SM raises the flag while this kernel runs)
-          t = (*reinterpret_cast<volatile int*>(&p.ws[1]) != 0) ? p.total_tasks : (long long)(unsigned)atomicAdd(&p.ws[0], 1);
+          t = (!mine || *reinterpret_cast<volatile int*>(&p.ws[1]) != 0) ? p.total_tasks : (long long)(unsigned)atomicAdd(&p.ws[0], 1);
         t = __shfl_sync(0xffffffffu, t, 0);
         t_out = t;
         Task tk{};
@@ -1957,7 +1988,7 @@ k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     tc_fence_after();
     tmem_dealloc(tmem_base, G::TMEM_COLS);
   }
-  if (tid == 0) {
+  if (tid == 0 && *pick_word(p) == 0) {
     const long long dt = clock64() - t_start;
     atomicMax(&p.ws[4], (int)(dt > 0x7fffffffll ? 0x7fffffffll : dt));
   }
@@ -2026,14 +2057,26 @@ __global__ void __launch_bounds__(kTailTasks) k_task_table(AttnParams p, int blo
 }
 
 // the same for a table that is there already (64-row blocks: pairs are formed first)
-__global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* table) {
+__global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* table, int* pick, int n_parts, int share) {
   waveal::let_next_kernel_start();
   waveal::wait_for_previous_kernel();
   const long long t = p.first_tail + threadIdx.x;
   const bool live = t < p.total_tasks;
   Task tk{};
   if (live) tk = table[t];
-  const int at = tail_place(tk.row2 >= 0 ? 2 * tk.n : tk.n, live);      // (a pair: two items a tile)
+  // which kernel: see k_bsattn_fwd_rows64
+  __shared__ int tiles[2];
+  if (threadIdx.x < 2) tiles[threadIdx.x] = 0;
+  __syncthreads();
+  int all = 0, paired = 0;
+  for (int i = threadIdx.x; i < n_parts; i += kTailTasks) { all += pick[2 + 2 * i]; paired += pick[3 + 2 * i]; }
+  all = __reduce_add_sync(0xffffffffu, all);
+  paired = __reduce_add_sync(0xffffffffu, paired);
+  if ((threadIdx.x & 31) == 0) { atomicAdd(&tiles[0], all); atomicAdd(&tiles[1], paired); }
+  __syncthreads();
+  const bool pairs = 100ll * tiles[1] > (long long)share * tiles[0];
+  if (threadIdx.x == 0) pick[0] = pairs;
+  const int at = tail_place(tk.row2 >= 0 && !pairs ? 2 * tk.n : tk.n, live);      // (a pair: two items a tile)
   if (live) table[p.first_tail + at] = tk;
 }
 
@@ -2051,7 +2094,9 @@ __global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* ta
 // before the block's own (a thread each, so the block reads the row lengths of its head once).  One thread
 // per row that counted and compared alone took 488 us on 32 heads of 1536 rows, a tenth of them full.
 constexpr int kPairRows = 64, kPairThreads = 256;
-__global__ void __launch_bounds__(kPairThreads) k_task_table_pairs(AttnParams p, Task* table, int chunks) {
+// COUNT: also the tiles in all and of pairs, for k_sort_tail (a test in the kernel instead took calls of 80 short rows from 18.6 to 19.7 us)
+template <bool COUNT>
+__global__ void __launch_bounds__(kPairThreads) k_task_table_pairs(AttnParams p, Task* table, int* pick, int chunks) {
   __shared__ int s_row[kPairRows], s_lo[kPairRows], s_len[kPairRows];      // (len -1: takes no part)
   __shared__ int s_mate[kPairRows];                 // list start of the candidate partner, -1: none
   __shared__ int s_mate_row[kPairRows], s_mate_pos[kPairRows], s_same[kPairRows];   // its row; its position here, -1: elsewhere
@@ -2137,8 +2182,7 @@ __global__ void __launch_bounds__(kPairThreads) k_task_table_pairs(AttnParams p,
     if (lane == 0) { s_same[e] = same; if (mpos >= 0) s_same[mpos] = same; }
   }
   __syncthreads();
-  if (!live) return;
-  if (s_same[tid]) {
+  if (live && s_same[tid]) {
     const int mpos = s_mate_pos[tid];
     // the first of the two in the order: partners elsewhere stand before (odd number) or behind (even)
     bool first = mpos > tid;
@@ -2151,7 +2195,14 @@ __global__ void __launch_bounds__(kPairThreads) k_task_table_pairs(AttnParams p,
     else tk.n = kAbsorbed;
   }
   tk.pad2 = 0;
-  table[p.interleaved ? (long long)pos * p.heads + h : (long long)hb + pos] = tk;
+  if (live) table[p.interleaved ? (long long)pos * p.heads + h : (long long)hb + pos] = tk;
+  if constexpr (!COUNT) return;
+  if (tid < kPairRows) {
+    const int n = live ? max(tk.n, 0) : 0, all = __reduce_add_sync(0xffffffffu, n), paired = __reduce_add_sync(0xffffffffu, tk.row2 >= 0 ? n : 0);
+    if (lane == 0) { s_lo[warp] = all; s_len[warp] = paired; }
+  }
+  __syncthreads();
+  if (tid == 0) { pick[2 + 2 * blockIdx.x] = s_lo[0] + s_lo[1]; pick[3 + 2 * blockIdx.x] = s_len[0] + s_len[1]; }
 }
 
 // ------------------------------------------------------------------ host side
@@ -2227,14 +2278,12 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
     if ((s = make_map(&tv2, V, D, d->seq_kv, d->heads, d->v_stride[0], d->v_stride[1], 128, "V (128-row boxes)")) != WAVEAL_OK) return s;
     to = tq;
   }
-  if constexpr (BLOCK == 64)
-    WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd_rows64<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Geo64<D>::SMEM_BYTES));
-  else
-    WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd<BLOCK, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES));
+  WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd<BLOCK, D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES));
   WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd<BLOCK, D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES));
   long long grid = p.total_tasks < sms ? p.total_tasks : sms;
   Task* table = reinterpret_cast<Task*>(reinterpret_cast<char*>(p.ws) + table_offset(p.total_tasks));
   p.table = table;
+  int* pick = nullptr;
   p.redo_pass = 0;
   p.wait_limit = kTimeoutCycles;
   p.drop_tile = 0;
@@ -2251,10 +2300,12 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   int launches = 1;
   if (BLOCK == 64) {
     const int chunks = (p.m_b + kPairRows - 1) / kPairRows;
-    k_task_table_pairs<<<(unsigned)((long long)p.heads * chunks), kPairThreads, 0, st>>>(p, table, chunks);
-    if (p.total_tasks > sms) {            // (else all tasks start at once)
+    if (p.total_tasks > sms) pick = reinterpret_cast<int*>(table + p.total_tasks);
+    if (pick) k_task_table_pairs<true><<<(unsigned)((long long)p.heads * chunks), kPairThreads, 0, st>>>(p, table, pick, chunks);
+    else k_task_table_pairs<false><<<(unsigned)((long long)p.heads * chunks), kPairThreads, 0, st>>>(p, table, pick, chunks);
+    if (pick) {                           // (else all tasks start at once)
       WAVEAL_CUDA_OK(cudaGetLastError());
-      WAVEAL_CUDA_OK(waveal::launch_chained(k_sort_tail, dim3(1), kTailTasks, 0, st, p, table));
+      WAVEAL_CUDA_OK(waveal::launch_chained(k_sort_tail, dim3(1), kTailTasks, 0, st, p, table, pick, p.heads * chunks, D == 128 ? 47 : 64));
       ++launches;
     }
   } else {
@@ -2270,9 +2321,18 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   // first pass: reference fixed after the first tile of a task; second pass: the tasks the
   // first one listed (normally none: its CTAs leave at once), max of every block
   p.redo_pass = 0;
-  if constexpr (BLOCK == 64)
-    WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd_rows64<D>, dim3((unsigned)grid), kThreads64, Geo64<D>::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, p));
-  else
+  if constexpr (BLOCK == 64) {
+    // Calls of no more tasks than SMs run as their longest task does, with products of 128 rows; of the others k_sort_tail
+    // says which kernel is quicker, and the other one leaves at once.
+    if (pick) {
+      WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd_rows64<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Geo64<D>::SMEM_BYTES));
+      WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd_rows64<D>, dim3((unsigned)grid), kThreads64, Geo64<D>::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, p));
+      WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd<64, D, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES));
+      WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<64, D, true, true>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, to, p));
+      ++launches;
+    }
+  }
+  if (!pick)
     WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, true>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, to, p));
   p.redo_pass = 1;
   p.direct = 0;
@@ -2290,7 +2350,9 @@ extern "C" waveal_status waveal_bsattn_workspace_bytes(const waveal_attn_desc* d
   // 32 bytes of counters and flags, one (head, query block) pair per task for the redo list,
   // then the 32-byte task of every ticket
   const long long tasks = (long long)desc->heads * ((desc->seq_q + desc->block_q - 1) / desc->block_q);
-  *bytes = (size_t)((table_offset(tasks) + 32 * tasks + 255) / 256 * 256);
+  // (64-row blocks: and two counts of every 64 positions of a head)
+  const long long parts = desc->block_q == 64 ? 8 + (long long)desc->heads * ((desc->seq_q + 64 * kPairRows - 1) / (64 * kPairRows)) * 8 : 0;
+  *bytes = (size_t)((table_offset(tasks) + 32 * tasks + parts + 255) / 256 * 256);
   return WAVEAL_OK;
 }
 

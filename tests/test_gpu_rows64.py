@@ -65,6 +65,33 @@ def test_items_of_single_and_shared_blocks(D, nb, cut):
         assert ((lse[0, rows].double() - s.logsumexp(-1)).abs() <= 1.5e-4).all(), i
 
 
+# pairs have all of the tiles, half or a few of them: products of 128 rows or of 64, with the same bits as the blocks on their own
+@pytest.mark.parametrize("D", [128, 64])
+@pytest.mark.parametrize("full", [200, 80, 12])
+def test_either_kernel_gives_the_same_bits(D, full):
+    nb = 200
+    g = torch.Generator().manual_seed(full)
+    lists = [torch.arange(nb) if i < full else torch.randperm(nb, generator=g)[:40 + i % 7].sort().values for i in range(nb)]
+    ptr = torch.tensor([0] + [len(l) for l in lists]).cumsum(0).int().cuda()
+    gg = torch.Generator("cuda")
+    gg.manual_seed(full)
+    T = nb * 64 - 21
+    q, k, v = (torch.randn((1, nb * 64, D), generator=gg, device="cuda").to(torch.bfloat16) for _ in range(3))
+    idx = torch.cat(lists).int().cuda()
+    o, lse, w, st = _call(q, k, v, ptr, idx, T)
+    alone, lse_alone, w_alone, _ = _call(q, k, v, ptr, idx, T, flags=wb.ATTN_NO_ROW_PAIRING)
+    assert st == [0] * 4 and w[6] == full // 2 and w_alone[6] == 0 and w[7] == w_alone[7] - full // 2 * nb // 2
+    assert torch.equal(o[:, :T], alone[:, :T]) and torch.equal(lse, lse_alone)
+    for i in (0, 1, full - 1, min(full, nb - 1), nb - 1):
+        rows = slice(i * 64, min((i + 1) * 64, T))
+        sel = (lists[i][:, None] * 64 + torch.arange(64)).flatten().cuda()
+        sel = sel[sel < T]
+        p = (q[0, rows].double() @ k[0, sel].double().T / D ** 0.5).softmax(-1)
+        ref = p @ v[0, sel].double()
+        bound = 2.0 ** -8 * (p @ v[0, sel].double().abs()) + 2.0 ** -8 * ref.abs() + 1e-6      # as in the test above
+        assert ((o[0, rows].double() - ref).abs() <= bound).all(), i
+
+
 @pytest.mark.parametrize("D", [128, 64])
 def test_a_tile_that_never_comes(D):
     q, k, v, ptr, idx, lists, T = _case(D, 400, 17, 5)
