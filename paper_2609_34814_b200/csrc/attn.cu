@@ -1398,12 +1398,14 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 // which the group of a block's last item runs while the others go on.
 // Which kernel a call takes: two blocks that share their tiles (a pair) fill a product of 128 rows, which takes 1,327 clk a tile
 // (1,140 at head_dim 64) against their two items' 1,770 (1,370), a lone block's tile as long against its item's 886
-// (735): products of 64 rows are quicker until pairs have 47 % (64 %) of the tiles.  k_sort_tail, which has the counts, picks; the kernel not
-// picked leaves at once (~3 us).  (8 heads of the LTX recipe, a quarter: 11.2 -> 9.3 ms; 2 dense heads of 512 rows, all: 892 us with the
-// one, 1,100 with the other.)  Calls of no more tasks than SMs last as long as their longest task and stay with products of 128 rows.
+// (735): products of 64 rows are quicker until pairs have 47 % (64 %) of the tiles, or the longest pair outlasts an SM's share of the
+// work.  k_sort_tail, which has the counts, picks; the kernel not picked leaves at once (~3 us).  (8 heads of the LTX recipe, a quarter: 11.2 -> 9.3 ms; 2 dense heads of 512 rows, all: 892 us with the
+// one, 1,100 with the other.)  Calls of no more tasks than SMs last as long as their longest task and stay with products of 128
+// rows, and so do small ones (launch()).
 // Pairs: two blocks with the very same list are items 2 i and 2 i + 1 of tile i, each with an accumulator of its own.  Everything a row
 // sees is as it would be alone: the products in the same order, a reference from the same first 128 keys, and the same
 // sums, which a lone block has by tile mod 4 (its groups) and a pair's groups keep two of.
+constexpr long long kRows64Tiles = 320;              // tiles an SM that the lists of a call may have, from which this kernel is launched
 constexpr int kThreads64 = 704, kLoadWarps64 = 20;   // 22 warps: those of the kernel above and two more loaders
 
 template <int D>
@@ -2057,26 +2059,36 @@ __global__ void __launch_bounds__(kTailTasks) k_task_table(AttnParams p, int blo
 }
 
 // the same for a table that is there already (64-row blocks: pairs are formed first)
-__global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* table, int* pick, int n_parts, int share) {
+template <bool PICK>
+__global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* table, int* pick, int n_parts, int d, int sms) {
   waveal::let_next_kernel_start();
   waveal::wait_for_previous_kernel();
   const long long t = p.first_tail + threadIdx.x;
   const bool live = t < p.total_tasks;
   Task tk{};
   if (live) tk = table[t];
-  // which kernel: see k_bsattn_fwd_rows64
-  __shared__ int tiles[2];
-  if (threadIdx.x < 2) tiles[threadIdx.x] = 0;
-  __syncthreads();
-  int all = 0, paired = 0;
-  for (int i = threadIdx.x; i < n_parts; i += kTailTasks) { all += pick[2 + 2 * i]; paired += pick[3 + 2 * i]; }
-  all = __reduce_add_sync(0xffffffffu, all);
-  paired = __reduce_add_sync(0xffffffffu, paired);
-  if ((threadIdx.x & 31) == 0) { atomicAdd(&tiles[0], all); atomicAdd(&tiles[1], paired); }
-  __syncthreads();
-  const bool pairs = 100ll * tiles[1] > (long long)share * tiles[0];
-  if (threadIdx.x == 0) pick[0] = pairs;
-  const int at = tail_place(tk.row2 >= 0 && !pairs ? 2 * tk.n : tk.n, live);      // (a pair: two items a tile)
+  int n = tk.n;
+  if constexpr (PICK) {
+    // which kernel: see k_bsattn_fwd_rows64.  Either takes as long as its share of the work an SM, or its longest task (of
+    // the last 1,024, all of a call where that matters)
+    __shared__ int tiles[4];                          // in all, of pairs, of the longest block on its own and pair
+    if (threadIdx.x < 4) tiles[threadIdx.x] = 0;
+    __syncthreads();
+    int all = 0, paired = 0;
+    for (int i = threadIdx.x; i < n_parts; i += kTailTasks) { all += pick[2 + 2 * i]; paired += pick[3 + 2 * i]; }
+    all = __reduce_add_sync(0xffffffffu, all);
+    paired = __reduce_add_sync(0xffffffffu, paired);
+    const bool pair = live && tk.row2 >= 0;
+    const int lone_n = __reduce_max_sync(0xffffffffu, pair ? 0 : max(tk.n, 0)), pair_n = __reduce_max_sync(0xffffffffu, pair ? tk.n : 0);
+    if ((threadIdx.x & 31) == 0) { atomicAdd(&tiles[0], all); atomicAdd(&tiles[1], paired); atomicMax(&tiles[2], lone_n); atomicMax(&tiles[3], pair_n); }
+    __syncthreads();
+    const long long c128 = d == 128 ? 1327 : 1140, c_lone = d == 128 ? 886 : 735, c_pair = d == 128 ? 1772 : 1372;
+    const long long t128 = max(c128 * tiles[0] / sms, c128 * max(tiles[2], tiles[3]));
+    const long long t64 = max((c_lone * (tiles[0] - tiles[1]) + c_pair * tiles[1]) / sms, max(c_lone * tiles[2], c_pair * tiles[3]));
+    if (threadIdx.x == 0) pick[0] = t128 < t64;
+    if (pair && t128 >= t64) n *= 2;                  // (a pair: two items a tile)
+  }
+  const int at = tail_place(n, live);
   if (live) table[p.first_tail + at] = tk;
 }
 
@@ -2300,12 +2312,17 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   int launches = 1;
   if (BLOCK == 64) {
     const int chunks = (p.m_b + kPairRows - 1) / kPairRows;
-    if (p.total_tasks > sms) pick = reinterpret_cast<int*>(table + p.total_tasks);
+    // (The kernel not picked is ~3 us more of launches, worth it from a few thousand cycles of work an SM on, of which the host knows
+    // only the most that a mask can select.  us a call with one kernel / the other, by that many tiles an SM: 17: 28.7 / 31.4,
+    // 140: 51.6 / 59.6, 249: 71.8 / 72.5, 280: 75.8 / 90.2 and 81.8 / 67.7, 324: 49.4 / 47.1, 331: 68.9 / 64.4, 373: 100 / 89,
+    // 553: 144 / 111, 622: 155 / 132, 648: 72.6 / 67.7)
+    const bool many = p.total_tasks > sms;            // (else all tasks start at once)
+    if (many && p.total_tasks * ((p.n_b + 1) / 2) >= kRows64Tiles * sms) pick = reinterpret_cast<int*>(table + p.total_tasks);
     if (pick) k_task_table_pairs<true><<<(unsigned)((long long)p.heads * chunks), kPairThreads, 0, st>>>(p, table, pick, chunks);
     else k_task_table_pairs<false><<<(unsigned)((long long)p.heads * chunks), kPairThreads, 0, st>>>(p, table, pick, chunks);
-    if (pick) {                           // (else all tasks start at once)
+    if (many) {
       WAVEAL_CUDA_OK(cudaGetLastError());
-      WAVEAL_CUDA_OK(waveal::launch_chained(k_sort_tail, dim3(1), kTailTasks, 0, st, p, table, pick, p.heads * chunks, D == 128 ? 47 : 64));
+      WAVEAL_CUDA_OK(waveal::launch_chained(pick ? k_sort_tail<true> : k_sort_tail<false>, dim3(1), kTailTasks, 0, st, p, table, pick, p.heads * chunks, D, sms));
       ++launches;
     }
   } else {
@@ -2322,8 +2339,7 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   // first one listed (normally none: its CTAs leave at once), max of every block
   p.redo_pass = 0;
   if constexpr (BLOCK == 64) {
-    // Calls of no more tasks than SMs run as their longest task does, with products of 128 rows; of the others k_sort_tail
-    // says which kernel is quicker, and the other one leaves at once.
+    // k_sort_tail says which kernel is quicker; the other one leaves at once
     if (pick) {
       WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd_rows64<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Geo64<D>::SMEM_BYTES));
       WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd_rows64<D>, dim3((unsigned)grid), kThreads64, Geo64<D>::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, p));

@@ -37,7 +37,7 @@ def _case(D, nb, cut, seed):
 
 
 @pytest.mark.parametrize("D", [128, 64])
-@pytest.mark.parametrize("nb,cut", [(3, 1), (90, 63), (700, 0), (701, 40)])
+@pytest.mark.parametrize("nb,cut", [(3, 1), (90, 63), (310, 1), (700, 0), (701, 40)])
 def test_items_of_single_and_shared_blocks(D, nb, cut):
     q, k, v, ptr, idx, lists, T = _case(D, nb, cut, nb + D)
     o, lse, w, st = _call(q, k, v, ptr, idx, T)
@@ -67,10 +67,9 @@ def test_items_of_single_and_shared_blocks(D, nb, cut):
 
 # pairs have all of the tiles, half or a few of them: products of 128 rows or of 64, with the same bits as the blocks on their own
 @pytest.mark.parametrize("D", [128, 64])
-@pytest.mark.parametrize("full", [200, 80, 12])
-def test_either_kernel_gives_the_same_bits(D, full):
-    nb = 200
-    g = torch.Generator().manual_seed(full)
+@pytest.mark.parametrize("nb,full", [(320, 320), (320, 120), (320, 12), (200, 80)])
+def test_either_kernel_gives_the_same_bits(D, nb, full):
+    g = torch.Generator().manual_seed(full)                   # (320 rows: up to 346 tiles an SM, 200: 135)
     lists = [torch.arange(nb) if i < full else torch.randperm(nb, generator=g)[:40 + i % 7].sort().values for i in range(nb)]
     ptr = torch.tensor([0] + [len(l) for l in lists]).cumsum(0).int().cuda()
     gg = torch.Generator("cuda")
@@ -94,7 +93,7 @@ def test_either_kernel_gives_the_same_bits(D, full):
 
 @pytest.mark.parametrize("D", [128, 64])
 def test_a_tile_that_never_comes(D):
-    q, k, v, ptr, idx, lists, T = _case(D, 400, 17, 5)
+    q, k, v, ptr, idx, lists, T = _case(D, 400, 17, 5)        # (541 tiles an SM: products of 64 rows)
     good, _, _, st = _call(q, k, v, ptr, idx, T)
     assert st == [0] * 4
     t0 = time.perf_counter()
