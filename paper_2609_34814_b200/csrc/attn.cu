@@ -8,7 +8,7 @@
 // SM, take tickets from a global counter, so a freed SM starts the next row of the list at
 // once - the streaming "wave" behaviour of Section 2.3 that the schedule is built for.
 //
-// Structure of one CTA (640 threads; the first launch of 64-row blocks has a kernel of its own, k_bsattn_fwd_rows64):
+// Structure of one CTA (640 threads; calls of many 64-row blocks have k_bsattn_fwd_rows64 as their first launch):
 //   warp 0      producer: takes tickets, publishes tasks, issues TMA loads of the Q tile and of the K
 //               tiles (128-byte-swizzled slabs) into shared-memory rings, as far ahead as the rings allow
 //   warp 19     requests the V tiles (a box costs the warp that requests it ~150 clk)
@@ -353,7 +353,7 @@ __host__ __device__ constexpr uint32_t make_idesc(int m, int n, bool b_mn_major)
 // n: KV tiles of the task (a tile = 128 keys = 128/block consecutive entries of the row's list),
 // len: entries of the list, tail_valid: keys of the last tile that exist.
 // row2 (64-row query blocks only): a second query block with the very same list, or -1; its rows
-// fill the other half of the 128-row MMA tile, so the pair costs what one block costs.  The
+// fill the other half of a 128-row product, so the pair costs what one block costs there.  The
 // ticket of the second block of a pair carries n = kAbsorbed and is skipped by whoever draws it.
 struct Task { int h, row, lo, n, tail_valid, len, row2, pad2; };
 constexpr int kAbsorbed = -2;
@@ -2092,7 +2092,7 @@ __global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* ta
   if (live) table[p.first_tail + at] = tk;
 }
 
-// The same for 64-row query blocks, where two blocks with the very same list share one 128-row tile.
+// The same for 64-row query blocks, where two blocks with the very same list share their tiles.
 // Candidates:
 //  - rows that select every KV block (list length = N_B: rows that attend to everything), wherever
 //    they stand: the 1st and 2nd, the 3rd and 4th, ... such row of the head's order form pairs,
