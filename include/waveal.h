@@ -230,6 +230,7 @@ waveal_status waveal_bsattn_workspace_bytes(const waveal_attn_desc* desc /*host*
  * more blocks than that runs in this order alone, whatever row_order and order_heads_interleaved say, but for the first
  * ticket of every SM with 128-row blocks and at least two blocks an SM); each output
  * tile is written at its original rows, so no inverse permutation pass exists.
+ * A head has the same bits alone and among any number of others, whichever kernels a call of that size takes.
  * Q, K, V, O: dev bf16, 16-byte aligned, strides multiples of 8 elements, head_dim
  * contiguous; query tokens >= seq_q are not written; keys >= seq_kv are ignored.
  * lse: dev float [heads][seq_q] or NULL (natural-log sum-exp per query token; -inf for a

@@ -385,6 +385,8 @@ struct AttnParams {
                       // the redo pass, [8 + 2i], [9 + 2i] = (head, query block) of redo entry i
   int redo_pass;      // 0: all tasks by ticket; 1: only the tasks the first pass listed
   const Task* table;         // task of every ticket of the first pass (k_task_table)
+  const int* pick;           // large calls of 64-row blocks, else null: [0] 1: products of 128 rows for this call, 0: of 64 (k_sort_tail);
+                             // [2 + 2i], [3 + 2i]: tiles in all and of pairs in block i of k_task_table_pairs
   int direct;         // CTAs that take the ticket of their own number before the table is there (0: none, else the grid)
   long long first_tail;      // tickets before this one are in the caller's order, the rest longest first
   int* dev_status;
@@ -397,10 +399,6 @@ struct AttnParams {
   float sl2;          // scale * log2(e)
 };
 
-
-// 64-row blocks, behind the table: [0] 1: products of 128 rows for this call, 0: of 64 (k_sort_tail); [2 + 2i], [3 + 2i]: tiles in all
-// and of pairs in block i of k_task_table_pairs
-__device__ __forceinline__ const int* pick_word(const AttnParams& p) { return reinterpret_cast<const int*>(p.table + p.total_tasks); }
 
 // Task of every ticket (head-major or position-major over the planned order), so that the
 // persistent CTAs need one load behind a ticket instead of a chain through row_order, the row
@@ -618,9 +616,9 @@ __device__ __noinline__ void list_task_call(int* ws, int* listed, int task_no, i
   list_task(ws, listed, task_no, h, row, row2);
 }
 
-// MOD4 (64-row blocks, first launch): the row sums by tile mod 4, as k_bsattn_fwd_rows64 has them, whose place this kernel takes in
-// calls of many pairs: the same bits, whichever of the two runs
-template <int BLOCK, int D, bool FAST, bool MOD4 = false>
+// First launch of 64-row blocks: this kernel does small calls and, where k_sort_tail picks it, large ones, all others are
+// k_bsattn_fwd_rows64's.  It sums the rows by tile mod 4 as that one does, so that a head has the same bits in every call.
+template <int BLOCK, int D, bool FAST>
 __global__ void __launch_bounds__(kThreads, 1)
 k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
              const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmK2,
@@ -629,6 +627,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   // two blocks of a tile lie next to each other in memory (for 128-key blocks they equal tmK / tmV).
   // tmO: O in boxes of 32 rows and half of head_dim, what a warp stores (128-row blocks only)
   using G = Geo<BLOCK, D>;
+  constexpr bool MOD4 = FAST && BLOCK == 64;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   const uint32_t sbase = smem_u32(smem);
@@ -639,10 +638,10 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 
   // second pass with nothing listed (or after an abort): leave before anything is set up
   if (p.redo_pass && (p.ws[2] == 0 || p.ws[1] != 0)) return;
-  // 64-row blocks of a call that k_bsattn_fwd_rows64 has done
-  if (MOD4) {
+  // a call that k_bsattn_fwd_rows64 has done
+  if (MOD4 && p.pick) {
     waveal::wait_for_previous_kernel();
-    if (*pick_word(p) == 0 || p.ws[1] != 0) return;
+    if (*p.pick == 0 || p.ws[1] != 0) return;
   }
 
   const uint32_t bar0 = sbase + G::OFF_BAR;
@@ -1590,7 +1589,7 @@ k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     TileLoader<G, true> k_tiles{0};
     int n_tiles = 0, n_pairs = 0;        // words 7 and 6 of the workspace
     bool ok = true;
-    const bool mine = *pick_word(p) == 0;
+    const bool mine = *p.pick == 0;
     auto draw = [&](long long& t_out) -> Task {
       for (;;) {
         long long t = 0;
@@ -1992,7 +1991,7 @@ k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     tc_fence_after();
     tmem_dealloc(tmem_base, G::TMEM_COLS);
   }
-  if (tid == 0 && *pick_word(p) == 0) {
+  if (tid == 0 && *p.pick == 0) {
     const long long dt = clock64() - t_start;
     atomicMax(&p.ws[4], (int)(dt > 0x7fffffffll ? 0x7fffffffll : dt));
   }
@@ -2298,6 +2297,7 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   Task* table = reinterpret_cast<Task*>(reinterpret_cast<char*>(p.ws) + table_offset(p.total_tasks));
   p.table = table;
   int* pick = nullptr;
+  p.pick = nullptr;
   p.redo_pass = 0;
   p.wait_limit = kTimeoutCycles;
   p.drop_tile = 0;
@@ -2342,16 +2342,14 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   p.redo_pass = 0;
   if constexpr (BLOCK == 64) {
     // k_sort_tail says which kernel is quicker; the other one leaves at once
+    p.pick = pick;
     if (pick) {
       WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd_rows64<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Geo64<D>::SMEM_BYTES));
       WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd_rows64<D>, dim3((unsigned)grid), kThreads64, Geo64<D>::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, p));
-      WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd<64, D, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, G::SMEM_BYTES));
-      WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<64, D, true, true>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, to, p));
       ++launches;
     }
   }
-  if (!pick)
-    WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, true>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, to, p));
+  WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, true>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, to, p));
   p.redo_pass = 1;
   p.direct = 0;
   WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd<BLOCK, D, false>, dim3((unsigned)grid), kThreads, G::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, to, p));

@@ -91,6 +91,24 @@ def test_either_kernel_gives_the_same_bits(D, nb, full):
         assert ((o[0, rows].double() - ref).abs() <= bound).all(), i
 
 
+# calls on either side of the number of tiles from which the choice of kernel is made on the device, and of as many blocks as SMs
+@pytest.mark.parametrize("D", [128, 64])
+@pytest.mark.parametrize("nb,heads", [(100, 9), (200, 4)])
+def test_a_head_has_the_same_bits_in_every_call(D, nb, heads):
+    _, _, _, ptr, idx, lists, T = _case(D, nb, 13, nb + D)
+    g = torch.Generator("cuda")
+    g.manual_seed(nb)
+    q, k, v = (torch.randn((heads, nb * 64, D), generator=g, device="cuda").to(torch.bfloat16) for _ in range(3))
+    n = ptr[-1]
+    all_ptr = torch.cat([ptr[:1]] + [ptr[1:] + h * n for h in range(heads)])
+    o, lse, w, st = _call(q, k, v, all_ptr, idx.repeat(heads), T)
+    assert st == [0] * 4 and w[2] == 0
+    for h in range(heads):
+        one, lse_one, w, st = _call(q[h:h + 1], k[h:h + 1], v[h:h + 1], ptr, idx, T)
+        assert st == [0] * 4 and w[2] == 0
+        assert torch.equal(one[0, :T], o[h, :T]) and torch.equal(lse_one[0], lse[h]), h
+
+
 @pytest.mark.parametrize("D", [128, 64])
 def test_a_tile_that_never_comes(D):
     q, k, v, ptr, idx, lists, T = _case(D, 400, 17, 5)        # (541 tiles an SM: products of 64 rows)
