@@ -42,7 +42,11 @@ constexpr int kMaxMerge = (kSmemMax - 2048) / 24;     // rows whose two sort buf
 // whether all are in range, and sets a bit for each (lanes of an ascending list then mostly have words of their own).
 // Collecting the bits of a word in a register first, with the branches that takes, and entry by entry range checks: 45 us for the
 // 19.7 M entries of 49,152 rows, now 27.  A run that sticks out of the row reads the row's first or last entry again instead.
+// PIECES: rows of more than kCsrCols columns, which read their list once a piece; most runs of an ascending list lie in one piece,
+// in front of it or behind it, and the others keep their eight entries in registers too (2,048 rows of 16,384 columns, a tenth
+// set: 8.0 us, with the entries loaded again one by one 20.7).  The form for one piece does not carry the offset.
 constexpr int kCsrCols = 8192, kCsrWarps = 8;
+template <bool PIECES>
 __global__ void __launch_bounds__(kCsrWarps * 32) k_csr_to_bitmap(const int* __restrict__ row_ptr, const int* __restrict__ idx,
                                                                   u64* __restrict__ bits, long long n_rows, int wq, int n_kv,
                                                                   int m_b, int* __restrict__ nnz, int* __restrict__ nnz_out,
@@ -73,24 +77,36 @@ __global__ void __launch_bounds__(kCsrWarps * 32) k_csr_to_bitmap(const int* __r
 #pragma unroll
         for (int i = 0; i < kRun; ++i) j[i] = list[min(max(e + i, 0), len - 1)];
       }
-      unsigned top = 0;
+      auto set = [&](int v) { atomicOr(&my[(PIECES ? v - c0 : v) >> 5], 1u << (v & 31)); };
+      auto report = [&](int v) {
+        if (c0 == 0 && dev_status && atomicCAS(dev_status, 0, WAVEAL_ERR_BAD_MASK) == 0) {
+          dev_status[1] = 1; dev_status[2] = (int)(row / m_b); dev_status[3] = v;
+        }
+      };
+      unsigned top = 0, bottom = ~0u, entry = 0;     // positions in this piece, and the entries themselves
 #pragma unroll
-      for (int i = 0; i < kRun; ++i) top = max(top, (unsigned)j[i]);
-      if (top < (unsigned)cols && c0 == 0) {
+      for (int i = 0; i < kRun; ++i) {
+        const unsigned k = (unsigned)j[i] - (PIECES ? (unsigned)c0 : 0u);
+        top = max(top, k);
+        if (PIECES) { bottom = min(bottom, k); entry = max(entry, (unsigned)j[i]); }
+      }
+      if (top < (unsigned)cols) {
 #pragma unroll
-        for (int i = 0; i < kRun; ++i) atomicOr(&my[j[i] >> 5], 1u << (j[i] & 31));
-      } else {                                       // a row of several pieces, or an entry out of range
+        for (int i = 0; i < kRun; ++i) set(j[i]);
+      } else if (PIECES) {
+        if (bottom < (unsigned)cols || entry >= (unsigned)n_kv) {      // (else all eight belong to other pieces)
+#pragma unroll
+          for (int i = 0; i < kRun; ++i) {
+            if ((unsigned)j[i] - (unsigned)c0 < (unsigned)cols) set(j[i]);
+            else if ((unsigned)j[i] >= (unsigned)n_kv) report(j[i]);
+          }
+        }
+      } else {                                       // an entry out of range
 #pragma unroll 1
         for (int i = 0; i < kRun; ++i) {
           const int v = list[min(max(e + i, 0), len - 1)];
-          const unsigned k = (unsigned)(v - c0);
-          if (v < 0 || v >= n_kv) {
-            if (c0 == 0 && dev_status && atomicCAS(dev_status, 0, WAVEAL_ERR_BAD_MASK) == 0) {
-              dev_status[1] = 1; dev_status[2] = (int)(row / m_b); dev_status[3] = v;
-            }
-          } else if (k < (unsigned)cols) {
-            atomicOr(&my[k >> 5], 1u << (k & 31));
-          }
+          if ((unsigned)v < (unsigned)n_kv) set(v);
+          else report(v);
         }
       }
     }
@@ -1401,7 +1417,7 @@ waveal_status plan_common(const waveal_plan_desc* d, const u64* mask_bits, const
   if (!M) {
     u64* bm = reinterpret_cast<u64*>(w + L.off_bitmap);
     long long rows = (long long)(H * m);
-    k_csr_to_bitmap<<<(unsigned)((rows + kCsrWarps - 1) / kCsrWarps), kCsrWarps * 32, 0, st>>>(
+    (n <= kCsrCols ? k_csr_to_bitmap<false> : k_csr_to_bitmap<true>)<<<(unsigned)((rows + kCsrWarps - 1) / kCsrWarps), kCsrWarps * 32, 0, st>>>(
         row_ptr, idx, bm, rows, L.wq, (int)n, (int)m, reinterpret_cast<int*>(w + L.off_nnz), out->row_nnz, out->dev_status);
     ++launches;
     M = bm;

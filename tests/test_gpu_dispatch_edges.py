@@ -209,6 +209,30 @@ def test_list_conversions(H, m, n):
         assert torch.equal(a.col_count, b.col_count) and torch.equal(a.row_nnz, b.row_nnz) and a.dev_status.tolist() == [0] * 4
 
 
+# one piece of 8,192 columns, and rows of two and three: runs of eight entries inside a piece, across its end, repeated, descending
+# and with entries out of range in them
+@pytest.mark.parametrize("n", [8191, 8192, 8193, 16384, 20000])
+def test_lists_of_any_order_with_entries_out_of_range(n):
+    rng = np.random.default_rng(n)
+    bad = np.array([-1, n, n + 5, -2 ** 31, 2 ** 31 - 1])
+    lists = [rng.permutation(n)[:1000], np.arange(n), np.arange(n)[::-1], np.repeat(rng.integers(0, n, 50), 3), [], [n - 1],
+             np.arange(max(0, 8192 - 21), min(n, 8192 + 20)), np.concatenate([rng.integers(0, n, 101), bad, rng.integers(0, n, 7)]),
+             np.insert(np.sort(rng.permutation(n)[:300]), [0, 13, 100, 299, 300], bad)]
+    lists = [np.asarray(l, dtype=np.int64) for l in lists]
+    mask = np.zeros((len(lists), n), dtype=bool)
+    for i, l in enumerate(lists):
+        mask[i, l[(l >= 0) & (l < n)]] = True
+    d = wb.plan_desc_default(heads=1, n_q_blocks=len(lists), n_kv_blocks=n, wave_size=148, mode=wb.FORCE_NATURAL)
+    for keep in (lists[:7] + [np.zeros(0, np.int64)] * 2, lists):
+        ptr = torch.tensor([0] + [len(l) for l in keep]).cumsum(0).int().cuda()
+        r = wb.plan_csr(d, ptr, torch.from_numpy(np.concatenate(keep)).int().cuda(), debug=True)
+        rows = 7 if keep is not lists else 9
+        assert r.row_nnz[0, :rows].tolist() == mask[:rows].sum(1).tolist()
+        assert np.array_equal(r.col_count[0].cpu().numpy(), mask[:rows].sum(0))
+        st = r.dev_status.tolist()
+        assert st == [0] * 4 if rows == 7 else (st[:3] == [wb.ERR_BAD_MASK, 1, 0] and st[3] in bad)
+
+
 def test_host_threads_plan_different_sizes():
     """A small plan must not take from a large one, between that one's set-up and its launches, the shared
     memory they need."""
