@@ -132,9 +132,24 @@ __device__ __forceinline__ void tc_commit(uint32_t bar) {   // whole warp calls;
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // D[tmem] (+)= A[smem] * B[smem], bf16 inputs, fp32 accumulate, one CTA: four of them along K, 32 bytes of A and B further each.
-// (One election for the four instead of one each: 0.6 to 1.2 % of the cycles of 128-row calls, 488 k -> 484 k on 5 heads of 256
-// rows, 2,059 k -> 2,035 k on 3 dense heads.  For the products with A in tensor memory, below, it lost 3 %.)
+// ONE: one election for the four instead of one each.  128-row blocks: 0.6 to 1.2 % of the cycles less (488 k -> 484 k on 5 heads of
+// 256 rows, 2,059 k -> 2,035 k on 3 dense heads); 64-row blocks, head_dim 128: 1 to 2 % more (300.3 k -> 306.7 k on 300 rows of 150 blocks,
+// 91.4 k -> 93.0 k on 200 of 60; at head_dim 64 the same), so those elect each time.  For the products with A in tensor memory,
+// below, it lost 3 %.
+template <bool ONE>
 __device__ __forceinline__ void umma4_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
+  if constexpr (!ONE) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (elect_one())
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "setp.ne.b32 p, %4, 0;\n\t"
+            "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+            ::"r"(d_tmem), "l"(a_desc + 2 * k), "l"(b_desc + 2 * k), "r"(idesc), "r"(k ? 1u : accumulate)
+            : "memory");
+    return;
+  }
   asm volatile(
       "{\n\t.reg .b32 rx;\n\t.reg .pred e, p, t;\n\t.reg .b64 a, b;\n\t"
       "elect.sync rx|e, 0xFFFFFFFF;\n\tsetp.ne.b32 p, %4, 0;\n\tsetp.eq.b32 t, %3, %3;\n\t"
@@ -897,7 +912,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
           const uint32_t d_s = tmem_base + sb * G::S_STRIDE;
 #pragma unroll
           for (int s = 0; s < G::SLABS; ++s)
-            umma4_bf16(d_s, qdesc + (uint64_t)((s * 128 * 128) >> 4), kd + (uint64_t)((s * G::KV_SLAB_BYTES) >> 4), IDESC_QK, s);
+            umma4_bf16<BLOCK == 128>(d_s, qdesc + (uint64_t)((s * 128 * 128) >> 4), kd + (uint64_t)((s * G::KV_SLAB_BYTES) >> 4), IDESC_QK, s);
           tc_commit(BAR(B_K_EMPTY + k_st));
           tc_commit(BAR(B_S_FULL + sb));
           if (j == n - 1) tc_commit(BAR(B_Q_EMPTY + qb));
