@@ -216,7 +216,8 @@ typedef struct waveal_attn_desc {
  * after its first task could start, number of query-block pairs that shared their tiles, number of 128-key tiles of K and V that the
  * call went through, those of a pair counted once),
  * 8 bytes per (head, query block) for the list of tasks to compute again and
- * 32 bytes per (head, query block) for the table that maps a ticket to its task.  The counters
+ * 32 bytes per (head, query block) for the table that maps a ticket to its task (that table at a multiple of 32
+ * bytes, the whole a multiple of 256).  The counters
  * are live state of the call (tickets are drawn from them): calls that may overlap on the GPU
  * must not share a workspace.  Host-only. */
 waveal_status waveal_bsattn_workspace_bytes(const waveal_attn_desc* desc /*host*/, size_t* bytes /*host*/);

@@ -374,7 +374,9 @@ __host__ __device__ constexpr uint32_t make_idesc(int m, int n, bool b_mn_major)
 // row2 (64-row query blocks only): a second query block with the very same list, or -1; its rows
 // fill the other half of a 128-row product, so the pair costs what one block costs there.  The
 // ticket of the second block of a pair carries n = kAbsorbed and is skipped by whoever draws it.
-struct Task { int h, row, lo, n, tail_valid, len, row2, pad2; };
+// pick: large calls of 64-row blocks, in the table's first entry: 1 if the call runs in products of 128 rows, 0: of 64 (k_sort_tail).
+// Every other entry's is not read.
+struct Task { int h, row, lo, n, tail_valid, len, row2, pick; };
 constexpr int kAbsorbed = -2;
 
 // tiles, list length and valid keys of the last tile from a list of `len` blocks of `block` keys
@@ -400,8 +402,7 @@ struct AttnParams {
                       // the redo pass, [8 + 2i], [9 + 2i] = (head, query block) of redo entry i
   int redo_pass;      // 0: all tasks by ticket; 1: only the tasks the first pass listed
   const Task* table;         // task of every ticket of the first pass (k_task_table)
-  const int* pick;           // large calls of 64-row blocks, else null: [0] 1: products of 128 rows for this call, 0: of 64 (k_sort_tail);
-                             // [2 + 2i], [3 + 2i]: tiles in all and of pairs in block i of k_task_table_pairs
+  const int* pick;           // large calls of 64-row blocks: `pick` of the table's first entry, else null
   int direct;         // CTAs that take the ticket of their own number before the table is there (0: none, else the grid)
   long long first_tail;      // tickets before this one are in the caller's order, the rest longest first
   int* dev_status;
@@ -443,14 +444,14 @@ __device__ __forceinline__ Task make_task(const AttnParams& p, int block_k, int 
     if (last < 0 || last >= p.n_b) { report(33, last); len = 0; }
   }
   fill_tiles(tk, len, block_k, last, p.n_b, p.seq_kv);
-  if (bad) tk.pad2 = 1;                             // takes no part in pairing
+  if (bad) tk.pick = 1;                             // (on its way into the table: takes no part in pairing)
   return tk;
 }
 
 __device__ __forceinline__ Task task_of_ticket(const AttnParams& p, int block_k, long long t) {
   const int h = p.interleaved ? (int)(t % p.heads) : (int)(t / p.m_b), pos = p.interleaved ? (int)(t / p.heads) : (int)(t % p.m_b);
   Task tk = make_task(p, block_k, h, pos);
-  tk.pad2 = 0;
+  tk.pick = 0;
   return tk;
 }
 
@@ -2074,9 +2075,17 @@ __global__ void __launch_bounds__(kTailTasks) k_task_table(AttnParams p, int blo
   }
 }
 
+// 64-row blocks: what k_task_table_pairs<true> leaves k_sort_tail<true> for every 32 positions of a head, tiles in all and of pairs.  It
+// lies where the list of tasks to compute again (8 bytes a task) has its entry for the first of them: that list is empty until the
+// first launch.
+__device__ __forceinline__ int head_parts(const AttnParams& p) { return (p.m_b + 31) / 32; }
+__device__ __forceinline__ int2* part_counts(const AttnParams& p, int h, int pos) {
+  return reinterpret_cast<int2*>(p.ws + 8) + (size_t)h * p.m_b + pos;
+}
+
 // the same for a table that is there already (64-row blocks: pairs are formed first)
 template <bool PICK>
-__global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* table, int* pick, int n_parts, int d, int sms) {
+__global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* table, int d, int sms) {
   waveal::let_next_kernel_start();
   waveal::wait_for_previous_kernel();
   const long long t = p.first_tail + threadIdx.x;
@@ -2084,6 +2093,7 @@ __global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* ta
   Task tk{};
   if (live) tk = table[t];
   int n = tk.n;
+  bool rows128 = false;
   if constexpr (PICK) {
     // which kernel: see k_bsattn_fwd_rows64.  Either takes as long as its share of the work an SM, or its longest task (of
     // the last 1,024, all of a call where that matters)
@@ -2091,7 +2101,11 @@ __global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* ta
     if (threadIdx.x < 4) tiles[threadIdx.x] = 0;
     __syncthreads();
     int all = 0, paired = 0;
-    for (int i = threadIdx.x; i < n_parts; i += kTailTasks) { all += pick[2 + 2 * i]; paired += pick[3 + 2 * i]; }
+    const int per_head = head_parts(p);
+    for (int i = threadIdx.x; i < p.heads * per_head; i += kTailTasks) {
+      const int2 c = *part_counts(p, i / per_head, i % per_head * 32);
+      all += c.x; paired += c.y;
+    }
     all = __reduce_add_sync(0xffffffffu, all);
     paired = __reduce_add_sync(0xffffffffu, paired);
     const bool pair = live && tk.row2 >= 0;
@@ -2101,11 +2115,15 @@ __global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* ta
     const long long c128 = d == 128 ? 1327 : 1140, c_lone = d == 128 ? 886 : 735, c_pair = d == 128 ? 1772 : 1372;
     const long long t128 = max(c128 * tiles[0] / sms, c128 * max(tiles[2], tiles[3]));
     const long long t64 = max((c_lone * (tiles[0] - tiles[1]) + c_pair * tiles[1]) / sms, max(c_lone * tiles[2], c_pair * tiles[3]));
-    if (threadIdx.x == 0) pick[0] = t128 < t64;
-    if (pair && t128 >= t64) n *= 2;                  // (a pair: two items a tile)
+    rows128 = t128 < t64;
+    if (pair && !rows128) n *= 2;                     // (a pair: two items a tile)
   }
   const int at = tail_place(n, live);
   if (live) table[p.first_tail + at] = tk;
+  if constexpr (PICK) {
+    __syncthreads();
+    if (threadIdx.x == 0) table[0].pick = rows128;
+  }
 }
 
 // The same for 64-row query blocks, where two blocks with the very same list share their tiles.
@@ -2124,7 +2142,7 @@ __global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* ta
 constexpr int kPairRows = 64, kPairThreads = 256;
 // COUNT: also the tiles in all and of pairs, for k_sort_tail (a test in the kernel instead took calls of 80 short rows from 18.6 to 19.7 us)
 template <bool COUNT>
-__global__ void __launch_bounds__(kPairThreads) k_task_table_pairs(AttnParams p, Task* table, int* pick, int chunks) {
+__global__ void __launch_bounds__(kPairThreads) k_task_table_pairs(AttnParams p, Task* table, int chunks) {
   __shared__ int s_row[kPairRows], s_lo[kPairRows], s_len[kPairRows];      // (len -1: takes no part)
   __shared__ int s_mate[kPairRows];                 // list start of the candidate partner, -1: none
   __shared__ int s_mate_row[kPairRows], s_mate_pos[kPairRows], s_same[kPairRows];   // its row; its position here, -1: elsewhere
@@ -2141,7 +2159,7 @@ __global__ void __launch_bounds__(kPairThreads) k_task_table_pairs(AttnParams p,
   const bool live = tid < kPairRows && pos < p.m_b;
   if (tid == 0) { s_before = 0; s_prev = -1; s_next = p.m_b; s_n_full = 0; }
   if (live) tk = make_task(p, 64, h, pos);
-  const bool open = live && !tk.pad2 && tk.len > 0 && !p.no_pairing;
+  const bool open = live && !tk.pick && tk.len > 0 && !p.no_pairing;
   auto full_at = [&](int ps) {                      // the row at position ps if it selects everything by its length, else -1
     const int r = p.row_order ? p.row_order[hb + ps] : ps;
     return (r < 0 || r >= p.m_b || p.row_ptr[hb + r + 1] - p.row_ptr[hb + r] != p.n_b) ? -1 : r;
@@ -2222,15 +2240,12 @@ __global__ void __launch_bounds__(kPairThreads) k_task_table_pairs(AttnParams p,
     if (first) tk.row2 = s_mate_row[tid];
     else tk.n = kAbsorbed;
   }
-  tk.pad2 = 0;
+  tk.pick = 0;
   if (live) table[p.interleaved ? (long long)pos * p.heads + h : (long long)hb + pos] = tk;
-  if constexpr (!COUNT) return;
-  if (tid < kPairRows) {
+  if (COUNT && tid < kPairRows) {
     const int n = live ? max(tk.n, 0) : 0, all = __reduce_add_sync(0xffffffffu, n), paired = __reduce_add_sync(0xffffffffu, tk.row2 >= 0 ? n : 0);
-    if (lane == 0) { s_lo[warp] = all; s_len[warp] = paired; }
+    if (lane == 0 && live) *part_counts(p, h, pos) = make_int2(all, paired);
   }
-  __syncthreads();
-  if (tid == 0) { pick[2 + 2 * blockIdx.x] = s_lo[0] + s_lo[1]; pick[3 + 2 * blockIdx.x] = s_len[0] + s_len[1]; }
 }
 
 // ------------------------------------------------------------------ host side
@@ -2311,8 +2326,8 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   long long grid = p.total_tasks < sms ? p.total_tasks : sms;
   Task* table = reinterpret_cast<Task*>(reinterpret_cast<char*>(p.ws) + table_offset(p.total_tasks));
   p.table = table;
-  int* pick = nullptr;
   p.pick = nullptr;
+  bool pick = false;
   p.redo_pass = 0;
   p.wait_limit = kTimeoutCycles;
   p.drop_tile = 0;
@@ -2334,12 +2349,11 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
     // 140: 51.6 / 59.6, 249: 71.8 / 72.5, 280: 75.8 / 90.2 and 81.8 / 67.7, 324: 49.4 / 47.1, 331: 68.9 / 64.4, 373: 100 / 89,
     // 553: 144 / 111, 622: 155 / 132, 648: 72.6 / 67.7)
     const bool many = p.total_tasks > sms;            // (else all tasks start at once)
-    if (many && p.total_tasks * ((p.n_b + 1) / 2) >= kRows64Tiles * sms) pick = reinterpret_cast<int*>(table + p.total_tasks);
-    if (pick) k_task_table_pairs<true><<<(unsigned)((long long)p.heads * chunks), kPairThreads, 0, st>>>(p, table, pick, chunks);
-    else k_task_table_pairs<false><<<(unsigned)((long long)p.heads * chunks), kPairThreads, 0, st>>>(p, table, pick, chunks);
+    pick = many && p.total_tasks * ((p.n_b + 1) / 2) >= kRows64Tiles * sms;
+    (pick ? k_task_table_pairs<true> : k_task_table_pairs<false>)<<<(unsigned)((long long)p.heads * chunks), kPairThreads, 0, st>>>(p, table, chunks);
     if (many) {
       WAVEAL_CUDA_OK(cudaGetLastError());
-      WAVEAL_CUDA_OK(waveal::launch_chained(pick ? k_sort_tail<true> : k_sort_tail<false>, dim3(1), kTailTasks, 0, st, p, table, pick, p.heads * chunks, D, sms));
+      WAVEAL_CUDA_OK(waveal::launch_chained(pick ? k_sort_tail<true> : k_sort_tail<false>, dim3(1), kTailTasks, 0, st, p, table, D, sms));
       ++launches;
     }
   } else {
@@ -2357,8 +2371,8 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   p.redo_pass = 0;
   if constexpr (BLOCK == 64) {
     // k_sort_tail says which kernel is quicker; the other one leaves at once
-    p.pick = pick;
     if (pick) {
+      p.pick = &table->pick;
       WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd_rows64<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Geo64<D>::SMEM_BYTES));
       WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd_rows64<D>, dim3((unsigned)grid), kThreads64, Geo64<D>::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, p));
       ++launches;
@@ -2381,9 +2395,7 @@ extern "C" waveal_status waveal_bsattn_workspace_bytes(const waveal_attn_desc* d
   // 32 bytes of counters and flags, one (head, query block) pair per task for the redo list,
   // then the 32-byte task of every ticket
   const long long tasks = (long long)desc->heads * ((desc->seq_q + desc->block_q - 1) / desc->block_q);
-  // (64-row blocks: and two counts of every 64 positions of a head)
-  const long long parts = desc->block_q == 64 ? 8 + (long long)desc->heads * ((desc->seq_q + 64 * kPairRows - 1) / (64 * kPairRows)) * 8 : 0;
-  *bytes = (size_t)((table_offset(tasks) + 32 * tasks + parts + 255) / 256 * 256);
+  *bytes = (size_t)((table_offset(tasks) + 32 * tasks + 255) / 256 * 256);
   return WAVEAL_OK;
 }
 

@@ -147,3 +147,13 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(wb, "LIB_PATH", str(tmp_path / "nope.so"))
     with pytest.raises(RuntimeError, match="no CPU fallback"):
         wb.load()
+
+
+@pytest.mark.parametrize("block", [64, 128])
+@pytest.mark.parametrize("heads,seq_q", [(1, 64), (1, 20000), (8, 20480), (32, 98304), (40, 75600)])
+def test_attention_workspace_is_the_sum_of_its_listed_parts(lib, block, heads, seq_q):
+    d = wb.AttnDesc(heads=heads, seq_q=seq_q, seq_kv=seq_q, head_dim=128, block_q=block, block_kv=block)
+    for name in ("q_stride", "k_stride", "v_stride", "o_stride"):
+        getattr(d, name)[0], getattr(d, name)[1] = seq_q * 128, 128
+    tasks = heads * -(-seq_q // block)
+    assert wb.bsattn_workspace_bytes(d) == -(-(-(-(32 + 8 * tasks) // 32) * 32 + 32 * tasks) // 256) * 256
