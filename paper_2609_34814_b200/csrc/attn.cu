@@ -1425,6 +1425,10 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 constexpr long long kRows64Tiles = 320;              // tiles an SM that the lists of a call may have, from which this kernel is launched
 constexpr int kThreads64 = 704, kLoadWarps64 = 20;   // 22 warps: those of the kernel above and two more loaders
 
+// clk a tile of 128 keys in products of 128 rows, and in products of 64 of a block on its own, of a pair, and of a long pair that
+// starts with the call
+struct Pace { int rows128, lone, pair, first_pair; };
+
 template <int D>
 struct Geo64 {
   static constexpr int BQ = 64, BK = 128;            // a KV tile is 128 keys: two consecutive entries of the row's list
@@ -1455,6 +1459,11 @@ struct Geo64 {
   static_assert(SMEM_BYTES <= 232448, "shared memory of a CTA");
   // tensor memory: an S buffer of 64 columns per softmax group, then two sets of output accumulators (by task) for two blocks
   static constexpr uint32_t S_STRIDE = 64, O_COL = NG * 64, O_STRIDE = 64, TMEM_COLS = 512;
+  // As measured on the kernels as they are: to be measured again when the pace of either changes (dense heads; 8 heads of the LTX
+  // recipe without pairs; rows that are all in pairs; a pair of 350 or 750 tiles among the first rows, the others 10 to 30 tiles).
+  // Over 300 mixes of both (long rows none to a third, first, last or spread; none, half or all of the others in pairs; 1 to 16
+  // heads) the kernel picked takes 0.15 % longer than the quicker one on average, 7.6 % at most; the other one up to 20 % or 47 %.
+  static constexpr Pace PACE = D == 128 ? Pace{1327, 886, 1772, 1615} : Pace{1140, 735, 1372, 1372};
 };
 
 // One K or V tile of a task into its ring stage (called by a whole warp); see load_kv_tile.  done: the product that read the
@@ -2075,8 +2084,9 @@ __global__ void __launch_bounds__(kTailTasks) k_task_table(AttnParams p, int blo
   }
 }
 
-// 64-row blocks: what k_task_table_pairs<true> leaves k_sort_tail<true> for every 32 positions of a head, tiles in all and of pairs.  It
-// lies where the list of tasks to compute again (8 bytes a task) has its entry for the first of them: that list is empty until the
+// 64-row blocks: what k_task_table_pairs<true> leaves k_sort_tail<true> for every 32 positions of a head: [0] tiles in all and of pairs,
+// [1] tiles of the longest block on its own and of the longest pair (a single position has no room for it: its [0] says the same).  It
+// lies where the list of tasks to compute again (8 bytes a task) has its entries for those positions: that list is empty until the
 // first launch.
 __device__ __forceinline__ int head_parts(const AttnParams& p) { return (p.m_b + 31) / 32; }
 __device__ __forceinline__ int2* part_counts(const AttnParams& p, int h, int pos) {
@@ -2085,38 +2095,47 @@ __device__ __forceinline__ int2* part_counts(const AttnParams& p, int h, int pos
 
 // the same for a table that is there already (64-row blocks: pairs are formed first)
 template <bool PICK>
-__global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* table, int d, int sms) {
+__global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* table, Pace pace, int sms) {
   waveal::let_next_kernel_start();
   waveal::wait_for_previous_kernel();
   const long long t = p.first_tail + threadIdx.x;
   const bool live = t < p.total_tasks;
   Task tk{};
+  tk.row2 = -1;
   if (live) tk = table[t];
   int n = tk.n;
   bool rows128 = false;
   if constexpr (PICK) {
-    // which kernel: see k_bsattn_fwd_rows64.  Either takes as long as its share of the work an SM, or its longest task (of
-    // the last 1,024, all of a call where that matters)
-    __shared__ int tiles[4];                          // in all, of pairs, of the longest block on its own and pair
-    if (threadIdx.x < 4) tiles[threadIdx.x] = 0;
+    // Which kernel: see k_bsattn_fwd_rows64.  Either takes as long as its share of the work an SM, or its longest task.  In products
+    // of 64 rows a long pair that starts with the call runs faster than one that the last 1,024 tickets begin with (pace.first_pair;
+    // of those 1,024 alone, 2 heads of 700 rows with a long pair among the first took 365 us there instead of 310 in products of 128).
+    __shared__ int tiles[5];                          // in all, of pairs; of the longest block on its own, pair, and pair in the tail
+    if (threadIdx.x < 5) tiles[threadIdx.x] = 0;
     __syncthreads();
-    int all = 0, paired = 0;
+    int all = 0, paired = 0, lone_n = 0, pair_n = 0;
     const int per_head = head_parts(p);
     for (int i = threadIdx.x; i < p.heads * per_head; i += kTailTasks) {
-      const int2 c = *part_counts(p, i / per_head, i % per_head * 32);
+      const int pos = i % per_head * 32;
+      const int2* part = part_counts(p, i / per_head, pos);
+      const int2 c = part[0], most = pos + 1 < p.m_b ? part[1] : make_int2(c.x - c.y, c.y);
       all += c.x; paired += c.y;
+      lone_n = max(lone_n, most.x); pair_n = max(pair_n, most.y);
     }
     all = __reduce_add_sync(0xffffffffu, all);
     paired = __reduce_add_sync(0xffffffffu, paired);
-    const bool pair = live && tk.row2 >= 0;
-    const int lone_n = __reduce_max_sync(0xffffffffu, pair ? 0 : max(tk.n, 0)), pair_n = __reduce_max_sync(0xffffffffu, pair ? tk.n : 0);
-    if ((threadIdx.x & 31) == 0) { atomicAdd(&tiles[0], all); atomicAdd(&tiles[1], paired); atomicMax(&tiles[2], lone_n); atomicMax(&tiles[3], pair_n); }
+    lone_n = __reduce_max_sync(0xffffffffu, lone_n);
+    pair_n = __reduce_max_sync(0xffffffffu, pair_n);
+    const int tail_pair_n = __reduce_max_sync(0xffffffffu, tk.row2 >= 0 ? tk.n : 0);
+    if ((threadIdx.x & 31) == 0) {
+      atomicAdd(&tiles[0], all); atomicAdd(&tiles[1], paired);
+      atomicMax(&tiles[2], lone_n); atomicMax(&tiles[3], pair_n); atomicMax(&tiles[4], tail_pair_n);
+    }
     __syncthreads();
-    const long long c128 = d == 128 ? 1327 : 1140, c_lone = d == 128 ? 886 : 735, c_pair = d == 128 ? 1772 : 1372;
-    const long long t128 = max(c128 * tiles[0] / sms, c128 * max(tiles[2], tiles[3]));
-    const long long t64 = max((c_lone * (tiles[0] - tiles[1]) + c_pair * tiles[1]) / sms, max(c_lone * tiles[2], c_pair * tiles[3]));
+    const long long t128 = max(pace.rows128 * (long long)tiles[0] / sms, pace.rows128 * (long long)max(tiles[2], tiles[3]));
+    const long long t64 = max(max((pace.lone * (long long)(tiles[0] - tiles[1]) + pace.pair * (long long)tiles[1]) / sms, pace.lone * (long long)tiles[2]),
+                              max(pace.first_pair * (long long)tiles[3], pace.pair * (long long)tiles[4]));
     rows128 = t128 < t64;
-    if (pair && !rows128) n *= 2;                     // (a pair: two items a tile)
+    if (tk.row2 >= 0 && !rows128) n *= 2;                     // (a pair: two items a tile)
   }
   const int at = tail_place(n, live);
   if (live) table[p.first_tail + at] = tk;
@@ -2140,7 +2159,7 @@ __global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* ta
 // before the block's own (a thread each, so the block reads the row lengths of its head once).  One thread
 // per row that counted and compared alone took 488 us on 32 heads of 1536 rows, a tenth of them full.
 constexpr int kPairRows = 64, kPairThreads = 256;
-// COUNT: also the tiles in all and of pairs, for k_sort_tail (a test in the kernel instead took calls of 80 short rows from 18.6 to 19.7 us)
+// COUNT: also what k_sort_tail picks the kernel by (a test in the kernel instead took calls of 80 short rows from 18.6 to 19.7 us)
 template <bool COUNT>
 __global__ void __launch_bounds__(kPairThreads) k_task_table_pairs(AttnParams p, Task* table, int chunks) {
   __shared__ int s_row[kPairRows], s_lo[kPairRows], s_len[kPairRows];      // (len -1: takes no part)
@@ -2243,8 +2262,13 @@ __global__ void __launch_bounds__(kPairThreads) k_task_table_pairs(AttnParams p,
   tk.pick = 0;
   if (live) table[p.interleaved ? (long long)pos * p.heads + h : (long long)hb + pos] = tk;
   if (COUNT && tid < kPairRows) {
-    const int n = live ? max(tk.n, 0) : 0, all = __reduce_add_sync(0xffffffffu, n), paired = __reduce_add_sync(0xffffffffu, tk.row2 >= 0 ? n : 0);
-    if (lane == 0 && live) *part_counts(p, h, pos) = make_int2(all, paired);
+    const int n = live ? max(tk.n, 0) : 0, pair_n = live && tk.row2 >= 0 ? n : 0, lone_n = n - pair_n;
+    const int2 sum = make_int2(__reduce_add_sync(0xffffffffu, n), __reduce_add_sync(0xffffffffu, pair_n));
+    const int2 most = make_int2(__reduce_max_sync(0xffffffffu, lone_n), __reduce_max_sync(0xffffffffu, pair_n));
+    if (lane == 0 && live) {
+      part_counts(p, h, pos)[0] = sum;
+      if (pos + 1 < p.m_b) part_counts(p, h, pos)[1] = most;
+    }
   }
 }
 
@@ -2353,7 +2377,7 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
     (pick ? k_task_table_pairs<true> : k_task_table_pairs<false>)<<<(unsigned)((long long)p.heads * chunks), kPairThreads, 0, st>>>(p, table, chunks);
     if (many) {
       WAVEAL_CUDA_OK(cudaGetLastError());
-      WAVEAL_CUDA_OK(waveal::launch_chained(pick ? k_sort_tail<true> : k_sort_tail<false>, dim3(1), kTailTasks, 0, st, p, table, D, sms));
+      WAVEAL_CUDA_OK(waveal::launch_chained(pick ? k_sort_tail<true> : k_sort_tail<false>, dim3(1), kTailTasks, 0, st, p, table, Geo64<D>::PACE, sms));
       ++launches;
     }
   } else {

@@ -21,6 +21,11 @@ def _call(q, k, v, ptr, idx, T, order=None, flags=0, ws=None):
     return o, lse, ws.view(torch.int32), st.tolist()
 
 
+def _rows128(w, tasks):
+    """The choice that the call made on the device: products of 128 rows (1) or of 64 (0)."""
+    return w[(32 + 8 * tasks + 31) // 32 * 8 + 7].item()
+
+
 def _case(D, nb, cut, seed):
     """Rows of 0 to 45 blocks; every fifth row has its neighbour's list, every eleventh selects everything."""
     g = torch.Generator().manual_seed(seed)
@@ -89,6 +94,25 @@ def test_either_kernel_gives_the_same_bits(D, nb, full):
         ref = p @ v[0, sel].double()
         bound = 2.0 ** -8 * (p @ v[0, sel].double().abs()) + 2.0 ** -8 * ref.abs() + 1e-6      # as in the test above
         assert ((o[0, rows].double() - ref).abs() <= bound).all(), i
+
+
+# one pair of 350 tiles among blocks of 10 to 15: it outlasts the call in products of 64 rows, in front of the last 1,024 tickets too
+@pytest.mark.parametrize("D", [128, 64])
+@pytest.mark.parametrize("at", [0, 1376])
+def test_a_long_pair_decides_wherever_it_stands(D, at):
+    heads, nb = 2, 700
+    g = torch.Generator().manual_seed(at)
+    lists = [torch.arange(nb) if t in (at, at + 1) else torch.randperm(nb, generator=g)[:20 + t % 11].sort().values for t in range(heads * nb)]
+    ptr = torch.tensor([0] + [len(l) for l in lists]).cumsum(0).int().cuda()
+    gg = torch.Generator("cuda")
+    gg.manual_seed(at)
+    q, k, v = (torch.randn((heads, nb * 64, D), generator=gg, device="cuda").to(torch.bfloat16) for _ in range(3))
+    idx = torch.cat(lists).int().cuda()
+    o, lse, w, st = _call(q, k, v, ptr, idx, nb * 64)
+    alone, lse_alone, w_alone, st_alone = _call(q, k, v, ptr, idx, nb * 64, flags=wb.ATTN_NO_ROW_PAIRING)
+    assert st == [0] * 4 and st_alone == [0] * 4 and w[6] == 1 and w_alone[6] == 0
+    assert _rows128(w, heads * nb) == 1 and _rows128(w_alone, heads * nb) == 0
+    assert torch.equal(o, alone) and torch.equal(lse, lse_alone)
 
 
 # calls on either side of the number of tiles from which the choice of kernel is made on the device, and of as many blocks as SMs
