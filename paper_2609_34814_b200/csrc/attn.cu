@@ -2373,7 +2373,7 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
     // 140: 51.6 / 59.6, 249: 71.8 / 72.5, 280: 75.8 / 90.2 and 81.8 / 67.7, 324: 49.4 / 47.1, 331: 68.9 / 64.4, 373: 100 / 89,
     // 553: 144 / 111, 622: 155 / 132, 648: 72.6 / 67.7)
     const bool many = p.total_tasks > sms;            // (else all tasks start at once)
-    pick = many && p.total_tasks * ((p.n_b + 1) / 2) >= kRows64Tiles * sms;
+    pick = many && !(d->flags & WAVEAL_ATTN_ONLINE_MAX_ONLY) && p.total_tasks * ((p.n_b + 1) / 2) >= kRows64Tiles * sms;
     (pick ? k_task_table_pairs<true> : k_task_table_pairs<false>)<<<(unsigned)((long long)p.heads * chunks), kPairThreads, 0, st>>>(p, table, chunks);
     if (many) {
       WAVEAL_CUDA_OK(cudaGetLastError());

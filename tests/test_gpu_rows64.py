@@ -115,6 +115,21 @@ def test_a_long_pair_decides_wherever_it_stands(D, at):
     assert torch.equal(o, alone) and torch.equal(lse, lse_alone)
 
 
+# the single-launch variant has one kernel: nothing is chosen, and long pairs are not put in front of longer blocks
+@pytest.mark.parametrize("D", [128, 64])
+def test_the_single_launch_variant_chooses_nothing(D):
+    nb, heads = 320, 2
+    lists = [torch.arange(nb) if t % 8 < 2 else torch.arange(0, nb, 2) if t % 8 < 4 else torch.arange(t % 7, 250 + t % 7) for t in range(heads * nb)]
+    ptr = torch.tensor([0] + [len(l) for l in lists]).cumsum(0).int().cuda()
+    q, k, v = (torch.randn((heads, nb * 64, D), generator=torch.Generator("cuda").manual_seed(D), device="cuda").to(torch.bfloat16) for _ in range(3))
+    o, _, w, st = _call(q, k, v, ptr, torch.cat(lists).int().cuda(), nb * 64, flags=wb.ATTN_ONLINE_MAX_ONLY)
+    tasks = heads * nb
+    table = w[(32 + 8 * tasks + 31) // 32 * 8:][:8 * tasks].view(tasks, 8)
+    n = table[:, 3].tolist()                       # tiles of a ticket, longest first (absorbed ones last); 160 and 80 of the pairs
+    assert st == [0] * 4 and wb.last_launch_count() == 3 and w[6] == tasks // 4 and not table[:, 7].any()
+    assert n == sorted(n, reverse=True) and max(n) == 160
+
+
 # calls on either side of the number of tiles from which the choice of kernel is made on the device, and of as many blocks as SMs
 @pytest.mark.parametrize("D", [128, 64])
 @pytest.mark.parametrize("nb,heads", [(100, 9), (200, 4)])
