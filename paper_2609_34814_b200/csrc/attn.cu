@@ -1416,8 +1416,9 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 // Which kernel a call takes: two blocks that share their tiles (a pair) fill a product of 128 rows, which takes 1,327 clk a tile
 // (1,140 at head_dim 64) against their two items' 1,770 (1,370), a lone block's tile as long against its item's 886
 // (735): products of 64 rows are quicker until pairs have 47 % (64 %) of the tiles, or the longest pair outlasts an SM's share of the
-// work.  k_sort_tail, which has the counts, picks; the kernel not picked leaves at once (~3 us).  (8 heads of the LTX recipe, a quarter: 11.2 -> 9.3 ms; 2 dense heads of 512 rows, all: 892 us with the
-// one, 1,100 with the other.)  Calls of no more tasks than SMs last as long as their longest task and stay with products of 128
+// work.  k_sort_tail, which has the counts, picks; the kernel not picked leaves at once (with the counts 4 to 5 us where products of 128
+// rows run, 1 to 2 where the others do).  (8 heads of the LTX recipe, a quarter: 11.2 -> 9.3 ms; 2 dense heads of 512 rows, all: 892 us
+// with the one, 1,100 with the other.)  Calls of no more tasks than SMs last as long as their longest task and stay with products of 128
 // rows, and so do small ones (launch()).
 // Pairs: two blocks with the very same list are items 2 i and 2 i + 1 of tile i, each with an accumulator of its own.  Everything a row
 // sees is as it would be alone: the products in the same order, a reference from the same first 128 keys, and the same
@@ -1462,7 +1463,8 @@ struct Geo64 {
   // As measured on the kernels as they are: to be measured again when the pace of either changes (dense heads; 8 heads of the LTX
   // recipe without pairs; rows that are all in pairs; a pair of 350 or 750 tiles among the first rows, the others 10 to 30 tiles).
   // Over 300 mixes of both (long rows none to a third, first, last or spread; none, half or all of the others in pairs; 1 to 16
-  // heads) the kernel picked takes 0.15 % longer than the quicker one on average, 7.6 % at most; the other one up to 20 % or 47 %.
+  // heads) the kernel picked takes 0.15 % longer than the quicker one on average, 7.6 % at most
+  // (products of 64 rows always 20 %, of 128 always 47 % at most).
   static constexpr Pace PACE = D == 128 ? Pace{1327, 886, 1772, 1615} : Pace{1140, 735, 1372, 1372};
 };
 
@@ -1607,19 +1609,21 @@ k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   const long long t_start = clock64();
 
   // every role walks the same sequence of tasks and, inside a task, of items
-  if (warp == kProducerWarp) {
+  const bool mine = *p.pick == 0;
+  if (!mine) {
+    // (the other kernel's call)
+  } else if (warp == kProducerWarp) {
     // ============================================================== producer: tickets, Q, every second K tile
     if (lane == 0) { prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmV); prefetch_tmap(&tmK2); prefetch_tmap(&tmV2); }
     uint32_t task_it = 0, q_it = 0, q_armed = 0, q_parity = 0;
     TileLoader<G, true> k_tiles{0};
     int n_tiles = 0, n_pairs = 0;        // words 7 and 6 of the workspace
     bool ok = true;
-    const bool mine = *p.pick == 0;
     auto draw = [&](long long& t_out) -> Task {
       for (;;) {
         long long t = 0;
         if (lane == 0)                   // (volatile: another SM raises the flag while this kernel runs)
-          t = (!mine || *reinterpret_cast<volatile int*>(&p.ws[1]) != 0) ? p.total_tasks : (long long)(unsigned)atomicAdd(&p.ws[0], 1);
+          t = *reinterpret_cast<volatile int*>(&p.ws[1]) != 0 ? p.total_tasks : (long long)(unsigned)atomicAdd(&p.ws[0], 1);
         t = __shfl_sync(0xffffffffu, t, 0);
         t_out = t;
         Task tk{};
@@ -2016,7 +2020,7 @@ k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     tc_fence_after();
     tmem_dealloc(tmem_base, G::TMEM_COLS);
   }
-  if (tid == 0 && *p.pick == 0) {
+  if (tid == 0 && mine) {
     const long long dt = clock64() - t_start;
     atomicMax(&p.ws[4], (int)(dt > 0x7fffffffll ? 0x7fffffffll : dt));
   }
@@ -2109,9 +2113,10 @@ __global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* ta
     // Which kernel: see k_bsattn_fwd_rows64.  Either takes as long as its share of the work an SM, or its longest task.  In products
     // of 64 rows a long pair that starts with the call runs faster than one that the last 1,024 tickets begin with (pace.first_pair;
     // of those 1,024 alone, 2 heads of 700 rows with a long pair among the first took 365 us there instead of 310 in products of 128).
-    __shared__ int tiles[5];                          // in all, of pairs; of the longest block on its own, pair, and pair in the tail
-    if (threadIdx.x < 5) tiles[threadIdx.x] = 0;
-    __syncthreads();
+    // (This stands in front of every large call: sums by warp and floats instead of atomics and 64-bit division, and a kernel not picked
+    // that leaves from where it waited: 0.8 to 2 us less.)
+    __shared__ int sums[5][kTailTasks / 32];          // by warp: tiles in all, of pairs; of the longest block on its own, pair, and pair in the tail
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int all = 0, paired = 0, lone_n = 0, pair_n = 0;
     const int per_head = head_parts(p);
     for (int i = threadIdx.x; i < p.heads * per_head; i += kTailTasks) {
@@ -2126,14 +2131,17 @@ __global__ void __launch_bounds__(kTailTasks) k_sort_tail(AttnParams p, Task* ta
     lone_n = __reduce_max_sync(0xffffffffu, lone_n);
     pair_n = __reduce_max_sync(0xffffffffu, pair_n);
     const int tail_pair_n = __reduce_max_sync(0xffffffffu, tk.row2 >= 0 ? tk.n : 0);
-    if ((threadIdx.x & 31) == 0) {
-      atomicAdd(&tiles[0], all); atomicAdd(&tiles[1], paired);
-      atomicMax(&tiles[2], lone_n); atomicMax(&tiles[3], pair_n); atomicMax(&tiles[4], tail_pair_n);
+    if (lane == 0) {
+      sums[0][warp] = all; sums[1][warp] = paired;
+      sums[2][warp] = lone_n; sums[3][warp] = pair_n; sums[4][warp] = tail_pair_n;
     }
     __syncthreads();
-    const long long t128 = max(pace.rows128 * (long long)tiles[0] / sms, pace.rows128 * (long long)max(tiles[2], tiles[3]));
-    const long long t64 = max(max((pace.lone * (long long)(tiles[0] - tiles[1]) + pace.pair * (long long)tiles[1]) / sms, pace.lone * (long long)tiles[2]),
-                              max(pace.first_pair * (long long)tiles[3], pace.pair * (long long)tiles[4]));
+    const float share = 1.f / (float)sms;
+    const float total = (float)__reduce_add_sync(0xffffffffu, sums[0][lane]) * share, pairs = (float)__reduce_add_sync(0xffffffffu, sums[1][lane]) * share;
+    const float lone_most = (float)__reduce_max_sync(0xffffffffu, sums[2][lane]), pair_most = (float)__reduce_max_sync(0xffffffffu, sums[3][lane]);
+    const float tail_most = (float)__reduce_max_sync(0xffffffffu, sums[4][lane]);
+    const float t128 = pace.rows128 * fmaxf(total, fmaxf(lone_most, pair_most));
+    const float t64 = fmaxf(fmaxf(pace.lone * (total - pairs) + pace.pair * pairs, pace.lone * lone_most), fmaxf(pace.first_pair * pair_most, pace.pair * tail_most));
     rows128 = t128 < t64;
     if (tk.row2 >= 0 && !rows128) n *= 2;                     // (a pair: two items a tile)
   }
@@ -2368,10 +2376,17 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   int launches = 1;
   if (BLOCK == 64) {
     const int chunks = (p.m_b + kPairRows - 1) / kPairRows;
-    // (The kernel not picked is ~3 us more of launches, worth it from a few thousand cycles of work an SM on, of which the host knows
-    // only the most that a mask can select.  us a call with one kernel / the other, by that many tiles an SM: 17: 28.7 / 31.4,
-    // 140: 51.6 / 59.6, 249: 71.8 / 72.5, 280: 75.8 / 90.2 and 81.8 / 67.7, 324: 49.4 / 47.1, 331: 68.9 / 64.4, 373: 100 / 89,
-    // 553: 144 / 111, 622: 155 / 132, 648: 72.6 / 67.7)
+    // The choice costs a launch and its counts, of which the host knows only the most that a mask can select.  us a call with products of
+    // 128 rows alone / with the choice, lists of 3 / 12 / 40 % of the blocks, none in pairs, and of all blocks (all in pairs: the choice falls
+    // on products of 128), by the tiles an SM that the lists may have, head_dim 128:
+    //    68 (2 heads of 100 rows): 24.7 / 24.7   30.9 / 30.9   50.9 / 45.6    62.5 / 67.7
+    //   135 (1 head of 200):       26.7 / 26.8   39.1 / 37.0   78.9 / 65.8   102.6 / 107.5
+    //   219 (2 heads of 180):      30.9 / 30.9   49.5 / 44.5   101.7 / 83.5  160.2 / 165.6
+    //   304 (1 head of 300):       35.0 / 32.9   62.2 / 53.7   150.1 / 114.8 253.1 / 258.0
+    // (head_dim 64: 56.8 -> 48.5 at 132 and 40 %, 102.6 -> 80.1 at 298; all in pairs + 4.5 .. 5).  The line lies where the 5 us are 2 to 4 %
+    // of a dense call; below it a call of lone blocks gives away up to a quarter.  From the line on the sparsest lists repay the choice
+    // (3 heads of 180 rows, 328: rows of 2 blocks 30.8 / 30.9, of 6 37.0 / 36.4, of 12 46.4 / 43.0; head_dim 64 28.6 / 29.8, 32.9 / 32.9, 41.0 / 39.0),
+    // short pairs do not (8 heads of 200 rows of 10 blocks, all in pairs, head_dim 64: 57.0 / 61.3).
     const bool many = p.total_tasks > sms;            // (else all tasks start at once)
     pick = many && !(d->flags & WAVEAL_ATTN_ONLINE_MAX_ONLY) && p.total_tasks * ((p.n_b + 1) / 2) >= kRows64Tiles * sms;
     (pick ? k_task_table_pairs<true> : k_task_table_pairs<false>)<<<(unsigned)((long long)p.heads * chunks), kPairThreads, 0, st>>>(p, table, chunks);
