@@ -392,6 +392,7 @@ __host__ __device__ inline void fill_tiles(Task& tk, int len, int block, int las
   }
 }
 
+// (a kernel's parameters travel with every launch: 8 bytes more than these 160 and the tensor maps took the smallest step 0.5 us of host time)
 struct AttnParams {
   __nv_bfloat16* O;
   float* lse;
@@ -401,8 +402,8 @@ struct AttnParams {
   int* ws;            // [0] ticket counter, [1] abort flag, [2] number of tasks to redo, [3] ticket counter of
                       // the redo pass, [8 + 2i], [9 + 2i] = (head, query block) of redo entry i
   int redo_pass;      // 0: all tasks by ticket; 1: only the tasks the first pass listed
+  int choose;         // first launch of large calls of 64-row blocks: `pick` of the table's first entry says whose they are
   const Task* table;         // task of every ticket of the first pass (k_task_table)
-  const int* pick;           // large calls of 64-row blocks: `pick` of the table's first entry, else null
   int direct;         // CTAs that take the ticket of their own number before the table is there (0: none, else the grid)
   long long first_tail;      // tickets before this one are in the caller's order, the rest longest first
   int* dev_status;
@@ -414,6 +415,7 @@ struct AttnParams {
   int no_pairing;         // 64-row blocks: never put two blocks with identical lists into one tile
   float sl2;          // scale * log2(e)
 };
+static_assert(sizeof(AttnParams) == 160, "parameters of the attention kernels");
 
 
 // Task of every ticket (head-major or position-major over the planned order), so that the
@@ -655,9 +657,9 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   // second pass with nothing listed (or after an abort): leave before anything is set up
   if (p.redo_pass && (p.ws[2] == 0 || p.ws[1] != 0)) return;
   // a call that k_bsattn_fwd_rows64 has done
-  if (MOD4 && p.pick) {
+  if (MOD4 && p.choose) {
     waveal::wait_for_previous_kernel();
-    if (*p.pick == 0 || p.ws[1] != 0) return;
+    if (p.table->pick == 0 || p.ws[1] != 0) return;
   }
 
   const uint32_t bar0 = sbase + G::OFF_BAR;
@@ -1609,7 +1611,7 @@ k_bsattn_fwd_rows64(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
   const long long t_start = clock64();
 
   // every role walks the same sequence of tasks and, inside a task, of items
-  const bool mine = *p.pick == 0;
+  const bool mine = p.table->pick == 0;
   if (!mine) {
     // (the other kernel's call)
   } else if (warp == kProducerWarp) {
@@ -2358,7 +2360,6 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   long long grid = p.total_tasks < sms ? p.total_tasks : sms;
   Task* table = reinterpret_cast<Task*>(reinterpret_cast<char*>(p.ws) + table_offset(p.total_tasks));
   p.table = table;
-  p.pick = nullptr;
   bool pick = false;
   p.redo_pass = 0;
   p.wait_limit = kTimeoutCycles;
@@ -2411,7 +2412,7 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
   if constexpr (BLOCK == 64) {
     // k_sort_tail says which kernel is quicker; the other one leaves at once
     if (pick) {
-      p.pick = &table->pick;
+      p.choose = 1;
       WAVEAL_CUDA_OK(cudaFuncSetAttribute(k_bsattn_fwd_rows64<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, Geo64<D>::SMEM_BYTES));
       WAVEAL_CUDA_OK(waveal::launch_chained(k_bsattn_fwd_rows64<D>, dim3((unsigned)grid), kThreads64, Geo64<D>::SMEM_BYTES, st, tq, tk, tv, tk2, tv2, p));
       ++launches;
