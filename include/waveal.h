@@ -179,7 +179,8 @@ size_t waveal_noalloc_max_rows(void);
  * results, lists the tasks where a sum reached 2^60 or a result is not finite and computes those again, with the max of
  * every block, in a second launch on the same stream.  Results agree to rounding; the flag exists for comparison runs.
  * Rows whose scores rise by more than about 41 nats (2^60) after their first 128 keys are computed twice: a call in which
- * all rows do, once, takes 2.1 times as long (64-row blocks, 320 rows of 21 tiles), with the flag 1.2 times. */
+ * all rows do, once, takes 2.3 to 2.4 times as long (64-row blocks, 4 heads of 320 rows of 21 tiles), with the flag 1.4 to 1.6
+ * times. */
 #define WAVEAL_ATTN_ONLINE_MAX_ONLY 1
 /* Self-test of the kernel's failure handling, never set in production: the loader leaves out
  * the first K tile of the first task and every bounded wait gives up after about 2 ms instead

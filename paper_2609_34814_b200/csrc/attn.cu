@@ -1418,7 +1418,7 @@ k_bsattn_fwd(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 // Which kernel a call takes: two blocks that share their tiles (a pair) fill a product of 128 rows, which takes 1,327 clk a tile
 // (1,140 at head_dim 64) against their two items' 1,770 (1,370), a lone block's tile as long against its item's 886
 // (735): products of 64 rows are quicker until pairs have 47 % (64 %) of the tiles, or the longest pair outlasts an SM's share of the
-// work.  k_sort_tail, which has the counts, picks; the kernel not picked leaves at once (with the counts 4 to 5 us where products of 128
+// work.  k_sort_tail, which has the counts, picks; the kernel not picked leaves at once (with the counts 4 to 6 us where products of 128
 // rows run, 1 to 2 where the others do).  (8 heads of the LTX recipe, a quarter: 11.2 -> 9.3 ms; 2 dense heads of 512 rows, all: 892 us
 // with the one, 1,100 with the other.)  Calls of no more tasks than SMs last as long as their longest task and stay with products of 128
 // rows, and so do small ones (launch()).
@@ -2387,7 +2387,7 @@ waveal_status launch(const waveal_attn_desc* d, const void* Q, const void* K, co
     // (head_dim 64: 56.8 -> 48.5 at 132 and 40 %, 102.6 -> 80.1 at 298; all in pairs + 4.5 .. 5).  The line lies where the 5 us are 2 to 4 %
     // of a dense call; below it a call of lone blocks gives away up to a quarter.  From the line on the sparsest lists repay the choice
     // (3 heads of 180 rows, 328: rows of 2 blocks 30.8 / 30.9, of 6 37.0 / 36.4, of 12 46.4 / 43.0; head_dim 64 28.6 / 29.8, 32.9 / 32.9, 41.0 / 39.0),
-    // short pairs do not (8 heads of 200 rows of 10 blocks, all in pairs, head_dim 64: 57.0 / 61.3).
+    // short pairs do not (8 heads of 200 rows of 10 blocks, all in pairs, head_dim 64: 56.9 / 60.7).
     const bool many = p.total_tasks > sms;            // (else all tasks start at once)
     pick = many && !(d->flags & WAVEAL_ATTN_ONLINE_MAX_ONLY) && p.total_tasks * ((p.n_b + 1) / 2) >= kRows64Tiles * sms;
     (pick ? k_task_table_pairs<true> : k_task_table_pairs<false>)<<<(unsigned)((long long)p.heads * chunks), kPairThreads, 0, st>>>(p, table, chunks);
